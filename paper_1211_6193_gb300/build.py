@@ -31,7 +31,7 @@ def _nvcc() -> str:
 
 def _inputs():
     files = [os.path.join(CSRC, s) for s in SOURCES]
-    files += [os.path.join(CSRC, h) for h in ("sr_internal.h", "host_prep.h")]
+    files += [os.path.join(CSRC, h) for h in ("sr_internal.h", "host_prep.h", "solo_loop.cuh")]
     files += [os.path.join(INCLUDE, "simtcheck.h"), __file__]
     return files
 

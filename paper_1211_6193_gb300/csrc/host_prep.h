@@ -3,6 +3,7 @@
 // of a kernel's per-block access log.  Internal; not part of the C ABI.
 #pragma once
 #include <algorithm>
+#include <cstdint>
 #include <cstdio>
 #include <vector>
 #include <cuda_runtime.h>
@@ -118,6 +119,173 @@ inline KernelBound bound_kernel(const sr_instr* code, uint32_t ncode, uint32_t e
   return kb;
 }
 
+// Words of a launch's shared array that its accesses can touch: 1 + the highest in-bounds
+// address of any LDS, STS or ATOMS, from intervals of the registers' values over the kernel's
+// control-flow graph (thread and block indices, parameters and immediates have known ranges,
+// loaded values none; a register still changing after a few visits of a loop is taken as
+// unknown).  At most shmem_words, which it is when an address is unknown.
+struct RangeScratch {
+  struct State {
+    int32_t lo[16], hi[16];
+    uint32_t visits;             // 0: not reached
+  };
+  std::vector<int32_t> leader;   // per pc: index of its state, -1 inside a straight line
+  std::vector<State> states;
+  std::vector<uint8_t> queued;
+};
+inline uint32_t shared_reach(const sr_instr* code, uint32_t ncode, uint32_t entry, const sr_launch& L, RangeScratch& w) {
+  const uint32_t shw = L.shmem_words;
+  if (!shw) return 0;
+  using State = RangeScratch::State;
+  // leaders: the entry, branch targets and what follows a branch
+  w.leader.assign(ncode + 1, -1);
+  w.states.clear();
+  auto lead = [&](uint32_t pc) {
+    if (pc < ncode && w.leader[pc] < 0) {
+      w.leader[pc] = (int32_t)w.states.size();
+      w.states.push_back(State{});
+    }
+  };
+  lead(entry);
+  for (uint32_t pc = 0; pc < ncode; ++pc) {
+    const uint32_t b = code[pc].op_d_a_b & 0x7Fu;
+    if (b == SR_OP_BRA || b == SR_OP_BRZ || b == SR_OP_BRNZ) {
+      lead((uint32_t)code[pc].imm);
+      lead(pc + 1);
+    }
+  }
+  w.queued.assign(ncode + 1, 0);
+  uint32_t reach = 0, next = ncode;              // next: the lowest queued leader
+  auto flow = [&](const State& s, uint32_t pc) { // join s into the leader at pc
+    if (pc >= ncode) return;
+    State& t = w.states[(size_t)w.leader[pc]];
+    bool changed = t.visits == 0;
+    for (uint32_t r = 0; r < 16; ++r) {
+      const int32_t lo = t.visits ? std::min(t.lo[r], s.lo[r]) : s.lo[r];
+      const int32_t hi = t.visits ? std::max(t.hi[r], s.hi[r]) : s.hi[r];
+      if (t.visits && (lo != t.lo[r] || hi != t.hi[r])) {
+        changed = true;
+        if (t.visits > 4) {                      // still changing: unknown
+          t.lo[r] = INT32_MIN;
+          t.hi[r] = INT32_MAX;
+          continue;
+        }
+      }
+      t.lo[r] = lo;
+      t.hi[r] = hi;
+    }
+    if (changed) {
+      ++t.visits;
+      w.queued[pc] = 1;
+      next = std::min(next, pc);
+    }
+  };
+  State s{};
+  for (uint32_t q = 0; q < 4 && q < L.nparams; ++q) s.lo[q] = s.hi[q] = L.params[q];
+  flow(s, entry);
+  const int64_t first = L.block_begin, blocks = L.block_count ? L.block_count : L.grid;
+  while (next < ncode) {
+    uint32_t pc = next;
+    w.queued[pc] = 0;
+    s = w.states[(size_t)w.leader[pc]];
+    next = ncode;
+    for (uint32_t i = pc + 1; i < ncode; ++i)
+      if (w.queued[i]) {
+        next = i;
+        break;
+      }
+    for (;;) {                                   // to the end of the straight line
+      const uint32_t word = code[pc].op_d_a_b, op = word & 0xFFu, b = op & 0x7Fu;
+      const uint32_t d = (word >> 8) & 0xFFu, ra = (word >> 16) & 0xFFu, rb = (word >> 24) & 0xFFu;
+      const int64_t imm = code[pc].imm;
+      const bool za = ra == SR_RZ || ra > 15, zb = rb == SR_RZ || rb > 15;
+      const int64_t al = za ? 0 : s.lo[ra], ah = za ? 0 : s.hi[ra];
+      int64_t bl = zb ? 0 : s.lo[rb], bh = zb ? 0 : s.hi[rb];
+      if (op & SR_BIMM) bl = bh = imm;
+      int64_t lo = INT32_MIN, hi = INT32_MAX;    // the result's interval (unknown)
+      switch (b) {
+        case SR_OP_MOV: lo = bl; hi = bh; break;
+        case SR_OP_ADD: lo = al + bl; hi = ah + bh; break;
+        case SR_OP_SUB: lo = al - bh; hi = ah - bl; break;
+        case SR_OP_MUL: {
+          const int64_t x[4] = {al * bl, al * bh, ah * bl, ah * bh};
+          lo = *std::min_element(x, x + 4);
+          hi = *std::max_element(x, x + 4);
+          break;
+        }
+        case SR_OP_DIV:
+          if (bl == bh && bl > 0) { lo = al / bl; hi = ah / bl; }
+          break;
+        case SR_OP_REM:
+          if (bl == bh && bl > 0) {
+            lo = al < 0 ? -(bl - 1) : 0;
+            hi = ah > 0 ? std::min(ah, bl - 1) : 0;
+          }
+          break;
+        case SR_OP_AND:
+          if (bl >= 0 || al >= 0) {
+            lo = 0;
+            hi = bl < 0 ? ah : al < 0 ? bh : std::min(ah, bh);
+          }
+          break;
+        case SR_OP_OR:
+        case SR_OP_XOR:
+          if (al >= 0 && bl >= 0) {
+            int64_t m = 1;
+            while (m <= ah || m <= bh) m <<= 1;
+            lo = 0;
+            hi = m - 1;
+          }
+          break;
+        case SR_OP_SHL:
+          if (bl == bh) { lo = al * ((int64_t)1 << (bl & 31)); hi = ah * ((int64_t)1 << (bl & 31)); }
+          break;
+        case SR_OP_SHR:
+          if (bl == bh) { lo = al >> (bl & 31); hi = ah >> (bl & 31); }
+          break;
+        case SR_OP_MIN: lo = std::min(al, bl); hi = std::min(ah, bh); break;
+        case SR_OP_MAX: lo = std::max(al, bl); hi = std::max(ah, bh); break;
+        case SR_OP_SLT: case SR_OP_SLE: case SR_OP_SEQ: case SR_OP_SNE: case SR_OP_BARAND: case SR_OP_BAROR:
+          lo = 0; hi = 1;
+          break;
+        case SR_OP_BARPOPC: lo = 0; hi = L.block_dim; break;
+        case SR_OP_S2R:
+          if (imm == SR_SREG_TID) { lo = 0; hi = (int64_t)L.block_dim - 1; }
+          else if (imm == SR_SREG_BID) { lo = first; hi = first + blocks - 1; }
+          else if (imm == SR_SREG_BDIM) lo = hi = L.block_dim;
+          else if (imm == SR_SREG_GDIM) lo = hi = L.grid;
+          else lo = hi = 32;
+          break;
+        case SR_OP_LDS: case SR_OP_STS: case SR_OP_ATOMS: {
+          const int64_t l = al + imm, h = ah + imm;
+          if (l < INT32_MIN || h > INT32_MAX) reach = shw;
+          else if (h >= 0 && l < (int64_t)shw) reach = std::max(reach, (uint32_t)std::min<int64_t>(h + 1, shw));
+          break;
+        }
+        default: break;
+      }
+      if (op_writes_d(b) && d < 16) {
+        const bool fits = lo >= INT32_MIN && hi <= INT32_MAX;
+        s.lo[d] = fits ? (int32_t)lo : INT32_MIN;
+        s.hi[d] = fits ? (int32_t)hi : INT32_MAX;
+      }
+      if (reach == shw || b == SR_OP_EXIT) break;
+      if (b == SR_OP_BRA || b == SR_OP_BRZ || b == SR_OP_BRNZ) {
+        flow(s, (uint32_t)code[pc].imm);
+        if (b != SR_OP_BRA) flow(s, pc + 1);
+        break;
+      }
+      if (++pc >= ncode) break;
+      if (w.leader[pc] >= 0) {
+        flow(s, pc);
+        break;
+      }
+    }
+    if (reach == shw) break;
+  }
+  return reach;
+}
+
 inline int validate(const sr_program* p, char* msg, size_t len) {
   auto bad = [&](const char* fmt, uint32_t x, uint32_t y) {
     if (msg && len) snprintf(msg, len, fmt, x, y);
@@ -187,28 +355,146 @@ inline RegMap map_registers(const sr_program& P) {
 // that are RZ or absent become kNoDest
 inline uint2 pack(const sr_instr& in, const RegMap& m) {
   const uint32_t w = in.op_d_a_b, op = w & 0xFFu, b = op & 0x7Fu;
-  uint32_t d = (w >> 8) & 0xFFu, ra = (w >> 16) & 0xFFu, rb = (w >> 24) & 0xFFu;
+  const bool bimm = (op & SR_BIMM) != 0;
+  uint32_t d = (w >> 8) & 0xFFu, ra = (w >> 16) & 0xFFu, rb = (w >> 24) & 0xFFu, imm = (uint32_t)in.imm, form;
   const uint32_t zrow = m.nrows - 1;
   d = (op_writes_d(b) && d != SR_RZ) ? m.row[d] : sr::kNoDest;
   ra = (op_reads_a(b) && ra != SR_RZ) ? m.row[ra] : zrow;
   rb = (op_reads_b(op) && rb != SR_RZ) ? m.row[rb] : zrow;
-  return make_uint2(sr::pk_make(b, (op & SR_BIMM) ? 1u : 0u, d, ra, rb, 0), (uint32_t)in.imm);
+  auto of = [&](uint32_t f) { return bimm ? f : f + 1u; };
+  switch (b) {
+    case SR_OP_MOV:                              // (of a register: a plus the zero row)
+      form = bimm ? sr::F_MOVI : sr::F_MOVR;
+      ra = bimm ? zrow : rb;
+      rb = zrow;
+      break;
+    case SR_OP_ADD: form = bimm ? sr::F_ADDI : sr::F_ADDR; break;
+    case SR_OP_SUB:
+      form = bimm ? sr::F_ADDI : sr::F_SUBR;
+      if (bimm) imm = 0u - imm;
+      break;
+    case SR_OP_MUL: form = bimm ? sr::F_MULI : sr::F_MULR; break;
+    case SR_OP_SHL:
+      form = bimm ? sr::F_MULI : sr::F_SHL + 1u;
+      if (bimm) imm = 1u << (imm & 31u);
+      break;
+    case SR_OP_AND: form = of(sr::F_AND); break;
+    case SR_OP_OR: form = of(sr::F_OR); break;
+    case SR_OP_XOR: form = of(sr::F_XOR); break;
+    case SR_OP_SHR: form = of(sr::F_SHR); break;
+    case SR_OP_MIN: form = of(sr::F_MIN); break;
+    case SR_OP_MAX: form = of(sr::F_MAX); break;
+    case SR_OP_SLT: form = of(sr::F_SLT); break;
+    case SR_OP_SLE: form = of(sr::F_SLE); break;
+    case SR_OP_SEQ: form = of(sr::F_SEQ); break;
+    case SR_OP_SNE: form = of(sr::F_SNE); break;
+    case SR_OP_DIV: form = bimm ? sr::F_DIVI : sr::F_DIVR; break;
+    case SR_OP_REM: form = bimm ? sr::F_REMI : sr::F_REMR; break;
+    case SR_OP_S2R: form = sr::F_S2R; break;
+    case SR_OP_LDG: form = sr::F_LDG; break;
+    case SR_OP_STG: form = sr::F_STG; break;
+    case SR_OP_LDS: form = sr::F_LDS; break;
+    case SR_OP_STS: form = sr::F_STS; break;
+    case SR_OP_ATOMS: form = sr::F_ATOMS; break;
+    case SR_OP_BRA: form = sr::F_BRA; break;
+    case SR_OP_BRZ: form = sr::F_BRZ; break;
+    case SR_OP_BRNZ: form = sr::F_BRNZ; break;
+    case SR_OP_BAR: form = sr::F_BAR; break;
+    case SR_OP_BARAND: form = sr::F_BARAND; break;
+    case SR_OP_BAROR: form = sr::F_BAROR; break;
+    case SR_OP_BARPOPC: form = sr::F_BARPOPC; break;
+    default: form = sr::F_EXIT; break;
+  }
+  return make_uint2(sr::pk_make(form, d, ra, rb), imm);
 }
 
 // The EXIT sentinel after a program's last instruction (running past the end exits).
 inline uint2 exit_sentinel(const RegMap& m) {
-  return make_uint2(sr::pk_make(SR_OP_EXIT, 0, sr::kNoDest, m.nrows - 1, m.nrows - 1, 0), 0);
+  return make_uint2(sr::pk_make(sr::F_EXIT, sr::kNoDest, m.nrows - 1, m.nrows - 1), 0);
 }
 
-// Fill in the run lengths of n packed instructions (straight-line successors only: a run
-// never contains a branch, so it is valid from any entry pc).
-inline void set_run_lengths(uint2* code, uint32_t n) {
-  uint32_t next = 0;
+// Marks, chains and run lengths (sr_internal.h) of n packed instructions; run: one byte each;
+// target[pc]: a branch or an entry may lead there.  A run holds straight-line successors only and
+// no branch, so its length is right from any entry pc.  The interpreter ignores the operand mark of
+// the first instruction it executes of a run and the result mark of the last one, so the marks
+// hold wherever a run is entered or cut: a value is kept back only while the instructions up to
+// its overwriting follow in the same straight line.  Runs are cut between chains, and nothing
+// leads into a chain's middle, so no thread ever stands there (but for one whose block is out of
+// rounds, and stops).
+inline void set_runs(uint2* code, uint8_t* run, uint32_t n, const uint8_t* target) {
+  auto runs = [&](uint32_t pc) { return sr::pk_form(code[pc].x) < sr::F_LDS; };
+  uint32_t live = 0;                             // rows read later, or alive past the run
   for (uint32_t pc = n; pc-- > 0;) {
-    const uint32_t run = sr::pk_plain_alu(sr::pk_op(code[pc].x)) ? std::min(sr::kRunMax, 1 + next) : 0u;
-    code[pc].x = (code[pc].x & ((1u << 22) - 1)) | run << 22;
-    next = run;
+    if (!runs(pc)) continue;
+    uint32_t x = code[pc].x;
+    const uint32_t form = sr::pk_form(x), d = sr::pk_d(x);
+    uint32_t a = sr::pk_a(x), b = sr::pk_b(x);
+    if (pc + 1 >= n || !runs(pc + 1)) live = ~0u;   // (the last of its run)
+    if (d != sr::kNoDest) {
+      if (!((live >> d) & 1u)) x |= sr::kDeadD;
+      live &= ~(1u << d);
+    }
+    // the previous instruction's result as operand a, swapped there where the operation allows
+    const uint32_t before = pc && runs(pc - 1) ? sr::pk_d(code[pc - 1].x) : sr::kNoDest;
+    const bool commutes = form == sr::F_ADDR || form == sr::F_MULR || form == sr::F_AND + 1u || form == sr::F_OR + 1u ||
+                          form == sr::F_XOR + 1u || form == sr::F_MIN + 1u || form == sr::F_MAX + 1u ||
+                          form == sr::F_SEQ + 1u || form == sr::F_SNE + 1u;
+    if (commutes && b == before && a != before) std::swap(a, b);
+    if (form == sr::F_MOVI || (a == before && before != sr::kNoDest))
+      x |= sr::kFwdA;                            // (MOVI: no operand a to load)
+    else
+      live |= 1u << a;
+    if (!sr::pk_imm(form)) live |= 1u << b;
+    if (form <= sr::F_MULI) b = 1;               // (a chain of one)
+    code[pc].x = (x & 0xFFFFu) | a << 16 | b << 24;
   }
+  for (uint32_t pc = 0; pc < n;) {               // chains
+    uint32_t len = 1;
+    if (sr::pk_form(code[pc].x) <= sr::F_MULI) {
+      uint32_t last = code[pc].x;
+      while (len < sr::kRunMax && pc + len < n && !target[pc + len] && (last & sr::kDeadD)) {
+        uint2& e = code[pc + len];
+        if (sr::pk_form(e.x) > sr::F_MULI || !(e.x & sr::kFwdA)) break;
+        last = e.x;
+        const uint32_t form = sr::pk_form(e.x);
+        e = form == sr::F_MULI ? make_uint2(e.y, 0u) : make_uint2(form, e.y);   // (MOVI 0, ADDI 1)
+        ++len;
+      }
+      code[pc].x = (code[pc].x & ~(0xFF000000u | 0xFF00u | sr::kDeadD)) | (last & (0xFF00u | sr::kDeadD)) | len << 24;
+    }
+    run[pc] = (uint8_t)len;
+    for (uint32_t i = 1; i < len; ++i) run[pc + i] = 0;
+    pc += len;
+  }
+  // from the lengths of single instructions and chains, those of runs (never past kRunMax)
+  uint32_t next = 0;                             // the run length after this place
+  for (uint32_t pc = n; pc-- > 0;) {
+    if (!run[pc]) continue;                      // (inside a chain)
+    const uint32_t len = run[pc];
+    if (!runs(pc)) {
+      run[pc] = 0;
+      next = 0;
+      continue;
+    }
+    next = len + next <= sr::kRunMax ? len + next : len;
+    run[pc] = (uint8_t)next;
+  }
+}
+
+// A program as it is staged: out holds packed_words(ncode) pairs.
+inline uint32_t packed_words(uint32_t ncode) { return sr::ir_smem_bytes(ncode) / 8u; }
+inline void pack_program(const sr_program& P, const RegMap& m, uint2* out) {
+  const uint32_t n = P.ncode + 1;
+  uint8_t target[SR_MAX_CODE + 1] = {};
+  for (uint32_t pc = 0; pc < P.ncode; ++pc) {
+    out[pc] = pack(P.code[pc], m);
+    const uint32_t b = P.code[pc].op_d_a_b & 0x7Fu;
+    if (b == SR_OP_BRA || b == SR_OP_BRZ || b == SR_OP_BRNZ) target[(uint32_t)P.code[pc].imm] = 1;
+  }
+  for (uint32_t k = 0; k < P.nkernels; ++k) target[P.kernel_entry[k]] = 1;
+  for (uint32_t i = P.ncode; i < packed_words(P.ncode); ++i) out[i] = make_uint2(0u, 0u);
+  for (uint32_t i = P.ncode; i < sr::ir_code_bytes(P.ncode) / 8u; ++i) out[i] = exit_sentinel(m);
+  set_runs(out, reinterpret_cast<uint8_t*>(out) + sr::ir_code_bytes(P.ncode), n, target);
 }
 
 inline uint32_t key_bits_for(uint32_t shw) {

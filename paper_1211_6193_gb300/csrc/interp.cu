@@ -1,4 +1,4 @@
-// interp.cu - the SIMT interpreter: one real warp per simulated warp.
+// interp.cu - the SIMT interpreter: one real warp per 1, 2 or 4 simulated warps.
 //
 // What it computes (Hathhorn et al., SSV 2012): every thread of every block runs the
 // kernel (Sec. 3 "Threads and memory"), blocks own a dynamic shared array (same
@@ -8,12 +8,20 @@
 // check of check.cu.  At each barrier the block's waiting threads are examined for
 // divergence and deadlock (Sec. 3.1, last paragraph).
 //
-// GPU design.  A simulated block of B threads runs on ceil(B/32) real warps; simulated
-// registers (row-major [reg][tid]) and the simulated shared array live in shared
-// memory, the program's code is staged into shared memory with a TMA bulk copy.  The
-// canonical schedule is round-lockstep across the block, but warps are NOT barrier-
+// GPU design.  A block's simulated warps are agents; a real warp runs V of them (block_vec), slot
+// j of lane l being thread 32 (V w + j) + l, and nearly always executes one instruction for all
+// of them at once: what bounds the interpreter is the latency and the issue slots of decoding
+// and dispatch, and these are then paid once for V simulated warps.  A lane's V values of a
+// register lie side by side (one 16-byte shared access for V = 4).  Registers, the simulated
+// shared array and the program's code (staged by a TMA bulk copy) live in shared memory.
+// Small blocks take a smaller V: a block keeps two real warps from 64 threads on, so that
+// latencies overlap.  Instructions run in solo_loop (solo_loop.cuh); what it does not take -
+// agents of a warp at different pcs, colliding or out-of-bounds addresses, barriers with
+// something to report - runs in the general steps of run_block.
+//
+// The canonical schedule is round-lockstep across the block, but warps are NOT barrier-
 // synchronised every round: each warp counts its own rounds (within a barrier interval
-// a warp executes exactly one instruction per round while it has runnable lanes) and
+// an agent executes exactly one instruction per round while it has runnable threads) and
 // publishes a logical clock 4*round + stage in shared memory.  Only memory
 // instructions wait, and only for what the round semantics needs:
 //   stage 0 (loads)   : every other warp has finished all earlier rounds;
@@ -22,11 +30,20 @@
 //                       (highest tid wins; within a warp via __match_any_sync);
 //   stage 2 (atomics) : every other warp has done its stores of this round.
 // ALU and branch instructions never wait, so warps drift freely between memory
-// operations.  A warp whose lanes all wait at a barrier or exited publishes +inf; when
-// all warps of the block have parked, warp 0 resolves the barrier.  Every wait is
-// bounded (spin_limit) and reports SR_ST_INTERNAL instead of hanging.
+// operations.  A clock carries the parity of its barrier interval in bit 31, and a warp whose
+// threads all wait at a barrier or exited publishes the highest clock of its parity; then every
+// warp reads all warps' park entries behind one CTA barrier, and if the release is plain all go
+// on; otherwise warp 0 resolves it and a second CTA barrier follows.  Every wait is bounded
+// (spin_limit) and reports SR_ST_INTERNAL instead of hanging.
+//
+// Measured (GB300, interpreter stage; before: one real warp per simulated warp, everything
+// compiled C++): the reduction of 2^24 values 3,917 -> 2,098 us, 256 generated programs
+// 19,912 -> 8,098 us, 96 of them with default shapes 5,893 -> 2,004 us, the 2048^2 stencil in 16
+// launches 11,302 -> 6,207 us.
+#include <algorithm>
 #include <climits>
 
+#include "solo_loop.cuh"
 #include "sr_internal.h"
 
 namespace sr {
@@ -36,12 +53,13 @@ constexpr uint32_t FULL = 0xFFFFFFFFu;
 enum : uint32_t { DEC_RELEASE = 1, DEC_DONE = 2, DEC_STOP = 3 };
 
 struct BlockVars {
+  uint32_t decision, any_race[2], n_misc;   // any_race: fused race check, words are marked (by interval parity)
   uint32_t cursor;             // log records reserved by the block (stops growing past the log)
-  uint32_t n_misc, epoch, k0, flags, decision, err_dirty, status;
+  uint32_t flags, err_dirty, status;
   uint32_t bar_np, bar_nw;     // at a release: true predicates, released threads
   uint32_t race_out;           // fused race check: race entries written so far
   uint32_t gcursor;            // global-log records reserved by the block
-  uint32_t pad[4];
+  uint32_t sreg[4];            // S2R BID, BDIM, GDIM, WARPSIZE
 };
 static_assert(sizeof(BlockVars) <= 64, "block vars");
 
@@ -52,14 +70,6 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   uint32_t m;
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
   return m;
-}
-__device__ __forceinline__ uint32_t ld_acquire_cta(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_release_cta(uint32_t* p, uint32_t v) {
-  asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
 __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
   uint32_t v;
@@ -104,6 +114,10 @@ __device__ __forceinline__ bool stage_wait(unsigned long long* bar, uint32_t pha
   return ok;
 }
 
+// A value that is the same in every lane, through a broadcast: the compiler then knows it to be
+// warp-uniform, and what depends on it needs no handling of divergence.
+__device__ __forceinline__ uint32_t same(uint32_t v) { return __shfl_sync(FULL, v, 0); }
+
 // Shared-memory accesses by 32-bit shared-window address (cheaper address arithmetic than
 // generic pointers in the interpreter's tight loops).
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
@@ -114,66 +128,79 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
 __device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) {
   asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
+__device__ __forceinline__ uint32_t lds_acquire(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+// The same under a predicate inside the statement: around a statement that the compiler cannot
+// look into, an `if` becomes a branch with its reconvergence instead of a predicated access.
+__device__ __forceinline__ uint32_t lds_if(bool p, uint32_t a) {
+  uint32_t v;
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %2, 0; mov.u32 %0, 0; @q ld.shared.u32 %0, [%1]; }"
+               : "=&r"(v) : "r"(a), "r"((uint32_t)p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts_if(bool p, uint32_t a, uint32_t v) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q st.shared.u32 [%0], %1; }" ::"r"(a), "r"(v), "r"((uint32_t)p)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t atom_add_if(bool p, uint32_t a, uint32_t v, uint32_t otherwise) {
+  uint32_t o;
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %3, 0; mov.u32 %0, %4; @q atom.shared.add.u32 %0, [%1], %2; }"
+               : "=&r"(o) : "r"(a), "r"(v), "r"((uint32_t)p), "r"(otherwise) : "memory");
+  return o;
+}
+__device__ __forceinline__ void st_release_if(bool p, uint32_t a, uint32_t v) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q st.release.cta.shared.u32 [%0], %1; }" ::"r"(a), "r"(v),
+               "r"((uint32_t)p)
+               : "memory");
+}
+__device__ __forceinline__ void sts_u128_if(bool p, uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t u) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %5, 0; @q st.shared.v4.u32 [%0], {%1, %2, %3, %4}; }" ::"r"(a), "r"(x),
+               "r"(y), "r"(z), "r"(u), "r"((uint32_t)p)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t lds_u8(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
 __device__ __forceinline__ uint2 lds_u64(uint32_t a) {
   uint2 v;
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
   return v;
 }
 
-__device__ __forceinline__ void group_sync(uint32_t id, uint32_t nthr) {
+// The simulated block's warps (named barrier 1: a CTA may hold warps that the block does not use).
+__device__ __forceinline__ void block_sync(uint32_t nthr) {
   if (nthr == 32)
     __syncwarp();
   else
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthr) : "memory");
-}
-
-// int32 ALU of the IR: two's-complement wrap, C division (x/0 and x%0 flagged)
-__device__ __forceinline__ int32_t alu(uint32_t op, int32_t x, int32_t y, bool& dz) {
-  switch (op) {
-    case SR_OP_MOV: return y;
-    case SR_OP_ADD: return (int32_t)((uint32_t)x + (uint32_t)y);
-    case SR_OP_SUB: return (int32_t)((uint32_t)x - (uint32_t)y);
-    case SR_OP_MUL: return (int32_t)((uint32_t)x * (uint32_t)y);
-    case SR_OP_DIV:
-      if (y == 0) { dz = true; return 0; }
-      return y == -1 ? (int32_t)(0u - (uint32_t)x) : x / y;   // -INT_MIN wraps to INT_MIN
-    case SR_OP_REM:
-      if (y == 0) { dz = true; return 0; }
-      return y == -1 ? 0 : x % y;
-    case SR_OP_AND: return x & y;
-    case SR_OP_OR: return x | y;
-    case SR_OP_XOR: return x ^ y;
-    case SR_OP_SHL: return (int32_t)((uint32_t)x << (y & 31));
-    case SR_OP_SHR: return x >> (y & 31);                        // arithmetic
-    case SR_OP_MIN: return min(x, y);
-    case SR_OP_MAX: return max(x, y);
-    case SR_OP_SLT: return x < y;
-    case SR_OP_SLE: return x <= y;
-    case SR_OP_SEQ: return x == y;
-    default: return x != y;                                      // SNE
-  }
+    asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
 }
 
 // Wait until every other warp of the block has published a clock >= need.  With
 // `order` (store stage), also wait for lower warps whose store of this same round
-// (clock == need) touches an overlapping range of the same memory space.
-// `omin` is a lower bound of the other warps' clocks (clocks only grow within a
-// barrier interval); when it already decides the wait, no clock is read.
-__device__ __forceinline__ bool wait_clocks(const uint32_t* clk, const int32_t* rlo, const int32_t* rhi,
-                                            const uint32_t* rsp, uint32_t nw, uint32_t w, uint32_t lane,
+// (clock == need) touches an overlapping range of the same memory space (ranges: {lowest,
+// highest address, space, -} per warp).  clks: shared address of clock `lane`; pad: the lane
+// stands for no other warp of the block.  Clocks and `need` carry the barrier interval's parity
+// in bit 31, so that a warp still parked at the last barrier (other parity, all other bits set)
+// reads as lower.
+__device__ __forceinline__ bool wait_clocks(uint32_t clks, uint32_t ranges, bool pad, uint32_t w, uint32_t lane,
                                             uint32_t need, bool order, int32_t lo, int32_t hi, uint32_t sp,
-                                            uint32_t limit, uint32_t& omin) {
-  if (omin > need || (!order && omin == need)) return true;
+                                            uint32_t limit) {
   for (uint32_t it = 0; it < limit; ++it) {
-    bool ok = true;
-    uint32_t c = kInf;
-    if (lane < nw && lane != w) {
-      c = ld_acquire_cta(clk + lane);
-      ok = c >= need;
-      if (ok && order && lane < w && c == need) ok = !(rsp[lane] == sp && rlo[lane] <= hi && lo <= rhi[lane]);
+    const uint32_t c = lds_acquire(clks);
+    bool ok = (int32_t)(c - need) >= 0;
+    if (order) {
+      int32_t l, h;
+      uint32_t s;
+      asm volatile("ld.shared.v2.u32 {%0, %1}, [%3];\nld.shared.u32 %2, [%3 + 8];"
+                   : "=r"(l), "=r"(h), "=r"(s) : "r"(ranges + 16u * lane) : "memory");
+      ok = ok && !(lane < w && c == need && (s == sp || s == 2u) && l <= hi && lo <= h);
     }
-    if (__all_sync(FULL, ok)) {
-      omin = __reduce_min_sync(FULL, c);
+    if (__all_sync(FULL, ok || pad)) {
       __syncwarp();
       return true;
     }
@@ -194,29 +221,6 @@ __device__ __forceinline__ void note_err(uint32_t* err, BlockVars* bv, uint32_t 
 // The 8-byte access-log record (layout in sr_internal.h) from its parts.
 __device__ __forceinline__ unsigned long long rec_of(uint32_t epoch_hi, uint32_t low_bits, uint32_t addr) {
   return (unsigned long long)(epoch_hi | addr >> 8) << 32 | (low_bits | addr << 24);
-}
-
-// Append one record per lane with `me` to the block's access log (warp-aggregated:
-// one 32-bit shared atomic per warp, consecutive 8-byte slots -> coalesced stores).
-// Once the log is full nothing more is reserved, so the cursor cannot wrap.
-__device__ __forceinline__ void log_access(BlockVars* bv, unsigned long long* region, uint32_t front_cap,
-                                           bool me, unsigned long long rec, uint32_t lane) {
-  const uint32_t m = __ballot_sync(FULL, me);
-  if (m == 0) return;
-  const uint32_t leader = __ffs(m) - 1;
-  uint32_t base = 0;
-  if (lane == leader) {
-    base = *reinterpret_cast<volatile uint32_t*>(&bv->cursor);
-    if (base < front_cap) base = atomicAdd(&bv->cursor, (uint32_t)__popc(m));
-  }
-  base = __shfl_sync(FULL, base, leader);
-  if (me) {
-    const uint32_t pos = base + __popc(m & lanemask_lt());
-    if (base < front_cap && pos < front_cap)
-      region[pos] = rec;
-    else
-      atomicOr(&bv->flags, BF_OVERFLOW);
-  }
 }
 
 // Append one 16-byte global-log record per lane with `me` to the block's global log (the
@@ -297,23 +301,37 @@ __device__ __forceinline__ void tuple_clear(uint32_t* T, uint32_t tps) {
 // End of an interval, every warp of the block: words 32 j .. 32 j + 31 for its share of j.
 // A racy word keeps its pair and class|pcs in planes 0 and 1 and is marked in the bitmap;
 // every other touched word is cleared for the next interval.
-__device__ __forceinline__ void tuples_mark(uint32_t* tup, uint32_t tps, uint32_t* rbm, uint32_t w, uint32_t nw,
-                                            uint32_t lane) {
-  for (uint32_t j = w; j < tps / 32u; j += nw) {
-    uint32_t* T = tup + 32u * j + lane;
-    bool racy = false;
-    if (T[6u * tps] != kTupleEmpty) {
-      uint32_t b, c;
-      racy = tuple_race(T, tps, b, c);
-      if (racy) {
-        T[0] = b;
-        T[tps] = c;
-      } else {
-        tuple_clear(T, tps);
+__device__ __forceinline__ void tuples_mark(uint32_t* tup, uint32_t tps, uint32_t* rbm, uint32_t* any, uint32_t w,
+                                            uint32_t nw, uint32_t lane) {
+  const uint32_t nbw = tps / 32u;
+  for (uint32_t j0 = w; j0 < nbw; j0 += 4u * nw) {
+    uint32_t lo[4];                              // the lowest pcs: is the word touched?
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i) {
+      const uint32_t j = j0 + i * nw;
+      lo[i] = j < nbw ? tup[6u * tps + 32u * j + lane] : kTupleEmpty;
+    }
+#pragma unroll 1
+    for (uint32_t i = 0, j = j0; i < 4 && j < nbw; ++i, j += nw) {
+      uint32_t* T = tup + 32u * j + lane;
+      bool racy = false;
+      if (lo[0] != kTupleEmpty) {
+        uint32_t b, c;
+        racy = tuple_race(T, tps, b, c);
+        if (racy) {
+          T[0] = b;
+          T[tps] = c;
+        } else {
+          tuple_clear(T, tps);
+        }
+      }
+      lo[0] = lo[1]; lo[1] = lo[2]; lo[2] = lo[3];
+      const uint32_t m = __ballot_sync(FULL, racy);
+      if (lane == 0) {
+        rbm[j] = m;
+        if (m) *any = 1u;
       }
     }
-    const uint32_t m = __ballot_sync(FULL, racy);
-    if (lane == 0) rbm[j] = m;
   }
 }
 
@@ -330,28 +348,20 @@ __device__ void tuples_emit(uint32_t* tup, uint32_t tps, const uint32_t* rbm, Bl
   bool over = false;
   uint4* out = reinterpret_cast<uint4*>(region);
   for (uint32_t base = 0; base < nbw; base += 32) {
-    const uint32_t wd = base + lane;
-    uint32_t word = wd < nbw ? rbm[wd] : 0u;
-    const uint32_t cnt = __popc(word);
-    uint32_t inc = cnt;
-#pragma unroll
-    for (uint32_t o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(FULL, inc, o);
-      if (lane >= o) inc += y;
+    const uint32_t word = base + lane < nbw ? rbm[base + lane] : 0u;
+    for (uint32_t nz = __ballot_sync(FULL, word != 0); nz; nz &= nz - 1u) {
+      const uint32_t i = __ffs(nz) - 1, m = __shfl_sync(FULL, word, i);
+      if ((m >> lane) & 1u) {
+        const uint32_t a = (base + i) * 32u + lane, pos = ro + __popc(m & ((1u << lane) - 1u));
+        uint32_t* T = tup + a;
+        if (pos < cap)
+          out[pos] = make_uint4(epoch, a, T[0], T[tps]);
+        else
+          over = true;
+        tuple_clear(T, tps);
+      }
+      ro += __popc(m);
     }
-    uint32_t pos = ro + inc - cnt;
-    while (word) {
-      const uint32_t a = wd * 32u + (__ffs(word) - 1);
-      word &= word - 1;
-      uint32_t* T = tup + a;
-      if (pos < cap)
-        out[pos] = make_uint4(epoch, a, T[0], T[tps]);
-      else
-        over = true;
-      ++pos;
-      tuple_clear(T, tps);
-    }
-    ro += __shfl_sync(FULL, inc, 31);
   }
   ro = min(ro, cap);
   if (__any_sync(FULL, over) && lane == 0) bv->flags |= BF_OVERFLOW;
@@ -392,10 +402,10 @@ __device__ void flush_errors(BlockVars* bv, uint32_t* err, uint32_t* un, const u
       } else if (pc < ncode) {
         cnt = err[2 * pc];
         if (cnt) {
-          const uint32_t op = ir[pc].x & 0x3Fu;
-          const uint32_t k2 = (op == SR_OP_LDS || op == SR_OP_STS || op == SR_OP_ATOMS) ? SR_REP_ERR_OOB_SHARED
-                              : (op == SR_OP_LDG || op == SR_OP_STG)                   ? SR_REP_ERR_OOB_GLOBAL
-                                                                                        : SR_REP_ERR_DIV0;
+          const uint32_t f = pk_form(ir[pc].x);
+          const uint32_t k2 = (f == F_LDS || f == F_STS || f == F_ATOMS) ? SR_REP_ERR_OOB_SHARED
+                              : (f == F_LDG || f == F_STG)               ? SR_REP_ERR_OOB_GLOBAL
+                                                                         : SR_REP_ERR_DIV0;
           hit = (k2 == kind);
           mt = err[2 * pc + 1];
         }
@@ -422,520 +432,249 @@ __device__ void flush_errors(BlockVars* bv, uint32_t* err, uint32_t* un, const u
   if (lane == 0) bv->err_dirty = 0;
 }
 
-// Run one simulated block on warps [0, nw) of a group (bar_id = its named barrier).  The
-// fused race check is compiled in only where Fused is set, and the logging of global
-// accesses only where Global is set, so that the default kernels keep their register budget.
-template <bool Fused, bool Global>
-__device__ void run_block(const RunArgs& A, const LaunchDev* Ls, uint32_t block, const uint2* __restrict__ ir,
-                          unsigned char* gsm, uint32_t w, uint32_t nw, uint32_t bar_id) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t nthr = nw * 32;
-  const uint32_t tid = w * 32 + lane;
-  const uint32_t bdim = Ls->bdim, shw = Ls->shw, ncode = Ls->ncode, log_cap = Ls->log_cap, nrows = Ls->nrows;
-  const bool uninit = Ls->uninit != 0;
-  const bool fused = Fused && Ls->fused != 0 && A.check_races != 0;
-  const GroupLayout G = group_layout(nthr, shw, ncode, nrows, Ls->uninit, Ls->fused);
-  uint32_t* regs = reinterpret_cast<uint32_t*>(gsm + G.regs);
-  int32_t* sh = reinterpret_cast<int32_t*>(gsm + G.sh);
-  uint32_t* clk = reinterpret_cast<uint32_t*>(gsm + kGroupClk);
-  int32_t* rlo = reinterpret_cast<int32_t*>(gsm + kGroupRlo);
-  int32_t* rhi = reinterpret_cast<int32_t*>(gsm + kGroupRhi);
-  uint32_t* rsp = reinterpret_cast<uint32_t*>(gsm + kGroupRsp);
-  uint32_t* park = reinterpret_cast<uint32_t*>(gsm + kGroupPark);
-  uint32_t* err = reinterpret_cast<uint32_t*>(gsm + G.err);
-  uint32_t* un = reinterpret_cast<uint32_t*>(gsm + G.un);      // with `uninit` only
-  uint32_t* wb = reinterpret_cast<uint32_t*>(gsm + G.wb);      // with `uninit` only
-  uint32_t* tup = reinterpret_cast<uint32_t*>(gsm + G.tup);    // with `fused` only
-  const uint32_t tps = tuple_plane_words(shw);
-  uint32_t* rbm = reinterpret_cast<uint32_t*>(gsm + G.rbm);
-  BlockVars* bv = reinterpret_cast<BlockVars*>(gsm + kGroupBv);
-  int32_t* arena = A.arena + Ls->arena_off;
-  const uint32_t arena_words = (uint32_t)Ls->arena_words;
-  unsigned long long* region = A.log + Ls->log_base + (unsigned long long)block * log_cap;
-  const bool logging = A.check_races != 0;
-  // global log of this block (with Global, for launches whose glog_cap is set)
-  const uint32_t gcap = Global ? Ls->glog_cap : 0u;
-  const uint32_t gb = Ls->block_base + block;
-  uint4* gregion = Global ? A.glog + Ls->glog_base + (unsigned long long)block * gcap : nullptr;
-  const uint32_t budget = A.budget, spin = A.spin_limit;
-  uint32_t* myregs = regs + tid;                 // row r of this thread: myregs[r * nthr]
-  // the same as 32-bit shared-window addresses, for the fast paths
-  const uint32_t rs = smem_u32(myregs), rstride = nthr * 4u, shs = smem_u32(sh), irs = smem_u32(ir);
+// ---- one simulated thread per (lane, slot): warp w of a block runs the simulated warps
+// V w .. V w + V - 1 ("agents"), slot j of its lane l being thread 32 (V w + j) + l.  A row of
+// the register file holds a lane's V values side by side, so that one 4 V-byte access moves
+// an operand of all of them.
+template <int V>
+__device__ __forceinline__ void lds_v(uint32_t a, uint32_t (&v)[V]) {
+  if constexpr (V == 4)
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(a) : "memory");
+  else if constexpr (V == 2)
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(a) : "memory");
+  else
+    v[0] = lds_u32(a);
+}
+template <int V>
+__device__ __forceinline__ void sts_v(uint32_t a, const uint32_t (&v)[V]) {
+  if constexpr (V == 4)
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+  else if constexpr (V == 2)
+    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v[0]), "r"(v[1]) : "memory");
+  else
+    sts_u32(a, v[0]);
+}
+template <int V>
+__device__ __forceinline__ void sts_v_if(bool p, uint32_t a, const uint32_t (&v)[V]) {
+  if constexpr (V == 4)
+    sts_u128_if(p, a, v[0], v[1], v[2], v[3]);
+  else if constexpr (V == 2)
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %3, 0; @q st.shared.v2.u32 [%0], {%1, %2}; }" ::"r"(a), "r"(v[0]),
+                 "r"(v[1]), "r"((uint32_t)p)
+                 : "memory");
+  else
+    sts_if(p, a, v[0]);
+}
+// Row d of the active slots `am` (kNoDest: nothing): one store when every slot whose register
+// still matters is active (`whole`, the same for the warp), else slot by slot.
+template <int V>
+__device__ __forceinline__ void put_row(uint32_t rs, uint32_t stride, uint32_t d, const uint32_t (&v)[V], uint32_t am,
+                                        bool whole) {
+  const uint32_t a = rs + d * stride;
+  sts_v_if<V>(whole && d != kNoDest, a, v);
+  if (!whole) {
+#pragma unroll
+    for (int j = 0; j < V; ++j) sts_if(((am >> j) & 1u) && d != kNoDest, a + 4u * j, v[j]);
+  }
+}
 
-  // ---- block start: registers = params then zeros (the last row stays zero), shared zeroed
-  for (uint32_t r = 0; r < nrows; ++r) myregs[r * nthr] = (r < Ls->nparams) ? (uint32_t)Ls->params[r] : 0u;
-  for (uint32_t i = tid; i < shw; i += nthr) sh[i] = 0;
-  for (uint32_t i = tid; i <= ncode; i += nthr) {
-    err[2 * i] = 0;
-    err[2 * i + 1] = kInf;
+// A run of instructions for the general steps: as in solo_loop, from the one at shared
+// address q with words (x, y) to the one before qend.  Returns the words at qend.
+// rs + r * stride: this lane's row r; am: the slots to write when not all are (whole = 0).
+#define SR_RPUT(i) "and.b32 t, %9, 1 << " #i ";\nsetp.ne.u32 pf, t, 0;\n@pf st.shared.u32 [ro + 4 * " #i "], c" #i ";\n"
+// the result's store, and the next instruction or the end
+#define SR_RTAIL(STC)                                                                                        \
+  "setp.ge.u32 pe, q, %5;\n"                                                             \
+  "and.b32 t, x, 128;\nsetp.eq.or.u32 ps, t, 0, pe;\n"                                                     \
+  "prmt.b32 ro, x, 0, 0x4441;\nsetp.ne.and.u32 ps, ro, 31, ps;\nmad.lo.u32 ro, ro, %7, %6;\n"             \
+  "@!pw bra.uni LPART;\n@ps " STC "mov.u32 x, nx;\nmov.u32 y, ny;\nmov.u32 keep, 64;\n"                    \
+  "@!pe bra.uni LTOP;\nbra.uni LX;\n"
+#define SR_RUN_ASM(REGS, LDC, LDB, STC, E)                                                                  \
+  asm volatile(                                                                                             \
+      "{\n"                                                                                                 \
+      ".reg .pred pa, pb, pc, pd, pf, pe, ps, pw;\n.reg .b32 x, y, nx, ny, m, n, t, u, ro, keep, q;\n"      \
+      ".reg .b32 " REGS ";\n"                                                                               \
+      "mov.u32 x, %2;\nmov.u32 y, %3;\nmov.u32 q, %4;\nmov.u32 keep, 0;\nsetp.ne.u32 pw, %8, 0;\n"          \
+      "LTOP:\n"                                                                                             \
+      "and.b32 t, x, keep;\nsetp.eq.u32 pf, t, 0;\n"                                                        \
+      "prmt.b32 ro, x, 0, 0x4442;\nmad.lo.u32 ro, ro, %7, %6;\n@pf " LDC                                    \
+      "and.b32 u, x, 63;\nsetp.gt.u32 pf, u, 2;\n@pf bra.uni LGEN;\n"                                       \
+      /* 0 MOV, 1 ADD, 2 MUL with an immediate: c * m + n */                                                \
+      "prmt.b32 t, x, 0, 0x4443;\nmad.lo.u32 q, t, 8, q;\nld.shared.v2.u32 {nx, ny}, [q];\n"               \
+      "setp.eq.u32 pf, u, 2;\nselp.u32 m, y, u, pf;\nselp.u32 n, 0, y, pf;\n" E(SR_MAD)                    \
+      "sub.u32 t, t, 1;\nshl.b32 u, t, 3;\nsub.u32 u, q, u;\n"                                             \
+      "LCHAIN:\nsetp.eq.u32 pf, t, 0;\n@pf bra.uni LCHAINED;\nld.shared.v2.u32 {m, n}, [u];\n" E(SR_MAD)  \
+      "add.u32 u, u, 8;\nsub.u32 t, t, 1;\nbra.uni LCHAIN;\nLCHAINED:\n" SR_RTAIL(STC)                     \
+      "LGEN:\nadd.u32 q, q, 8;\nld.shared.v2.u32 {nx, ny}, [q];\n"                                                                                             \
+      "prmt.b32 ro, x, 0, 0x4443;\nmad.lo.u32 ro, ro, %7, %6;\nsetp.ge.u32 pf, u, 8;\n@pf bra.uni LREST;\n" \
+      /* 3 MOV (operand b is zero), 4 ADD, 5 SUB, 6 MUL of registers */                                     \
+      LDB "setp.eq.u32 pf, u, 5;\nselp.b32 m, 0xFFFFFFFF, 1, pf;\nsetp.eq.u32 pa, u, 6;\n" E(SR_REGOP)      \
+      SR_RTAIL(STC)                                                                                          \
+      "LREST:\n"                                                                                            \
+      E(SR_SPLAT) "and.b32 t, u, 1;\nsetp.ne.u32 pf, t, 0;\n@pf " LDB                                       \
+      "setp.ge.u32 pf, u, 22;\n@pf bra.uni LCMP;\nsetp.ge.u32 pf, u, 14;\n@pf bra.uni LSHIFT;\n"            \
+      /* 8 AND, 10 OR, 12 XOR (+ 1: of registers) */                                                        \
+      "setp.lt.u32 pa, u, 10;\nsetp.ge.u32 pb, u, 12;\nor.pred pc, pa, pb;\nnot.pred pc, pc;\n"             \
+      E(SR_LOGIC) SR_RTAIL(STC)                                                                              \
+      "LSHIFT:\n" /* 14 SHL, 16 SHR, 18 MIN, 20 MAX */                                                      \
+      "setp.lt.u32 pa, u, 16;\nsetp.ge.u32 pd, u, 20;\nsetp.ge.u32 pb, u, 18;\nnot.pred pc, pd;\n"          \
+      "and.pred pc, pc, pb;\nor.pred pb, pb, pa;\nnot.pred pb, pb;\n" E(SR_SHIFT) SR_RTAIL(STC)              \
+      "LCMP:\n" /* 22 SLT, 24 SLE, 26 SEQ, 28 SNE: (lt and pa) or (eq and pb), inverted under pc */         \
+      "setp.lt.u32 pa, u, 26;\nsetp.ge.u32 pb, u, 24;\nsetp.ge.u32 pc, u, 28;\n" E(SR_COMPARE) SR_RTAIL(STC) \
+      "LPART:\n@!ps bra.uni LNEXT;\n" E(SR_RPUT)                                                             \
+      "LNEXT:\nmov.u32 x, nx;\nmov.u32 y, ny;\nmov.u32 keep, 64;\n@!pe bra.uni LTOP;\n"                     \
+      "LX:\nmov.u32 %0, x;\nmov.u32 %1, y;\n"                                                               \
+      "}\n"                                                                                                 \
+      : "=r"(out.x), "=r"(out.y)                                                                            \
+      : "r"(x), "r"(y), "r"(q), "r"(qend), "r"(rs), "r"(stride), "r"(whole ? 1u : 0u), "r"(am)              \
+      : "memory")
+template <int V>
+__device__ __forceinline__ uint2 alu_run(uint32_t x, uint32_t y, uint32_t q, uint32_t qend, uint32_t rs,
+                                         uint32_t stride, bool whole, uint32_t am) {
+  uint2 out;
+  if constexpr (V == 4)
+    SR_RUN_ASM("c0, c1, c2, c3, b0, b1, b2, b3", "ld.shared.v4.u32 {c0, c1, c2, c3}, [ro];\n",
+               "ld.shared.v4.u32 {b0, b1, b2, b3}, [ro];\n", "st.shared.v4.u32 [ro], {c0, c1, c2, c3};\n", SR_E4);
+  else if constexpr (V == 2)
+    SR_RUN_ASM("c0, c1, b0, b1", "ld.shared.v2.u32 {c0, c1}, [ro];\n", "ld.shared.v2.u32 {b0, b1}, [ro];\n",
+               "st.shared.v2.u32 [ro], {c0, c1};\n", SR_E2);
+  else
+    SR_RUN_ASM("c0, b0", "ld.shared.u32 c0, [ro];\n", "ld.shared.u32 b0, [ro];\n", "st.shared.u32 [ro], c0;\n", SR_E1);
+  return out;
+}
+#undef SR_RUN_ASM
+
+// Append one access record per slot of `im` to the block's log (one 32-bit shared atomic per
+// warp and instruction; consecutive 8-byte slots, so coalesced stores).  `low` holds the low
+// record bits of slot 0 without the address.  A warp that found the log full reserves nothing
+// more, so the cursor cannot wrap.  log_all: slots 0 .. ns - 1
+// of every lane, at the place that log_reserve gave lane 0.
+__device__ __forceinline__ uint32_t log_reserve(BlockVars* bv, bool go, uint32_t n, uint32_t lane) {
+  return atom_add_if(go && lane == 0, smem_u32(&bv->cursor), n, 0xFFFFFFFFu);
+}
+template <int V>
+__device__ __forceinline__ void log_wide(BlockVars* bv, unsigned long long* region, uint32_t front_cap, uint32_t im,
+                                         const uint32_t (&ad)[V], uint32_t epoch_hi, uint32_t low, uint32_t lane,
+                                         bool& full) {
+  uint32_t total = 0, pos[V];
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    const uint32_t m = __ballot_sync(FULL, (im >> j) & 1u);
+    pos[j] = total + __popc(m & lanemask_lt());
+    total += __popc(m);
   }
-  if (uninit) {
-    for (uint32_t i = tid; i <= ncode; i += nthr) {
-      un[2 * i] = 0;
-      un[2 * i + 1] = kInf;
-    }
-    for (uint32_t i = tid; i < (shw + 31u) / 32u; i += nthr) wb[i] = 0;
+  if (total == 0) return;
+  const uint32_t base = same(log_reserve(bv, !full, total, lane));
+  if (base >= front_cap || front_cap - base < total) {
+    full = true;
+    if (lane == 0) atomicOr(&bv->flags, BF_OVERFLOW);
   }
-  if (fused) {
-    for (uint32_t i = tid; i < 8u * tps; i += nthr) tup[i] = i < 7u * tps ? kTupleEmpty : 0u;
-    for (uint32_t i = tid; i < (shw + 31u) / 32u; i += nthr) rbm[i] = 0;
+#pragma unroll
+  for (int j = 0; j < V; ++j)
+    if (((im >> j) & 1u) && base < front_cap && base + pos[j] < front_cap)
+      region[base + pos[j]] = rec_of(epoch_hi, low + ((32u * j) << 14), ad[j]);
+}
+
+template <int V>
+__device__ __forceinline__ void log_all(BlockVars* bv, unsigned long long* region, uint32_t front_cap, uint32_t reserved,
+                                        uint32_t ns, const uint32_t (&ad)[V], uint32_t epoch_hi, uint32_t low,
+                                        uint32_t lane, bool& full) {
+  const uint32_t base = same(reserved);
+  if (base < front_cap && front_cap - base >= 32u * ns) {
+    unsigned long long* out = region + base + lane;
+#pragma unroll
+    for (int j = 0; j < V; ++j)
+      if ((uint32_t)j < ns) out[32 * j] = rec_of(epoch_hi, low + ((32u * j) << 14), ad[j]);
+    return;
   }
-  if (tid == 0) {
+  full = true;                                   // (the part that fits)
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    const uint32_t pos = base + 32u * j + lane;
+    if ((uint32_t)j < ns && base < front_cap && pos < front_cap)
+      region[pos] = rec_of(epoch_hi, low + ((32u * j) << 14), ad[j]);
+  }
+  if (lane == 0) atomicOr(&bv->flags, BF_OVERFLOW);
+}
+
+// Sum of a per-lane count over the warp (counts below 2^32, their sum may exceed it).
+__device__ __forceinline__ unsigned long long warp_sum(uint32_t n) {
+  return (unsigned long long)__reduce_add_sync(FULL, n & 0xFFFFu) +
+         ((unsigned long long)__reduce_add_sync(FULL, n >> 16) << 16);
+}
+
+// Per-thread state word: pc (13 bits) | status << 16 | for a thread at a reducing barrier:
+// destination row << 18 | kind (0 plain, 1 and, 2 or, 3 count) << 23 | predicate << 25.
+__device__ __forceinline__ uint32_t ts_pc(uint32_t t) { return t & 0x1FFFu; }
+__device__ __forceinline__ uint32_t ts_st(uint32_t t) { return (t >> 16) & 3u; }
+
+// The start of a block, in the warps that run it: registers = params then zeros (the last row
+// stays zero), shared memory and the block's records cleared.  Before the CTA waits for the
+// launches it follows, and for its code; apart from run_block, whose registers it does not need.
+template <int V, bool Fused>
+__device__ __forceinline__ void start_block(const RunArgs& A, const LaunchDev* Ls, uint32_t block, const void* ir,
+                                            unsigned char* gsm) {
+  const uint32_t t = threadIdx.x, nw = Ls->nw, nthr = nw * 32u, sha = Ls->sha, ncode = Ls->ncode, nrows = Ls->nrows;
+  const GroupLayout G = group_layout(nthr * V, sha, ncode, nrows, Ls->uninit, Ls->fused);
+  const uint32_t rs = smem_u32(gsm + G.regs) + t * (4u * V), rstride = nthr * (4u * V);
+  for (uint32_t r = 0; r < nrows; ++r) {
+    uint32_t v[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) v[j] = r < Ls->nparams ? (uint32_t)Ls->params[r & 3u] : 0u;
+    sts_v<V>(rs + r * rstride, v);
+  }
+  auto fill2 = [&](uint32_t off) {               // error records: none
+    for (uint32_t i = t; i <= ncode; i += nthr) reinterpret_cast<uint2*>(gsm + off)[i] = make_uint2(0u, kInf);
+  };
+  auto fill4 = [&](uint32_t off, uint32_t words, uint32_t v) {
+    for (uint32_t i = t; i < words / 4u; i += nthr) reinterpret_cast<uint4*>(gsm + off)[i] = make_uint4(v, v, v, v);
+  };
+  auto clear = [&](uint32_t off, uint32_t words) {
+    for (uint32_t i = t; i < words; i += nthr) reinterpret_cast<uint32_t*>(gsm + off)[i] = 0;
+  };
+  fill4(G.sh, sha + 3u, 0);
+  fill2(G.err);
+  if (Ls->uninit) {
+    fill2(G.un);
+    clear(G.wb, (sha + 31u) / 32u);
+  }
+  const uint32_t tps = tuple_plane_words(sha);
+  if (Fused && Ls->fused && A.check_races) {
+    fill4(G.tup, 7u * tps, kTupleEmpty);
+    fill4(G.tup + 28u * tps, tps, 0);
+    clear(G.rbm, (sha + 31u) / 32u);
+  }
+  if ((t & 31u) == 0) reinterpret_cast<uint32_t*>(gsm + kGroupClk)[t >> 5] = 0;
+  if (t == 0) {
+    BlockVars* bv = reinterpret_cast<BlockVars*>(gsm + kGroupBv);
     bv->cursor = 0;
-    bv->n_misc = 0; bv->epoch = 0; bv->k0 = 0; bv->flags = 0;
+    bv->n_misc = 0; bv->flags = 0;
     bv->decision = 0; bv->err_dirty = 0; bv->status = 0;
     bv->race_out = 0;
+    bv->any_race[0] = 0; bv->any_race[1] = 0;
     bv->gcursor = 0;
-  }
-  if (lane == 0) clk[w] = 0;
-  group_sync(bar_id, nthr);
-
-  uint32_t pc = Ls->entry, st = tid < bdim ? ST_RUN : ST_NONE, wpc = 0;
-  // at a barrier: destination row | kind << 5 (0 plain, 1 and, 2 or, 3 count) | predicate << 7
-  uint32_t bst = 0;
-  uint32_t k = 0, epoch = 0, front_cap = log_cap, omin = 0;
-  // pn: the pc the warp issues next (the lowest pc of its runnable lanes, kInf if none);
-  // while every runnable lane sits at pn (conv) it is advanced without a reduction
-  bool conv = true;
-  uint32_t pn = Ls->entry;
-  uint32_t n_instr = 0, n_gacc = 0;              // per lane: executed instructions, global accesses
-  uint32_t n_sacc = 0;                           // per lane, fused race check: shared accesses
-  // a log record is built from 32-bit halves: low = addr << 24 | tid << 14 | kind << 12 | pc,
-  // high = epoch << 6 | addr >> 8
-  const uint32_t lane_rec = tid << 14;
-  uint32_t epoch_hi = 0;                         // epoch << 6
-
-  for (;;) {  // barrier intervals
-    bool limit = false, timeout = false;
-    for (;;) {  // rounds
-      const uint32_t p = pn;
-      if (p == kInf) break;                      // no runnable lane
-      if (k >= budget) { limit = true; break; }
-      const bool act = (st == ST_RUN) && (pc == p);
-      const uint2 ins = ir[p];
-      const uint32_t op = ins.x & 0x3Fu;
-      if (conv && pk_run(ins.x)) {
-        // Converged warp at a run of MOV / ADD / MUL instructions (the bulk of straight-line code):
-        // every runnable lane is at p and the run touches no memory, so its last round can be
-        // published at once (other warps wait on a clock only for memory effects), and the
-        // run executes in this tight loop, one instruction per round.
-        const bool runl = st == ST_RUN;
-        const uint32_t len = min(pk_run(ins.x), budget - k);      // (k < budget here)
-        if (lane == 0) st_release_cta(&clk[w], 4u * (k + len));
-        uint32_t q = p;
-        uint2 in = ins;
-        bool bad = false;                        // (debug build: an index check failed)
-        for (uint32_t i = 0;;) {
-          const uint32_t o = pk_op(in.x), dd = pk_d(in.x);
-          if (!dbg_ok(q <= ncode && pk_a(in.x) < nrows && pk_b(in.x) < nrows && (dd < nrows || dd == kNoDest),
-                      &A.prog_status[Ls->prog], SR_ST_BOUNDS)) {
-            bad = true;
-            break;
-          }
-          const uint32_t a = lds_u32(rs + pk_a(in.x) * rstride);
-          const uint32_t b = pk_imm(in.x) ? in.y : lds_u32(rs + pk_b(in.x) * rstride);
-          const uint32_t r = o == SR_OP_ADD ? a + b : o == SR_OP_MUL ? a * b : b;   // ADD, MUL, MOV
-          if (runl && dd != kNoDest) sts_u32(rs + dd * rstride, r);
-          ++q;
-          if (++i == len) break;
-          in = lds_u64(irs + q * 8u);
-        }
-        if (bad) {                               // stop the block the way a wait that gave up does
-          timeout = true;
-          break;
-        }
-        n_instr += runl ? len : 0u;
-        if (runl) pc = q;
-        pn = q;
-        k += len;
-        continue;
-      }
-      const uint32_t d = pk_d(ins.x), ra = pk_a(ins.x), rb = pk_b(ins.x);
-      const int32_t imm = (int32_t)ins.y;
-      if (!dbg_ok(p <= ncode && ra < nrows && rb < nrows && (d < nrows || d == kNoDest), &A.prog_status[Ls->prog],
-                  SR_ST_BOUNDS)) {
-        timeout = true;                          // (debug build) stop the block like a failed wait
-        break;
-      }
-      if (conv && (op == SR_OP_LDS || op == SR_OP_STS) && !uninit && !fused) {
-        // Converged warp, shared load or store without the optional checks: the general
-        // path's steps for this one case (every runnable lane is at p, the next pc is p + 1).
-        const bool runl = st == ST_RUN;
-        const int32_t addr = (int32_t)(lds_u32(rs + ra * rstride) + (uint32_t)imm);
-        const bool inb = runl && (uint32_t)addr < shw;
-        uint32_t kind;
-        if (op == SR_OP_LDS) {
-          kind = K_R;
-          if (nw > 1 && !wait_clocks(clk, rlo, rhi, rsp, nw, w, lane, 4u * k, false, 0, 0, 0, spin, omin)) {
-            timeout = true;
-            break;
-          }
-          const uint32_t v = inb ? lds_u32(shs + (uint32_t)addr * 4u) : 0u;
-          if (runl && d != kNoDest) sts_u32(rs + d * rstride, v);
-        } else {
-          kind = K_W;
-          const uint32_t vb = lds_u32(rs + rb * rstride);
-          if (nw > 1) {
-            const int32_t lo = __reduce_min_sync(FULL, inb ? addr : INT_MAX);
-            const int32_t hi = __reduce_max_sync(FULL, inb ? addr : INT_MIN);
-            if (lane == 0) {
-              rlo[w] = lo;
-              rhi[w] = hi;
-              rsp[w] = 1u;
-              st_release_cta(&clk[w], 4u * k + 1u);
-            }
-            if (!wait_clocks(clk, rlo, rhi, rsp, nw, w, lane, 4u * k + 1u, true, lo, hi, 1u, spin, omin)) {
-              timeout = true;
-              break;
-            }
-          }
-          // several lanes on one word: the highest tid's store is kept (see the general path)
-          const uint32_t sm = __ballot_sync(FULL, inb);
-          const int32_t off = __shfl_sync(FULL, addr - (int32_t)lane, sm ? __ffs(sm) - 1 : 0);
-          bool last = inb;
-          if (!__all_sync(FULL, !inb || addr - (int32_t)lane == off)) {
-            const uint32_t grp = __match_any_sync(FULL, inb ? (uint32_t)addr : (0x80000000u | lane));
-            last = inb && lane == 31u - __clz(grp);
-          }
-          if (last) sts_u32(shs + (uint32_t)addr * 4u, vb);
-        }
-        const uint32_t em = __ballot_sync(FULL, runl && !inb);
-        if (em) note_err(err, bv, p, w, em, lane);
-        if (logging) log_access(bv, region, front_cap, inb, rec_of(epoch_hi, lane_rec | kind << 12 | p, (uint32_t)addr), lane);
-        n_instr += runl;
-        if (runl) pc = p + 1;
-        pn = p + 1;
-        ++k;
-        __syncwarp();
-        if (lane == 0) st_release_cta(&clk[w], 4u * k);
-        continue;
-      }
-      const int32_t va = (int32_t)myregs[ra * nthr];
-      const int32_t vb = pk_imm(ins.x) ? imm : (int32_t)myregs[rb * nthr];
-      const bool wr = act && d != kNoDest;
-      uint32_t npc = p + 1, cn = p + 1;         // cn: the warp's next pc while converged
-      bool memop = false;
-      n_instr += act;
-
-      if (op <= SR_OP_SNE) {
-        bool dz = false;
-        const int32_t r = alu(op, va, vb, dz);
-        if (wr) myregs[d * nthr] = (uint32_t)r;
-        if (op == SR_OP_DIV || op == SR_OP_REM) {
-          const uint32_t em = __ballot_sync(FULL, act && dz);
-          if (em) note_err(err, bv, p, w, em, lane);
-        }
-      } else {
-        switch (op) {
-          case SR_OP_S2R: {
-            const uint32_t v = imm == SR_SREG_TID    ? tid
-                               : imm == SR_SREG_BID  ? block + Ls->block_off
-                               : imm == SR_SREG_BDIM ? bdim
-                               : imm == SR_SREG_GDIM ? Ls->gdim
-                                                     : 32u;
-            if (wr) myregs[d * nthr] = v;
-            break;
-          }
-          case SR_OP_LDS:
-          case SR_OP_LDG: {
-            memop = true;
-            const bool shared = op == SR_OP_LDS;
-            const int32_t addr = (int32_t)((uint32_t)va + (uint32_t)imm);
-            const bool inb = act && (uint32_t)addr < (shared ? shw : arena_words);
-            if (nw > 1 && !wait_clocks(clk, rlo, rhi, rsp, nw, w, lane, 4u * k, false, 0, 0, 0, spin, omin)) {
-              timeout = true;
-              break;
-            }
-            int32_t v = 0;
-            if (inb) v = shared ? sh[addr] : arena[addr];
-            if (wr) myregs[d * nthr] = (uint32_t)v;
-            const uint32_t em = __ballot_sync(FULL, act && !inb);
-            if (em) note_err(err, bv, p, w, em, lane);
-            if (shared && uninit) {                // words no store or atomic of an earlier round wrote
-              const uint32_t um = __ballot_sync(FULL, inb && !((wb[addr >> 5] >> (addr & 31)) & 1u));
-              if (um) note_err(un, bv, p, w, um, lane);
-            }
-            if (shared) {
-              if (logging) {
-                if (fused) {
-                  tuple_add(tup, tps, inb, (uint32_t)addr, tid, K_R, p);
-                  n_sacc += inb;
-                } else {
-                  log_access(bv, region, front_cap, inb,
-                           rec_of(epoch_hi, lane_rec | K_R << 12 | p, (uint32_t)addr),
-                           lane);
-                }
-              }
-            } else {
-              n_gacc += act;
-              if (Global && gcap)
-                log_global(bv, gregion, gcap, inb, make_uint4((uint32_t)addr, epoch, tid << 16 | p, gb), lane);
-            }
-            break;
-          }
-          case SR_OP_STS:
-          case SR_OP_STG: {
-            memop = true;
-            const bool shared = op == SR_OP_STS;
-            const int32_t addr = (int32_t)((uint32_t)va + (uint32_t)imm);
-            const bool inb = act && (uint32_t)addr < (shared ? shw : arena_words);
-            if (nw > 1) {
-              const int32_t lo = __reduce_min_sync(FULL, inb ? addr : INT_MAX);
-              const int32_t hi = __reduce_max_sync(FULL, inb ? addr : INT_MIN);
-              if (lane == 0) {
-                rlo[w] = lo;
-                rhi[w] = hi;
-                rsp[w] = shared;
-                st_release_cta(&clk[w], 4u * k + 1u);
-              }
-              if (!wait_clocks(clk, rlo, rhi, rsp, nw, w, lane, 4u * k + 1u, true, lo, hi, shared, spin, omin)) {
-                timeout = true;
-                break;
-              }
-            }
-            // several lanes of the warp on one word: the highest tid's store is the one kept.
-            // Consecutive addresses, one per lane (addr - lane equal across the storing lanes),
-            // cannot collide; any other pattern groups the lanes by address.
-            const uint32_t sm = __ballot_sync(FULL, inb);
-            const int32_t off = __shfl_sync(FULL, addr - (int32_t)lane, sm ? __ffs(sm) - 1 : 0);
-            bool last = inb;
-            if (!__all_sync(FULL, !inb || addr - (int32_t)lane == off)) {
-              const uint32_t grp = __match_any_sync(FULL, inb ? (uint32_t)addr : (0x80000000u | lane));
-              last = inb && lane == 31u - __clz(grp);
-            }
-            if (last) {
-              if (shared)
-                sh[addr] = vb;
-              else
-                arena[addr] = vb;
-            }
-            if (shared && uninit && inb) atomicOr(&wb[addr >> 5], 1u << (addr & 31));
-            const uint32_t em = __ballot_sync(FULL, act && !inb);
-            if (em) note_err(err, bv, p, w, em, lane);
-            if (shared) {
-              if (logging) {
-                if (fused) {
-                  tuple_add(tup, tps, inb, (uint32_t)addr, tid, K_W, p);
-                  n_sacc += inb;
-                } else {
-                  log_access(bv, region, front_cap, inb,
-                           rec_of(epoch_hi, lane_rec | K_W << 12 | p, (uint32_t)addr),
-                           lane);
-                }
-              }
-            } else {
-              n_gacc += act;
-              if (Global && gcap)
-                log_global(bv, gregion, gcap, inb, make_uint4((uint32_t)addr, epoch, tid << 16 | 1u << 12 | p, gb),
-                           lane);
-            }
-            break;
-          }
-          case SR_OP_ATOMS: {
-            memop = true;
-            const int32_t addr = (int32_t)((uint32_t)va + (uint32_t)imm);
-            const bool inb = act && (uint32_t)addr < shw;
-            if (nw > 1) {
-              if (lane == 0) st_release_cta(&clk[w], 4u * k + 2u);
-              if (!wait_clocks(clk, rlo, rhi, rsp, nw, w, lane, 4u * k + 2u, false, 0, 0, 0, spin, omin)) {
-                timeout = true;
-                break;
-              }
-            }
-            if (inb) atomicAdd(&sh[addr], vb);
-            if (uninit && inb) atomicOr(&wb[addr >> 5], 1u << (addr & 31));
-            const uint32_t em = __ballot_sync(FULL, act && !inb);
-            if (em) note_err(err, bv, p, w, em, lane);
-            if (logging) {
-                if (fused) {
-                  tuple_add(tup, tps, inb, (uint32_t)addr, tid, K_A, p);
-                  n_sacc += inb;
-                } else {
-                  log_access(bv, region, front_cap, inb,
-                         rec_of(epoch_hi, lane_rec | K_A << 12 | p, (uint32_t)addr),
-                         lane);
-                }
-              }
-            break;
-          }
-          case SR_OP_BRA: npc = cn = (uint32_t)imm; break;
-          case SR_OP_BRZ:
-          case SR_OP_BRNZ: {
-            const bool taken = (va == 0) == (op == SR_OP_BRZ);
-            npc = taken ? (uint32_t)imm : p + 1;
-            if (conv) {                          // a split branch ends the converged run
-              const uint32_t tm = __ballot_sync(FULL, act && taken);
-              if (tm != 0 && tm != __ballot_sync(FULL, act)) conv = false;
-              if (tm) cn = (uint32_t)imm;
-            }
-            break;
-          }
-          case SR_OP_BAR:
-          case SR_OP_BARAND:
-          case SR_OP_BAROR:
-          case SR_OP_BARPOPC:
-            // __syncthreads and its reducing forms: wait; a reducing form hands in its
-            // predicate and keeps the row its result goes to
-            if (act) {
-              st = ST_WAIT;
-              wpc = p;
-              bst = op == SR_OP_BAR ? 0u : (d | (op - SR_OP_BARAND + 1u) << 5 | (va != 0 ? 1u : 0u) << 7);
-            }
-            conv = false;
-            break;
-          default:  // EXIT, and the EXIT sentinel after the last instruction
-            if (act) st = ST_EXIT;
-            conv = false;
-            break;
-        }
-      }
-      if (timeout) break;
-      if (act) pc = npc;
-      ++k;
-      if (conv) {
-        pn = cn;
-      } else {
-        pn = __reduce_min_sync(FULL, st == ST_RUN ? pc : kInf);
-        conv = __all_sync(FULL, st != ST_RUN || pc == pn);
-      }
-      // publish progress; after a memory instruction every lane's access must be
-      // ordered before the clock (warp barrier, then a release by lane 0)
-      if (memop) __syncwarp();
-      if (lane == 0) st_release_cta(&clk[w], 4u * k);
-    }
-
-    // ---- no runnable lane in this warp: publish its state and park
-    // (`uni`: every waiting lane at one barrier pc and none runnable, the usual case: its
-    // lanes all resume together after that barrier)
-    bool uni = false;
-    uint32_t upc = 0;
-    {
-      const uint32_t wm = __ballot_sync(FULL, st == ST_WAIT);
-      const uint32_t xm = __ballot_sync(FULL, st == ST_EXIT);
-      const uint32_t rm = __ballot_sync(FULL, st == ST_RUN);
-      const uint32_t tm = __ballot_sync(FULL, st == ST_WAIT && (bst >> 7));   // true predicates
-      uint32_t pmn = kInf, pmx = 0, rpc = kInf;
-      if (wm) {
-        upc = __shfl_sync(FULL, wpc, __ffs(wm) - 1);
-        uni = rm == 0 && __all_sync(FULL, st != ST_WAIT || wpc == upc);
-        if (uni) {
-          pmn = pmx = upc;
-        } else {
-          pmn = __reduce_min_sync(FULL, st == ST_WAIT ? wpc : kInf);
-          pmx = __reduce_max_sync(FULL, st == ST_WAIT ? wpc : 0u);
-        }
-      }
-      if (rm) rpc = __reduce_min_sync(FULL, st == ST_RUN ? pc : kInf);
-      if (lane == 0) {
-        uint32_t* P = park + w * 8;
-        P[0] = __popc(wm); P[1] = __popc(xm); P[2] = __popc(rm);
-        P[3] = pmn; P[4] = pmx; P[5] = rpc; P[6] = k;
-        P[7] = (limit ? 1u : 0u) | (timeout ? 2u : 0u) | (uint32_t)__popc(tm) << 8;
-        st_release_cta(&clk[w], kInf);
-      }
-    }
-    group_sync(bar_id, nthr);
-    if (fused) {                                 // the interval's touched words, all warps
-      tuples_mark(tup, tps, rbm, w, nw, lane);
-      group_sync(bar_id, nthr);
-    }
-
-    // ---- barrier resolution by warp 0 of the block
-    if (w == 0) {
-      const bool v = lane < nw;
-      const uint4 pa = reinterpret_cast<const uint4*>(park)[2 * lane];      // warp `lane`'s entry
-      const uint4 pb = reinterpret_cast<const uint4*>(park)[2 * lane + 1];
-      const uint32_t nW = __reduce_add_sync(FULL, v ? pa.x : 0u);
-      const uint32_t nX = __reduce_add_sync(FULL, v ? pa.y : 0u);
-      const uint32_t nR = __reduce_add_sync(FULL, v ? pa.z : 0u);
-      const uint32_t pmn = __reduce_min_sync(FULL, v ? pa.w : kInf);
-      const uint32_t pmx = __reduce_max_sync(FULL, v ? pb.x : 0u);
-      const uint32_t rpc = __reduce_min_sync(FULL, v ? pb.y : kInf);
-      const uint32_t kmax = __reduce_max_sync(FULL, v ? pb.z : 0u);
-      const uint32_t fl = __reduce_or_sync(FULL, v ? pb.w & 0xFFu : 0u);
-      const uint32_t nP = __reduce_add_sync(FULL, v ? pb.w >> 8 : 0u);
-      const uint32_t ep = bv->epoch;
-      if (fused) tuples_emit(tup, tps, rbm, bv, region, log_cap - 2u * bv->n_misc, ep, lane);
-      uint32_t dec, kind = 0, a = 0, b = 0, c = 0, stbits = 0;
-      if (fl & 2u) {
-        dec = DEC_STOP;
-        if (lane == 0) bv->flags |= BF_INTERNAL;
-      } else if (fl & 1u) {            // out of rounds
-        dec = DEC_STOP; kind = SR_REP_STEP_LIMIT; a = budget; b = nR; c = rpc; stbits = SR_ST_STEP_LIMIT;
-      } else if (nW == 0) {            // every thread exited
-        dec = DEC_DONE;
-      } else if (nX > 0) {             // some wait at a barrier that exited threads never reach
-        dec = DEC_STOP; kind = SR_REP_DEADLOCK; a = pmn; b = pmx; c = nW << 16 | nX; stbits = SR_ST_DEADLOCK;
-      } else {                         // all wait: release, flag differing barrier pcs
-        dec = DEC_RELEASE;
-        if (pmn != pmx) { kind = SR_REP_DIVERGENCE; a = pmn; b = pmx; c = nW << 16; }
-      }
-      if (lane == 0 && kind) push_misc(bv, region, log_cap, kind, ep, a, b, c);
-      __syncwarp();
-      if (bv->err_dirty) flush_errors(bv, err, uninit ? un : nullptr, ir, ncode, region, log_cap, ep, lane);
-      if (lane == 0) {
-        bv->decision = dec;
-        bv->status |= stbits;
-        if (dec == DEC_RELEASE) {
-          bv->epoch = ep + 1;
-          bv->k0 = kmax;
-          bv->bar_np = nP;
-          bv->bar_nw = nW;
-        }
-      }
-      if (dec == DEC_RELEASE && v) clk[lane] = 4u * kmax;
-    }
-    group_sync(bar_id, nthr);
-    if (bv->decision != DEC_RELEASE) break;
-    if (st == ST_WAIT) {
-      // a reducing barrier's result, over every released thread's predicate
-      const uint32_t kind = (bst >> 5) & 3u, row = bst & 31u;
-      if (kind && row != kNoDest) {
-        const uint32_t np = bv->bar_np;
-        myregs[row * nthr] = kind == 1 ? (np == bv->bar_nw ? 1u : 0u) : kind == 2 ? (np ? 1u : 0u) : np;
-      }
-      st = ST_RUN;
-    }
-    if (uni) {                                   // every released lane resumes after its barrier
-      pn = upc + 1;
-      conv = true;
-    } else {
-      pn = __reduce_min_sync(FULL, st == ST_RUN ? pc : kInf);
-      conv = __all_sync(FULL, st != ST_RUN || pc == pn);
-    }
-    k = bv->k0;
-    omin = 4u * k;                               // every clock was reset to 4 * k0
-    epoch = bv->epoch;
-    epoch_hi = epoch << 6;
-    front_cap = log_cap - 2u * bv->n_misc;
-  }
-
-  // ---- block finished
-  const uint32_t wi = __reduce_add_sync(FULL, n_instr), wg = __reduce_add_sync(FULL, n_gacc);
-  const uint32_t ws = __reduce_add_sync(FULL, n_sacc);
-  if (lane == 0) {
-    atomicAdd(&A.counters->thread_instrs, (unsigned long long)wi);
-    if (wg) atomicAdd(&A.counters->global_accesses, (unsigned long long)wg);
-    if (ws) atomicAdd(&A.counters->shared_accesses, (unsigned long long)ws);
-  }
-  if (tid == 0) {
-    const uint32_t front = log_cap - 2u * bv->n_misc;
-    BlockRes r;
-    r.n_log = fused ? 0u : (bv->cursor < front ? bv->cursor : front);   // fused: no records to check
-    r.n_race = fused ? bv->race_out : 0u;
-    r.n_misc = bv->n_misc;
-    r.flags = bv->flags;
-    A.blocks[Ls->block_base + block] = r;
-    if (Global && gcap) {
-      const uint32_t ng = bv->gcursor < gcap ? bv->gcursor : gcap;
-      A.glog_n[gb] = ng;
-      if (ng) atomicAdd(&A.counters->global_records, (unsigned long long)ng);
-    }
-    if (r.n_log) atomicAdd(&A.counters->shared_accesses, (unsigned long long)r.n_log);
-    const uint32_t bits = bv->status | ((bv->flags & BF_OVERFLOW) ? (uint32_t)SR_ST_LOG_OVERFLOW : 0u) |
-                          ((bv->flags & BF_INTERNAL) ? (uint32_t)SR_ST_INTERNAL : 0u);
-    if (bits) atomicOr(&A.prog_status[Ls->prog], bits);
-    if (bits & (SR_ST_DEADLOCK | SR_ST_STEP_LIMIT | SR_ST_INTERNAL)) atomicOr(&A.launch_dead[Ls->index], 1u);
+    bv->sreg[0] = block + Ls->block_off;
+    bv->sreg[1] = Ls->bdim;
+    bv->sreg[2] = Ls->gdim;
+    bv->sreg[3] = 32u;
+    SoloConst* sc = reinterpret_cast<SoloConst*>(gsm + kGroupConst);
+    sc->irs = smem_u32(ir);
+    sc->rb = smem_u32(ir) + ir_code_bytes(ncode) - smem_u32(ir) / 8u;
+    sc->shs = smem_u32(gsm + G.sh);
+    sc->sha = sha;
+    sc->arena = reinterpret_cast<unsigned long long>(A.arena + Ls->arena_off);
+    sc->arena_words = (uint32_t)Ls->arena_words;
+    sc->spin = A.spin_limit;
+    sc->budget4 = 4u * A.budget;
+    sc->nthr = nthr;
+    sc->nw = nw;
+    sc->tup = smem_u32(gsm + G.tup);
+    sc->tps4 = 4u * tps;
+    sc->region = reinterpret_cast<unsigned long long>(A.log + Ls->log_base + (unsigned long long)block * Ls->log_cap);
+    sc->wb = smem_u32(gsm + G.wb);
+    sc->gcap = Ls->glog_cap;
+    sc->gblock = Ls->block_base + block;
+    sc->gregion = reinterpret_cast<unsigned long long>(A.glog + Ls->glog_base + (unsigned long long)block * Ls->glog_cap);
   }
 }
 
@@ -946,174 +685,809 @@ __device__ __forceinline__ bool deps_dead(const RunArgs& A, const LaunchDev& L) 
   return (L.dep_prev != kNoDep && dead[L.dep_prev]) || (L.dep_wait != kNoDep && dead[L.dep_wait]);
 }
 
-// Thread 0 of a CTA, batched mode: wait (bounded) until every block of the launches L follows
+// Warp 0 of a CTA, batched mode: wait (bounded) until every block of the launches L follows
 // (the previous launch of its stream, the one it waits for) has completed - they hold earlier
 // places in the queue, so CTAs that never wait on L's blocks run them - and decide whether L is
-// skipped: a wait that gave up marks the program SR_ST_INTERNAL, and a launch that stopped or
-// was skipped skips L (deps_dead).  A skipped launch is marked in launch_dead.
-__device__ __forceinline__ bool wait_deps(const RunArgs& A, const LaunchDev& L) {
-  bool skip = false;
-  const uint32_t deps[2] = {L.dep_prev, L.dep_wait};
-  for (uint32_t j = 0; j < 2 && !skip; ++j) {
-    if (deps[j] == kNoDep) continue;
-    const uint32_t need = A.launches[deps[j]].grid;
-    bool ok = false;
-    for (uint32_t s = 0; s < A.spin_limit; ++s) {
-      if (ld_acquire_gpu(&A.launch_done[deps[j]]) >= need) { ok = true; break; }
-      __nanosleep(128);
-    }
-    if (!ok) {
-      skip = true;
-      atomicOr(&A.prog_status[L.prog], (uint32_t)SR_ST_INTERNAL);
+// skipped (*skip set): a wait that gave up marks the program SR_ST_INTERNAL, and a launch that
+// stopped or was skipped skips L (deps_dead).  A skipped launch is marked in launch_dead.
+__device__ __forceinline__ void wait_deps(const RunArgs& A, const LaunchDev& L, uint32_t* skip) {
+  bool give_up = false;
+#pragma unroll 1
+  for (uint32_t j = 0; j < 2 && !give_up; ++j) {
+    const uint32_t dep = same(j ? L.dep_wait : L.dep_prev);
+    if (dep == kNoDep) continue;
+    const uint32_t need = same(A.launches[dep].grid);
+    uint32_t s = 0;
+    while (same(ld_acquire_gpu(&A.launch_done[dep])) < need) {
+      if (++s >= A.spin_limit) {
+        give_up = true;
+        break;
+      }
+      __nanosleep(32);
     }
   }
-  if (!skip && deps_dead(A, L)) skip = true;
-  if (skip) atomicOr(&A.launch_dead[L.index], 1u);
-  return skip;
+  if (threadIdx.x == 0) {
+    if (give_up) atomicOr(&A.prog_status[L.prog], (uint32_t)SR_ST_INTERNAL);
+    if (give_up || deps_dead(A, L)) {
+      atomicOr(&A.launch_dead[L.index], 1u);
+      *skip = 1u;
+    }
+  }
+  __syncwarp();
+}
+
+// Run one simulated block on warps [0, Ls->nw) of the CTA, V simulated warps per warp.  The fused race check is compiled in only where Fused is set, and
+// the logging of global accesses only where Global is set, so that the default kernels keep
+// their register budget.
+//
+// Each agent (simulated warp) has its round count and next pc; the warp executes one
+// instruction for a set of agents at the same pc and round.  Nearly always the set holds
+// every agent that can run (`solo`): then only (p, k) are kept, in registers, and the decoding
+// and dispatch of an instruction is paid once for V simulated warps.  Threads of an agent
+// that wait at a higher pc for the lowest-pc rule to reach them do not end that (`wpc`: the
+// lowest such pc).  Otherwise the agents' states sit in lanes 0..V-1 (ap next pc, ak round,
+// aw lowest waiting pc) and the set with the lowest round runs, at one round first loads and
+// everything that touches no memory, then stores, then atomics.
+template <int V, bool Fused, bool Global>
+__device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls, uint32_t block,
+                                          const uint2* __restrict__ ir, unsigned char* gsm) {
+  const uint32_t w = same(threadIdx.x >> 5), nw = same(Ls->nw);
+  constexpr uint32_t ALL = (1u << V) - 1u;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t nthr = nw * 32;
+  const uint32_t t = w * 32 + lane;              // thread of the group
+  const uint32_t tid0 = w * 32 * V + lane;       // simulated thread of slot 0 (slot j: + 32 j)
+  const uint32_t bdim = Ls->bdim, shw = same(Ls->shw), sha = same(Ls->sha), ncode = same(Ls->ncode), log_cap = same(Ls->log_cap);
+  const uint32_t nrows = same(Ls->nrows);
+  const bool uninit = same(Ls->uninit) != 0;
+  const bool fused = Fused && same(Ls->fused) != 0 && A.check_races != 0;
+  const GroupLayout G = group_layout(nthr * V, sha, ncode, nrows, Ls->uninit, Ls->fused);
+  int32_t* sh = reinterpret_cast<int32_t*>(gsm + G.sh);
+  uint32_t* clk = reinterpret_cast<uint32_t*>(gsm + kGroupClk);
+  const uint32_t gb = same(smem_u32(gsm)), clks = gb + kGroupClk + 4u * lane, myclk = gb + kGroupClk + 4u * w;
+  const uint32_t ranges = gb + kGroupRange;
+  const bool pad = lane >= nw || lane == w;      // (of wait_clocks)
+  uint32_t* err = reinterpret_cast<uint32_t*>(gsm + G.err);
+  uint32_t* un = reinterpret_cast<uint32_t*>(gsm + G.un);      // with `uninit` only
+  uint32_t* wb = reinterpret_cast<uint32_t*>(gsm + G.wb);      // with `uninit` only
+  uint32_t* tup = reinterpret_cast<uint32_t*>(gsm + G.tup);    // with `fused` only
+  const uint32_t tps = tuple_plane_words(sha);
+  uint32_t* rbm = reinterpret_cast<uint32_t*>(gsm + G.rbm);
+  BlockVars* bv = reinterpret_cast<BlockVars*>(gsm + kGroupBv);
+  int32_t* arena = A.arena + Ls->arena_off;
+  const uint32_t arena_words = same((uint32_t)Ls->arena_words);
+  unsigned long long* region = A.log + Ls->log_base + (unsigned long long)block * log_cap;
+  const bool logging = A.check_races != 0;
+  // global log of this block (with Global, for launches whose glog_cap is set)
+  const uint32_t gcap = Global ? Ls->glog_cap : 0u;
+  const uint32_t gblock = Ls->block_base + block;
+  uint4* gregion = Global ? A.glog + Ls->glog_base + (unsigned long long)block * gcap : nullptr;
+  const uint32_t budget = A.budget, spin = A.spin_limit;
+  // 32-bit shared-window addresses: row r of this lane is at rs + r * rstride
+  const uint32_t rs = smem_u32(gsm + G.regs) + t * (4u * V), rstride = nthr * (4u * V);
+  const uint32_t shs = smem_u32(sh), irs = smem_u32(ir);
+  const bool pub = lane == 0 && nw > 1;          // this thread publishes the warp's clock
+
+  uint32_t ts[V], xm = 0;                        // state words; xm: slots without a thread, or exited
+  uint32_t p = same(Ls->entry), k = 0, wpc = kInf;     // the running set: pc, round, lowest waiting pc
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    const bool none = tid0 + 32u * j >= bdim;
+    ts[j] = p | (none ? ST_NONE : ST_RUN) << 16;
+    xm |= (none ? 1u : 0u) << j;
+  }
+  uint32_t am = ALL & ~xm;                       // its active slots of this lane
+  // every slot whose registers still matter is active; ns: slots 0 .. ns - 1 are active in every
+  // lane and no others (0: the active threads form no such shape)
+  bool whole;
+  uint32_t ns;
+  auto set_shape = [&]() {
+    whole = __all_sync(FULL, (am | xm) == ALL);
+    const uint32_t m = same(am);
+    ns = __all_sync(FULL, am == m) && (m & (m + 1u)) == 0 ? __popc(m) : 0u;
+  };
+  set_shape();
+  uint32_t nexit = 0;                            // exited threads of the warp
+  bool errs = false;                             // the warp noted errors in this interval
+  uint32_t sub = ALL;                            // its agents
+  bool solo = true;                              // it holds every agent that can run
+  uint32_t ak = 0, ap = kInf, aw = kInf;         // lanes 0..V-1: the agents, while not solo
+  uint32_t epoch = 0, front_cap = log_cap;
+  uint32_t par = 0;                              // the barrier interval's parity, in bit 31
+  uint32_t n_instr = 0, n_gacc = 0;              // per lane: executed instructions, global accesses
+  uint32_t n_sacc = 0;                           // per lane, fused race check: shared accesses
+  bool lfull = false;
+  // a log record is built from 32-bit halves: low = addr << 24 | tid << 14 | kind << 12 | pc,
+  // high = epoch << 6 | addr >> 8
+  const uint32_t lane_rec = tid0 << 14;
+  uint32_t epoch_hi = 0;                         // epoch << 6
+  enum : uint32_t { GO, PICK, RESCHED };
+  uint32_t how = GO;
+  uint32_t kn = 0;                               // not solo: the lowest round of the other agents, if memory may be
+                                                 // accessed in the rounds below it (else 0)
+  const uint32_t solo_flags = (nw > 1 ? kSoloMany : 0u) | (logging && !fused ? kSoloLog : 0u) | (fused ? kSoloFused : 0u);
+  const uint32_t solo_mem = (uninit ? kSoloUninit : kSoloShared) | (Global && gcap ? kSoloGlog : kSoloGlobal);
+
+  // (debug build) every row of the run of `len` instructions at p is in the register file
+  auto rows_ok = [&](uint32_t p, uint32_t len) {
+    bool ok = true;
+    if (kDebugBounds)
+      for (uint32_t q = p, x; q < p + len; q += pk_form(x) <= F_MULI ? pk_b(x) : 1u) {
+        x = ir[q].x;
+        ok = ok && dbg_ok(q < ncode && pk_a(x) < nrows && (pk_imm(pk_form(x)) || pk_b(x) < nrows) &&
+                              (pk_d(x) < nrows || pk_d(x) == kNoDest),
+                          &A.prog_status[Ls->prog], SR_ST_BOUNDS);
+      }
+    return ok;
+  };
+
+  for (;;) {  // barrier intervals
+    bool at_bar = false;                         // the warp's threads wait at barrier p, their states not written
+    uint32_t stop = 0;                           // 1: out of rounds, 2: a wait gave up
+    for (;;) {  // steps of the running set
+      bool multi_st = false;                     // stores of other pcs share this round
+      bool moved = false;                        // solo_loop ran some instructions
+      if (how != GO) {
+        if (how == RESCHED) {                    // the agents' next and waiting pcs from the threads'
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            const uint32_t c = ts_st(ts[j]) == ST_RUN ? ts_pc(ts[j]) : kInf;
+            const uint32_t m = __reduce_min_sync(FULL, c);
+            const uint32_t m2 = __reduce_min_sync(FULL, c != m ? c : kInf);
+            if (lane == (uint32_t)j) {
+              ap = m;
+              aw = m2;
+            }
+          }
+        }
+        const uint32_t can = __ballot_sync(FULL, ap != kInf);
+        if (!can) break;
+        k = __reduce_min_sync(FULL, ap != kInf ? ak : kInf);
+        if (k >= budget) {
+          stop = 1;
+          break;
+        }
+        const bool cand = ap != kInf && ak == k;
+        p = __shfl_sync(FULL, ap, __ffs(__ballot_sync(FULL, cand)) - 1);
+        sub = __ballot_sync(FULL, cand && ap == p);
+        solo = sub == can;
+        kn = 0;
+        if (!solo) {
+          // among the agents at this round: what touches no memory and loads, one pc at a time;
+          // then stores (agent by agent when they are at several pcs); then atomics
+          uint32_t cls = 3;
+          if (cand) {
+            const uint32_t o = pk_form(ir[ap].x);
+            cls = (o == F_STS || o == F_STG) ? 1u : o == F_ATOMS ? 2u : 0u;
+          }
+          const uint32_t first = __reduce_min_sync(FULL, cls);
+          const uint32_t of = __ballot_sync(FULL, cls == first);
+          p = __shfl_sync(FULL, ap, __ffs(of) - 1);
+          sub = __ballot_sync(FULL, cls == first && ap == p);
+          if (first == 1 && (sub != of || clk[w] == 4u * k + 1u + par)) {
+            multi_st = true;                     // (also for the last of them)
+            sub &= 0u - sub;
+          }
+        }
+        wpc = __reduce_min_sync(FULL, (sub >> lane) & 1u ? aw : kInf);
+        am = 0;
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+          if (((sub >> j) & 1u) && ts_st(ts[j]) == ST_RUN && ts_pc(ts[j]) == p) am |= 1u << j;
+        set_shape();
+        __syncwarp();
+        st_release_if(pub && 4u * k + par > clk[w], myclk, 4u * k + par);
+        how = GO;
+      } else if (k >= budget) {                  // (solo)
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+          if ((am >> j) & 1u) ts[j] = p;
+        ak = k;
+        stop = 1;
+        break;
+      }
+      if (!kDebugBounds) {
+        // Most instructions run in solo_loop; what it does not take is left at (p, k).  While other
+        // agents are at later rounds, it runs up to their lowest; with some at the same round, it runs
+        // ahead over what touches no memory.
+        const uint32_t k_in = k;
+        uint32_t q = same(irs + p * 8u), k4 = same(4u * k + par), eh = same(epoch_hi);
+        uint32_t qw = same(wpc == kInf ? 0xFFFFFFF8u : irs + wpc * 8u);
+        uint32_t fl = solo_flags | (whole ? kSoloWhole : 0u) | (ns ? kSoloRegular : 0u) | (lfull ? kSoloFull : 0u);
+        if (solo) fl |= kSoloSolo;
+        if (solo || kn) fl |= kSoloPub | solo_mem;
+        if (solo && whole && nexit == 0 && !errs && !fused && wpc == kInf) fl |= kSoloBar;
+        fl = same(fl);
+        const uint32_t mask = solo_loop<V, Fused>(q, k4, n_gacc, n_sacc, eh, n_instr, fl, qw, gb, w, rs, rstride, am,
+                                                  same(front_cap), same(4u * (solo || !kn ? budget : kn) + par));
+        fl = same(fl);
+        lfull = (fl & kSoloFull) != 0;
+        p = (same(q) - irs) >> 3;
+        k4 = same(k4);
+        par = k4 & 0x80000000u;
+        k = (k4 - par) >> 2;
+        epoch_hi = same(eh);
+        epoch = epoch_hi >> 6;
+        moved = k != k_in;
+        if (fl & kSoloNested) {
+          // some threads wait at a higher pc (at a barrier: agents without a running thread have
+          // executed it)
+          wpc = (same(qw) - irs) >> 3;
+          am = mask & ALL;
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            const bool at = (fl & kSoloAgents) && !__any_sync(FULL, (am >> j) & 1u);
+            if ((mask >> (4 + j)) & 1u) {
+              ts[j] = at ? (wpc + 1u) | ST_WAIT << 16 : wpc;
+              n_instr += at;
+            }
+          }
+          set_shape();
+        }
+        if (fl & kSoloAtBar) {
+          at_bar = true;
+          break;
+        }
+        if (fl & kSoloTimeout) {
+          stop = 2;
+          break;
+        }
+        if (solo && k >= budget) continue;
+      }
+      if (p < wpc && (solo || !moved)) {
+      const uint2 in = lds_u64(irs + p * 8u);
+      const uint32_t f = pk_form(in.x), run = f < F_LDS ? lds_u8(irs + ir_code_bytes(ncode) + p) : 0u;
+      if (run) {
+        // A run of instructions that touch no memory and do not branch executes in a tight loop,
+        // one instruction per round; its last round is published at once (other warps wait on
+        // a clock only for memory effects).
+        const uint32_t len = min(min(run, budget - k), wpc - p);
+        if (!rows_ok(p, len)) {                  // stop the block the way a wait that gave up does
+          stop = 2;
+          break;
+        }
+        st_release_if(solo && pub, myclk, 4u * (k + len) + par);
+        alu_run<V>(in.x, in.y, irs + p * 8u, irs + (p + len) * 8u, rs, rstride, whole, am);
+        n_instr += len * __popc(am);
+        p += len;
+        k += len;
+      } else {
+        const uint32_t d = pk_d(in.x), ra = rs + pk_a(in.x) * rstride, rb = rs + pk_b(in.x) * rstride;
+        const uint32_t imm = in.y;
+        if (!dbg_ok(p <= ncode && pk_a(in.x) < nrows && pk_b(in.x) < nrows && (d < nrows || d == kNoDest),
+                    &A.prog_status[Ls->prog], SR_ST_BOUNDS)) {
+          stop = 2;                              // (debug build) stop the block like a failed wait
+          break;
+        }
+        n_instr += __popc(am);
+        if (f <= F_STS || (f >= F_LDG && f <= F_ATOMS)) {
+          const bool shared = f != F_LDG && f != F_STG;
+          const uint32_t bound = shared ? sha : arena_words;
+          uint32_t ad[V], im = 0;                // addresses; im: active slots whose address is in bounds
+          bool past = false;                     // a shared address in bounds that shared_reach ruled out
+          lds_v<V>(ra, ad);
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            ad[j] += imm;
+            im |= (ad[j] < bound ? 1u : 0u) << j;
+            past = past || (((am >> j) & 1u) && shared && ad[j] >= sha && ad[j] < shw);
+          }
+          im &= am;
+          if (__any_sync(FULL, past)) {          // (never: stop the block rather than leave it out)
+            stop = 2;
+            break;
+          }
+          uint32_t kind = K_R;
+          if (f == F_LDS || f == F_LDG) {
+            if (nw > 1 && !wait_clocks(clks, ranges, pad, w, lane, 4u * k + par, false, 0, 0, 0, spin)) {
+              stop = 2;
+              break;
+            }
+            uint32_t v[V];
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+              const bool me = (im >> j) & 1u;
+              v[j] = lds_if(me && shared, shs + ad[j] * 4u);
+              if (me && !shared) v[j] = (uint32_t)arena[ad[j]];
+            }
+            put_row<V>(rs, rstride, d, v, am, whole);
+            if (shared && uninit) {              // words no store or atomic of an earlier round wrote
+#pragma unroll
+              for (int j = 0; j < V; ++j) {
+                const uint32_t um = __ballot_sync(
+                    FULL, ((im >> j) & 1u) && !((wb[ad[j] >> 5] >> (ad[j] & 31u)) & 1u));
+                if (um) {
+                  errs = true;
+                  note_err(un, bv, p, w * V + j, um, lane);
+                }
+              }
+            }
+          } else if (f == F_ATOMS) {
+            kind = K_A;
+            uint32_t v[V];
+            lds_v<V>(rb, v);
+            if (nw > 1) {
+              st_release_if(pub, myclk, 4u * k + 2u + par);
+              if (!wait_clocks(clks, ranges, pad, w, lane, 4u * k + 2u + par, false, 0, 0, 0, spin)) {
+                stop = 2;
+                break;
+              }
+            }
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+              if ((im >> j) & 1u) atomicAdd(&sh[ad[j]], (int32_t)v[j]);
+          } else {
+            kind = K_W;
+            uint32_t v[V];
+            lds_v<V>(rb, v);
+            if (nw > 1) {
+              int32_t lo = INT_MAX, hi = INT_MIN;
+#pragma unroll
+              for (int j = 0; j < V; ++j)
+                if ((im >> j) & 1u) {
+                  lo = min(lo, (int32_t)ad[j]);
+                  hi = max(hi, (int32_t)ad[j]);
+                }
+              lo = __reduce_min_sync(FULL, lo);
+              hi = __reduce_max_sync(FULL, hi);
+              // stores of several pcs in this round: any address of either space, from the first on
+              sts_u128_if(pub, ranges + 16u * w, (uint32_t)(multi_st ? INT_MIN : lo), (uint32_t)(multi_st ? INT_MAX : hi),
+                          multi_st ? 2u : shared ? 1u : 0u, 0u);
+              st_release_if(pub, myclk, 4u * k + 1u + par);
+              if (!wait_clocks(clks, ranges, pad, w, lane, 4u * k + 1u + par, true, lo, hi, shared ? 1u : 0u, spin)) {
+                stop = 2;
+                break;
+              }
+            }
+            // Several threads on one word: the highest tid's store is the one kept.  Consecutive
+            // addresses (address - tid equal over the storing threads) cannot collide; any other
+            // pattern stores slot by slot (tids ascend with the slot), in each slot the highest
+            // lane of a word.
+            const uint32_t m0 = __ballot_sync(FULL, im & 1u);
+            const uint32_t ref = __shfl_sync(FULL, ad[0] - lane, m0 ? __ffs(m0) - 1 : 0);
+            bool consec = m0 != 0 || !(im & 1u);
+#pragma unroll
+            for (int j = 0; j < V; ++j) consec = consec && (!((im >> j) & 1u) || ad[j] - lane - 32u * j == ref);
+            if (m0 != 0 && __all_sync(FULL, consec)) {
+#pragma unroll
+              for (int j = 0; j < V; ++j)
+              {
+                const bool me = (im >> j) & 1u;
+                sts_if(me && shared, shs + ad[j] * 4u, v[j]);
+                if (me && !shared) arena[ad[j]] = (int32_t)v[j];
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < V; ++j) {
+                const bool me = (im >> j) & 1u;
+                const uint32_t m = __ballot_sync(FULL, me);
+                if (m) {
+                  const uint32_t off = __shfl_sync(FULL, ad[j] - lane, __ffs(m) - 1);
+                  bool last = me;
+                  if (!__all_sync(FULL, !me || ad[j] - lane == off)) {
+                    const uint32_t grp = __match_any_sync(FULL, me ? ad[j] : (0x80000000u | lane));
+                    last = me && lane == 31u - __clz(grp);
+                  }
+                  sts_if(last && shared, shs + ad[j] * 4u, v[j]);
+                  if (last && !shared) arena[ad[j]] = (int32_t)v[j];
+                  __syncwarp();
+                }
+              }
+            }
+          }
+          if (shared && uninit && kind != K_R) {
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+              if ((im >> j) & 1u) atomicOr(&wb[ad[j] >> 5], 1u << (ad[j] & 31u));
+          }
+          if (__any_sync(FULL, im != am)) {
+            errs = true;
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+              const uint32_t em = __ballot_sync(FULL, ((am & ~im) >> j) & 1u);
+              if (em) note_err(err, bv, p, w * V + j, em, lane);
+            }
+          }
+          if (shared) {
+            if (fused) {
+#pragma unroll
+              for (int j = 0; j < V; ++j) tuple_add(tup, tps, (im >> j) & 1u, ad[j], tid0 + 32u * j, kind, p);
+              n_sacc += __popc(im);
+            } else if (logging) {
+              log_wide<V>(bv, region, front_cap, im, ad, epoch_hi, lane_rec | kind << 12 | p, lane, lfull);
+            }
+          } else {
+            n_gacc += __popc(am);
+            if (Global && gcap) {
+#pragma unroll
+              for (int j = 0; j < V; ++j)
+                log_global(bv, gregion, gcap, (im >> j) & 1u,
+                           make_uint4(ad[j], epoch, (tid0 + 32u * j) << 16 | kind << 12 | p, gblock), lane);
+            }
+          }
+          ++p;
+          ++k;
+          // every lane's access is ordered before the clock (warp barrier, then a release)
+          __syncwarp();
+        } else if (f >= F_DIVR && f <= F_REMI) {
+          uint32_t a[V], b[V], zm = 0;
+          lds_v<V>(ra, a);
+          if (f == F_DIVI || f == F_REMI) {
+#pragma unroll
+            for (int j = 0; j < V; ++j) b[j] = imm;
+          } else {
+            lds_v<V>(rb, b);
+          }
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            const int32_t x = (int32_t)a[j], y = (int32_t)b[j];
+            const int32_t s = (y == 0 || y == -1) ? 1 : y;   // (INT_MIN / -1 would trap)
+            const int32_t qt = x / s;
+            if (y == 0) {
+              zm |= 1u << j;
+              a[j] = 0u;
+            } else if (f <= F_DIVI) {
+              a[j] = y == -1 ? 0u - (uint32_t)x : (uint32_t)qt;   // -INT_MIN wraps to INT_MIN
+            } else {
+              a[j] = y == -1 ? 0u : (uint32_t)(x - qt * s);
+            }
+          }
+          put_row<V>(rs, rstride, d, a, am, whole);
+          zm &= am;
+          if (__any_sync(FULL, zm != 0)) {
+            errs = true;
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+              const uint32_t em = __ballot_sync(FULL, (zm >> j) & 1u);
+              if (em) note_err(err, bv, p, w * V + j, em, lane);
+            }
+          }
+          ++p;
+          ++k;
+        } else if (f == F_S2R) {
+          const uint32_t u = imm == SR_SREG_BID    ? block + Ls->block_off
+                             : imm == SR_SREG_BDIM ? bdim
+                             : imm == SR_SREG_GDIM ? Ls->gdim
+                                                   : 32u;
+          uint32_t v[V];
+#pragma unroll
+          for (int j = 0; j < V; ++j) v[j] = imm == SR_SREG_TID ? tid0 + 32u * j : u;
+          put_row<V>(rs, rstride, d, v, am, whole);
+          ++p;
+          ++k;
+        } else if (f == F_BRA) {
+          p = imm;
+          ++k;
+        } else if (f == F_BRZ || f == F_BRNZ) {
+          uint32_t a[V], tm = 0;                 // tm: active slots that take the branch
+          lds_v<V>(ra, a);
+#pragma unroll
+          for (int j = 0; j < V; ++j) tm |= ((a[j] == 0) == (f == F_BRZ) ? 1u : 0u) << j;
+          tm &= am;
+          ++k;
+          if (!__any_sync(FULL, tm != 0)) {
+            ++p;
+          } else if (!__any_sync(FULL, tm != am)) {
+            p = imm;
+          } else {                               // both ways: the threads' pcs part
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+              if ((am >> j) & 1u) ts[j] = (tm >> j) & 1u ? imm : p + 1u;
+            if ((sub >> lane) & 1u) ak = k;
+            how = RESCHED;
+            continue;
+          }
+        } else {
+          // barriers: the thread waits; a reducing form hands in its predicate and keeps the row
+          // its result goes to.  EXIT, and the EXIT sentinel after the last instruction.
+          const bool bar = f != F_EXIT;
+          uint32_t a[V];
+#pragma unroll
+          for (int j = 0; j < V; ++j) a[j] = 0;
+          uint32_t word = p | ST_EXIT << 16;
+          if (bar) {
+            word = (p + 1u) | ST_WAIT << 16;
+            if (f != F_BAR) {
+              lds_v<V>(ra, a);
+              word |= d << 18 | (f - F_BAR) << 23;
+            }
+          } else {
+            xm |= am;
+            nexit += __reduce_add_sync(FULL, __popc(am));
+          }
+#pragma unroll
+          for (int j = 0; j < V; ++j)
+            if ((am >> j) & 1u) ts[j] = word | (a[j] != 0 ? 1u << 25 : 0u);
+          ++k;
+          if ((sub >> lane) & 1u) ak = k;
+          if (solo && wpc == kInf) break;        // no thread of the warp can run
+          how = RESCHED;
+          continue;
+        }
+      }
+      // (p, k): the set's next instruction
+      if (solo && p < wpc) {
+        st_release_if(pub, myclk, 4u * k + par);
+        continue;
+      }
+      }
+#pragma unroll
+      for (int j = 0; j < V; ++j)
+        if ((am >> j) & 1u) ts[j] = p;
+      if ((sub >> lane) & 1u) {
+        ak = k;
+        ap = p;
+      }
+      how = p < wpc ? PICK : RESCHED;
+    }
+
+    // ---- no runnable thread in this warp (or it stopped): publish its state and park
+    // (`uni`: every waiting thread at one barrier pc and none runnable, the usual case: they
+    // all resume together after that barrier)
+    bool uni = at_bar;
+    uint32_t upc = p;
+    const uint32_t parks = gb + kGroupPark + (par ? 32u * kMaxWarps : 0u);   // the interval's park entries
+    if (!at_bar) {                               // (else solo_loop wrote it and passed the CTA barrier)
+      uint32_t n = 0, np = 0, mn = kInf, mx = 0, rp = kInf;   // counts: wait | exit << 10 | run << 20
+#pragma unroll
+      for (int j = 0; j < V; ++j) {
+        const uint32_t st = ts_st(ts[j]), c = ts_pc(ts[j]);
+        if (st == ST_WAIT) {
+          n += 1u;
+          np += ts[j] >> 25 | ((ts[j] >> 23) & 3u ? 1u << 16 : 0u);   // predicates; reducing barriers << 16
+          mn = min(mn, c - 1u);
+          mx = max(mx, c - 1u);
+        } else if (st == ST_EXIT) {
+          n += 1u << 10;
+        } else if (st == ST_RUN) {
+          n += 1u << 20;
+          rp = min(rp, c);
+        }
+      }
+      n = __reduce_add_sync(FULL, n);
+      np = __reduce_add_sync(FULL, np);
+      mn = __reduce_min_sync(FULL, mn);
+      mx = __reduce_max_sync(FULL, mx);
+      rp = __reduce_min_sync(FULL, rp);
+      const uint32_t kx = __reduce_max_sync(FULL, lane < (uint32_t)V ? ak : 0u);
+      uni = (n >> 20) == 0 && (n & 0x3FFu) != 0 && mn == mx;
+      upc = mn;
+      sts_u128_if(lane == 0, parks + 32u * w, n & 0x3FFu, (n >> 10) & 0x3FFu, n >> 20, mn);
+      sts_u128_if(lane == 0, parks + 32u * w + 16u, mx, rp, kx, stop | (errs ? 4u : 0u) | np << 8);
+      st_release_if(pub, myclk, par | 0x7FFFFFFFu);
+      block_sync(nthr);
+    }
+    if (fused) {                                 // the interval's touched words, all warps
+      tuples_mark(tup, tps, rbm, &bv->any_race[par >> 31], w, nw, lane);
+      block_sync(nthr);
+    }
+
+    // ---- barrier resolution.  Every thread of the block waits at one plain barrier and there is
+    // nothing to report: each warp sees that in the park entries and goes on by itself (the other
+    // interval's entries are written next, so none is overwritten while a warp still reads it).
+    // Otherwise warp 0 resolves the barrier and a second CTA barrier follows.
+    const bool v = lane < nw;
+    uint4 pa, pb;                                // warp `lane`'s entry
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(pa.x), "=r"(pa.y), "=r"(pa.z), "=r"(pa.w) : "r"(parks + 32u * (lane & 7u)) : "memory");
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(pb.x), "=r"(pb.y), "=r"(pb.z), "=r"(pb.w) : "r"(parks + 32u * (lane & 7u) + 16u) : "memory");
+    const uint32_t kmax = __reduce_max_sync(FULL, v ? pb.z : 0u);
+    const uint32_t pc0 = same(pa.w);
+    if (!(fused && same(bv->any_race[par >> 31])) &&
+        __all_sync(FULL, !v || (pa.x && !(pa.y | pa.z | pb.w) && pa.w == pc0 && pb.x == pc0))) {
+      epoch += 1u;
+    } else {
+      if (w == 0) {
+        const uint32_t nW = __reduce_add_sync(FULL, v ? pa.x : 0u);
+        const uint32_t nX = __reduce_add_sync(FULL, v ? pa.y : 0u);
+        const uint32_t nR = __reduce_add_sync(FULL, v ? pa.z : 0u);
+        const uint32_t pmn = __reduce_min_sync(FULL, v ? pa.w : kInf);
+        const uint32_t pmx = __reduce_max_sync(FULL, v ? pb.x : 0u);
+        const uint32_t rpc = __reduce_min_sync(FULL, v ? pb.y : kInf);
+        const uint32_t fl = __reduce_or_sync(FULL, v ? pb.w & 0xFFu : 0u);
+        const uint32_t nP = __reduce_add_sync(FULL, v ? (pb.w >> 8) & 0xFFFFu : 0u);
+        if (fused && bv->any_race[par >> 31]) {
+          tuples_emit(tup, tps, rbm, bv, region, log_cap - 2u * bv->n_misc, epoch, lane);
+          if (lane == 0) bv->any_race[par >> 31] = 0;
+        }
+        uint32_t dec = DEC_RELEASE, kind = 0, a = 0, b = 0, c = 0, stbits = 0;
+        if (fl & 2u) {
+          dec = DEC_STOP;
+          if (lane == 0) bv->flags |= BF_INTERNAL;
+        } else if (fl & 1u) {          // out of rounds
+          dec = DEC_STOP; kind = SR_REP_STEP_LIMIT; a = budget; b = nR; c = rpc; stbits = SR_ST_STEP_LIMIT;
+        } else if (nW == 0) {          // every thread exited
+          dec = DEC_DONE;
+        } else if (nX > 0) {           // some wait at a barrier that exited threads never reach
+          dec = DEC_STOP; kind = SR_REP_DEADLOCK; a = pmn; b = pmx; c = nW << 16 | nX; stbits = SR_ST_DEADLOCK;
+        } else if (pmn != pmx) {       // all wait: release, flag differing barrier pcs
+          kind = SR_REP_DIVERGENCE; a = pmn; b = pmx; c = nW << 16;
+        }
+        if (lane == 0 && kind) push_misc(bv, region, log_cap, kind, epoch, a, b, c);
+        __syncwarp();
+        if (bv->err_dirty) flush_errors(bv, err, uninit ? un : nullptr, ir, ncode, region, log_cap, epoch, lane);
+        if (lane == 0) {
+          bv->decision = dec;
+          bv->status |= stbits;
+          bv->bar_np = nP;
+          bv->bar_nw = nW;
+        }
+      }
+      block_sync(nthr);
+      if (same(bv->decision) != DEC_RELEASE) break;
+      front_cap = log_cap - 2u * same(bv->n_misc);
+      epoch += 1u;
+    }
+    k = ak = kmax;
+    par ^= 0x80000000u;
+    errs = false;
+    epoch_hi = epoch << 6;
+    st_release_if(pub, myclk, 4u * k + par);
+    if (at_bar) {
+      ++p;                                       // (the set stays as it is)
+    } else {
+      am = 0;
+#pragma unroll
+      for (int j = 0; j < V; ++j)
+        if (ts_st(ts[j]) == ST_WAIT) {
+          // a reducing barrier's result, over every released thread's predicate
+          const uint32_t kind = (ts[j] >> 23) & 3u, row = (ts[j] >> 18) & 31u;
+          if (kind && row != kNoDest) {
+            const uint32_t np = bv->bar_np;
+            sts_u32(rs + row * rstride + 4u * j,
+                    kind == 1 ? (np == bv->bar_nw ? 1u : 0u) : kind == 2 ? (np ? 1u : 0u) : np);
+          }
+          ts[j] = ts_pc(ts[j]);                  // runs on after its barrier
+          am |= 1u << j;
+        }
+      set_shape();
+      how = RESCHED;
+      if (uni) {                                 // every released thread resumes after its barrier
+        p = upc + 1u;
+        wpc = kInf;
+        sub = ALL;
+        solo = true;
+        how = GO;
+      }
+    }
+  }
+
+  // ---- block finished
+  const unsigned long long wi = warp_sum(n_instr), wg = warp_sum(n_gacc);
+  const unsigned long long ws = Fused ? warp_sum(n_sacc) : 0ull;
+  if (lane == 0) {
+    atomicAdd(&A.counters->thread_instrs, wi);
+    if (wg) atomicAdd(&A.counters->global_accesses, wg);
+    if (ws) atomicAdd(&A.counters->shared_accesses, ws);
+  }
+  if (t == 0) {
+    const uint32_t front = log_cap - 2u * bv->n_misc;
+    BlockRes r;
+    r.n_log = fused ? 0u : (bv->cursor < front ? bv->cursor : front);   // fused: no records to check
+    r.n_race = fused ? bv->race_out : 0u;
+    r.n_misc = bv->n_misc;
+    r.flags = bv->flags;
+    A.blocks[Ls->block_base + block] = r;
+    if (Global && gcap) {
+      const uint32_t ng = bv->gcursor < gcap ? bv->gcursor : gcap;
+      A.glog_n[gblock] = ng;
+      if (ng) atomicAdd(&A.counters->global_records, (unsigned long long)ng);
+    }
+    if (r.n_log) atomicAdd(&A.counters->shared_accesses, (unsigned long long)r.n_log);
+    const uint32_t bits = bv->status | ((bv->flags & BF_OVERFLOW) ? (uint32_t)SR_ST_LOG_OVERFLOW : 0u) |
+                          ((bv->flags & BF_INTERNAL) ? (uint32_t)SR_ST_INTERNAL : 0u);
+    if (bits) atomicOr(&A.prog_status[Ls->prog], bits);
+    if (bits & (SR_ST_DEADLOCK | SR_ST_STEP_LIMIT | SR_ST_INTERNAL)) atomicOr(&A.launch_dead[Ls->index], 1u);
+  }
+}
+
+// Warp 0 of a CTA: its launch's descriptor into shared memory.
+__device__ __forceinline__ void copy_launch(LaunchDev* dst, const LaunchDev* src) {
+  static_assert(sizeof(LaunchDev) % 4 == 0, "copied by words");
+  for (uint32_t i = threadIdx.x; i < sizeof(LaunchDev) / 4; i += 32)
+    reinterpret_cast<uint32_t*>(dst)[i] = __ldg(reinterpret_cast<const uint32_t*>(src) + i);
+  __syncwarp();
+}
+
+// The CTA's block once its launch is known and its code is under way: clear, wait for the code,
+// run (unless warp 0 has found, before it comes here, that the launch is skipped).
+template <int V, bool Fused, bool Global>
+__device__ __forceinline__ void run_staged(const RunArgs& A, const LaunchDev* Ls, uint32_t block, unsigned char* smem,
+                                           unsigned long long* mbar, const uint32_t* skip) {
+  // every thread must take the same branch before the block's named barriers
+  const bool mine = __all_sync(FULL, (threadIdx.x >> 5) < Ls->nw);
+  if (mine) start_block<V, Fused>(A, Ls, block, smem, smem + Ls->ir_bytes);
+  bool drained;
+  if (!__any_sync(FULL, stage_wait(mbar, 0, drained))) {           // (its barrier also ends the clearing)
+    if (threadIdx.x == 0) atomicOr(&A.prog_status[Ls->prog], (uint32_t)SR_ST_INTERNAL);
+  } else if (mine && !same(*skip)) {
+    run_block<V, Fused, Global>(A, Ls, block, reinterpret_cast<const uint2*>(smem), smem + Ls->ir_bytes);
+  }
 }
 
 // One CTA per simulated block; one kernel launch per (program, launch), in an order that
-// respects every stream and wait.  MINB = 2 caps registers so that two 1024-thread CTAs fit
-// an SM.
-template <int MINB, bool Fused, bool Global>
-__global__ void __launch_bounds__(1024, MINB) k_interp_plain(RunArgs A, uint32_t li) {
+// respects every stream and wait.  A block takes block_warps(bdim, V) warps: at most 8 with
+// V = 4, two with V = 1 and 2 (block_vec).  MINB: CTAs of that many warps the registers allow.
+template <int V, int MINB, bool Fused, bool Global>
+__global__ void __launch_bounds__(V == 4 ? 256 : 64, MINB) k_interp_plain(RunArgs A, uint32_t li) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ LaunchDev Ls;
   __shared__ __align__(8) unsigned long long mbar;
   __shared__ uint32_t s_skip;
-  if (threadIdx.x == 0) {
-    Ls = A.launches[li];
-    // (the launches before this one have completed: they ran earlier on this CUDA stream)
-    s_skip = deps_dead(A, Ls);
-    if (s_skip) atomicOr(&A.launch_dead[Ls.index], 1u);
-    if (!s_skip) {
-      mbar_init(&mbar);
-      bulk_load(smem, A.code + Ls.code_off, Ls.ir_bytes, &mbar);
-    }
-  }
-  __syncthreads();
-  if (s_skip) return;
-  // every thread must take the same branch before the block's named barriers
-  bool drained;
-  if (!stage_wait(&mbar, 0, drained)) {
-    if (threadIdx.x == 0) atomicOr(&A.prog_status[Ls.prog], (uint32_t)SR_ST_INTERNAL);
-    return;
-  }
-  run_block<Fused, Global>(A, &Ls, blockIdx.x, reinterpret_cast<const uint2*>(smem), smem + Ls.ir_bytes,
-                           threadIdx.x >> 5, blockDim.x >> 5, 1);
-}
-
-// Persistent: CTAs pop (launch, first block) items from a device queue; an item's
-// `item_blocks` simulated blocks run `groups` at a time side by side, each group on its own
-// warps and named barrier, a group taking the item's next unclaimed block when it finishes one.
-// Items are ordered launch-wave by launch-wave, and an item waits (bounded) until every
-// block of the launches it follows (the previous launch of its stream, the one it waits
-// for) has completed; launches of other streams run meanwhile.
-template <int MINB, bool Fused, bool Global>
-__global__ void __launch_bounds__(1024, MINB) k_interp_batched(RunArgs A) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ LaunchDev Ls;
-  __shared__ __align__(8) unsigned long long mbar;
-  __shared__ uint32_t s_item, s_skip, s_next, s_claim[32];
-  uint32_t phase = 0;
-  if (threadIdx.x == 0) mbar_init(&mbar);
-  __syncthreads();
-  for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(A.queue_head, 1u);
-    __syncthreads();
-    const uint32_t item = s_item;
-    if (item >= A.nitems) break;
-    const uint2 it = A.items[item];
+  if (threadIdx.x < 32) {
+    copy_launch(&Ls, A.launches + li);
     if (threadIdx.x == 0) {
-      Ls = A.launches[it.x];
-      const uint32_t skip = wait_deps(A, Ls) ? 1u : 0u;
-      if (!skip) bulk_load(smem, A.code + Ls.code_off, Ls.ir_bytes, &mbar);
-      s_skip = skip;
-      s_next = Ls.groups;
-    }
-    __syncthreads();
-    const uint32_t nblk = min(Ls.item_blocks, Ls.grid - it.y);
-    bool drained = true;
-    if (!s_skip) {
-      const bool ok = stage_wait(&mbar, phase, drained);
-      phase ^= 1u;
-      const uint32_t nw = (Ls.bdim + 31) >> 5;
-      const uint32_t wid = threadIdx.x >> 5, g = wid / nw;
-      if (ok && g < Ls.groups) {
-        // block j of the item: the first `groups` one per group, the rest claimed in turn; the
-        // group barrier after each block also keeps the next block's set-up behind the last
-        // reads of this one
-        for (uint32_t j = g; j < nblk;) {
-          run_block<Fused, Global>(A, &Ls, it.y + j, reinterpret_cast<const uint2*>(smem),
-                                   smem + Ls.ir_bytes + g * Ls.group_bytes, wid - g * nw, nw, 1 + g);
-          if (wid == g * nw && (threadIdx.x & 31) == 0) s_claim[g] = atomicAdd(&s_next, 1u);
-          group_sync(1 + g, nw * 32);
-          j = s_claim[g];
-        }
+      // (the launches before this one have completed: they ran earlier on this CUDA stream)
+      s_skip = deps_dead(A, Ls);
+      if (s_skip) atomicOr(&A.launch_dead[Ls.index], 1u);
+      if (!s_skip) {
+        mbar_init(&mbar);
+        bulk_load(smem, A.code + Ls.code_off, Ls.ir_bytes, &mbar);
       }
-      if (!ok && threadIdx.x == 0) atomicOr(&A.prog_status[Ls.prog], (uint32_t)SR_ST_INTERNAL);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      atomicAdd(&A.launch_done[it.x], nblk);
-    }
-    // a staging copy still in flight owns the code buffer and the mbarrier: this CTA takes no
-    // further item (the others drain the queue)
-    if (!drained) break;
   }
+  __syncthreads();
+  if (same(s_skip)) return;
+  run_staged<V, Fused, Global>(A, &Ls, blockIdx.x, smem, &mbar, &s_skip);
 }
 
-// Batched mode with two CTAs per SM: the programs whose every launch would take one group per
-// persistent CTA (blocks of more than 512 threads, or blocks whose shared memory leaves room for
-// one) run here, one simulated block per 1024-thread CTA and two CTAs per SM, the blocks of all
-// such launches of a wave in one grid - the occupancy of the plain kernel without a launch per
-// (program, launch).  Each CTA takes the next ticket of the wave's queue; tickets follow launch
-// level, then launch index, then block, so the launches a block's launch follows hold smaller
-// tickets, taken by CTAs that are already running, and the CTA waits for them (bounded) as the
-// persistent kernel does.  No loop surrounds the block and its warps are chosen by a warp vote:
-// the block then runs with the plain kernel's register allocation (a persistent loop around it,
-// or a branch the compiler cannot see to be warp-uniform, costs several times its spills).
-__global__ void __launch_bounds__(1024, 2) k_interp_blocks(RunArgs A) {
+// Batched mode: the blocks of many launches in one grid, one simulated block per CTA.  The host
+// puts launches together that take the same kernel form and warps and about the same shared
+// memory (a bucket), so that the CTAs an SM holds follow from what these blocks need; the
+// buckets of a wave run side by side on streams of their own.  A block's place in the bucket's
+// queue is its ticket: where launches follow others, the CTAs take tickets from a counter, in
+// the order of launch level, launch and block, so that the launches a block's launch follows
+// hold smaller tickets, taken by CTAs that are already running, and the CTA waits for them
+// (bounded); else it is the CTA's index.  No loop surrounds the block and its warps are chosen
+// by a warp vote: a persistent loop around it cost several hundred bytes of spills.
+template <int V, int MINB, bool Fused, bool Global>
+__global__ void __launch_bounds__(V == 4 ? 256 : 64, MINB) k_interp_blocks(RunArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ LaunchDev Ls;
   __shared__ __align__(8) unsigned long long mbar;
-  __shared__ uint32_t s_skip, s_block, s_li;
-  if (threadIdx.x == 0) {
-    const uint32_t t = atomicAdd(A.bq_head, 1u);    // one ticket per CTA: t < the grid size
-    // the queue entry holding ticket t: the last one whose first ticket is <= t
+  __shared__ uint32_t s_skip, s_bad, s_block, s_li;
+  if (threadIdx.x < 32) {
+    const uint32_t lane = threadIdx.x;
+    uint32_t t = blockIdx.x;
+    if (A.bq_head) {                                // one ticket per CTA: t < the grid size
+      if (lane == 0) t = atomicAdd(A.bq_head, 1u);
+      t = __shfl_sync(FULL, t, 0);
+    }
+    // the queue entry holding ticket t: the last one whose first ticket is <= t; the lanes probe
+    // 32 places of [lo, hi) at a time
     uint32_t lo = 0, hi = A.bq_n;
     while (hi - lo > 1) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (A.bq_first[mid] <= t) lo = mid; else hi = mid;
+      const uint32_t step = (hi - lo + 31u) / 32u, at = lo + lane * step;
+      const uint32_t m = __ballot_sync(FULL, at < hi && __ldg(A.bq_first + at) <= t);   // (lane 0 always)
+      const uint32_t last = 31u - __clz(m);
+      lo += last * step;
+      hi = min(hi, lo + step);
     }
     const uint32_t li = A.bq_launch[lo];
-    Ls = A.launches[li];
-    s_li = li;
-    s_block = t - A.bq_first[lo];
-    bool skip = wait_deps(A, Ls);
-    if (!skip && s_block >= Ls.grid) {              // (a corrupt queue: never from load_programs)
-      skip = true;
-      atomicOr(&A.prog_status[Ls.prog], (uint32_t)SR_ST_INTERNAL);
+    copy_launch(&Ls, A.launches + li);
+    if (lane == 0) {
+      s_li = li;
+      s_block = t - A.bq_first[lo];
+      const bool bad = s_block >= Ls.grid;          // (a corrupt queue: never from load_programs)
+      if (bad) {
+        atomicOr(&A.prog_status[Ls.prog], (uint32_t)SR_ST_INTERNAL);
+      } else {
+        mbar_init(&mbar);
+        bulk_load(smem, A.code + Ls.code_off, Ls.ir_bytes, &mbar);
+      }
+      s_bad = bad ? 1u : 0u;
+      s_skip = 0;
     }
-    if (!skip) {
-      mbar_init(&mbar);
-      bulk_load(smem, A.code + Ls.code_off, Ls.ir_bytes, &mbar);
-    }
-    s_skip = skip ? 1u : 0u;
+    __syncwarp();
+    // the other warps clear their part of the block's memory while this one waits
+    asm volatile("bar.arrive 2, %0;" ::"r"(blockDim.x) : "memory");
+    if (A.bq_head && !same(s_bad)) wait_deps(A, Ls, &s_skip);
+  } else {
+    asm volatile("bar.sync 2, %0;" ::"r"(blockDim.x) : "memory");
   }
-  __syncthreads();
-  if (!s_skip) {
-    bool drained;
-    if (!stage_wait(&mbar, 0, drained)) {
-      if (threadIdx.x == 0) atomicOr(&A.prog_status[Ls.prog], (uint32_t)SR_ST_INTERNAL);
-    } else {
-      const uint32_t nw = (Ls.bdim + 31) >> 5;
-      if (__all_sync(FULL, (threadIdx.x >> 5) < nw))
-        run_block<false, false>(A, &Ls, s_block, reinterpret_cast<const uint2*>(smem), smem + Ls.ir_bytes,
-                                threadIdx.x >> 5, nw, 1);
-    }
-  }
+  if (!same(s_bad)) run_staged<V, Fused, Global>(A, &Ls, s_block, smem, &mbar, &s_skip);
+  if (!A.bq_head) return;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -1124,8 +1498,7 @@ __global__ void __launch_bounds__(1024, 2) k_interp_blocks(RunArgs A) {
 }  // namespace
 
 uint32_t interp_plain_smem(const LaunchDev& L) {
-  const uint32_t nthr = ((L.bdim + 31) / 32) * 32;
-  return L.ir_bytes + group_layout(nthr, L.shw, L.ncode, L.nrows, L.uninit, L.fused).total;
+  return L.ir_bytes + group_layout(L.nw * 32u * L.vec, L.sha, L.ncode, L.nrows, L.uninit, L.fused).total;
 }
 
 // dynamic shared memory may use what the kernel's static shared memory leaves of the opt-in limit
@@ -1138,73 +1511,58 @@ static cudaError_t allow_dynamic_smem(K kernel, uint32_t smem_optin) {
                               (int)(smem_optin - (uint32_t)fa.sharedSizeBytes));
 }
 
+// The kernels: simulated warps per warp x register budget x fused race check x global log.
+typedef void (*PlainKernel)(RunArgs, uint32_t);
+typedef void (*BlocksKernel)(RunArgs);
+template <int V, int MINB>
+static PlainKernel plain_of(bool fused, bool global) {
+  if (global) return k_interp_plain<V, MINB, false, true>;
+  return fused ? k_interp_plain<V, MINB, true, false> : k_interp_plain<V, MINB, false, false>;
+}
+static PlainKernel plain_kernel(uint32_t vec, uint32_t variant, bool fused, bool global) {
+  if (vec == 1) return plain_of<1, 12>(fused, global);
+  if (vec == 2) return plain_of<2, 12>(fused, global);
+  return variant == 2 ? plain_of<4, 4>(fused, global) : plain_of<4, 3>(fused, global);
+}
+template <int V, int MINB>
+static BlocksKernel blocks_of(bool fused, bool global) {
+  if (global) return k_interp_blocks<V, MINB, false, true>;
+  return fused ? k_interp_blocks<V, MINB, true, false> : k_interp_blocks<V, MINB, false, false>;
+}
+static BlocksKernel blocks_kernel(uint32_t vec, uint32_t variant, bool fused, bool global) {
+  if (vec == 1) return blocks_of<1, 12>(fused, global);
+  if (vec == 2) return blocks_of<2, 12>(fused, global);
+  return variant == 2 ? blocks_of<4, 4>(fused, global) : blocks_of<4, 3>(fused, global);
+}
+
 cudaError_t init_interp_attributes(uint32_t smem_optin) {
-  cudaError_t e = allow_dynamic_smem(k_interp_plain<1, false, false>, smem_optin);
-  if (e == cudaSuccess) e = allow_dynamic_smem(k_interp_plain<2, false, false>, smem_optin);
-  if (e == cudaSuccess) e = allow_dynamic_smem(k_interp_plain<1, true, false>, smem_optin);
-  if (e == cudaSuccess) e = allow_dynamic_smem(k_interp_plain<2, true, false>, smem_optin);
-  if (e == cudaSuccess) e = allow_dynamic_smem(k_interp_plain<1, false, true>, smem_optin);
-  if (e == cudaSuccess) e = allow_dynamic_smem(k_interp_plain<2, false, true>, smem_optin);
-  if (e == cudaSuccess) e = allow_dynamic_smem(k_interp_batched<1, false, false>, smem_optin);
-  if (e == cudaSuccess) e = allow_dynamic_smem(k_interp_blocks, smem_optin);
-  // (two CTAs of up to half the SM's shared memory each: the largest shared-memory carveout)
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_interp_blocks, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess) e = allow_dynamic_smem(k_interp_batched<1, true, false>, smem_optin);
-  return e == cudaSuccess ? allow_dynamic_smem(k_interp_batched<1, false, true>, smem_optin) : e;
+  cudaError_t e = cudaSuccess;
+  for (uint32_t vec = 1; vec <= 4 && e == cudaSuccess; vec *= 2)
+    for (uint32_t variant = 1; variant <= 2 && e == cudaSuccess; ++variant)
+      for (uint32_t f = 0; f < 3 && e == cudaSuccess; ++f) {
+        e = allow_dynamic_smem(plain_kernel(vec, variant, f == 1, f == 2), smem_optin);
+        if (e == cudaSuccess) e = allow_dynamic_smem(blocks_kernel(vec, variant, f == 1, f == 2), smem_optin);
+      }
+  return e;
 }
 
-// The plain-mode kernel for one launch: MINB (register budget) x fused race check x global log.
-template <int MINB>
-static void (*plain_kernel(bool fused, bool global))(RunArgs, uint32_t) {
-  if (global) return k_interp_plain<MINB, false, true>;
-  return fused ? k_interp_plain<MINB, true, false> : k_interp_plain<MINB, false, false>;
-}
-
-// variant: 1 = one CTA per SM budget (no register cap), 2 = two CTAs per SM, 0 = the one
-// with more resident warps for this launch (ties: 1)
-cudaError_t launch_interp_plain(const RunArgs& a, uint32_t li, const LaunchDev& L, uint32_t variant, cudaStream_t s) {
-  const uint32_t threads = ((L.bdim + 31) / 32) * 32;
+// variant: 1 = the larger register budget, 2 = more CTAs per SM, 0 = the one with more resident
+// warps for this launch (ties: 1)
+cudaError_t launch_interp_plain(const RunArgs& a, uint32_t li, const LaunchDev& L, uint32_t variant,
+                                uint32_t smem_per_sm, cudaStream_t s) {
+  const uint32_t threads = L.nw * 32u;
   const uint32_t smem = interp_plain_smem(L);
   const bool global = L.glog_cap != 0;
   const bool fused = L.fused != 0 && !global;
-  if (variant == 0) {
-    int b1 = 0, b2 = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, plain_kernel<1>(fused, global), (int)threads, smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, plain_kernel<2>(fused, global), (int)threads, smem);
-    variant = b2 > b1 ? 2 : 1;
-  }
-  if (variant == 2)
-    plain_kernel<2>(fused, global)<<<L.grid, threads, smem, s>>>(a, li);
-  else
-    plain_kernel<1>(fused, global)<<<L.grid, threads, smem, s>>>(a, li);
+  if (variant == 0) variant = std::min(32u / L.nw, smem_per_sm / (smem + kBlocksStaticSmem)) > 24u / L.nw ? 2 : 1;
+  plain_kernel(L.vec, variant, fused, global)<<<L.grid, threads, smem, s>>>(a, li);
   return cudaGetLastError();
 }
 
-cudaError_t launch_interp_batched(const RunArgs& a, uint32_t ctas, uint32_t smem, bool fused, bool global,
-                                  cudaStream_t s) {
-  auto k = global ? k_interp_batched<1, false, true>
-           : fused ? k_interp_batched<1, true, false> : k_interp_batched<1, false, false>;
-  k<<<ctas, 1024, smem, s>>>(a);
+cudaError_t launch_interp_blocks(const RunArgs& a, uint32_t vec, uint32_t variant, uint32_t warps, uint32_t nblocks,
+                                 uint32_t smem, bool fused, bool global, cudaStream_t s) {
+  blocks_kernel(vec, variant, fused, global)<<<nblocks, warps * 32u, smem, s>>>(a);
   return cudaGetLastError();
-}
-
-cudaError_t launch_interp_blocks(const RunArgs& a, uint32_t nblocks, uint32_t smem, cudaStream_t s) {
-  k_interp_blocks<<<nblocks, 1024, smem, s>>>(a);
-  return cudaGetLastError();
-}
-
-// Two CTAs per SM: each may use half the SM's shared memory, less the 1 KB the hardware reserves
-// per CTA and the kernel's static shared memory.
-uint32_t interp_blocks_smem_cap(uint32_t smem_per_sm) {
-  cudaFuncAttributes fa;
-  if (cudaFuncGetAttributes(&fa, k_interp_blocks) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  const uint32_t half = smem_per_sm / 2u, fixed = 1024u + (uint32_t)fa.sharedSizeBytes;
-  return half > fixed ? half - fixed : 0u;
 }
 
 }  // namespace sr

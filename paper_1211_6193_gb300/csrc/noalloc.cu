@@ -41,7 +41,7 @@ struct NoallocWave {
 // Host staging of one call (~150 KB): thread-local, so that a call needs neither heap
 // memory nor a large stack (callers on threads with small stacks).
 struct HostStaging {
-  uint2 code[SR_MAX_CODE + 2];
+  uint2 code[SR_MAX_CODE + 2 + (SR_MAX_CODE + 16) / 8];
   uint8_t colour[SR_MAX_CODE + 1];
   uint32_t acc[SR_MAX_CODE + 1], bar[SR_MAX_CODE + 1], spc[SR_MAX_CODE + 1], snx[SR_MAX_CODE + 1];
   uint32_t gacc[SR_MAX_CODE + 1];
@@ -98,11 +98,8 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
   const uint32_t ncode = prog->ncode;
   uint2* code = T.code;
   const RegMap rm = map_registers(*prog);
-  for (uint32_t pc = 0; pc < ncode; ++pc) code[pc] = pack(prog->code[pc], rm);
-  code[ncode] = exit_sentinel(rm);
-  set_run_lengths(code, ncode + 1);
-  uint32_t npacked = ncode + 1;
-  if (npacked & 1) code[npacked++] = exit_sentinel(rm);
+  pack_program(*prog, rm, code);
+  const uint32_t npacked = packed_words(ncode);
 
   const BoundScratch ws{T.colour, T.acc, T.bar, T.spc, T.snx, T.gacc};
   sr::LaunchDev* L = T.L;
@@ -134,10 +131,10 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
     d.arena_words = prog->global_words;
     d.ir_bytes = sr::ir_smem_bytes(ncode);
     d.nrows = rm.nrows;
-    const uint32_t nw = (pl.block_dim + 31) / 32;
-    d.group_bytes = sr::group_layout(nw * 32, pl.shmem_words, ncode, rm.nrows, 0, 0).total;
-    d.groups = 1;
-    d.item_blocks = 1;
+    d.sha = pl.shmem_words;                      // (shared_reach takes heap memory)
+    d.vec = sr::block_vec(pl.block_dim);
+    d.nw = sr::block_warps(pl.block_dim, d.vec);
+    d.group_bytes = sr::group_layout(d.nw * 32 * d.vec, pl.shmem_words, ncode, rm.nrows, 0, 0).total;
     d.check_group = sr::check_group_for(d.log_cap);
     d.check_item = (uint32_t)check_items;
     check_items += (d.grid + d.check_group - 1) / d.check_group;
@@ -220,7 +217,7 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
   uint32_t* heads = reinterpret_cast<uint32_t*>(base + o_heads);
   for (uint32_t wi = 0; wi < nwaves; ++wi) {
     const NoallocWave& w = waves[wi];
-    for (uint32_t li = w.li0; li < w.li1; ++li) NA_TRY(sr::launch_interp_plain(ra, li, L[li], 0, s));
+    for (uint32_t li = w.li0; li < w.li1; ++li) NA_TRY(sr::launch_interp_plain(ra, li, L[li], 0, (uint32_t)optin + 1024u, s));
     sr::CheckArgs ca{};
     ca.launches = ra.launches;
     ca.li0 = w.li0;

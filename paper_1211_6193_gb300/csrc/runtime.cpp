@@ -4,10 +4,11 @@
 //                fields remapped so RZ and unused operands read the zero row), bounds
 //                every launch's per-block access log statically, groups launches into
 //                waves whose logs fit the log budget, and uploads everything.
-// run_and_check  per wave: interpreter (one launch per (program, launch) in plain mode;
-//                in batched mode one persistent launch, preceded with two CTAs per SM by
-//                one grid of the programs that run one block per CTA), race check, report
-//                scan and emission.  Everything is enqueued on the caller's stream.
+// run_and_check  per wave: interpreter (one launch per (program, launch) in plain mode, the
+//                programs on the context's side streams; in batched mode one grid per
+//                bucket of launches that take the same kernel form, the buckets on the
+//                side streams), race check, report scan and emission.  Everything is
+//                enqueued behind the caller's stream, which waits for the side streams.
 // fetch_*        synchronise the stream and copy results to the host.
 #include <algorithm>
 #include <cstdarg>
@@ -30,18 +31,26 @@ struct DevBuf {
   size_t bytes = 0;
 };
 
+// Batched mode: launches of a wave that run in one grid (k_interp_blocks).
+struct Bucket {
+  uint32_t vec, variant, warps, smem;   // the kernel form; CTA size and dynamic shared memory
+  uint32_t bq0, bq1;      // entries of the block queue
+  uint32_t blocks;        // and the blocks (tickets) they hold
+  uint32_t ordered;       // launches of it follow others: tickets from a counter
+};
+
 struct Wave {
   uint32_t li0, li1;      // launch index range
   uint32_t gb0, gb1;      // global block range
-  uint32_t item0, item1;  // batched work items
-  uint32_t bq0, bq1;      // batched mode, two CTAs per SM: entries of the block queue
-  uint32_t bq_blocks;     // and the blocks (tickets) they hold
+  uint32_t bk0, bk1;      // batched mode: buckets
   uint64_t log_records;
   uint64_t glog_records;  // global-memory race check: records of the wave's global logs
   uint32_t addr_bits;     // and the bits of its largest global word address
 };
 
 }  // namespace
+
+constexpr uint32_t kSideStreams = 12;
 
 struct sr_ctx {
   sr_opts opts{};
@@ -53,28 +62,28 @@ struct sr_ctx {
   size_t smem_optin = 0;
   size_t smem_per_sm = 0;
   cudaMemPool_t pool = nullptr;   // without a caller allocator: this context's own memory pool
+  // streams on which independent kernels of one run are enqueued side by side: each waits for
+  // the caller's stream (fork), which waits for it again (join)
+  cudaStream_t side[kSideStreams] = {};
+  cudaEvent_t fork = nullptr, join[kSideStreams] = {};
 };
 
 struct sr_batch {
   uint32_t nprogs = 0;
   std::vector<LaunchDev> launches;
   std::vector<uint64_t> arena_off, arena_words;
-  std::vector<uint2> items;
   std::vector<uint32_t> item_launch;       // race check: launch of every work item
-  // batched mode, two CTAs per SM: the launches run one block per CTA (k_interp_blocks), per
-  // wave in ticket order, and the first ticket of each
-  std::vector<uint8_t> one_per_cta;        // per launch
+  // batched mode: the launches of every bucket in ticket order, and the first ticket of each
+  std::vector<Bucket> buckets;
   std::vector<uint32_t> bq_launch, bq_first;
-  uint32_t blocks_smem = 0;
-  uint64_t bq_blocks = 0;                  // blocks of all waves run one per CTA
+  uint64_t wide_blocks = 0;                // blocks run in kernel variant 2 (ctas_per_sm 2)
   std::vector<Wave> waves;
   uint32_t nblocks = 0;
   uint32_t check_items = 0;                // race-check work items of all waves
   uint32_t max_key_bits = 1;
-  uint32_t batched_smem = 0;
   uint64_t total_code = 0, total_arena = 0, log_records = 0;
-  DevBuf code, launches_d, arena_init, arena_work, log, blocks, prog_status, launch_dead, counters, items_d,
-      queue_head, launch_done, scratch, work_head, err_flag, offsets, partials, out, total, item_launch_d,
+  DevBuf code, launches_d, arena_init, arena_work, log, blocks, prog_status, launch_dead, counters,
+      launch_done, scratch, work_head, err_flag, offsets, partials, out, total, item_launch_d,
       bq_launch_d, bq_first_d, bq_head;
   uint64_t out_cap = 0;
   // global-memory race check (opts.check_global)
@@ -145,7 +154,7 @@ int alloc_buf(sr_ctx* c, DevBuf& b, size_t bytes, cudaStream_t s, const char* wh
 
 void free_batch_buffers(sr_ctx* c, sr_batch* b, cudaStream_t s) {
   DevBuf* all[] = {&b->code, &b->launches_d, &b->arena_init, &b->arena_work, &b->log, &b->blocks,
-                   &b->prog_status, &b->launch_dead, &b->counters, &b->items_d, &b->queue_head,
+                   &b->prog_status, &b->launch_dead, &b->counters,
                    &b->launch_done, &b->scratch, &b->work_head, &b->err_flag, &b->offsets, &b->partials,
                    &b->out, &b->total, &b->item_launch_d, &b->glog, &b->glog_n, &b->goff, &b->gpartials,
                    &b->gtotal, &b->sort_a, &b->sort_b, &b->hist, &b->status, &b->tile_ctr, &b->ord_bits,
@@ -258,38 +267,52 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
   ra.prog_status = (uint32_t*)b->prog_status.p;
   ra.launch_dead = (uint32_t*)b->launch_dead.p;
   ra.counters = (sr::Counters*)b->counters.p;
-  ra.items = (const uint2*)b->items_d.p;
   ra.launch_done = (uint32_t*)b->launch_done.p;
   ra.glog = (uint4*)b->glog.p;
   ra.glog_n = (uint32_t*)b->glog_n.p;
 
   for (size_t wi = 0; wi < b->waves.size(); ++wi) {
     const Wave& w = b->waves[wi];
-    if (o.mode == SR_MODE_BATCHED) {
-      if (w.bq_blocks) {         // (two CTAs per SM) the wave's launches that run one block per CTA
-        ra.bq_launch = (const uint32_t*)b->bq_launch_d.p + w.bq0;
-        ra.bq_first = (const uint32_t*)b->bq_first_d.p + w.bq0;
-        ra.bq_n = w.bq1 - w.bq0;
-        ra.bq_head = (uint32_t*)b->bq_head.p + wi;
-        CUDA_TRY(c, cudaMemsetAsync(ra.bq_head, 0, 4, s));
-        CUDA_TRY(c, sr::launch_interp_blocks(ra, w.bq_blocks, b->blocks_smem, s));
+    // Independent kernels - the buckets, or in plain mode the programs - run side by side: alone, a
+    // kernel of a few blocks leaves the chip idle for the 20 to 90 us that its blocks take.
+    const bool batched = o.mode == SR_MODE_BATCHED;
+    const uint32_t nprogs = batched ? 0u : b->launches[w.li1 - 1].prog - b->launches[w.li0].prog + 1u;
+    const uint32_t nside = std::min(kSideStreams, batched ? w.bk1 - w.bk0 : nprogs);
+    const bool fork = nside > 1;
+    if (fork) {
+      CUDA_TRY(c, cudaEventRecord(c->fork, s));
+      for (uint32_t i = 0; i < nside; ++i) CUDA_TRY(c, cudaStreamWaitEvent(c->side[i], c->fork, 0));
+    }
+    cudaError_t e = cudaSuccess;
+    if (batched) {
+      for (uint32_t bk = w.bk0; bk < w.bk1 && e == cudaSuccess; ++bk) {
+        const Bucket& B = b->buckets[bk];
+        const cudaStream_t bs = fork ? c->side[(bk - w.bk0) % nside] : s;
+        ra.bq_launch = (const uint32_t*)b->bq_launch_d.p + B.bq0;
+        ra.bq_first = (const uint32_t*)b->bq_first_d.p + B.bq0;
+        ra.bq_n = B.bq1 - B.bq0;
+        ra.bq_head = B.ordered ? (uint32_t*)b->bq_head.p + bk : nullptr;
+        if (B.ordered) e = cudaMemsetAsync(ra.bq_head, 0, 4, bs);
+        if (e == cudaSuccess)
+          e = sr::launch_interp_blocks(ra, B.vec, B.variant, B.warps, B.blocks, B.smem,
+                                       o.fused_check && o.check_races && !o.check_global, o.check_global != 0, bs);
         b->kernels += 1;
       }
-      ra.items = (const uint2*)b->items_d.p + w.item0;
-      ra.nitems = w.item1 - w.item0;
-      ra.queue_head = (uint32_t*)b->queue_head.p + wi;
-      CUDA_TRY(c, cudaMemsetAsync(ra.queue_head, 0, 4, s));
-      const uint32_t ctas = std::min<uint32_t>(ra.nitems, (uint32_t)c->sms);
-      if (ctas)
-        CUDA_TRY(c, sr::launch_interp_batched(ra, ctas, b->batched_smem,
-                                              o.fused_check && o.check_races && !o.check_global, o.check_global != 0,
-                                              s));
-      b->kernels += ctas ? 1 : 0;
     } else {
-      for (uint32_t li = w.li0; li < w.li1; ++li)
-        CUDA_TRY(c, sr::launch_interp_plain(ra, li, b->launches[li], o.interp_variant, s));
+      for (uint32_t li = w.li0; li < w.li1 && e == cudaSuccess; ++li) {
+        const LaunchDev& L = b->launches[li];
+        e = sr::launch_interp_plain(ra, li, L, o.interp_variant, (uint32_t)c->smem_per_sm,
+                                    fork ? c->side[L.prog % nside] : s);
+      }
       b->kernels += w.li1 - w.li0;
     }
+    if (fork)                                    // (also after an error: nothing stays unjoined)
+      for (uint32_t i = 0; i < nside; ++i) {
+        cudaError_t j = cudaEventRecord(c->join[i], c->side[i]);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(s, c->join[i], 0);
+        if (e == cudaSuccess) e = j;
+      }
+    if (e != cudaSuccess) return fail(c, SR_E_CUDA, "interpreter launch: %s", cudaGetErrorString(e));
     mark();
     if (o.check_races) {
       sr::CheckArgs ca{};
@@ -360,6 +383,11 @@ int sr_create(sr_ctx** out, const sr_opts* opts) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device);
   c->smem_per_sm = (size_t)per_sm;
   if (e == cudaSuccess) e = sr::init_kernel_attributes((uint32_t)optin);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
+  for (uint32_t i = 0; i < kSideStreams && e == cudaSuccess; ++i) {
+    e = cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->join[i], cudaEventDisableTiming);
+  }
   if (e == cudaSuccess && !c->custom_alloc) {
     // a pool of its own that keeps freed memory (batch after batch reuses it instead of
     // returning it to the driver at every synchronisation)
@@ -380,8 +408,7 @@ int sr_create(sr_ctx** out, const sr_opts* opts) {
   }
   if (e != cudaSuccess) {
     cudaGetLastError();
-    if (c->pool) cudaMemPoolDestroy(c->pool);
-    delete c;
+    sr_destroy(c);
     return fail(nullptr, SR_E_CUDA, "device setup failed: %s", cudaGetErrorString(e));
   }
   *out = c;
@@ -390,6 +417,11 @@ int sr_create(sr_ctx** out, const sr_opts* opts) {
 
 void sr_destroy(sr_ctx* c) {
   if (!c) return;
+  for (uint32_t i = 0; i < kSideStreams; ++i) {
+    if (c->join[i]) cudaEventDestroy(c->join[i]);
+    if (c->side[i]) cudaStreamDestroy(c->side[i]);   // (returns at once; released when its work is done)
+  }
+  if (c->fork) cudaEventDestroy(c->fork);
   if (c->pool) cudaMemPoolDestroy(c->pool);   // released once frees still in flight complete
   delete c;
 }
@@ -422,22 +454,19 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   b->arena_words.resize(n);
   uint64_t arena_total = 0;
   uint64_t nblocks = 0, check_items = 0;
+  RangeScratch ranges;
   // shared memory of a CTA of the plain or the persistent batched kernel (one per SM)
   const uint32_t smem_budget =
       (uint32_t)std::min<size_t>(c->smem_optin ? c->smem_optin : 227 * 1024, 227 * 1024) - 1024;
-  // batched mode with two CTAs per SM: a program whose every launch takes one group per
-  // persistent CTA, and whose blocks fit two CTAs per SM, runs one block per CTA instead
-  const bool hybrid = o.mode == SR_MODE_BATCHED && o.ctas_per_sm >= 2 && !o.fused_check && !o.check_global;
-  const uint32_t blocks_cap =
-      hybrid ? std::min<uint32_t>(smem_budget, sr::interp_blocks_smem_cap((uint32_t)c->smem_per_sm)) : 0u;
+  const bool batched = o.mode == SR_MODE_BATCHED;
+  const bool wide = batched && o.ctas_per_sm >= 2 && !o.fused_check && !o.check_global;
+  std::vector<uint8_t> large;                  // per launch: of a program that ctas_per_sm 2 is about
   for (uint32_t i = 0; i < n; ++i) {
     const sr_program& P = progs[i];
     code_off[i] = (uint32_t)code.size();
     const RegMap rm = map_registers(P);
-    for (uint32_t pc = 0; pc < P.ncode; ++pc) code.push_back(pack(P.code[pc], rm));
-    code.push_back(exit_sentinel(rm));
-    set_run_lengths(code.data() + code_off[i], P.ncode + 1);
-    if (code.size() & 1) code.push_back(exit_sentinel(rm));
+    code.resize(code.size() + packed_words(P.ncode));
+    pack_program(P, rm, code.data() + code_off[i]);
     b->arena_off[i] = arena_total;
     b->arena_words[i] = P.global_words;
     arena_total += (P.global_words + 3) & ~3ull;
@@ -449,7 +478,11 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       for (uint32_t k = 0; k < P.nkernels; ++k) kb[k] = bound_kernel(P.code, P.ncode, P.kernel_entry[k], ws);
     }
     const uint32_t first_launch = (uint32_t)b->launches.size();   // the program's launches are contiguous
-    bool one_all = P.nlaunches > 0;            // every launch of the program runs one block per CTA
+    bool one_all = wide && P.nlaunches > 0;    // every launch's blocks are large
+    // batched mode: a program's launches run in one grid, so they share the kernel form
+    uint32_t pvec = 0;
+    if (batched)
+      for (uint32_t l = 0; l < P.nlaunches; ++l) pvec = std::max(pvec, sr::block_vec(P.launches[l].block_dim));
     // the global-memory race check of a program whose launches are not all ordered needs its
     // launch-order matrix (and all its launches in one wave)
     uint32_t ord_off = sr::kNoDep;
@@ -503,30 +536,25 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       d.arena_words = P.global_words;
       d.ir_bytes = sr::ir_smem_bytes(P.ncode);
       d.nrows = rm.nrows;
-      const uint32_t nw = (L.block_dim + 31) / 32;
+      const uint32_t nsw = (L.block_dim + 31) / 32;         // simulated warps
+      d.sha = shared_reach(P.code, P.ncode, d.entry, L, ranges);
+      d.vec = pvec ? pvec : sr::block_vec(L.block_dim);
+      d.nw = sr::block_warps(L.block_dim, d.vec);
+      const uint32_t lanes = d.nw * 32 * d.vec;
       d.uninit = o.check_uninit ? 1u : 0u;
       // the fused race check where its summaries fit beside the block, else the access log
       d.fused = (o.fused_check && o.check_races && !o.check_global && L.shmem_words) ? 1u : 0u;
-      d.group_bytes = sr::group_layout(nw * 32, L.shmem_words, P.ncode, rm.nrows, d.uninit, d.fused).total;
+      d.group_bytes = sr::group_layout(lanes, d.sha, P.ncode, rm.nrows, d.uninit, d.fused).total;
       if (d.fused && d.ir_bytes + d.group_bytes > smem_budget) {
         d.fused = 0;
-        d.group_bytes = sr::group_layout(nw * 32, L.shmem_words, P.ncode, rm.nrows, d.uninit, 0).total;
+        d.group_bytes = sr::group_layout(lanes, d.sha, P.ncode, rm.nrows, d.uninit, 0).total;
       }
       if (d.ir_bytes + d.group_bytes > smem_budget) {
         delete b;
         return fail(c, SR_E_INVAL, "program %u launch %u: %u bytes of shared memory needed, %u available", i, l,
                     d.ir_bytes + d.group_bytes, smem_budget);
       }
-      uint32_t g = std::min<uint32_t>(32 / nw, (smem_budget - d.ir_bytes) / d.group_bytes);
-      one_all = one_all && hybrid && g == 1 && d.ir_bytes + d.group_bytes <= blocks_cap;
-      if (nw >= 2) g = std::min<uint32_t>(g, 15);
-      d.groups = std::max<uint32_t>(1, std::min<uint32_t>(g, d.grid));
-      // blocks per work item: up to 8 rounds of `groups` while the launch still makes two
-      // items per SM, so that a group that finishes early takes another block of the item
-      // instead of waiting for the item's slowest block
-      const uint32_t rounds = std::max<uint32_t>(1, std::min<uint32_t>(
-          8, d.grid / std::max<uint32_t>(1, d.groups * 2u * (uint32_t)c->sms)));
-      d.item_blocks = d.groups * rounds;
+      one_all = one_all && (nsw > 16 || (smem_budget - d.ir_bytes) / d.group_bytes == 1);
       d.check_group = sr::check_group_for(d.log_cap);
       d.check_item = (uint32_t)check_items;
       check_items += (d.grid + d.check_group - 1) / d.check_group;
@@ -538,9 +566,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       }
       b->launches.push_back(d);
     }
-    // (a program as a whole: the launches a launch follows are of its own program, and each of
-    // the two kernels waits only on launches that it runs itself)
-    b->one_per_cta.resize(b->launches.size(), one_all ? 1 : 0);
+    large.resize(b->launches.size(), one_all ? 1 : 0);
   }
   b->nblocks = (uint32_t)nblocks;
   b->check_items = (uint32_t)check_items;
@@ -602,36 +628,59 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   b->glog_records = gwave_max;
   b->entry_cap = std::max<uint64_t>(1024, std::min<uint64_t>(gwave_max, o.report_cap ? o.report_cap : 1u << 20));
 
-  // ---- batched work items: per wave, launch-index order, blocks in chunks of `item_blocks`;
-  // with two CTAs per SM the launches that run one block per CTA go to the wave's block queue
-  // instead, in the same order
-  b->batched_smem = 0;
-  b->blocks_smem = 0;
-  b->bq_blocks = 0;
-  for (Wave& w : b->waves) {
-    w.item0 = (uint32_t)b->items.size();
-    w.bq0 = (uint32_t)b->bq_launch.size();
-    w.bq_blocks = 0;
-    uint32_t maxl = 0;
-    for (uint32_t li = w.li0; li < w.li1; ++li) maxl = std::max(maxl, b->launches[li].launch);
-    for (uint32_t lv = 0; lv <= maxl; ++lv)
-      for (uint32_t li = w.li0; li < w.li1; ++li) {
-        const LaunchDev& d = b->launches[li];
-        if (d.launch != lv || d.grid == 0) continue;
-        if (b->one_per_cta[li]) {
-          b->bq_launch.push_back(li);
-          b->bq_first.push_back(w.bq_blocks);
-          w.bq_blocks += d.grid;
-          b->blocks_smem = std::max(b->blocks_smem, d.ir_bytes + d.group_bytes);
-          continue;
+  // ---- batched mode: the buckets of every wave.  Launches share one when they take the same kernel
+  // form and warps per block and the same number of their blocks fits an SM by shared memory (so that
+  // none is held down by another's footprint); a program's launches go together, and those of
+  // programs with several launches apart from the others (tickets from a counter).  Buckets are
+  // enqueued by falling work; in one, launches follow level, then index.
+  if (batched)
+    for (Wave& w : b->waves) {
+      w.bk0 = (uint32_t)b->buckets.size();
+      struct Entry { uint64_t key; uint32_t level, li; };
+      std::vector<Entry> es;
+      std::vector<uint64_t> work;              // per launch of the wave: simulated warps x code length
+      for (uint32_t li = w.li0; li < w.li1;) {
+        const LaunchDev& f = b->launches[li];
+        uint32_t end = li, warps = 0, smem = 0;
+        for (; end < w.li1 && b->launches[end].prog == f.prog; ++end) {
+          warps = std::max(warps, b->launches[end].nw);
+          smem = std::max(smem, b->launches[end].ir_bytes + b->launches[end].group_bytes);
         }
-        for (uint32_t blk = 0; blk < d.grid; blk += d.item_blocks) b->items.push_back(make_uint2(li, blk));
-        b->batched_smem = std::max(b->batched_smem, d.ir_bytes + d.groups * d.group_bytes);
+        const uint32_t variant = large[li] ? 2u : 1u;
+        // CTAs per SM that registers (24 or 32 warps) and shared memory allow
+        const uint32_t by_regs = (variant == 2u ? 32u : 24u) / warps;
+        const uint32_t by_smem = (uint32_t)c->smem_per_sm / (smem + sr::kBlocksStaticSmem);
+        const uint64_t key = (uint64_t)f.vec << 32 | variant << 24 | warps << 16 |
+                             std::max(1u, std::min(by_regs, by_smem)) << 8 | (f.nl_prog > 1 ? 1u : 0u);
+        for (; li < end; ++li) es.push_back({key, b->launches[li].launch, li});
       }
-    w.item1 = (uint32_t)b->items.size();
-    w.bq1 = (uint32_t)b->bq_launch.size();
-    b->bq_blocks += w.bq_blocks;
-  }
+      std::stable_sort(es.begin(), es.end(), [](const Entry& x, const Entry& y) {
+        return x.key != y.key ? x.key < y.key : x.level < y.level;
+      });
+      for (size_t i = 0; i < es.size(); ++i) {
+        const LaunchDev& d = b->launches[es[i].li];
+        if (i == 0 || es[i].key != es[i - 1].key) {
+          b->buckets.push_back({(uint32_t)(es[i].key >> 32), (uint32_t)(es[i].key >> 24) & 0xFFu,
+                                (uint32_t)(es[i].key >> 16) & 0xFFu, 0, (uint32_t)b->bq_launch.size(), 0, 0,
+                                (uint32_t)es[i].key & 0xFFu});
+          work.push_back(0);
+        }
+        Bucket& B = b->buckets.back();
+        b->bq_launch.push_back(es[i].li);
+        b->bq_first.push_back(B.blocks);
+        B.bq1 = (uint32_t)b->bq_launch.size();
+        B.blocks += d.grid;
+        B.smem = std::max(B.smem, d.ir_bytes + d.group_bytes);
+        if (B.variant == 2) b->wide_blocks += d.grid;
+        work.back() += (uint64_t)d.grid * d.nw * d.ncode;
+      }
+      w.bk1 = (uint32_t)b->buckets.size();
+      std::vector<uint32_t> order(w.bk1 - w.bk0);
+      for (uint32_t i = 0; i < order.size(); ++i) order[i] = i;
+      std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) { return work[x] > work[y]; });
+      const std::vector<Bucket> unsorted(b->buckets.begin() + w.bk0, b->buckets.end());
+      for (uint32_t i = 0; i < order.size(); ++i) b->buckets[w.bk0 + i] = unsorted[order[i]];
+    }
   b->check_ctas = (uint32_t)c->sms * sr::check_ctas_per_sm(o.check_variant);
 
   // ---- device buffers
@@ -649,8 +698,6 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       {&b->prog_status, (size_t)n * 4, "status"},
       {&b->launch_dead, std::max<size_t>(1, b->launches.size()) * 4, "launch stop marks"},
       {&b->counters, sizeof(sr::Counters), "counters"},
-      {&b->items_d, std::max<size_t>(1, b->items.size()) * 8, "work items"},
-      {&b->queue_head, (size_t)nwaves * 4, "queue heads"},
       {&b->launch_done, std::max<size_t>(1, nl) * 4, "launch completion"},
       {&b->scratch, (size_t)b->check_ctas * sr::kScratchWords * 16, "checker scratch"},
       {&b->work_head, (size_t)nwaves * 4, "checker queue"},
@@ -662,7 +709,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       {&b->item_launch_d, std::max<size_t>(1, b->item_launch.size()) * 4, "check item table"},
       {&b->bq_launch_d, std::max<size_t>(1, b->bq_launch.size()) * 4, "block queue launches"},
       {&b->bq_first_d, std::max<size_t>(1, b->bq_first.size()) * 4, "block queue tickets"},
-      {&b->bq_head, (size_t)nwaves * 4, "block queue heads"},
+      {&b->bq_head, b->buckets.size() * 4, "block queue heads"},
       // global-memory race check (16-byte stand-ins when off)
       {&b->glog, (size_t)b->glog_records * 16, "global logs"},
       {&b->glog_n, o.check_global ? (size_t)b->nblocks * 4 : 0, "global log counts"},
@@ -696,7 +743,6 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   };
   cudaError_t e = up(b->code, code.data(), code.size() * 8);
   if (e == cudaSuccess) e = up(b->launches_d, b->launches.data(), nl * sizeof(LaunchDev));
-  if (e == cudaSuccess) e = up(b->items_d, b->items.data(), b->items.size() * 8);
   if (e == cudaSuccess) e = up(b->item_launch_d, b->item_launch.data(), b->item_launch.size() * 4);
   if (e == cudaSuccess) e = up(b->bq_launch_d, b->bq_launch.data(), b->bq_launch.size() * 4);
   if (e == cudaSuccess) e = up(b->bq_first_d, b->bq_first.data(), b->bq_first.size() * 4);
@@ -863,7 +909,7 @@ int sr_batch_stats(sr_ctx* c, sr_batch* b, sr_stats* out) {
   out->blocks = b->nblocks;
   out->waves = (uint32_t)b->waves.size();
   out->kernels = b->kernels;
-  out->one_per_cta_blocks = b->bq_blocks;
+  out->one_per_cta_blocks = b->wide_blocks;
   out->global_records = k.global_records;
   if (c->opts.profile && b->nevents_used >= 2) {
     float ms = 0;

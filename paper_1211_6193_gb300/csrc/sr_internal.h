@@ -8,28 +8,43 @@
 
 namespace sr {
 
-// Packed instructions (device copy), x word: op:6 | immediate operand:1 | d:5 | a:5 | b:5 |
-// run:10, y word: the immediate.  Register fields are rows of the program's compacted
-// register file (only the registers the program uses, plus one zero row last); a destination
-// of kNoDest drops the write (RZ or an opcode without a result).  `run` is the number of
-// consecutive MOV, ADD and MUL instructions starting at this one, at most kRunMax, 0 for any
-// other instruction: such a run touches no memory and needs no ALU dispatch (the interpreter's
-// tight loop selects among the three; every other operation takes the general path).
+// Packed instructions (device copy), x word: form:6 | marks:2 | d:8 | a:8 | b:8, y word: the
+// immediate; the register fields are whole bytes, which one permute extracts.  Register fields
+// are rows of the program's compacted register file (only the registers the program uses, plus
+// one zero row last); a destination of kNoDest drops the write (RZ or an opcode without a
+// result).  The forms below F_LDS come in runs: they touch no memory, do not branch and report
+// nothing.  After the code, a byte per instruction holds the number of them in a row from it on (at
+// most kRunMax; 0 for other forms).  MOV, ADD and MUL with an immediate each on the result of the
+// one before, which nothing else reads, form a chain: the first one's word names the chain's
+// operand a and its length (b) and the last one's result, and the slots of the others hold their
+// factors (x) and addends (y).  Marks of an instruction or chain of a run (set_runs): operand a is the
+// previous one's result; its own result is overwritten in the run before any read but the next
+// one's operand a.
 constexpr uint32_t kNoDest = 31;
-constexpr uint32_t kRunMax = 1023;
-__host__ __device__ constexpr uint32_t pk_op(uint32_t x) { return x & 0x3Fu; }
-__host__ __device__ constexpr uint32_t pk_imm(uint32_t x) { return (x >> 6) & 1u; }
-__host__ __device__ constexpr uint32_t pk_d(uint32_t x) { return (x >> 7) & 31u; }
-__host__ __device__ constexpr uint32_t pk_a(uint32_t x) { return (x >> 12) & 31u; }
-__host__ __device__ constexpr uint32_t pk_b(uint32_t x) { return (x >> 17) & 31u; }
-__host__ __device__ constexpr uint32_t pk_run(uint32_t x) { return x >> 22; }
-__host__ __device__ constexpr uint32_t pk_make(uint32_t op, uint32_t imm, uint32_t d, uint32_t a, uint32_t b,
-                                               uint32_t run) {
-  return op | imm << 6 | d << 7 | a << 12 | b << 17 | run << 22;
+constexpr uint32_t kRunMax = 255;
+constexpr uint32_t kFwdA = 1u << 6, kDeadD = 1u << 7;
+enum : uint32_t {
+  F_MOVI = 0, F_ADDI, F_MULI,             // one multiply-add (SUB and SHL by an immediate become these)
+  F_MOVR, F_ADDR, F_SUBR, F_MULR,         // of registers
+  F_AND = 8, F_OR = 10, F_XOR = 12, F_SHL = 14, F_SHR = 16, F_MIN = 18, F_MAX = 20, F_SLT = 22, F_SLE = 24,
+  F_SEQ = 26, F_SNE = 28,                 // with an immediate; + 1 of registers
+  F_LDS = 32, F_STS, F_BRZ, F_BRNZ, F_LDG, F_STG, F_ATOMS, F_BRA, F_S2R, F_BAR, F_BARAND, F_BAROR, F_BARPOPC,
+  F_DIVR, F_DIVI, F_REMR, F_REMI, F_EXIT
+};
+__host__ __device__ constexpr uint32_t pk_form(uint32_t x) { return x & 0x3Fu; }
+__host__ __device__ constexpr uint32_t pk_d(uint32_t x) { return (x >> 8) & 0xFFu; }
+__host__ __device__ constexpr uint32_t pk_a(uint32_t x) { return (x >> 16) & 0xFFu; }
+__host__ __device__ constexpr uint32_t pk_b(uint32_t x) { return x >> 24; }
+__host__ __device__ constexpr uint32_t pk_make(uint32_t form, uint32_t d, uint32_t a, uint32_t b) {
+  return form | d << 8 | a << 16 | b << 24;
 }
-__host__ __device__ constexpr bool pk_plain_alu(uint32_t op) {
-  return op == SR_OP_MOV || op == SR_OP_ADD || op == SR_OP_MUL;
-}
+// (bit f: a form of runs whose second operand is an immediate)
+constexpr uint32_t kImmForms = 7u | 0x15555500u;
+__host__ __device__ constexpr bool pk_imm(uint32_t form) { return form < F_LDS && ((kImmForms >> form) & 1u); }
+// Simulated warps per real warp of the interpreter for a block of bdim threads, and the real
+// warps the block then takes (at most 8).
+__host__ __device__ constexpr uint32_t block_vec(uint32_t bdim) { return bdim <= 64 ? 1u : bdim <= 128 ? 2u : 4u; }
+__host__ __device__ constexpr uint32_t block_warps(uint32_t bdim, uint32_t vec) { return (bdim + 32u * vec - 1u) / (32u * vec); }
 constexpr uint32_t kInf = 0xFFFFFFFFu;
 constexpr uint32_t kMaxBudget = 1u << 26;  // epochs and rounds stay below 2^26
 // Polls of an mbarrier that only a CTA's own bulk copy (global -> its shared memory) completes.
@@ -41,6 +56,11 @@ constexpr uint32_t kCopyWaitLimit = 1u << 24;
 // Debug build (-DSR_DEBUG_BOUNDS): internal indices are checked before each access; a failed
 // check sets `flag_bits` in *flag and the access is skipped (no trap, no fault: the kernel
 // goes on and the host reports the failure).  In the default build the check is compiled away.
+#if defined(SR_DEBUG_BOUNDS)
+constexpr bool kDebugBounds = true;
+#else
+constexpr bool kDebugBounds = false;
+#endif
 #if defined(SR_DEBUG_BOUNDS) && defined(__CUDACC__)
 __device__ __forceinline__ bool dbg_ok(bool ok, uint32_t* flag, uint32_t flag_bits) {
   if (!ok) atomicOr(flag, flag_bits);
@@ -79,7 +99,7 @@ struct LaunchDev {
   uint32_t nparams, block_base, log_cap, key_bits;   // log_cap records per block (even)
   uint64_t log_base;                     // record offset of block 0's region
   uint64_t arena_off, arena_words;       // word offset of the program's working arena
-  uint32_t groups, group_bytes;          // batched mode: blocks per CTA, smem per block
+  uint32_t group_bytes, pad0;            // smem of a block beside the staged code
   uint32_t ir_bytes, nrows;              // smem bytes of the staged code; register rows (zero row last)
   uint32_t check_group, check_item;      // race check: blocks per work item, index of the first item
   uint32_t uninit;                       // 1 = report shared loads of words no thread wrote
@@ -95,9 +115,11 @@ struct LaunchDev {
   // the blocks run are [block_off, block_off + grid) of a grid of gdim blocks (S2R BID and
   // reports add block_off; S2R GDIM reads gdim)
   uint32_t block_off, gdim;
-  // batched mode: blocks per work item, a multiple of `groups` (a group that finishes its block
-  // claims the item's next one)
-  uint32_t item_blocks;
+  // the interpreter's simulated warps per real warp (1, 2 or 4) and real warps per block
+  uint32_t vec, nw;
+  // words of the shared array that exist: no access reaches past them (shared_reach), so that
+  // more blocks share an SM than the declared array would let in
+  uint32_t sha;
 };
 constexpr uint32_t kNoDep = 0xFFFFFFFFu;
 
@@ -120,17 +142,12 @@ struct RunArgs {
   uint32_t* prog_status;        // SR_ST_* bits
   uint32_t* launch_dead;        // per launch: 1 = a block stopped it, or it was skipped
   Counters* counters;
-  // batched mode
-  const uint2* items;           // (launch index, first block)
-  uint32_t nitems;
-  uint32_t* queue_head;
-  uint32_t* launch_done;        // completed blocks per launch
+  uint32_t* launch_done;        // batched mode: completed blocks per launch
   // global-memory race check: per-block global-log regions and per-block record counts
   uint4* glog;
   uint32_t* glog_n;
-  // batched mode, two CTAs per SM: the wave's block queue of the one-block-per-CTA kernel -
-  // its launches in ticket order and the first ticket of each (bq_first[0] = 0), and the
-  // ticket counter
+  // batched mode: a bucket's block queue - its launches in ticket order and the first ticket of
+  // each (bq_first[0] = 0), and the ticket counter (NULL: tickets are CTA indices)
   const uint32_t* bq_launch;
   const uint32_t* bq_first;
   uint32_t bq_n;
@@ -139,7 +156,7 @@ struct RunArgs {
 
 // Shared-memory footprint of one simulated block in the interpreter.
 struct GroupLayout {
-  uint32_t regs, sh, clk, rlo, rhi, rsp, park, err, bv, un, wb, tup, rbm, total;
+  uint32_t regs, sh, err, un, wb, tup, rbm, total;
 };
 // The summary of one shared word in the fused race check: the two smallest distinct tids of
 // each access kind (kTupleEmpty none) and the lowest and highest pc, eight planes of this
@@ -149,19 +166,21 @@ __host__ __device__ inline uint32_t tuple_plane_words(uint32_t shw) { return (sh
 __host__ __device__ inline uint32_t align16(uint32_t x) { return (x + 15u) & ~15u; }
 // The fixed-size arrays come first, at offsets known at compile time; the arrays whose
 // size depends on the launch follow.
-constexpr uint32_t kGroupClk = 0, kGroupRlo = 128, kGroupRhi = 256, kGroupRsp = 384, kGroupPark = 512,
-                   kGroupBv = 512 + 32 * 8 * 4, kGroupFixed = kGroupBv + 64;
+// (clocks: 32 words; address ranges of the warps' stores, 16 bytes each; park entries of two
+// intervals, 8 of 32 bytes each; SoloConst; BlockVars.  A block has at most 8 warps: block_vec.)
+#define SR_GROUP_RANGE 128
+#define SR_GROUP_PARK 256
+#define SR_GROUP_CONST 768
+#define SR_GROUP_BV 864
+constexpr uint32_t kGroupClk = 0, kGroupRange = SR_GROUP_RANGE, kGroupPark = SR_GROUP_PARK, kGroupConst = SR_GROUP_CONST,
+                   kGroupBv = SR_GROUP_BV, kGroupFixed = kGroupBv + 64;
+constexpr uint32_t kMaxWarps = 8;
+static_assert(kGroupPark >= kGroupRange + 16 * kMaxWarps && kGroupConst >= kGroupPark + 2 * 32 * kMaxWarps, "group layout");
 // With `uninit`: per-pc counters of loads of unwritten words, and the bitmap of written words.
 // With `fused`: the eight summary planes and a bitmap of the interval's racy words.
 __host__ __device__ inline GroupLayout group_layout(uint32_t nthr, uint32_t shw, uint32_t ncode, uint32_t nrows,
                                                    uint32_t uninit, uint32_t fused) {
   GroupLayout g;
-  g.clk = kGroupClk;
-  g.rlo = kGroupRlo;
-  g.rhi = kGroupRhi;
-  g.rsp = kGroupRsp;
-  g.park = kGroupPark;
-  g.bv = kGroupBv;
   uint32_t o = kGroupFixed;
   g.regs = o; o += align16(nrows * nthr * 4u);
   g.sh = o;   o += align16(shw * 4u);
@@ -179,25 +198,27 @@ __host__ __device__ inline GroupLayout group_layout(uint32_t nthr, uint32_t shw,
   g.total = o;
   return g;
 }
-__host__ __device__ inline uint32_t ir_smem_bytes(uint32_t ncode) {
-  return align16(((ncode + 2u) & ~1u) * 8u);   // ncode + EXIT sentinel, even count
-}
+// Staged code of a program: its instructions with the EXIT sentinel (an even count), then the run
+// lengths, one byte each.
+__host__ __device__ inline uint32_t ir_code_bytes(uint32_t ncode) { return ((ncode + 2u) & ~1u) * 8u; }
+__host__ __device__ inline uint32_t ir_smem_bytes(uint32_t ncode) { return ir_code_bytes(ncode) + align16(ncode + 1u); }
 
 // kernel launchers (defined in the .cu files); attributes are set once per process
 cudaError_t init_kernel_attributes(uint32_t smem_optin);
 cudaError_t init_interp_attributes(uint32_t smem_optin);
 cudaError_t init_check_attributes(uint32_t smem_optin);
-cudaError_t launch_interp_plain(const RunArgs& a, uint32_t li, const LaunchDev& L, uint32_t variant, cudaStream_t s);
-// fused: run the instantiation with the fused race check (launches whose `fused` is 0 still
-// log their accesses in it); global: the instantiation that logs global accesses (launches
-// whose glog_cap is 0 log none in it; it has no fused race check)
-cudaError_t launch_interp_batched(const RunArgs& a, uint32_t ctas, uint32_t smem, bool fused, bool global,
-                                  cudaStream_t s);
-// batched mode, two CTAs per SM: one simulated block per 1024-thread CTA for the wave's block
-// queue (a.bq_*), `nblocks` CTAs, `smem` bytes of dynamic shared memory each
-cudaError_t launch_interp_blocks(const RunArgs& a, uint32_t nblocks, uint32_t smem, cudaStream_t s);
-// dynamic shared memory of one CTA of the one-block-per-CTA kernel that still lets two share an SM
-uint32_t interp_blocks_smem_cap(uint32_t smem_optin);
+cudaError_t launch_interp_plain(const RunArgs& a, uint32_t li, const LaunchDev& L, uint32_t variant,
+                                uint32_t smem_per_sm, cudaStream_t s);
+// Shared memory of a CTA beside the dynamic part (its static variables and what the hardware keeps).
+constexpr uint32_t kBlocksStaticSmem = 1024 + 256;
+// batched mode: one simulated block per CTA of `warps` warps for the bucket's block queue (a.bq_*),
+// `nblocks` CTAs, `smem` bytes of dynamic shared memory each; vec, variant: the kernel form
+// (variant 2: registers for four CTAs of 8 warps per SM instead of three).  fused: the instantiation with the
+// fused race check (launches whose `fused` is 0 still log their accesses in it); global: the
+// instantiation that logs global accesses (launches whose glog_cap is 0 log none in it; it has no
+// fused race check)
+cudaError_t launch_interp_blocks(const RunArgs& a, uint32_t vec, uint32_t variant, uint32_t warps, uint32_t nblocks,
+                                 uint32_t smem, bool fused, bool global, cudaStream_t s);
 
 // Global-log record (16 bytes): x = word address in the program's arena, y = epoch (barrier
 // interval of the block), z = tid << 16 | kind << 12 | pc (kind 1 = store, 0 = load),
@@ -241,7 +262,7 @@ constexpr uint32_t kCheckMaxGroup = 32;        // blocks per check work item at 
 // touching words past the table are checked in the CTA's spill table instead.
 inline uint32_t check_table_words(const LaunchDev* L, uint32_t li0, uint32_t li1, uint32_t cap) {
   uint32_t m = 8;
-  for (uint32_t i = li0; i < li1; ++i) m = L[i].shw > m ? L[i].shw : m;
+  for (uint32_t i = li0; i < li1; ++i) m = L[i].sha > m ? L[i].sha : m;
   m = (4u * m + 31u) & ~31u;
   return m < cap ? m : cap;
 }
