@@ -758,10 +758,7 @@ cudaError_t launch_gcheck(const GcheckArgs& G, uint32_t& kernels, cudaStream_t s
   e = radix_sort<Rec16, AddrDigit>(reinterpret_cast<Rec16*>(G.sort_a), reinterpret_cast<Rec16*>(G.sort_b),
                                    G.gtotal, G.rec_cap, G.addr_passes, G, g_pass_ctas16, &sorted, kernels, s);
   if (e != cudaSuccess) return e;
-  // 3. the run scan
-  e = cudaMemsetAsync(G.gn, 0, 8, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(G.gcount + G.gb0, 0, (size_t)(G.gb1 - G.gb0) * 4, s);
-  if (e != cudaSuccess) return e;
+  // 3. the run scan (gn and gcount start from zero: launch_reset)
   GrunArgs R{};
   R.rec = reinterpret_cast<const uint4*>(sorted);
   R.n_ptr = G.gtotal;

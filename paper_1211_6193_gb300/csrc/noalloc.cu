@@ -135,7 +135,7 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
     d.vec = sr::block_vec(pl.block_dim);
     d.nw = sr::block_warps(pl.block_dim, d.vec);
     d.group_bytes = sr::group_layout(d.nw * 32 * d.vec, pl.shmem_words, ncode, rm.nrows, 0, 0).total;
-    d.check_group = sr::check_group_for(d.log_cap);
+    d.check_group = sr::check_group_for(d.log_cap, sr::kCheckMaxGroup);
     d.check_item = (uint32_t)check_items;
     check_items += (d.grid + d.check_group - 1) / d.check_group;
     if (d.ir_bytes + d.group_bytes + 1024 > (uint32_t)optin) return SR_E_RANGE;
@@ -238,7 +238,8 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
     ka.nlaunches = nl;
     ka.gb0 = w.gb0;
     ka.gb1 = w.gb1;
-    ka.total = reinterpret_cast<unsigned long long*>(base + o_total);
+    ka.total_out = reinterpret_cast<unsigned long long*>(base + o_total);
+    ka.total_in = ka.total_out;
     ka.log = ra.log;
     ka.blocks = ra.blocks;
     ka.offsets = reinterpret_cast<unsigned long long*>(base + o_offsets);

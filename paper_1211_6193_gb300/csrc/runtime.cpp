@@ -82,8 +82,10 @@ struct sr_batch {
   uint32_t check_items = 0;                // race-check work items of all waves
   uint32_t max_key_bits = 1;
   uint64_t total_code = 0, total_arena = 0, log_records = 0;
+  // (total: the running report count before each wave and after the last, then the error flag: what
+  // fetch_reports reads first, in one copy)
   DevBuf code, launches_d, arena_init, arena_work, log, blocks, prog_status, launch_dead, counters,
-      launch_done, scratch, work_head, err_flag, offsets, partials, out, total, item_launch_d,
+      launch_done, scratch, work_head, offsets, partials, out, total, item_launch_d,
       bq_launch_d, bq_first_d, bq_head;
   uint64_t out_cap = 0;
   // global-memory race check (opts.check_global)
@@ -155,7 +157,7 @@ int alloc_buf(sr_ctx* c, DevBuf& b, size_t bytes, cudaStream_t s, const char* wh
 void free_batch_buffers(sr_ctx* c, sr_batch* b, cudaStream_t s) {
   DevBuf* all[] = {&b->code, &b->launches_d, &b->arena_init, &b->arena_work, &b->log, &b->blocks,
                    &b->prog_status, &b->launch_dead, &b->counters,
-                   &b->launch_done, &b->scratch, &b->work_head, &b->err_flag, &b->offsets, &b->partials,
+                   &b->launch_done, &b->scratch, &b->work_head, &b->offsets, &b->partials,
                    &b->out, &b->total, &b->item_launch_d, &b->glog, &b->glog_n, &b->goff, &b->gpartials,
                    &b->gtotal, &b->sort_a, &b->sort_b, &b->hist, &b->status, &b->tile_ctr, &b->ord_bits,
                    &b->entries_a, &b->entries_b, &b->gn, &b->gcount, &b->gstart, &b->gn_sorted,
@@ -172,14 +174,17 @@ cudaEvent_t next_event(sr_batch* b) {
   return b->events[b->nevents_used++];
 }
 
-// Enqueue the whole pipeline for one run on stream s.
-sr::CompactArgs compact_args(sr_batch* b, const Wave& w) {
+uint32_t* err_flag(const sr_batch* b) { return (uint32_t*)((unsigned long long*)b->total.p + b->waves.size() + 1); }
+
+sr::CompactArgs compact_args(sr_batch* b, uint32_t wi) {
+  const Wave& w = b->waves[wi];
   sr::CompactArgs ka{};
   ka.launches = (const LaunchDev*)b->launches_d.p;
   ka.nlaunches = (uint32_t)b->launches.size();
   ka.gb0 = w.gb0;
   ka.gb1 = w.gb1;
-  ka.total = (unsigned long long*)b->total.p;
+  ka.total_in = (unsigned long long*)b->total.p + wi;
+  ka.total_out = (unsigned long long*)b->total.p + wi + 1;
   ka.log = (const unsigned long long*)b->log.p;
   ka.blocks = (const sr::BlockRes*)b->blocks.p;
   ka.offsets = (unsigned long long*)b->offsets.p;
@@ -187,7 +192,7 @@ sr::CompactArgs compact_args(sr_batch* b, const Wave& w) {
   ka.out = (sr_report*)b->out.p;
   ka.out_cap = b->out_cap;
   ka.counters = (sr::Counters*)b->counters.p;
-  ka.error_flag = (uint32_t*)b->err_flag.p;
+  ka.error_flag = err_flag(b);
   if (w.glog_records) {
     ka.gcount = (const uint32_t*)b->gcount.p;
     ka.gstart = (const unsigned long long*)b->gstart.p;
@@ -218,7 +223,7 @@ sr::GcheckArgs gcheck_args(sr_ctx* c, sr_batch* b, uint32_t wi) {
   g.hist = (unsigned long long*)b->hist.p;
   g.status = (unsigned long long*)b->status.p;
   g.tile_ctr = (uint32_t*)b->tile_ctr.p;
-  g.err = (uint32_t*)b->err_flag.p;
+  g.err = err_flag(b);
   g.spin_limit = c->opts.spin_limit;
   g.sms = (uint32_t)c->sms;
   g.ord_bits = (const uint32_t*)b->ord_bits.p;
@@ -243,15 +248,27 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
     return e;
   };
   mark();
-  CUDA_TRY(c, cudaMemcpyAsync(b->arena_work.p, b->arena_init.p, b->total_arena * 4, cudaMemcpyDeviceToDevice, s));
-  CUDA_TRY(c, cudaMemsetAsync(b->blocks.p, 0, (size_t)b->nblocks * sizeof(sr::BlockRes), s));
-  CUDA_TRY(c, cudaMemsetAsync(b->prog_status.p, 0, (size_t)b->nprogs * 4, s));
-  CUDA_TRY(c, cudaMemsetAsync(b->launch_dead.p, 0, std::max<size_t>(1, b->launches.size()) * 4, s));
-  CUDA_TRY(c, cudaMemsetAsync(b->counters.p, 0, sizeof(sr::Counters), s));
-  CUDA_TRY(c, cudaMemsetAsync(b->launch_done.p, 0, b->launches.size() * 4, s));
-  CUDA_TRY(c, cudaMemsetAsync(b->total.p, 0, 8, s));
-  CUDA_TRY(c, cudaMemsetAsync(b->err_flag.p, 0, 4, s));
-  if (o.check_global) CUDA_TRY(c, cudaMemsetAsync(b->glog_n.p, 0, (size_t)b->nblocks * 4, s));
+  // one kernel: a copy and nine memsets, each a launch of its own, took 14 us of the smallest runs
+  sr::ResetArgs za{};
+  za.src = (const uint4*)b->arena_init.p;
+  za.dst = (uint4*)b->arena_work.p;
+  za.words16 = b->total_arena / 4;               // (arenas are padded to 16 bytes)
+  auto zero = [&](const DevBuf& d, size_t bytes) { za.zero[za.nzero++] = {(uint32_t*)d.p, bytes / 4}; };
+  zero(b->blocks, (size_t)b->nblocks * sizeof(sr::BlockRes));
+  zero(b->prog_status, (size_t)b->nprogs * 4);
+  zero(b->launch_dead, b->launches.size() * 4);
+  zero(b->launch_done, b->launches.size() * 4);
+  zero(b->counters, sizeof(sr::Counters));
+  zero(b->total, (b->waves.size() + 1) * 8 + 4);
+  zero(b->work_head, b->waves.size() * 4);
+  zero(b->bq_head, b->buckets.size() * 4);
+  if (o.check_global) {
+    zero(b->glog_n, (size_t)b->nblocks * 4);
+    zero(b->gn, b->waves.size() * 8);
+    zero(b->gcount, (size_t)b->nblocks * 4);
+  }
+  CUDA_TRY(c, sr::launch_reset(za, (uint32_t)c->sms, s));
+  b->kernels += 1;
   mark();
 
   sr::RunArgs ra{};
@@ -292,10 +309,8 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
         ra.bq_first = (const uint32_t*)b->bq_first_d.p + B.bq0;
         ra.bq_n = B.bq1 - B.bq0;
         ra.bq_head = B.ordered ? (uint32_t*)b->bq_head.p + bk : nullptr;
-        if (B.ordered) e = cudaMemsetAsync(ra.bq_head, 0, 4, bs);
-        if (e == cudaSuccess)
-          e = sr::launch_interp_blocks(ra, B.vec, B.variant, B.warps, B.blocks, B.smem,
-                                       o.fused_check && o.check_races && !o.check_global, o.check_global != 0, bs);
+        e = sr::launch_interp_blocks(ra, B.vec, B.variant, B.warps, B.blocks, B.smem,
+                                     o.fused_check && o.check_races && !o.check_global, o.check_global != 0, bs);
         b->kernels += 1;
       }
     } else {
@@ -325,11 +340,10 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
       ca.blocks = ra.blocks;
       ca.scratch = (uint4*)b->scratch.p;
       ca.work_head = (uint32_t*)b->work_head.p + wi;
-      ca.error_flag = (uint32_t*)b->err_flag.p;
+      ca.error_flag = err_flag(b);
       ca.spin_limit = o.spin_limit;
       ca.table_words = sr::check_table_words(b->launches.data(), w.li0, w.li1, sr::check_table_cap(o.check_variant));
       ca.item_launch = (const uint32_t*)b->item_launch_d.p;
-      CUDA_TRY(c, cudaMemsetAsync(ca.work_head, 0, 4, s));
       const uint32_t ctas = std::min<uint32_t>(b->check_ctas, ca.item1 - ca.item0);
       if (ctas) CUDA_TRY(c, sr::launch_check(ca, o.check_variant, ctas, s));
       b->kernels += ctas ? 1 : 0;
@@ -337,7 +351,7 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
     mark();
     if (w.glog_records) CUDA_TRY(c, sr::launch_gcheck(gcheck_args(c, b, (uint32_t)wi), b->kernels, s));
     mark();
-    const sr::CompactArgs ka = compact_args(b, w);
+    const sr::CompactArgs ka = compact_args(b, (uint32_t)wi);
     CUDA_TRY(c, sr::launch_compact_scan(ka, s));
     CUDA_TRY(c, sr::launch_compact_emit(ka, s));
     b->kernels += sr::compact_kernels(ka);
@@ -555,12 +569,9 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
                     d.ir_bytes + d.group_bytes, smem_budget);
       }
       one_all = one_all && (nsw > 16 || (smem_budget - d.ir_bytes) / d.group_bytes == 1);
-      d.check_group = sr::check_group_for(d.log_cap);
-      d.check_item = (uint32_t)check_items;
-      check_items += (d.grid + d.check_group - 1) / d.check_group;
       b->max_key_bits = std::max(b->max_key_bits, d.key_bits);
       nblocks += d.grid;
-      if (nblocks >= (1ull << 31) || check_items >= (1ull << 31)) {
+      if (nblocks >= (1ull << 31)) {
         delete b;
         return fail(c, SR_E_INVAL, "too many simulated blocks in one batch");
       }
@@ -569,6 +580,11 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
     large.resize(b->launches.size(), one_all ? 1 : 0);
   }
   b->nblocks = (uint32_t)nblocks;
+  for (LaunchDev& d : b->launches) {             // (at most one item per block)
+    d.check_group = sr::check_group_for(d.log_cap, nblocks / ((uint64_t)c->sms * sr::check_ctas_per_sm(o.check_variant)));
+    d.check_item = (uint32_t)check_items;
+    check_items += (d.grid + d.check_group - 1) / d.check_group;
+  }
   b->check_items = (uint32_t)check_items;
   b->item_launch.resize(check_items);
   for (uint32_t li = 0; li < b->launches.size(); ++li) {
@@ -701,11 +717,10 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       {&b->launch_done, std::max<size_t>(1, nl) * 4, "launch completion"},
       {&b->scratch, (size_t)b->check_ctas * sr::kScratchWords * 16, "checker scratch"},
       {&b->work_head, (size_t)nwaves * 4, "checker queue"},
-      {&b->err_flag, 4, "error flag"},
       {&b->offsets, ((size_t)b->nblocks + 1) * 8, "report offsets"},
       {&b->partials, sr::compact_partials_count(b->nblocks) * 8, "scan partials"},
       {&b->out, b->out_cap * sizeof(sr_report), "reports"},
-      {&b->total, 8, "report total"},
+      {&b->total, ((size_t)nwaves + 1) * 8 + 8, "report totals and error flag"},
       {&b->item_launch_d, std::max<size_t>(1, b->item_launch.size()) * 4, "check item table"},
       {&b->bq_launch_d, std::max<size_t>(1, b->bq_launch.size()) * 4, "block queue launches"},
       {&b->bq_first_d, std::max<size_t>(1, b->bq_first.size()) * 4, "block queue tickets"},
@@ -830,9 +845,14 @@ int fetch_reports(sr_ctx* c, sr_batch* b, sr_report* dst, uint64_t cap, uint64_t
       if (rc) return rc;
     }
   }
-  unsigned long long total = 0;
-  CUDA_TRY(c, cudaMemcpyAsync(&total, b->total.p, 8, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(c, cudaStreamSynchronize(s));
+  struct { unsigned long long total; uint32_t err, pad; } fin{};   // the last running count, the error flag
+  auto fetch_fin = [&]() -> cudaError_t {
+    const cudaError_t e = cudaMemcpyAsync(&fin, (unsigned long long*)b->total.p + b->waves.size(), sizeof fin,
+                                          cudaMemcpyDeviceToHost, s);
+    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+  };
+  CUDA_TRY(c, fetch_fin());
+  unsigned long long& total = fin.total;
   if (total > b->out_cap) {
     // The report buffer was too small: grow it.  With one wave, that wave's logs, block
     // results and report offsets are all still on the device, so only the emission runs
@@ -847,24 +867,23 @@ int fetch_reports(sr_ctx* c, sr_batch* b, sr_report* dst, uint64_t cap, uint64_t
       b->graph = nullptr;
     }
     if (b->waves.size() == 1) {
-      CUDA_TRY(c, sr::launch_compact_emit(compact_args(b, b->waves[0]), s));
+      CUDA_TRY(c, sr::launch_compact_emit(compact_args(b, 0), s));
+      CUDA_TRY(c, fetch_fin());                  // (an index check of the debug build)
     } else {
       rc = run_and_check(c, b, s);
       if (rc) return rc;
-      CUDA_TRY(c, cudaMemcpyAsync(&total, b->total.p, 8, cudaMemcpyDeviceToHost, s));
-      CUDA_TRY(c, cudaStreamSynchronize(s));
+      CUDA_TRY(c, fetch_fin());
     }
   }
-  uint32_t err = 0;
-  CUDA_TRY(c, cudaMemcpyAsync(&err, b->err_flag.p, 4, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(c, cudaStreamSynchronize(s));
+  const uint32_t err = fin.err;
   if (n_total) *n_total = total;
   if (err & sr::kErrBounds) return fail(c, SR_E_BOUNDS, "an internal index check failed (debug build)");
   if (err & sr::kErrCorrupt) return fail(c, SR_E_TIMEOUT, "the race checker found an access log out of order");
   if (err) return fail(c, SR_E_TIMEOUT, "a device-side wait of the checks gave up");
   if (!dst) return SR_OK;
   if (cap < total) return fail(c, SR_E_RANGE, "report buffer holds %llu, %llu needed", (unsigned long long)cap, total);
-  if (total) CUDA_TRY(c, cudaMemcpyAsync(dst, b->out.p, total * sizeof(sr_report), cudaMemcpyDeviceToHost, s));
+  if (!total) return SR_OK;
+  CUDA_TRY(c, cudaMemcpyAsync(dst, b->out.p, total * sizeof(sr_report), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(c, cudaStreamSynchronize(s));
   return SR_OK;
 }

@@ -267,10 +267,14 @@ inline uint32_t check_table_words(const LaunchDev* L, uint32_t li0, uint32_t li1
   return m < cap ? m : cap;
 }
 
-// blocks per check work item for a launch whose blocks log at most `log_cap` records
-__host__ __device__ inline uint32_t check_group_for(uint32_t log_cap) {
-  const uint32_t g = (kCheckItemRecords + log_cap - 1) / (log_cap ? log_cap : 1);
-  return g < 1 ? 1 : (g > kCheckMaxGroup ? kCheckMaxGroup : g);
+// blocks per check work item for a launch whose blocks log at most `log_cap` records, when
+// `share` blocks come on each of the CTAs that fit the device (20 small blocks in one item took
+// one CTA 58 us, in 20 items 16 us)
+__host__ __device__ inline uint32_t check_group_for(uint32_t log_cap, uint64_t share) {
+  uint64_t g = (kCheckItemRecords + log_cap - 1) / (log_cap ? log_cap : 1);
+  g = g > kCheckMaxGroup ? kCheckMaxGroup : g;
+  g = g > share ? share : g;
+  return g < 1 ? 1u : (uint32_t)g;
 }
 
 // Global-memory race check of one wave (gcheck.cu).  Device buffers, all owned by the batch.
@@ -310,7 +314,10 @@ struct CompactArgs {
   const LaunchDev* launches;
   uint32_t nlaunches;
   uint32_t gb0, gb1;            // block range of the wave
-  unsigned long long* total;    // running report count over waves
+  // running report count over waves: read before the wave, written after it (with the same
+  // pointer for both the wave always takes launch_compact_scan's three kernels)
+  const unsigned long long* total_in;
+  unsigned long long* total_out;
   const unsigned long long* log;
   const BlockRes* blocks;
   unsigned long long* offsets;  // nblocks + 1
@@ -330,5 +337,19 @@ cudaError_t launch_compact_scan(const CompactArgs& a, cudaStream_t s);
 cudaError_t launch_compact_emit(const CompactArgs& a, cudaStream_t s);
 uint64_t compact_partials_count(uint32_t nblocks);
 uint32_t compact_kernels(const CompactArgs& a);   // kernel launches of launch_compact_scan + _emit
+
+// The start of a run in one kernel: the working arenas from the initial ones (words16 16-byte
+// words), and the run's counters and queues cleared.
+struct ResetArgs {
+  const uint4* src;
+  uint4* dst;
+  unsigned long long words16;
+  struct Zero {
+    uint32_t* p;
+    unsigned long long words;
+  } zero[12];
+  uint32_t nzero;
+};
+cudaError_t launch_reset(const ResetArgs& a, uint32_t sms, cudaStream_t s);
 
 }  // namespace sr
