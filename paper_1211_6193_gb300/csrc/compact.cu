@@ -129,7 +129,7 @@ __device__ __forceinline__ void emit_block(const CompactArgs& A, uint32_t gb, un
   const uint32_t block = lb + L->block_off;          // its index in the grid (reports)
   const uint4* reg4 = reinterpret_cast<const uint4*>(A.log + L->log_base + (unsigned long long)lb * L->log_cap);
   const uint32_t top = L->log_cap / 2 - 1;        // misc entry j lives at reg4[top - j]
-  const uint4* ge = ng ? A.gentries + 2 * A.gstart[gb - A.gb0] : nullptr;   // the block's global list
+  const uint4* ge = ng ? (*A.gwhere ? A.gentries_b : A.gentries) + 2 * A.gstart[gb - A.gb0] : nullptr;   // the block's global list
   // (debug build: both lists lie inside the block's region)
   if (!dbg_ok(2ull * (nr + nm) <= L->log_cap, A.error_flag, kErrBounds)) return;
   // misc entries (epoch order) with epoch below / at most `ep`

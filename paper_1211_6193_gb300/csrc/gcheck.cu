@@ -14,18 +14,18 @@
 // block's region (epoch order inside a block).  Per wave:
 //   1. gather   the blocks' records into one array, blocks in (program, launch, block) order;
 //   2. sort     stably by word address: an LSD radix sort with 8-bit digits, onesweep style -
-//               one upsweep pass builds the digit histograms of every pass, then each pass
-//               is one kernel in which a CTA ranks a tile staged in shared memory by a TMA
-//               bulk copy, learns the tile's offsets from its predecessors by decoupled
-//               look-back (bounded waits), and writes the tile out digit by digit.  Stable,
-//               so the records of one word keep (program, launch, block, epoch) order;
+//               one upsweep pass builds the digit histograms of every pass, then in each pass
+//               a CTA ranks a tile staged in shared memory by a TMA bulk copy, learns the
+//               tile's offsets from its predecessors by decoupled look-back (bounded waits),
+//               and writes the tile out digit by digit.  Stable, so the records of one word
+//               keep (program, launch, block, epoch) order;
 //   3. scan     each run of one (program, word) in one pass: sub-runs of one (block, epoch)
 //               give the interval check, of one launch the check between blocks, and the
 //               run's launches the check between unordered launches.  Every word keeps the
 //               two smallest distinct tids (blocks) of each access kind and the pc range,
 //               which decide the classes and the smallest conflicting pair exactly;
-//   4. order    the report entries by (block, epoch, kind, word) with the same radix sort,
-//               for the canonical merge in compact.cu.
+//   4. order    the report entries by (block, epoch, kind, word) with the same radix sort, its
+//               passes in one kernel, for the canonical merge in compact.cu.
 #include <algorithm>
 
 #include "sr_internal.h"
@@ -40,9 +40,11 @@ constexpr uint32_t RS_ITEMS = 8;                     // records per thread and t
 constexpr uint32_t RS_TILE = RS_T * RS_ITEMS;        // 2048 records per tile
 constexpr uint32_t RADIX = 256;
 constexpr uint32_t MAX_PASSES = 12;
+constexpr uint32_t kSortSyncLimit = 1u << 26;        // polls for the other CTAs of the sort
 constexpr unsigned long long ST_AGG = 1ull << 62;    // tile status: its own count is known
 constexpr unsigned long long ST_INC = 1ull << 63;    // tile status: its inclusive prefix is known
-constexpr unsigned long long ST_VAL = ST_AGG - 1;
+constexpr uint32_t ST_TAG = 56;                      // bits 56..61: the pass, from 1 (a word of an earlier pass is no news)
+constexpr unsigned long long ST_VAL = (1ull << ST_TAG) - 1;
 constexpr uint32_t NONE16 = 0xFFFFu;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -182,6 +184,35 @@ __global__ void __launch_bounds__(SC_T) k_count_offsets(const uint32_t* c, uint3
   }
 }
 
+// the same in one CTA, for a few chunks
+constexpr uint32_t SC_ONE = 4;
+__global__ void __launch_bounds__(SC_T) k_count_one(const uint32_t* c, uint32_t gb0, uint32_t gb1, unsigned long long* off,
+                                                    unsigned long long* total) {
+  __shared__ unsigned long long wsum[32];
+  __shared__ unsigned long long s_tot;
+  unsigned long long carry = 0;
+  for (uint32_t b0 = gb0; b0 < gb1; b0 += SC_CHUNK) {
+    const uint32_t base = b0 + threadIdx.x * SC_PER;
+    uint32_t v[SC_PER];
+    unsigned long long s = 0;
+    for (uint32_t i = 0; i < SC_PER; ++i) {
+      v[i] = base + i < gb1 ? c[base + i] : 0u;
+      s += v[i];
+    }
+    const unsigned long long inc = cta_inclusive(s, wsum);
+    unsigned long long run = carry + inc - s;
+    for (uint32_t i = 0; i < SC_PER; ++i) {
+      if (base + i < gb1) off[base + i - gb0] = run;
+      run += v[i];
+    }
+    if (threadIdx.x == SC_T - 1) s_tot = inc;
+    __syncthreads();
+    carry += s_tot;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *total = carry;
+}
+
 // ---------------------------------------------------------------- 1. gather
 // One warp per block: its records from its region to their place in the wave's array.
 __global__ void __launch_bounds__(256) k_ggather(const LaunchDev* launches, uint32_t li0, uint32_t li1,
@@ -208,19 +239,24 @@ __global__ void __launch_bounds__(256) k_ggather(const LaunchDev* launches, uint
 }
 
 // ---------------------------------------------------------------- 2. radix sort
-// Digit histograms of every pass in one read of the records.  Each warp reads UP_ITEMS rows
-// of 32 consecutive records; per pass and row, a digit that all 32 lanes share (the upper
-// digits of nearly sorted input) is counted by one shared atomic, other rows by one atomic
-// per lane.
+// Digit histograms of every pass in one read of the records (hist starts from zero), and the
+// tiles' states cleared.  Each warp reads UP_ITEMS rows of 32 consecutive records; per pass and
+// row, a digit that all 32 lanes share (the upper digits of nearly sorted input) is counted by one
+// shared atomic, other rows by one atomic per lane.  A kernel of its own: inside k_rs_sort, at the
+// sort's registers and CTAs per SM, it took 0.7 ms longer for 34 M records.
 constexpr uint32_t UP_ITEMS = 8;
 template <class Rec, class Digit>
 __global__ void __launch_bounds__(RS_T) k_rs_upsweep(const Rec* in, const unsigned long long* n_ptr,
-                                                     unsigned long long cap, uint32_t npasses,
-                                                     unsigned long long* hist) {
+                                                     unsigned long long cap, uint32_t npasses, unsigned long long* hist,
+                                                     unsigned long long* status) {
   __shared__ uint32_t h[MAX_PASSES * RADIX];
+  const unsigned long long n = min(*n_ptr, cap);
+  const unsigned long long states = (n + RS_TILE - 1) / RS_TILE * RADIX;
+  for (unsigned long long i = blockIdx.x * RS_T + threadIdx.x; i < states; i += (unsigned long long)gridDim.x * RS_T)
+    status[i] = 0;
+  if ((unsigned long long)blockIdx.x * RS_T * UP_ITEMS >= n) return;   // (no records for this CTA)
   for (uint32_t i = threadIdx.x; i < npasses * RADIX; i += RS_T) h[i] = 0;
   __syncthreads();
-  const unsigned long long n = min(*n_ptr, cap);
   const uint32_t lane = threadIdx.x & 31;
   constexpr uint32_t CHUNK = RS_T * UP_ITEMS;
   const unsigned long long stride = (unsigned long long)gridDim.x * CHUNK;
@@ -254,33 +290,39 @@ __global__ void __launch_bounds__(RS_T) k_rs_upsweep(const Rec* in, const unsign
     if (h[i]) atomicAdd(&hist[i], (unsigned long long)h[i]);
 }
 
-// Per pass, digit counts -> exclusive digit offsets (one CTA of RADIX threads).
-__global__ void __launch_bounds__(RADIX) k_rs_bins(unsigned long long* hist, uint32_t npasses) {
-  __shared__ unsigned long long wsum[RADIX / 32];
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (uint32_t p = 0; p < npasses; ++p) {
-    const unsigned long long v = hist[p * RADIX + threadIdx.x];
-    unsigned long long x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(FULL, x, o);
-      if (lane >= (uint32_t)o) x += y;
+// Every CTA of the sort arrives and waits (bounded) for the others: `count` reaches `target`.
+// What a CTA wrote before is then visible to the others, also to their bulk copies.
+__device__ __forceinline__ bool sort_sync(uint32_t* count, uint32_t target, uint32_t limit) {
+  asm volatile("fence.proxy.async;" ::: "memory");
+  __syncthreads();
+  bool ok = true;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(count, 1u);
+    ok = false;
+    for (uint32_t it = 0; it < limit && !ok; ++it) {
+      uint32_t v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+      ok = v >= target;
+      if (!ok) __nanosleep(20);
     }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    unsigned long long before = 0;
-    for (uint32_t w = 0; w < wid; ++w) before += wsum[w];
-    hist[p * RADIX + threadIdx.x] = before + x - v;
-    __syncthreads();
+    __threadfence();
   }
+  ok = !__syncthreads_or(!ok);
+  asm volatile("fence.proxy.async;" ::: "memory");
+  return ok;
 }
 
-// One pass of the stable LSD radix sort (onesweep): persistent CTAs claim tiles in order from
-// a counter, so every tile's predecessors are claimed by running CTAs and the look-back ends
+// The stable LSD radix sort (onesweep).  What bounds small sorts is launches: the report entries'
+// twelve passes, each a kernel with two memsets before it, took most of the 220 us of a small
+// check.  So their passes are one cooperative kernel, where a sort of one tile runs in one CTA
+// without any wait between CTAs, and no pass needs a memset.  A pass in which all records have the same digit changes nothing and is
+// left out there (the host bounds the digits by the widest possible key).  In a pass, CTAs claim tiles in
+// order from a counter, so every tile's predecessors are claimed by running CTAs and the look-back ends
 // (a CTA also holds the tile it prefetches, but that one comes after its current tile, so the
 // lowest unfinished tile is always some CTA's current tile).
 // status[tile * RADIX + d] holds ST_AGG | the tile's count of digit d, then ST_INC | the count
-// of digit d in tiles 0..tile (zero: not yet known); it is cleared before every pass.
+// of digit d in tiles 0..tile, both with the pass (ST_TAG); anything else: not yet known.
 // Two tile buffers: while a tile is ranked, placed and written from one, the CTA's next tile
 // streams into the other by a TMA bulk copy.  The tile's records are held in registers after
 // ranking, so it is placed in digit order in its own buffer.
@@ -299,30 +341,57 @@ __device__ __forceinline__ void claim_tile(const Rec* in, Rec* dst, unsigned lon
   }
 }
 
+struct SortArgs {
+  const unsigned long long* n_ptr;  // records; at most cap count
+  unsigned long long cap;
+  uint32_t npasses;
+  const unsigned long long* hist;   // npasses x RADIX digit counts
+  unsigned long long* status;
+  uint32_t* tile_ctr;               // per pass (zero before the launch)
+  uint32_t* sync;                   // arrivals of the CTAs (zero before the launch)
+  uint32_t* where;                  // out: the result is in the second buffer (zero before the launch)
+  uint32_t* err;
+  uint32_t spin_limit;
+};
+
+template <class Rec>
+struct SortSmem {
+  uint16_t whist[RS_WARPS][RADIX];                // per warp and digit: count, then offset
+  uint16_t tstart[RADIX];                         // tile-local start of each digit
+  uint32_t thist[RADIX];                          // the tile's count of each digit
+  unsigned long long gdst[RADIX];                 // output index of tile position 0 per digit
+  unsigned long long bins[RADIX], bsum[RS_WARPS]; // where each digit starts
+  uint32_t wsum[RS_WARPS];
+  unsigned long long mbar[2];
+  uint32_t s_tile[2];
+};
+
+// One pass (every thread of the CTA); cur, phases: the tile buffer and the buffers' mbarrier
+// parities, from pass to pass.  False: a copy did not land, the CTA takes no more tiles.
 template <class Rec, class Digit>
-__global__ void __launch_bounds__(RS_T, sizeof(Rec) == 16 ? 3 : 1)
-    k_rs_pass(const Rec* __restrict__ in, Rec* __restrict__ out, const unsigned long long* n_ptr,
-              unsigned long long cap, uint32_t pass, const unsigned long long* bins, unsigned long long* status,
-              uint32_t* tile_ctr, uint32_t* err, uint32_t spin_limit) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  Rec* const buf0 = reinterpret_cast<Rec*>(smem);
-  __shared__ uint16_t whist[RS_WARPS][RADIX];                // per warp and digit: count, then offset
-  __shared__ uint16_t tstart[RADIX];                         // tile-local start of each digit
-  __shared__ uint32_t thist[RADIX];                          // the tile's count of each digit
-  __shared__ unsigned long long gdst[RADIX];                 // output index of tile position 0 per digit
-  __shared__ uint32_t wsum[RS_WARPS];
-  __shared__ __align__(8) unsigned long long mbar[2];
-  __shared__ uint32_t s_tile[2];
+__device__ __forceinline__ bool rs_pass(const Rec* __restrict__ in, Rec* __restrict__ out, unsigned long long n,
+                                        uint32_t pass, const SortArgs& A, Rec* buf0, SortSmem<Rec>& S, uint32_t& cur,
+                                        uint32_t& phases) {
   const uint32_t tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
-  const unsigned long long n = min(*n_ptr, cap);
+  auto& whist = S.whist; auto& tstart = S.tstart; auto& thist = S.thist; auto& gdst = S.gdst; auto& bins = S.bins;
+  auto& wsum = S.wsum; auto& mbar = S.mbar; auto& s_tile = S.s_tile;
   const unsigned long long ntiles = (n + RS_TILE - 1) / RS_TILE;
-  if (tid == 0) {
-    mbar_init(&mbar[0]);
-    mbar_init(&mbar[1]);
-    claim_tile(in, buf0, n, ntiles, tile_ctr, &s_tile[0], &mbar[0]);
+  uint32_t* const tile_ctr = A.tile_ctr + pass;
+  // the digits' counts -> where each digit starts; all records in one digit: nothing to do
+  {
+    const unsigned long long dn = A.hist[pass * RADIX + tid];
+    unsigned long long bin = dn;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(FULL, bin, o);
+      if (lane >= (uint32_t)o) bin += y;
+    }
+    if (lane == 31) S.bsum[w] = bin;
+    if (tid == 0) claim_tile(in, buf0 + cur * RS_TILE, n, ntiles, tile_ctr, &s_tile[cur], &mbar[cur]);
+    __syncthreads();
+    for (uint32_t ww = 0; ww < w; ++ww) bin += S.bsum[ww];
+    bins[tid] = bin - dn;
   }
-  __syncthreads();
-  uint32_t cur = 0, phases = 0;                              // bit b: buffer b's mbarrier parity
   for (;;) {
     const unsigned long long tile = s_tile[cur];
     if (tile >= ntiles) break;
@@ -337,11 +406,11 @@ __global__ void __launch_bounds__(RS_T, sizeof(Rec) == 16 ? 3 : 1)
     // copies are drained before the CTA stops taking tiles
     const bool ok = !__syncthreads_or(!mbar_wait(&mbar[cur], (phases >> cur) & 1u, kCopyWaitLimit));
     if (!ok) {
-      if (tid == 0) atomicOr(err, 1u);
+      if (tid == 0) atomicOr(A.err, 1u);
       __syncthreads_or(!mbar_wait(&mbar[cur], (phases >> cur) & 1u, kCopyWaitLimit));
       if (s_tile[cur ^ 1u] < ntiles)
         __syncthreads_or(!mbar_wait(&mbar[cur ^ 1u], (phases >> (cur ^ 1u)) & 1u, kCopyWaitLimit));
-      break;
+      return false;
     }
     phases ^= 1u << cur;
 
@@ -364,7 +433,7 @@ __global__ void __launch_bounds__(RS_T, sizeof(Rec) == 16 ? 3 : 1)
       }
     }
     __syncthreads();
-    st_relaxed_u64(status + tile * RADIX + tid, (tile == 0 ? ST_INC : ST_AGG) | thist[tid]);   // digit tid
+    st_relaxed_u64(A.status + tile * RADIX + tid, (tile == 0 ? ST_INC : ST_AGG) | (unsigned long long)(pass + 1u) << ST_TAG | thist[tid]);   // digit tid
 
     // rank: warp w takes records [256 w, 256 w + 256) in 8 steps of 32 consecutive records;
     // a group of lanes with one digit adds itself to the warp's count in one step, in lane
@@ -413,7 +482,7 @@ __global__ void __launch_bounds__(RS_T, sizeof(Rec) == 16 ? 3 : 1)
     if (lane == 31) wsum[w] = x;
     // decoupled look-back for digit d: add the predecessors' counts until one whose inclusive
     // prefix is known, publish the inclusive prefix
-    unsigned long long* st = status + tile * RADIX + d;
+    unsigned long long* st = A.status + tile * RADIX + d;
     unsigned long long excl = 0;
     if (tile != 0) {                 // (the tile's count went out before the ranking)
       // the predecessors' words for digit d, LB tiles at a time (independent loads in flight
@@ -426,14 +495,14 @@ __global__ void __launch_bounds__(RS_T, sizeof(Rec) == 16 ? 3 : 1)
         unsigned long long v[LB];
 #pragma unroll
         for (uint32_t q = 0; q < LB; ++q)
-          if (q < k) v[q] = ld_relaxed_u64(status + (top - 1 - q) * RADIX + d);
+          if (q < k) v[q] = ld_relaxed_u64(A.status + (top - 1 - q) * RADIX + d);
 #pragma unroll
         for (uint32_t q = 0; q < LB; ++q) {
           if (q >= k || found || waited_out) break;
-          const unsigned long long* sp = status + (top - 1 - q) * RADIX + d;
+          const unsigned long long* sp = A.status + (top - 1 - q) * RADIX + d;
           unsigned long long y = v[q];
-          for (uint32_t it = 0; !(y & (ST_AGG | ST_INC)); ++it) {
-            if (it >= spin_limit) {
+          for (uint32_t it = 0; ((uint32_t)(y >> ST_TAG) & 63u) != pass + 1u; ++it) {
+            if (it >= A.spin_limit) {
               waited_out = true;
               break;
             }
@@ -446,8 +515,8 @@ __global__ void __launch_bounds__(RS_T, sizeof(Rec) == 16 ? 3 : 1)
         }
         top -= k;
       }
-      if (waited_out) atomicOr(err, 1u);
-      st_relaxed_u64(st, ST_INC | (excl + cnt));
+      if (waited_out) atomicOr(A.err, 1u);
+      st_relaxed_u64(st, ST_INC | (unsigned long long)(pass + 1u) << ST_TAG | (excl + cnt));
     }
     __syncthreads();
     uint32_t before = 0;
@@ -472,6 +541,64 @@ __global__ void __launch_bounds__(RS_T, sizeof(Rec) == 16 ? 3 : 1)
     __syncthreads();                 // the buffer is free for the copy issued next iteration
     cur ^= 1u;
   }
+  return true;
+}
+
+// Wide sorts: a kernel per pass (several passes in one kernel took twice as long: the pass's loads and
+// stores were then ordered against one another).
+template <class Rec, class Digit>
+__global__ void __launch_bounds__(RS_T, sizeof(Rec) == 16 ? 3 : 1)
+    k_rs_pass(const Rec* __restrict__ in, Rec* __restrict__ out, SortArgs A, uint32_t pass) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(8) SortSmem<Rec> S;
+  const unsigned long long n = min(*A.n_ptr, A.cap);
+  if (blockIdx.x * (unsigned long long)RS_TILE >= n) return;   // (no tile for this CTA)
+  if (threadIdx.x == 0) {
+    mbar_init(&S.mbar[0]);
+    mbar_init(&S.mbar[1]);
+  }
+  uint32_t cur = 0, phases = 0;
+  rs_pass<Rec, Digit>(in, out, n, pass, A, reinterpret_cast<Rec*>(smem), S, cur, phases);
+}
+
+// All passes in one cooperative kernel, for sorts that are mostly small (see above).
+template <class Rec, class Digit>
+__global__ void __launch_bounds__(RS_T, sizeof(Rec) == 16 ? 3 : 1) k_rs_sort(Rec* in, Rec* out, SortArgs A) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(8) SortSmem<Rec> S;
+  const uint32_t tid = threadIdx.x;
+  const unsigned long long n = min(*A.n_ptr, A.cap);
+  const unsigned long long ntiles = (n + RS_TILE - 1) / RS_TILE;
+  const uint32_t nctas = (uint32_t)min((unsigned long long)gridDim.x, ntiles);   // (the others have no tile)
+  if (blockIdx.x >= nctas) return;
+  uint32_t target = nctas;
+  auto sync = [&]() {
+    if (nctas == 1) {
+      asm volatile("fence.proxy.async;" ::: "memory");
+      __syncthreads();
+      return true;
+    }
+    const bool ok = sort_sync(A.sync, target, kSortSyncLimit);
+    target += nctas;
+    if (!ok && tid == 0) atomicOr(A.err, 1u);
+    return ok;
+  };
+  if (tid == 0) {
+    mbar_init(&S.mbar[0]);
+    mbar_init(&S.mbar[1]);
+  }
+  uint32_t cur = 0, phases = 0, swaps = 0;
+  bool dead = false;
+  for (uint32_t pass = 0; pass < A.npasses; ++pass) {
+    if (__syncthreads_or(A.hist[pass * RADIX + tid] == n)) continue;   // all records have the same digit
+    if (!dead) dead = !rs_pass<Rec, Digit>(in, out, n, pass, A, reinterpret_cast<Rec*>(smem), S, cur, phases);
+    if (!sync()) return;
+    Rec* const t = in;
+    in = out;
+    out = t;
+    swaps ^= 1u;
+  }
+  if (blockIdx.x == 0 && tid == 0) *A.where = swaps;
 }
 
 // ---------------------------------------------------------------- 3. run scan
@@ -556,25 +683,74 @@ __device__ __forceinline__ bool ordered(const GrunArgs& A, const LaunchDev& P0, 
   return (A.ord_bits[P0.ord_off + (bit >> 5)] >> (bit & 31u)) & 1u;
 }
 
-// One thread per run of equal (program, word); records of a run are in (launch, block, epoch)
-// order.  A thread looks at record i, and takes the run that starts there.
-__global__ void __launch_bounds__(256) k_grun(GrunArgs A) {
+// One thread per run of equal (program, word) of two records or more (one record holds no pair);
+// records of a run are in (launch, block, epoch) order.  What bounds it is latency: a run is a chain
+// of dependent reads, and runs start at a few lanes of a warp only.  So a CTA takes GR_T records
+// into shared memory, with GR_HALO behind them (a run that goes on past these is read from memory),
+// collects the places where runs start, and then every thread has a run.  With a thread per record
+// and no tile this kernel took 348 us for 6.3 M records of a stencil; the whole check of the
+// 1024^2 stencil's eight launches went from 2,230 to 1,310 us.
+constexpr uint32_t GR_T = 1024, GR_HALO = 256, GR_N = 256, GR_PROGS = 512;
+__global__ void __launch_bounds__(GR_N) k_grun(GrunArgs A) {
+  __shared__ uint4 tile[GR_T + GR_HALO + 1];       // records t0 - 1 .. t0 + GR_T + GR_HALO - 1
+  __shared__ uint16_t start[GR_T];
+  __shared__ uint32_t nstart;
+  __shared__ uint32_t pr[GR_T + GR_HALO + 1];      // with several programs: the records' programs
+  __shared__ uint32_t pfirst[GR_PROGS];            // with a few: the programs' first blocks
   const unsigned long long n = *A.n_ptr;
-  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const uint4 r0 = A.rec[i];
+  const uint32_t tid = threadIdx.x, lane = tid & 31u;
+  const uint32_t prog0 = A.launches[A.li0].prog;   // (launches are in program order)
+  const uint32_t nprog = A.launches[A.li1 - 1].prog - prog0 + 1u;
+  const bool one_prog = nprog == 1u, few = nprog <= GR_PROGS;
+  if (!one_prog && few) {
+    // (a program without launches gets the next one's first block, so the search passes over it)
+    for (uint32_t l = A.li0 + tid; l < A.li1; l += GR_N) {
+      const LaunchDev& L = A.launches[l];
+      for (uint32_t p = l == A.li0 ? prog0 : A.launches[l - 1].prog + 1u; p <= L.prog; ++p)
+        pfirst[p - prog0] = L.block_base;
+    }
+    __syncthreads();
+  }
+  auto prog_of = [&](uint32_t gb) {
+    if (!few) return A.launches[find_launch(A, gb)].prog;
+    uint32_t lo = 0, hi = nprog - 1;
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (pfirst[mid] <= gb) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+  };
+  // tile[i] and tile[i + 1] belong to one run
+  auto same_run = [&](uint32_t i) { return tile[i].x == tile[i + 1].x && (one_prog || pr[i] == pr[i + 1]); };
+  for (unsigned long long t0 = (unsigned long long)blockIdx.x * GR_T; t0 < n; t0 += (unsigned long long)gridDim.x * GR_T) {
+  const uint32_t nt = (uint32_t)min((unsigned long long)(GR_T + GR_HALO), n - t0), own = min(nt, GR_T);
+  __syncthreads();                                 // (the last tile's runs are done)
+  for (uint32_t i = tid; i <= nt; i += GR_N)
+    if (t0 + i > 0) {
+      const uint4 q = A.rec[t0 + i - 1];
+      tile[i] = q;
+      if (!one_prog) pr[i] = prog_of(q.w);
+    }
+  if (tid == 0) nstart = 0;
+  __syncthreads();
+  for (uint32_t i0 = 0; i0 < own; i0 += GR_N) {    // (the same trips for every thread of a warp)
+    const uint32_t i = i0 + tid;
+    const bool st = i < own && i + 1 < nt && (t0 + i == 0 || !same_run(i)) && same_run(i + 1);
+    const uint32_t m = __ballot_sync(FULL, st);
+    uint32_t at = 0;
+    if (lane == 0 && m) at = atomicAdd(&nstart, (uint32_t)__popc(m));
+    at = __shfl_sync(FULL, at, 0);
+    if (st) start[at + __popc(m & lanemask_lt())] = (uint16_t)i;
+  }
+  __syncthreads();
+  const uint32_t nst = nstart;
+  for (uint32_t x = tid; x < nst; x += GR_N) {
+    const unsigned long long i = t0 + start[x];
+    auto rec = [&](unsigned long long j) { return j - t0 < nt ? tile[j - t0 + 1] : A.rec[j]; };
+    const uint4 r0 = rec(i);
     uint32_t li = find_launch(A, r0.w);
     const uint32_t prog = A.launches[li].prog;
-    if (i > 0) {
-      const uint4 q = A.rec[i - 1];
-      if (q.x == r0.x && A.launches[find_launch(A, q.w)].prog == prog) continue;   // not a run start
-    }
-    // a run of one record holds no pair: nothing to decide
-    if (i + 1 >= n) continue;
-    {
-      const uint4 q = A.rec[i + 1];
-      if (q.x != r0.x || A.launches[find_launch(A, q.w)].prog != prog) continue;
-    }
+    uint32_t base = A.launches[li].block_base, grid = A.launches[li].grid;   // of launch li
     const uint32_t word = r0.x;
     const LaunchDev& P0 = A.launches[A.launches[li].first_launch];    // the program's launch 0
     const bool pairs = P0.ord_off != kNoDep;                          // unordered launches exist
@@ -590,10 +766,12 @@ __global__ void __launch_bounds__(256) k_grun(GrunArgs A) {
       uint4 q = make_uint4(0, 0, 0, 0);
       uint32_t qli = li;
       if (!end) {
-        q = A.rec[j];
-        const LaunchDev& Lc = A.launches[li];
-        qli = (q.w >= Lc.block_base && q.w - Lc.block_base < Lc.grid) ? li : find_launch(A, q.w);
-        end = q.x != word || A.launches[qli].prog != prog;
+        q = rec(j);
+        end = q.x != word;
+        if (!end && (q.w < base || q.w - base >= grid)) {
+          qli = find_launch(A, q.w);
+          end = A.launches[qli].prog != prog;
+        }
       }
       // interval boundary: (block, epoch) changes
       if (igb != kInf && (end || q.w != igb || q.y != iep)) {
@@ -616,11 +794,11 @@ __global__ void __launch_bounds__(256) k_grun(GrunArgs A) {
           const uint32_t l = L.launch;
           unsigned long long k = i;
           while (k < lstart) {
-            const uint32_t mli = find_launch(A, A.rec[k].w);
+            const uint32_t mli = find_launch(A, rec(k).w);
             const LaunchDev& M = A.launches[mli];
-            uint32_t mk = 1u << grec_write(A.rec[k]);      // (the first record is M's: progress)
-            for (++k; k < lstart && A.rec[k].w >= M.block_base && A.rec[k].w - M.block_base < M.grid; ++k)
-              mk |= 1u << grec_write(A.rec[k]);
+            uint32_t mk = 1u << grec_write(rec(k));      // (the first record is M's: progress)
+            for (++k; k < lstart && rec(k).w >= M.block_base && rec(k).w - M.block_base < M.grid; ++k)
+              mk |= 1u << grec_write(rec(k));
             const uint32_t m = M.launch;
             if (ordered(A, P0, m, l)) continue;
             uint32_t c = 0;
@@ -657,14 +835,19 @@ __global__ void __launch_bounds__(256) k_grun(GrunArgs A) {
         lk = 0;
         lstart = j;
       }
-      const uint32_t blk = q.w - A.launches[qli].block_base;
+      if (qli != li) {
+        li = qli;
+        base = A.launches[li].block_base;
+        grid = A.launches[li].grid;
+      }
+      const uint32_t blk = q.w - base;
       if (wr) min2_32(lW[0], lW[1], blk); else min2_32(lR[0], lR[1], blk);
       lpl = min(lpl, pc);
       lph = max(lph, pc);
       lk |= 1u << wr;
-      li = qli;
     }
     if (pcls) emit_entry(A, A.launches[P0.first_launch + b1].block_base, 2u, word, b2, pcls << 24);
+  }
   }
 }
 
@@ -681,14 +864,14 @@ cudaError_t init_gcheck_attributes(uint32_t smem_optin) {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rs_pass<Rec16, AddrDigit>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(2 * RS_TILE * sizeof(Rec16)));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_rs_pass<Rec32, EntryDigit>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_rs_sort<Rec32, EntryDigit>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(2 * RS_TILE * sizeof(Rec32)));
   int b16 = 0, b32 = 0;
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b16, k_rs_pass<Rec16, AddrDigit>, RS_T,
                                                       2 * RS_TILE * sizeof(Rec16));
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b32, k_rs_pass<Rec32, EntryDigit>, RS_T,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b32, k_rs_sort<Rec32, EntryDigit>, RS_T,
                                                       2 * RS_TILE * sizeof(Rec32));
   g_pass_ctas16 = (uint32_t)std::max(1, b16) * (uint32_t)sms;
   g_pass_ctas32 = (uint32_t)std::max(1, b32) * (uint32_t)sms;
@@ -703,43 +886,45 @@ static cudaError_t count_scan(const uint32_t* c, uint32_t gb0, uint32_t gb1, uns
                               unsigned long long* off, unsigned long long* total, uint32_t& kernels,
                               cudaStream_t s) {
   const uint32_t nchunks = (gb1 - gb0 + SC_CHUNK - 1) / SC_CHUNK;
-  if (nchunks) k_count_chunks<<<nchunks, SC_T, 0, s>>>(c, gb0, gb1, partials);
+  if (nchunks <= SC_ONE) {
+    k_count_one<<<1, SC_T, 0, s>>>(c, gb0, gb1, off, total);
+    ++kernels;
+    return cudaGetLastError();
+  }
+  k_count_chunks<<<nchunks, SC_T, 0, s>>>(c, gb0, gb1, partials);
   k_count_scan<<<1, SC_T, 0, s>>>(partials, nchunks, total);
-  if (nchunks) k_count_offsets<<<nchunks, SC_T, 0, s>>>(c, gb0, gb1, partials, off);
-  kernels += nchunks ? 3 : 1;
+  k_count_offsets<<<nchunks, SC_T, 0, s>>>(c, gb0, gb1, partials, off);
+  kernels += 3;
   return cudaGetLastError();
 }
 
-// sort n (device count, at most cap) records of `in` by `npasses` digits; returns the buffer
-// holding the result (in or tmp)
-template <class Rec, class Digit>
+// Sort n (device count, at most cap) records of `in` by `npasses` digits.  which: 0 or 1, the wave's
+// sort.  Small: mostly a few records; the passes are one kernel, and the result is in `tmp` where
+// G.where[which] is set.  Else it is in `tmp` after an odd number of passes.
+template <class Rec, class Digit, bool Small>
 static cudaError_t radix_sort(Rec* in, Rec* tmp, const unsigned long long* n_ptr, unsigned long long cap,
-                              uint32_t npasses, const GcheckArgs& G, uint32_t ctas, Rec** result,
-                              uint32_t& kernels, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(G.hist, 0, MAX_PASSES * RADIX * 8, s);
+                              uint32_t npasses, const GcheckArgs& G, uint32_t ctas, uint32_t which, uint32_t& kernels,
+                              cudaStream_t s) {
+  unsigned long long* hist = G.hist + which * MAX_PASSES * RADIX;
+  const uint32_t up = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(1, (cap + RS_T * UP_ITEMS - 1) / (RS_T * UP_ITEMS)),
+                                                   8ull * G.sms);
+  k_rs_upsweep<Rec, Digit><<<up, RS_T, 0, s>>>(in, n_ptr, cap, npasses, hist, G.status);
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const uint64_t tiles = gcheck_tiles(cap);
-  const uint32_t up = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(1, (cap + RS_T - 1) / RS_T), 8ull * G.sms);
-  k_rs_upsweep<Rec, Digit><<<up, RS_T, 0, s>>>(in, n_ptr, cap, npasses, G.hist);
-  k_rs_bins<<<1, RADIX, 0, s>>>(G.hist, npasses);
-  kernels += 2;
-  Rec* a = in;
-  Rec* b = tmp;
-  const uint32_t grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(tiles, ctas));
-  for (uint32_t p = 0; p < npasses; ++p) {
-    e = cudaMemsetAsync(G.status, 0, std::max<uint64_t>(1, tiles) * RADIX * 8, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(G.tile_ctr + p, 0, 4, s);
-    if (e != cudaSuccess) return e;
-    k_rs_pass<Rec, Digit><<<grid, RS_T, 2 * RS_TILE * sizeof(Rec), s>>>(a, b, n_ptr, cap, p, G.hist + p * RADIX,
-                                                                       G.status, G.tile_ctr + p, G.err,
-                                                                       G.spin_limit);
-    ++kernels;
-    Rec* t = a;
-    a = b;
-    b = t;
+  SortArgs A{n_ptr,         cap,           npasses, hist, G.status, G.tile_ctr + which * MAX_PASSES, G.sync + which,
+             G.where + which, G.err, G.spin_limit};
+  const uint32_t grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(gcheck_tiles(cap), ctas));
+  const size_t smem = 2 * RS_TILE * sizeof(Rec);
+  if constexpr (Small) {
+    void* args[] = {&in, &tmp, &A};
+    kernels += 2;
+    return cudaLaunchCooperativeKernel((const void*)k_rs_sort<Rec, Digit>, dim3(grid), dim3(RS_T), args, smem, s);
+  } else {
+    for (uint32_t p = 0; p < npasses; ++p)
+      k_rs_pass<Rec, Digit><<<grid, RS_T, smem, s>>>(p & 1u ? tmp : in, p & 1u ? in : tmp, A, p);
+    kernels += 1 + npasses;
+    return cudaGetLastError();
   }
-  *result = a;
-  return cudaGetLastError();
 }
 
 cudaError_t launch_gcheck(const GcheckArgs& G, uint32_t& kernels, cudaStream_t s) {
@@ -754,13 +939,12 @@ cudaError_t launch_gcheck(const GcheckArgs& G, uint32_t& kernels, cudaStream_t s
     ++kernels;
   }
   // 2. sort by word address
-  Rec16* sorted = nullptr;
-  e = radix_sort<Rec16, AddrDigit>(reinterpret_cast<Rec16*>(G.sort_a), reinterpret_cast<Rec16*>(G.sort_b),
-                                   G.gtotal, G.rec_cap, G.addr_passes, G, g_pass_ctas16, &sorted, kernels, s);
+  e = radix_sort<Rec16, AddrDigit, false>(reinterpret_cast<Rec16*>(G.sort_a), reinterpret_cast<Rec16*>(G.sort_b),
+                                   G.gtotal, G.rec_cap, G.addr_passes, G, g_pass_ctas16, 0, kernels, s);
   if (e != cudaSuccess) return e;
   // 3. the run scan (gn and gcount start from zero: launch_reset)
   GrunArgs R{};
-  R.rec = reinterpret_cast<const uint4*>(sorted);
+  R.rec = G.addr_passes & 1u ? G.sort_b : G.sort_a;
   R.n_ptr = G.gtotal;
   R.launches = G.launches;
   R.li0 = G.li0;
@@ -771,16 +955,14 @@ cudaError_t launch_gcheck(const GcheckArgs& G, uint32_t& kernels, cudaStream_t s
   R.gn = G.gn;
   R.gcount = G.gcount;
   {
-    const uint32_t ctas = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((G.rec_cap + 255) / 256, 16ull * G.sms));
-    k_grun<<<ctas, 256, 0, s>>>(R);
+    const uint32_t ctas = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((G.rec_cap + GR_T - 1) / GR_T, 8ull * G.sms));
+    k_grun<<<ctas, GR_N, 0, s>>>(R);
     ++kernels;
   }
   // 4. the entries in (block, epoch, kind, word) order, and each block's first entry
-  Rec32* ordered_entries = nullptr;
-  e = radix_sort<Rec32, EntryDigit>(reinterpret_cast<Rec32*>(G.entries_a), reinterpret_cast<Rec32*>(G.entries_b),
-                                    G.gn, G.entry_cap, MAX_PASSES, G, g_pass_ctas32, &ordered_entries, kernels, s);
+  e = radix_sort<Rec32, EntryDigit, true>(reinterpret_cast<Rec32*>(G.entries_a), reinterpret_cast<Rec32*>(G.entries_b),
+                                    G.gn, G.entry_cap, MAX_PASSES, G, g_pass_ctas32, 1, kernels, s);
   if (e != cudaSuccess) return e;
-  // (12 passes: the result is back in entries_a)
   return count_scan(G.gcount, G.gb0, G.gb1, G.partials, G.gstart, G.gn_sorted, kernels, s);
 }
 

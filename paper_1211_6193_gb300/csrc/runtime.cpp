@@ -90,7 +90,7 @@ struct sr_batch {
   uint64_t out_cap = 0;
   // global-memory race check (opts.check_global)
   DevBuf glog, glog_n, goff, gpartials, gtotal, sort_a, sort_b, hist, status, tile_ctr, ord_bits, entries_a, entries_b,
-      gn, gcount, gstart, gn_sorted;
+      gn, gcount, gstart, gn_sorted, gsync;       // (gsync: per wave two sorts' arrivals, then their results' places)
   std::vector<uint32_t> ord_bits_h;
   uint64_t glog_records = 0;               // largest wave's global-log records
   uint64_t entry_cap = 0;                  // report entries of one wave that fit
@@ -160,7 +160,7 @@ void free_batch_buffers(sr_ctx* c, sr_batch* b, cudaStream_t s) {
                    &b->launch_done, &b->scratch, &b->work_head, &b->offsets, &b->partials,
                    &b->out, &b->total, &b->item_launch_d, &b->glog, &b->glog_n, &b->goff, &b->gpartials,
                    &b->gtotal, &b->sort_a, &b->sort_b, &b->hist, &b->status, &b->tile_ctr, &b->ord_bits,
-                   &b->entries_a, &b->entries_b, &b->gn, &b->gcount, &b->gstart, &b->gn_sorted,
+                   &b->entries_a, &b->entries_b, &b->gn, &b->gcount, &b->gstart, &b->gn_sorted, &b->gsync,
                    &b->bq_launch_d, &b->bq_first_d, &b->bq_head};
   for (DevBuf* d : all) dev_free(c, *d, s);
 }
@@ -197,6 +197,8 @@ sr::CompactArgs compact_args(sr_batch* b, uint32_t wi) {
     ka.gcount = (const uint32_t*)b->gcount.p;
     ka.gstart = (const unsigned long long*)b->gstart.p;
     ka.gentries = (const uint4*)b->entries_a.p;
+    ka.gentries_b = (const uint4*)b->entries_b.p;
+    ka.gwhere = (const uint32_t*)b->gsync.p + 4 * wi + 3;
     ka.gcap = b->entry_cap;
   }
   return ka;
@@ -220,10 +222,12 @@ sr::GcheckArgs gcheck_args(sr_ctx* c, sr_batch* b, uint32_t wi) {
   g.sort_b = (uint4*)b->sort_b.p;
   g.rec_cap = w.glog_records;
   g.addr_passes = std::max(1u, (w.addr_bits + 7) / 8);
-  g.hist = (unsigned long long*)b->hist.p;
+  g.hist = (unsigned long long*)b->hist.p + (size_t)wi * 2 * 12 * 256;
   g.status = (unsigned long long*)b->status.p;
-  g.tile_ctr = (uint32_t*)b->tile_ctr.p;
+  g.tile_ctr = (uint32_t*)b->tile_ctr.p + (size_t)wi * 2 * 12;
   g.err = err_flag(b);
+  g.sync = (uint32_t*)b->gsync.p + 4 * wi;
+  g.where = g.sync + 2;
   g.spin_limit = c->opts.spin_limit;
   g.sms = (uint32_t)c->sms;
   g.ord_bits = (const uint32_t*)b->ord_bits.p;
@@ -265,6 +269,9 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
   if (o.check_global) {
     zero(b->glog_n, (size_t)b->nblocks * 4);
     zero(b->gn, b->waves.size() * 8);
+    zero(b->gsync, b->waves.size() * 16);
+    zero(b->hist, b->waves.size() * 2 * 12 * 256 * 8);
+    zero(b->tile_ctr, b->waves.size() * 2 * 12 * 4);
     zero(b->gcount, (size_t)b->nblocks * 4);
   }
   CUDA_TRY(c, sr::launch_reset(za, (uint32_t)c->sms, s));
@@ -733,10 +740,10 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       {&b->gtotal, 8, "global record total"},
       {&b->sort_a, (size_t)b->glog_records * 16, "global sort buffer"},
       {&b->sort_b, (size_t)b->glog_records * 16, "global sort buffer"},
-      {&b->hist, o.check_global ? (size_t)12 * 256 * 8 : 0, "digit histograms"},
+      {&b->hist, o.check_global ? (size_t)nwaves * 2 * 12 * 256 * 8 : 0, "digit histograms"},
       {&b->status, o.check_global ? sr::gcheck_tiles(std::max(b->glog_records, b->entry_cap)) * 256 * 8 : 0,
        "sort tile states"},
-      {&b->tile_ctr, 12 * 4, "sort tile counters"},
+      {&b->tile_ctr, (size_t)nwaves * 2 * 12 * 4, "sort tile counters"},
       {&b->ord_bits, std::max<size_t>(1, b->ord_bits_h.size()) * 4, "launch-order matrices"},
       {&b->entries_a, o.check_global ? (size_t)b->entry_cap * 32 : 0, "global race entries"},
       {&b->entries_b, o.check_global ? (size_t)b->entry_cap * 32 : 0, "global race entries"},
@@ -744,6 +751,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       {&b->gcount, o.check_global ? (size_t)b->nblocks * 4 : 0, "global entries per block"},
       {&b->gstart, o.check_global ? ((size_t)b->nblocks + 1) * 8 : 0, "global entry offsets"},
       {&b->gn_sorted, 8, "global entry total"},
+      {&b->gsync, (size_t)nwaves * 16, "sort progress"},
   };
   for (auto& a : allocs) {
     rc = alloc_buf(c, *a.buf, a.bytes, s, a.what);

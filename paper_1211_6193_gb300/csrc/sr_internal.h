@@ -290,9 +290,11 @@ struct GcheckArgs {
   uint4* sort_b;
   unsigned long long rec_cap;       // >= the wave's records
   uint32_t addr_passes;             // 8-bit digits of the largest word address of the wave
-  unsigned long long* hist;         // 12 x 256 digit counts
+  unsigned long long* hist;         // per sort of the wave 12 x 256 digit counts (zero at the start of the run)
   unsigned long long* status;       // gcheck_tiles(max(rec_cap, entry_cap)) x 256 tile states
-  uint32_t* tile_ctr;               // 12 tile counters
+  uint32_t* tile_ctr;               // per sort of the wave 12 tile counters (zero at the start of the run)
+  uint32_t* sync;                   // per sort of the wave: arrivals of its CTAs,
+  uint32_t* where;                  // and where its result is (both zero at the start of the run)
   uint32_t* err;                    // set when a bounded wait gave up
   uint32_t spin_limit;
   uint32_t sms;
@@ -329,7 +331,9 @@ struct CompactArgs {
   // the wave its first entry, and the entries in (block, epoch, kind, word) order
   const uint32_t* gcount;
   const unsigned long long* gstart;
-  const uint4* gentries;
+  const uint4* gentries;        // here, or, where *gwhere is set, there
+  const uint4* gentries_b;
+  const uint32_t* gwhere;
   unsigned long long gcap;      // entries the buffer holds (a wave that produced more is run again)
   uint32_t* error_flag;         // debug build: kErrBounds
 };
@@ -347,7 +351,7 @@ struct ResetArgs {
   struct Zero {
     uint32_t* p;
     unsigned long long words;
-  } zero[12];
+  } zero[16];
   uint32_t nzero;
 };
 cudaError_t launch_reset(const ResetArgs& a, uint32_t sms, cudaStream_t s);

@@ -140,3 +140,20 @@ def test_report_compaction_sizes(B, blocks):
     p = Program(a.assemble(), [0], [Launch(0, blocks, 32, 8, ())], np.zeros(4, np.int32))
     got = assert_same(B, [p], {"mode": "batched"}, {})
     assert len(got.reports) == 4 * ((blocks + 2) // 3)
+
+
+def test_global_check_groups_by_program(B):
+    """Racing programs with the same words, one without a launch among them, more runs than a tile."""
+    def prog(i):
+        a = Asm().s2r(r2, TID).s2r(r3, BID).mul(r4, r3, 64).add(r4, r4, r2).and_(r4, r4, 255).stg(r4, r2)
+        a.ldg(r5, r4, i % 3).exit()
+        return Program(a.assemble(), [0], [Launch(0, 9, 64, 1, ())] if i != 3 else [], np.zeros(300, np.int32))
+    for mode in ("plain", "batched"):
+        got = assert_same(B, [prog(i) for i in range(7)], {"mode": mode, "check_global": True}, {"check_global": True})
+        assert len(got.reports) > 1500
+    one = Asm().s2r(r2, BID).stg(r2, r2).exit()      # one record per word: no run
+    wide = Program(one.assemble(), [0], [Launch(0, 3000, 1, 1, ())], np.zeros(3000, np.int32))
+    assert len(assert_same(B, [wide], {"check_global": True}, {"check_global": True}).reports) == 0
+    zero = Asm().s2r(r2, BID).mov(r3, 0).ldg(r4, r3).brnz(r2, "end").stg(r3, r2).label("end").exit()
+    deep = Program(zero.assemble(), [0], [Launch(0, 3000, 1, 1, ())], np.zeros(4, np.int32))   # one long run
+    assert len(assert_same(B, [deep], {"check_global": True}, {"check_global": True}).reports) == 1
