@@ -37,9 +37,9 @@
 // (spin_limit) and reports SR_ST_INTERNAL instead of hanging.
 //
 // Measured (GB300, interpreter stage; before: one real warp per simulated warp, everything
-// compiled C++): the reduction of 2^24 values 3,917 -> 2,098 us, 256 generated programs
-// 19,912 -> 8,098 us, 96 of them with default shapes 5,893 -> 2,004 us, the 2048^2 stencil in 16
-// launches 11,302 -> 6,207 us.
+// compiled C++): the reduction of 2^24 values 3,917 -> 1,521 us, 256 generated programs
+// 19,912 -> 7,171 us, 96 of them with default shapes 5,893 -> 1,763 us, the 2048^2 stencil in 16
+// launches 11,302 -> 5,563 us.
 #include <algorithm>
 #include <climits>
 
@@ -853,21 +853,29 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
         solo = sub == can;
         kn = 0;
         if (!solo) {
-          // among the agents at this round: what touches no memory and loads, one pc at a time;
+          // among the agents at this round: what touches no memory, then loads, one pc at a time;
           // then stores (agent by agent when they are at several pcs); then atomics
-          uint32_t cls = 3;
+          uint32_t cls = 4;
           if (cand) {
             const uint32_t o = pk_form(ir[ap].x);
-            cls = (o == F_STS || o == F_STG) ? 1u : o == F_ATOMS ? 2u : 0u;
+            cls = (o == F_LDS || o == F_LDG) ? 1u : (o == F_STS || o == F_STG) ? 2u : o == F_ATOMS ? 3u : 0u;
           }
           const uint32_t first = __reduce_min_sync(FULL, cls);
           const uint32_t of = __ballot_sync(FULL, cls == first);
           p = __shfl_sync(FULL, ap, __ffs(of) - 1);
           sub = __ballot_sync(FULL, cls == first && ap == p);
-          if (first == 1 && (sub != of || clk[w] == 4u * k + 1u + par)) {
+          if (first == 2 && (sub != of || clk[w] == 4u * k + 1u + par)) {
             multi_st = true;                     // (also for the last of them)
             sub &= 0u - sub;
           }
+          // the only set at this round, about to access memory: it may, in the rounds up to the
+          // others' lowest (as long as nothing of this round is published; away from the budget,
+          // which runs of the set may pass otherwise)
+          const uint32_t o = same(pk_form(ir[p].x));
+          kn = __reduce_min_sync(FULL, ap != kInf && !((sub >> lane) & 1u) ? ak : kInf);
+          if (kn == k || multi_st || same(clk[w]) > 4u * k + par || kn + 256u > budget || o < F_LDS || o > F_ATOMS ||
+              o == F_BRZ || o == F_BRNZ)
+            kn = 0;
         }
         wpc = __reduce_min_sync(FULL, (sub >> lane) & 1u ? aw : kInf);
         am = 0;
@@ -910,17 +918,24 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
         epoch = epoch_hi >> 6;
         moved = k != k_in;
         if (fl & kSoloNested) {
-          // some threads wait at a higher pc (at a barrier: agents without a running thread have
-          // executed it)
+          // some threads wait at a higher pc (at a barrier or exit: agents without a running thread
+          // have executed it)
           wpc = (same(qw) - irs) >> 3;
           am = mask & ALL;
+          const bool exits = pk_form(lds_u64(irs + wpc * 8u).x) == F_EXIT;
+          uint32_t gone = 0;
 #pragma unroll
           for (int j = 0; j < V; ++j) {
             const bool at = (fl & kSoloAgents) && !__any_sync(FULL, (am >> j) & 1u);
             if ((mask >> (4 + j)) & 1u) {
-              ts[j] = at ? (wpc + 1u) | ST_WAIT << 16 : wpc;
+              ts[j] = !at ? wpc : exits ? wpc | ST_EXIT << 16 : (wpc + 1u) | ST_WAIT << 16;
               n_instr += at;
+              gone |= (at && exits ? 1u : 0u) << j;
             }
+          }
+          if (exits) {
+            xm |= gone;
+            nexit += __reduce_add_sync(FULL, __popc(gone));
           }
           set_shape();
         }
@@ -934,9 +949,11 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
         }
         if (solo && k >= budget) continue;
       }
-      if (p < wpc && (solo || !moved)) {
       const uint2 in = lds_u64(irs + p * 8u);
-      const uint32_t f = pk_form(in.x), run = f < F_LDS ? lds_u8(irs + ir_code_bytes(ncode) + p) : 0u;
+      const uint32_t f = pk_form(in.x);
+      // (what touches no memory may run ahead of other agents' earlier rounds)
+      if (p < wpc && (solo || !moved || (k < budget && (f > F_ATOMS || f == F_BRZ || f == F_BRNZ)))) {
+      const uint32_t run = f < F_LDS ? lds_u8(irs + ir_code_bytes(ncode) + p) : 0u;
       if (run) {
         // A run of instructions that touch no memory and do not branch executes in a tight loop,
         // one instruction per round; its last round is published at once (other warps wait on
@@ -1274,9 +1291,11 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
                  : "=r"(pb.x), "=r"(pb.y), "=r"(pb.z), "=r"(pb.w) : "r"(parks + 32u * (lane & 7u) + 16u) : "memory");
     const uint32_t kmax = __reduce_max_sync(FULL, v ? pb.z : 0u);
     const uint32_t pc0 = same(pa.w);
-    if (!(fused && same(bv->any_race[par >> 31])) &&
-        __all_sync(FULL, !v || (pa.x && !(pa.y | pa.z | pb.w) && pa.w == pc0 && pb.x == pc0))) {
+    const bool racy = fused && same(bv->any_race[par >> 31]);   // (cleared behind the second barrier)
+    if (!racy && __all_sync(FULL, !v || (pa.x && !(pa.y | pa.z | pb.w) && pa.w == pc0 && pb.x == pc0))) {
       epoch += 1u;
+    } else if (!racy && __all_sync(FULL, !v || !(pa.x | pa.z | pb.w))) {
+      break;                                     // every thread exited, nothing to report
     } else {
       if (w == 0) {
         const uint32_t nW = __reduce_add_sync(FULL, v ? pa.x : 0u);
@@ -1287,10 +1306,7 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
         const uint32_t rpc = __reduce_min_sync(FULL, v ? pb.y : kInf);
         const uint32_t fl = __reduce_or_sync(FULL, v ? pb.w & 0xFFu : 0u);
         const uint32_t nP = __reduce_add_sync(FULL, v ? (pb.w >> 8) & 0xFFFFu : 0u);
-        if (fused && bv->any_race[par >> 31]) {
-          tuples_emit(tup, tps, rbm, bv, region, log_cap - 2u * bv->n_misc, epoch, lane);
-          if (lane == 0) bv->any_race[par >> 31] = 0;
-        }
+        if (racy) tuples_emit(tup, tps, rbm, bv, region, log_cap - 2u * bv->n_misc, epoch, lane);
         uint32_t dec = DEC_RELEASE, kind = 0, a = 0, b = 0, c = 0, stbits = 0;
         if (fl & 2u) {
           dec = DEC_STOP;
@@ -1316,6 +1332,7 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
       }
       block_sync(nthr);
       if (same(bv->decision) != DEC_RELEASE) break;
+      if (t == 0) bv->any_race[par >> 31] = 0;   // (marked again behind the next CTA barrier at the earliest)
       front_cap = log_cap - 2u * same(bv->n_misc);
       epoch += 1u;
     }

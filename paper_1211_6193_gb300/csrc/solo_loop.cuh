@@ -38,14 +38,15 @@ struct SoloConst {
   unsigned long long gregion, pad2;  // the global log
 };
 static_assert(sizeof(SoloConst) == 96 && sizeof(SoloConst) <= kGroupBv - kGroupConst, "solo constants");
-// flags in: several warps; log accesses; barriers may be passed here; the log is full; shared and
-// global accesses may run here (or: with reads of unwritten words checked, with global accesses
-// logged; then the fast bounds checks fail and the access takes the path behind them); every slot whose registers still matter is active; the active
-// slots are slots 0..n-1 of every lane; no other agent can run; summaries instead of the log;
-// clocks are published (no other agent can run, or all others are at later rounds).  Flags out: the log is full; some threads wait at qw for the others to come
-// there (kSoloAgents: some agents as a whole, at a barrier); behind the CTA barrier of a simulated
-// barrier that is not a plain release; a wait gave up.  (One register of bits instead of
-// predicates: there are seven.)
+// Flags in: clocks are published (no other agent can run, or all others are at later rounds);
+// several warps; log accesses; barriers may be passed here; the log is full; shared and global
+// accesses may run here (or: with reads of unwritten words checked, with global accesses logged;
+// then the fast bounds checks fail and the access takes the path behind them); every slot whose
+// registers still matter is active; the active slots are slots 0..n-1 of every lane; no other agent
+// can run; summaries instead of the log.  Flags out: the log is full; some threads wait at qw for
+// the others to come there (kSoloAgents: some agents as a whole, at a barrier or exit); behind the
+// CTA barrier of a simulated barrier that is not a plain release; a wait gave up.  (One register of
+// bits instead of predicates: there are seven.)
 enum : uint32_t {
   kSoloPub = 1, kSoloMany = 2, kSoloLog = 4, kSoloBar = 8, kSoloFull = 16, kSoloShared = 32, kSoloGlobal = 64, kSoloWhole = 128,
   kSoloRegular = 256, kSoloSolo = 512, kSoloFused = 1024, kSoloNested = 2048, kSoloAgents = 4096,
@@ -267,9 +268,10 @@ enum : uint32_t {
       "LTOP:\n"                                                                                                     \
       "and.b32 u, x, 63;\nsetp.ge.u32 pm, u, 32;\n@pm bra.uni LMEM;\n" /* a run starts */                           \
       "ld.shared.u32 u, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 4];\nshr.u32 t, q, 3;\nadd.u32 t, t, u;\nld.shared.u8 t, [t];\n"                           \
-      "sub.u32 u, bud, k4;\nshr.u32 u, u, 2;\nmin.u32 t, t, u;\nsub.u32 u, qw, q;\nshr.u32 u, u, 3;\n"        \
+      "sub.u32 u, bud, k4;\nshr.u32 u, u, 2;\nand.b32 r0, fl, 513;\nsetp.eq.u32 pf, r0, 1;\n@pf mov.u32 u, 255;\n"   \
+      "min.u32 t, t, u;\nsub.u32 u, qw, q;\nshr.u32 u, u, 3;\n" /* (up to other agents' round: not cut, see bud) */  \
       "min.u32 t, t, u;\nmad.lo.u32 qend, t, 8, q;\nmad.lo.u32 k4, t, 4, k4;\n"                                     \
-      "@pp st.release.cta.shared.u32 [myclk], k4;\nmov.u32 keep, 0;\n"                                              \
+      "min.u32 r0, k4, bud;\n@pp st.release.cta.shared.u32 [myclk], r0;\nmov.u32 keep, 0;\n"                                              \
       "LALU:\n"                                                                                                     \
       "and.b32 t, x, keep;\nsetp.eq.u32 pf, t, 0;\n"                                                                \
       "prmt.b32 ro, x, 0, 0x4442;\nmad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n@pf " LDC                            \
@@ -440,12 +442,12 @@ enum : uint32_t {
       "LROWC:\n@!ps bra.uni LROWC1;\n" E(SR_PUT) "bra.uni LROWC1;\n"                                                \
       SR_FLUSH_ANY(E, "A") SR_FLUSH_ANY(E, "B") SR_FLUSH_ANY(E, "C") SR_FLUSH_ANY(E, "D")                           \
       /* A branch forward that parts the threads: those that take it wait at its target, as the lowest-pc rule has   \
-         it, while the others go on here, if every agent has some of these - or if a barrier stands at the target,   \
-         where agents that take it as a whole wait in any case.  Not nested. */                                     \
+         it, while the others go on here, if every agent has some of these - or if a barrier or an exit stands at    \
+         the target, where agents that take it as a whole wait in any case.  Not nested. */                                     \
       "LPARTS:\nsetp.eq.u32 pz, u, 34;\nsetp.ne.u32 pc, 0, 0;\n" E(SR_PARTS)                                        \
       "mad.lo.u32 need, y, 8, irs;\nand.b32 t, fl, 512;\nsetp.ne.u32 pa, t, 0;\nsetp.gt.and.u32 pa, need, q, pa;\n"    \
       "setp.eq.and.u32 pa, qw, 0xFFFFFFF8, pa;\nld.shared.u32 t, [need];\nand.b32 t, t, 63;\nsetp.eq.u32 pb, t, 41;\n" \
-      "and.b32 t, fl, 8;\nsetp.ne.and.u32 pb, t, 0, pb;\nnot.pred pd, pc;\nor.pred pb, pb, pd;\nand.pred pa, pa, pb;\n" \
+      "setp.eq.or.u32 pb, t, 49, pb;\nnot.pred pd, pc;\nor.pred pb, pb, pd;\nand.pred pa, pa, pb;\n"               \
       "selp.u32 t, 14336, 10240, pc;\n@pa or.b32 fl, fl, t;\nbra.uni LEND;\n" /* (kSoloToNest, Nested, Agents) */  \
       "LNEST:\nadd.u32 k4, k4, 4;\nadd.u32 q, q, 8;\nand.b32 t, k4, 0x7FFFFFFF;\nsub.u32 u, t, kst;\nshr.u32 u, u, 2;\n" \
       "mad.lo.u32 ni, u, cnt, ni;\nmov.u32 kst, t;\nmov.u32 qw, need;\nmov.u32 x, nx;\nmov.u32 y, ny;\n"             \
@@ -469,17 +471,18 @@ enum : uint32_t {
       : "+r"(q), "+r"(k4), "+r"(gacc), "+r"(sacc), "+r"(eh), "+r"(ni), "+r"(fl), "+r"(qw), "=r"(mask)               \
       : "r"(gb), "r"(w), "r"(rs), "r"(stride), "r"(am), "r"(fcap), "r"(bud)                                                 \
       : "memory")
-static_assert(F_LDS == 32 && F_STS == 33 && F_BRZ == 34 && F_LDG == 36 && F_ATOMS == 38 && F_S2R == 40 && F_BAR == 41 &&
+static_assert(F_LDS == 32 && F_STS == 33 && F_BRZ == 34 && F_LDG == 36 && F_ATOMS == 38 && F_S2R == 40 && F_BAR == 41 && F_EXIT == 49 &&
                   F_DIVR > 41 && kFwdA == 64 && kDeadD == 128 && kNoDest == 31,
               "forms in solo_loop");
 
 // Runs the set of the active slots `am` from instruction address q and clock k4 (4 * round with
 // the interval's parity in bit 31) while it stays below the address qw and the clock below bud
-// (with the parity too); q, k4, eh (the epoch field
-// of log records), fl (flags), qw and the per-lane counts of global and (fused) shared accesses and of
-// executed instructions are updated.  gb: the block's shared memory; rs, stride: this lane's row 0 and
-// the row stride; fcap: log records that fit.  Returns the slots active at the end, << 4 those that
-// wait at qw.
+// (with the parity too; when bud is other agents' round, a run of instructions that touch no memory
+// goes on past it, uncut - its parts may be one chain - and unpublished there: at most 255 rounds);
+// q, k4, eh (the epoch field of log records), fl (flags), qw and the per-lane counts of global and
+// (fused) shared accesses and of executed instructions are updated.  gb: the block's shared memory;
+// rs, stride: this lane's row 0 and the row stride; fcap: log records that fit.  Returns the slots
+// active at the end, << 4 those that wait at qw.
 template <int V, bool Fused>
 __device__ __forceinline__ uint32_t solo_loop(uint32_t& q, uint32_t& k4, uint32_t& gacc, uint32_t& sacc, uint32_t& eh,
                                               uint32_t& ni, uint32_t& fl, uint32_t& qw, uint32_t gb, uint32_t w,

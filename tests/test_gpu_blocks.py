@@ -157,3 +157,13 @@ def test_global_check_groups_by_program(B):
     zero = Asm().s2r(r2, BID).mov(r3, 0).ldg(r4, r3).brnz(r2, "end").stg(r3, r2).label("end").exit()
     deep = Program(zero.assemble(), [0], [Launch(0, 3000, 1, 1, ())], np.zeros(4, np.int32))   # one long run
     assert len(assert_same(B, [deep], {"check_global": True}, {"check_global": True}).reports) == 1
+
+
+def test_global_check_in_a_graph(B):
+    """The sort's cooperative kernel under capture, and the graph run again."""
+    progs = [random_program(rng.derive(7, i), 96) for i in range(6)]
+    want = oracle.run(progs, check_global=True)
+    with B.Context(mode="batched", check_global=True, use_graph=True) as ctx, ctx.load_programs(progs) as b:
+        for _ in range(3):
+            b.run_and_check()
+            assert [tuple(int(x) for x in r) for r in b.fetch_reports()] == want.report_tuples()
