@@ -14,8 +14,7 @@
 // and dispatch, and these are then paid once for V simulated warps.  A lane's V values of a
 // register lie side by side (one 16-byte shared access for V = 4).  Registers, the simulated
 // shared array and the program's code (staged by a TMA bulk copy) live in shared memory.
-// Small blocks take a smaller V: a block keeps two real warps from 64 threads on, so that
-// latencies overlap.  Instructions run in solo_loop (solo_loop.cuh); what it does not take -
+// Small blocks and small grids take a smaller V.  Instructions run in solo_loop (solo_loop.cuh); what it does not take -
 // agents of a warp at different pcs, colliding or out-of-bounds addresses, barriers with
 // something to report - runs in the general steps of run_block.
 //
@@ -1425,9 +1424,9 @@ __device__ __forceinline__ void run_staged(const RunArgs& A, const LaunchDev* Ls
 
 // One CTA per simulated block; one kernel launch per (program, launch), in an order that
 // respects every stream and wait.  A block takes block_warps(bdim, V) warps: at most 8 with
-// V = 4, two with V = 1 and 2 (block_vec).  MINB: CTAs of that many warps the registers allow.
+// V = 2 and 4, two with V = 1 (block_vec).  MINB: CTAs of that many warps the registers allow.
 template <int V, int MINB, bool Fused, bool Global>
-__global__ void __launch_bounds__(V == 4 ? 256 : 64, MINB) k_interp_plain(RunArgs A, uint32_t li) {
+__global__ void __launch_bounds__(V == 1 ? 64 : 256, MINB) k_interp_plain(RunArgs A, uint32_t li) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ LaunchDev Ls;
   __shared__ __align__(8) unsigned long long mbar;
@@ -1459,7 +1458,7 @@ __global__ void __launch_bounds__(V == 4 ? 256 : 64, MINB) k_interp_plain(RunArg
 // (bounded); else it is the CTA's index.  No loop surrounds the block and its warps are chosen
 // by a warp vote: a persistent loop around it cost several hundred bytes of spills.
 template <int V, int MINB, bool Fused, bool Global>
-__global__ void __launch_bounds__(V == 4 ? 256 : 64, MINB) k_interp_blocks(RunArgs A) {
+__global__ void __launch_bounds__(V == 1 ? 64 : 256, MINB) k_interp_blocks(RunArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ LaunchDev Ls;
   __shared__ __align__(8) unsigned long long mbar;
@@ -1538,7 +1537,7 @@ static PlainKernel plain_of(bool fused, bool global) {
 }
 static PlainKernel plain_kernel(uint32_t vec, uint32_t variant, bool fused, bool global) {
   if (vec == 1) return plain_of<1, 12>(fused, global);
-  if (vec == 2) return plain_of<2, 12>(fused, global);
+  if (vec == 2) return plain_of<2, 3>(fused, global);
   return variant == 2 ? plain_of<4, 4>(fused, global) : plain_of<4, 3>(fused, global);
 }
 template <int V, int MINB>
@@ -1548,7 +1547,7 @@ static BlocksKernel blocks_of(bool fused, bool global) {
 }
 static BlocksKernel blocks_kernel(uint32_t vec, uint32_t variant, bool fused, bool global) {
   if (vec == 1) return blocks_of<1, 12>(fused, global);
-  if (vec == 2) return blocks_of<2, 12>(fused, global);
+  if (vec == 2) return blocks_of<2, 3>(fused, global);
   return variant == 2 ? blocks_of<4, 4>(fused, global) : blocks_of<4, 3>(fused, global);
 }
 

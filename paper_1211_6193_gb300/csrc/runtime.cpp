@@ -503,7 +503,8 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
     // batched mode: a program's launches run in one grid, so they share the kernel form
     uint32_t pvec = 0;
     if (batched)
-      for (uint32_t l = 0; l < P.nlaunches; ++l) pvec = std::max(pvec, sr::block_vec(P.launches[l].block_dim));
+      for (uint32_t l = 0; l < P.nlaunches; ++l)
+        pvec = std::max(pvec, sr::block_vec(P.launches[l].block_dim, P.launches[l].grid, (uint32_t)c->sms));
     // the global-memory race check of a program whose launches are not all ordered needs its
     // launch-order matrix (and all its launches in one wave)
     uint32_t ord_off = sr::kNoDep;
@@ -559,7 +560,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       d.nrows = rm.nrows;
       const uint32_t nsw = (L.block_dim + 31) / 32;         // simulated warps
       d.sha = shared_reach(P.code, P.ncode, d.entry, L, ranges);
-      d.vec = pvec ? pvec : sr::block_vec(L.block_dim);
+      d.vec = pvec ? pvec : sr::block_vec(L.block_dim, d.grid, (uint32_t)c->sms);
       d.nw = sr::block_warps(L.block_dim, d.vec);
       const uint32_t lanes = d.nw * 32 * d.vec;
       d.uninit = o.check_uninit ? 1u : 0u;

@@ -41,10 +41,17 @@ __host__ __device__ constexpr uint32_t pk_make(uint32_t form, uint32_t d, uint32
 // (bit f: a form of runs whose second operand is an immediate)
 constexpr uint32_t kImmForms = 7u | 0x15555500u;
 __host__ __device__ constexpr bool pk_imm(uint32_t form) { return form < F_LDS && ((kImmForms >> form) & 1u); }
-// Simulated warps per real warp of the interpreter for a block of bdim threads, and the real
-// warps the block then takes (at most 8).
-__host__ __device__ constexpr uint32_t block_vec(uint32_t bdim) { return bdim <= 64 ? 1u : bdim <= 128 ? 2u : 4u; }
+// Real warps of a block of bdim threads with vec simulated warps each (at most 8), and the
+// simulated warps per real warp for a launch of `blocks` such blocks.  Decoding an instruction once
+// for four simulated warps is the fastest where the chip is full; a grid that fits it at 16 warps
+// per SM with two is bound by the latency of its blocks instead, and shorter steps pay: 162 blocks of
+// 192 threads 44 -> 35 us, 124 of 448 52 -> 44, eight small generated programs 430 -> 188; past that
+// line the other way round: 1449 of 192 59 -> 74, 1501 of 333 58 -> 102 (blocks above 512 threads
+// would need more than 8 warps).  A block keeps two warps from 64 threads on.
 __host__ __device__ constexpr uint32_t block_warps(uint32_t bdim, uint32_t vec) { return (bdim + 32u * vec - 1u) / (32u * vec); }
+__host__ __device__ constexpr uint32_t block_vec(uint32_t bdim, uint64_t blocks, uint32_t sms) {
+  return bdim <= 64 ? 1u : bdim <= 128 || (bdim <= 512 && blocks * block_warps(bdim, 2) <= 16ull * sms) ? 2u : 4u;
+}
 constexpr uint32_t kInf = 0xFFFFFFFFu;
 constexpr uint32_t kMaxBudget = 1u << 26;  // epochs and rounds stay below 2^26
 // Polls of an mbarrier that only a CTA's own bulk copy (global -> its shared memory) completes.
