@@ -132,7 +132,7 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
     d.ir_bytes = sr::ir_smem_bytes(ncode);
     d.nrows = rm.nrows;
     d.sha = pl.shmem_words;                      // (shared_reach takes heap memory)
-    d.vec = sr::block_vec(pl.block_dim, d.grid, (uint32_t)sms);
+    d.vec = sr::block_vec(pl.block_dim, d.grid, (uint32_t)sms, false);
     d.nw = sr::block_warps(pl.block_dim, d.vec);
     d.group_bytes = sr::group_layout(d.nw * 32 * d.vec, pl.shmem_words, ncode, rm.nrows, 0, 0).total;
     d.check_group = sr::check_group_for(d.log_cap, sr::kCheckMaxGroup);

@@ -480,6 +480,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   const uint32_t smem_budget =
       (uint32_t)std::min<size_t>(c->smem_optin ? c->smem_optin : 227 * 1024, 227 * 1024) - 1024;
   const bool batched = o.mode == SR_MODE_BATCHED;
+  const bool fused = o.fused_check && o.check_races && !o.check_global;
   const bool wide = batched && o.ctas_per_sm >= 2 && !o.fused_check && !o.check_global;
   std::vector<uint8_t> large;                  // per launch: of a program that ctas_per_sm 2 is about
   for (uint32_t i = 0; i < n; ++i) {
@@ -504,7 +505,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
     uint32_t pvec = 0;
     if (batched)
       for (uint32_t l = 0; l < P.nlaunches; ++l)
-        pvec = std::max(pvec, sr::block_vec(P.launches[l].block_dim, P.launches[l].grid, (uint32_t)c->sms));
+        pvec = std::max(pvec, sr::block_vec(P.launches[l].block_dim, P.launches[l].grid, (uint32_t)c->sms, fused));
     // the global-memory race check of a program whose launches are not all ordered needs its
     // launch-order matrix (and all its launches in one wave)
     uint32_t ord_off = sr::kNoDep;
@@ -560,7 +561,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       d.nrows = rm.nrows;
       const uint32_t nsw = (L.block_dim + 31) / 32;         // simulated warps
       d.sha = shared_reach(P.code, P.ncode, d.entry, L, ranges);
-      d.vec = pvec ? pvec : sr::block_vec(L.block_dim, d.grid, (uint32_t)c->sms);
+      d.vec = pvec ? pvec : sr::block_vec(L.block_dim, d.grid, (uint32_t)c->sms, fused);
       d.nw = sr::block_warps(L.block_dim, d.vec);
       const uint32_t lanes = d.nw * 32 * d.vec;
       d.uninit = o.check_uninit ? 1u : 0u;
