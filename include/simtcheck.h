@@ -199,7 +199,7 @@ typedef struct {
                                      sr_destroy) */
   uint32_t check_variant;    /* race-check kernel shape, 1..SR_CHECK_VARIANTS (consumer threads,
                                 records per stage, staging, CTAs per SM, address-table size);
-                                0 = the default */
+                                0 = chosen by the records per barrier interval */
   uint32_t check_uninit;     /* 1 = also report loads of shared words not yet written
                                 (SR_REP_ERR_UNINIT_SHARED); 0 = off */
   uint32_t fused_check;      /* 1 = the interpreter keeps each shared word's access summary itself

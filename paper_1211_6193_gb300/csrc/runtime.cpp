@@ -96,7 +96,7 @@ struct sr_batch {
   uint64_t entry_cap = 0;                  // report entries of one wave that fit
   cudaStream_t stream = nullptr;
   bool ran = false;
-  uint32_t check_ctas = 0;
+  uint32_t check_ctas = 0, check_variant = 0;   // race-check kernel: CTAs, shape
   // CUDA graph of run_and_check (batched mode with use_graph)
   cudaGraphExec_t graph = nullptr;
   cudaStream_t graph_stream = nullptr;
@@ -349,10 +349,10 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
       ca.work_head = (uint32_t*)b->work_head.p + wi;
       ca.error_flag = err_flag(b);
       ca.spin_limit = o.spin_limit;
-      ca.table_words = sr::check_table_words(b->launches.data(), w.li0, w.li1, sr::check_table_cap(o.check_variant));
+      ca.table_words = sr::check_table_words(b->launches.data(), w.li0, w.li1, sr::check_table_cap(b->check_variant));
       ca.item_launch = (const uint32_t*)b->item_launch_d.p;
       const uint32_t ctas = std::min<uint32_t>(b->check_ctas, ca.item1 - ca.item0);
-      if (ctas) CUDA_TRY(c, sr::launch_check(ca, o.check_variant, ctas, s));
+      if (ctas) CUDA_TRY(c, sr::launch_check(ca, b->check_variant, ctas, s));
       b->kernels += ctas ? 1 : 0;
     }
     mark();
@@ -474,6 +474,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   b->arena_off.resize(n);
   b->arena_words.resize(n);
   uint64_t arena_total = 0;
+  double interval_records = 0, interval_weight = 0;   // what the race check will find (bounds)
   uint64_t nblocks = 0, check_items = 0;
   RangeScratch ranges;
   // shared memory of a CTA of the plain or the persistent batched kernel (one per SM)
@@ -539,6 +540,12 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       d.key_bits = key_bits_for(std::max(1u, L.shmem_words));
       const KernelBound& k = kb[L.kernel];
       const uint64_t cap = launch_log_cap(k, L.block_dim, o.check_races, o.loop_log_records);
+      {
+        // records per barrier interval, weighted by records (a loop: as many as its log holds)
+        const double recs = k.cyclic ? o.loop_log_records : (double)k.accesses * L.block_dim;
+        interval_records += recs * d.grid;
+        interval_weight += recs * d.grid * (recs / (k.cyclic ? 1.0 : k.barriers + 1.0));
+      }
       if (cap >= (1ull << 31)) {
         delete b;
         return fail(c, SR_E_INVAL, "program %u launch %u: access log bound too large", i, l);
@@ -589,8 +596,11 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
     large.resize(b->launches.size(), one_all ? 1 : 0);
   }
   b->nblocks = (uint32_t)nblocks;
+  b->check_variant = o.check_variant ? o.check_variant
+                                     : sr::check_variant_for(interval_weight / std::max(1.0, interval_records));
+  b->check_ctas = (uint32_t)c->sms * sr::check_ctas_per_sm(b->check_variant);
   for (LaunchDev& d : b->launches) {             // (at most one item per block)
-    d.check_group = sr::check_group_for(d.log_cap, nblocks / ((uint64_t)c->sms * sr::check_ctas_per_sm(o.check_variant)));
+    d.check_group = sr::check_group_for(d.log_cap, nblocks / b->check_ctas);
     d.check_item = (uint32_t)check_items;
     check_items += (d.grid + d.check_group - 1) / d.check_group;
   }
@@ -706,7 +716,6 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       const std::vector<Bucket> unsorted(b->buckets.begin() + w.bk0, b->buckets.end());
       for (uint32_t i = 0; i < order.size(); ++i) b->buckets[w.bk0 + i] = unsorted[order[i]];
     }
-  b->check_ctas = (uint32_t)c->sms * sr::check_ctas_per_sm(o.check_variant);
 
   // ---- device buffers
   int rc = SR_OK;

@@ -254,6 +254,7 @@ struct CheckArgs {
 // race-check kernel shapes (variant 1..SR_CHECK_VARIANTS; 0 = default)
 uint32_t check_default_variant();
 uint32_t check_ctas_per_sm(uint32_t variant);
+uint32_t check_variant_for(double interval);   // the shape for so many records per barrier interval
 uint32_t check_table_cap(uint32_t variant);
 cudaError_t launch_check(const CheckArgs& a, uint32_t variant, uint32_t ctas, cudaStream_t s);
 constexpr uint32_t kCheckBins = 12288;         // the largest shared array (words)
