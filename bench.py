@@ -6,8 +6,8 @@ Default workload (batched): 4096 seed-generated programs (reduction / 1-D stenci
 blockDim 32-1024, shared arrays up to 48 KB, 20-400 instructions, 30% with one planted bug
 (SplitMix64 seed 3): 1.97M blocks, 1.0e9 simulated threads, 6.1e9 checked shared accesses.
 One step = one pass of the whole hot path over the resident batch: arena reset, SIMT
-interpretation of every launch with access logging (one persistent launch), race check of
-every barrier interval, barrier checks, canonical report ordering.
+interpretation of every launch with access logging (buckets of alike blocks side by side), race
+check of every barrier interval, barrier checks, canonical report ordering.
 
   value  : checked shared accesses / s, batched path, programs resident on the device
   plain_path : the same programs through one kernel launch per (program, launch)
@@ -70,10 +70,10 @@ def parse():
     ap.add_argument("--workload", default="batched", choices=sorted(WORKLOADS))
     ap.add_argument("--mode", default="plain", choices=["plain", "batched"])
     ap.add_argument("--interp-variant", type=int, default=0, choices=[0, 1, 2],
-                    help="plain interpreter kernel: 1 = one CTA/SM register budget, 2 = two CTAs/SM, 0 = auto")
+                    help="plain interpreter kernel, blocks of eight warps: 1 = registers for three CTAs/SM, 2 = four, 0 = auto")
     ap.add_argument("--ctas-per-sm", type=int, default=0, choices=[0, 1, 2],
-                    help="batched mode: 1 = every launch in the persistent interpreter (one CTA per SM), 2 = "
-                         "programs of one-group blocks one block per CTA, two CTAs per SM (0 = autotuner)")
+                    help="batched mode: 1 = registers for three CTAs of eight warps per SM, 2 = for four, for the "
+                         "programs of large blocks (0 = autotuner)")
     ap.add_argument("--check-variant", type=int, default=0, choices=[0, 1, 2, 3, 4, 5, 6, 7],
                     help="race-check kernel shape (0 = default); setting a shape flag skips the autotuner")
     ap.add_argument("--fused-check", action="store_true",
@@ -418,10 +418,8 @@ def run_native(args):
     alg = {"checked_shared_access": 16, "simulated_global_access": 4, "report": 32, "arena_word": 8}
     step_bytes = (alg["checked_shared_access"] * st.shared_accesses + alg["simulated_global_access"] *
                   st.global_accesses + alg["report"] * n_reports + alg["arena_word"] * arena_words)
-    # (batched mode with two CTAs per SM: the interpreter stage is two kernels, the one-block-per-CTA
-    # grid of the programs of one-group blocks, then the persistent kernel for the rest)
-    interp_kernel = ("k_interp_plain" if mode == "plain" else
-                     "k_interp_blocks + k_interp_batched" if opts.get("ctas_per_sm") == 2 else "k_interp_batched")
+    # (batched mode: one launch of it per bucket of alike blocks, side by side)
+    interp_kernel = "k_interp_plain" if mode == "plain" else "k_interp_blocks"
     achieved = step_bytes / (stage["interp"] / 1e3) / 1e9
     isha, csha = src_sha("interp.cu", "sr_internal.h"), src_sha("check.cu", "sr_internal.h")
     fused = bool(opts.get("fused_check"))

@@ -172,22 +172,19 @@ typedef struct {
 } sr_allocator;
 
 enum { SR_MODE_PLAIN = 0,    /* one kernel launch per (program, launch) */
-       SR_MODE_BATCHED = 1   /* one persistent launch over every block of every program */ };
+       SR_MODE_BATCHED = 1   /* alike blocks of all programs in one launch, such launches side by side */ };
 
 typedef struct {
   uint32_t check_races;      /* 1 = log + race check (default), 0 = interpreter + barrier check only */
   uint32_t round_budget;     /* rounds per block before STEP_LIMIT; 0 = 1 << 24 (max 1 << 26) */
   uint32_t mode;             /* SR_MODE_* */
-  uint32_t ctas_per_sm;      /* batched mode: 1 (0) = every launch in the persistent interpreter, one
-                                1024-thread CTA per SM; 2 = the programs whose every launch would take
-                                one group per persistent CTA (blocks of more than 512 threads, or
-                                shared arrays that leave room for one) and whose blocks fit two CTAs
-                                per SM run one simulated block per CTA, two CTAs per SM, all such
-                                launches of a wave in one grid; the other programs stay persistent.
+  uint32_t ctas_per_sm;      /* batched mode: register budget of the programs of large blocks (more than
+                                512 threads in every launch, or shared arrays that leave room for one
+                                such block): 1 (0) = three CTAs of eight warps per SM, 2 = four.
                                 Without effect with fused_check or check_global */
   uint32_t loop_log_records; /* log region (records per block) for kernels with loops; 0 = 65536 */
-  uint32_t interp_variant;   /* plain-mode interpreter: 1 = one 1024-thread CTA per SM budget,
-                                2 = registers capped for two per SM, 0 = pick by occupancy */
+  uint32_t interp_variant;   /* plain-mode interpreter, blocks of eight warps: 1 = registers for three
+                                CTAs per SM, 2 = for four, 0 = the one with more resident */
   uint32_t use_graph;        /* batched mode: capture run_and_check once, replay as a CUDA graph */
   uint32_t profile;          /* record CUDA events between stages (sr_batch_stats) */
   uint32_t spin_limit;       /* device wait iterations before SR_ST_INTERNAL; 0 = 1 << 26 */
@@ -229,7 +226,7 @@ typedef struct {
   uint32_t kernels;          /* kernel launches of the library enqueued by the last run */
   float ms_global;           /* last run, when opts.profile: the global-memory race check */
   uint64_t global_records;   /* global accesses logged for the global-memory race check (last run) */
-  uint64_t one_per_cta_blocks; /* batched mode, ctas_per_sm 2: blocks run one per CTA in a run */
+  uint64_t one_per_cta_blocks; /* batched mode, ctas_per_sm 2: blocks of the programs it applies to */
 } sr_stats;
 
 /* Create a context on the current CUDA device.  opts may be NULL (defaults). */

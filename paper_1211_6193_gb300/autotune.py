@@ -4,8 +4,9 @@ Four knobs of the library decide how the hot path maps onto the GPU, and the bes
 setting depends on the workload's block sizes, barrier-interval lengths and shared-array
 sizes:
 
-  * interpreter CTAs per SM (``ctas_per_sm``, batched mode) or the register budget of the
-    plain interpreter (``interp_variant``): how many simulated blocks share an SM;
+  * the register budget of the interpreter, for large blocks in batched mode
+    (``ctas_per_sm``) or in plain mode (``interp_variant``): how many simulated blocks share
+    an SM;
   * the race-check kernel shape (``check_variant``): consumer threads per CTA, records per
     stage, staging (TMA ring or registers) and CTAs per SM -- the log-tile width;
   * where the race check runs (``fused_check``): over the access log after the interpreter,

@@ -609,8 +609,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_check(CheckArgs A) {
 
   // -------------------------------------------------------------- consumer warps
   const uint32_t cbase = tid * C::PER;
-  uint4* const stage_out = A.scratch + (size_t)blockIdx.x * kScratchWords;
-  uint32_t* const gtab = reinterpret_cast<uint32_t*>(stage_out + kCheckBins);
+  uint4* const stage_out = A.scratch + (size_t)blockIdx.x * check_scratch_words(A.stage_entries);
+  uint32_t* const gtab = reinterpret_cast<uint32_t*>(stage_out + A.stage_entries);
   bool ovf = false, g_ready = false;
   uint32_t iv = 1, par = 0, tag = 1, tagw = 1u << 14;
   // per block
@@ -761,8 +761,8 @@ __global__ void __launch_bounds__(NC, MINB) k_check_reg(CheckArgs A) {
   volatile uint32_t* s_nep = misc + 4;           // [2] its epoch
   uint32_t* wtot = misc + 8;
   const uint32_t tid = threadIdx.x, cbase = tid * PER;
-  uint4* const stage_out = A.scratch + (size_t)blockIdx.x * kScratchWords;
-  uint32_t* const gtab = reinterpret_cast<uint32_t*>(stage_out + kCheckBins);
+  uint4* const stage_out = A.scratch + (size_t)blockIdx.x * check_scratch_words(A.stage_entries);
+  uint32_t* const gtab = reinterpret_cast<uint32_t*>(stage_out + A.stage_entries);
   bool ovf = false, g_ready = false;
 
   for (uint32_t i = tid; i < ntab; i += NC) tab[i] = 0;
@@ -888,8 +888,8 @@ __global__ void __launch_bounds__(32, 20) k_check_lean(CheckArgs A) {
   volatile uint32_t* s_racy = misc;              // [2] tag of the racy interval, by interval parity
   uint32_t* wtot = misc + 8;
   const uint32_t lane = threadIdx.x;
-  uint4* const stage_out = A.scratch + (size_t)blockIdx.x * kScratchWords;
-  uint32_t* const gtab = reinterpret_cast<uint32_t*>(stage_out + kCheckBins);
+  uint4* const stage_out = A.scratch + (size_t)blockIdx.x * check_scratch_words(A.stage_entries);
+  uint32_t* const gtab = reinterpret_cast<uint32_t*>(stage_out + A.stage_entries);
   bool g_ready = false, bad = false;
 
   for (uint32_t i = lane; i < ntab; i += 32) tab[i] = 0;

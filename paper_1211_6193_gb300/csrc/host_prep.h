@@ -482,7 +482,7 @@ inline void set_runs(uint2* code, uint8_t* run, uint32_t n, const uint8_t* targe
 }
 
 // A program as it is staged: out holds packed_words(ncode) pairs.
-inline uint32_t packed_words(uint32_t ncode) { return sr::ir_smem_bytes(ncode) / 8u; }
+inline uint32_t packed_words(uint32_t ncode) { return sr::packed_bytes(ncode) / 8u; }
 inline void pack_program(const sr_program& P, const RegMap& m, uint2* out) {
   const uint32_t n = P.ncode + 1;
   uint8_t target[SR_MAX_CODE + 1] = {};

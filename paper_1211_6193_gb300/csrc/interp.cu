@@ -400,13 +400,13 @@ __device__ void flush_errors(BlockVars* bv, uint32_t* err, uint32_t* un, const u
         mt = un[2 * pc + 1];
       } else if (pc < ncode) {
         cnt = err[2 * pc];
-        if (cnt) {
+        mt = err[2 * pc + 1];
+        if (cnt && mt != kInf) {                 // (else the length of a run)
           const uint32_t f = pk_form(ir[pc].x);
           const uint32_t k2 = (f == F_LDS || f == F_STS || f == F_ATOMS) ? SR_REP_ERR_OOB_SHARED
                               : (f == F_LDG || f == F_STG)               ? SR_REP_ERR_OOB_GLOBAL
                                                                          : SR_REP_ERR_DIV0;
           hit = (k2 == kind);
-          mt = err[2 * pc + 1];
         }
       }
       uint32_t hm = __ballot_sync(FULL, hit);
@@ -420,8 +420,10 @@ __device__ void flush_errors(BlockVars* bv, uint32_t* err, uint32_t* un, const u
     }
   }
   for (uint32_t pc = lane; pc <= ncode; pc += 32) {
-    err[2 * pc] = 0;
-    err[2 * pc + 1] = kInf;
+    if (err[2 * pc + 1] != kInf) {
+      err[2 * pc] = 0;
+      err[2 * pc + 1] = kInf;
+    }
     if (un) {
       un[2 * pc] = 0;
       un[2 * pc + 1] = kInf;
@@ -622,9 +624,9 @@ __device__ __forceinline__ void start_block(const RunArgs& A, const LaunchDev* L
     for (int j = 0; j < V; ++j) v[j] = r < Ls->nparams ? (uint32_t)Ls->params[r & 3u] : 0u;
     sts_v<V>(rs + r * rstride, v);
   }
-  auto fill2 = [&](uint32_t off) {               // error records: none
-    for (uint32_t i = t; i <= ncode; i += nthr) reinterpret_cast<uint2*>(gsm + off)[i] = make_uint2(0u, kInf);
-  };
+  // error records: none (no tid), with the run lengths in place of the counts
+  const uint8_t* runs = reinterpret_cast<const uint8_t*>(A.code + Ls->code_off) + ir_code_bytes(ncode);
+  for (uint32_t i = t; i <= ncode; i += nthr) reinterpret_cast<uint2*>(gsm + G.err)[i] = make_uint2(__ldg(runs + i), kInf);
   auto fill4 = [&](uint32_t off, uint32_t words, uint32_t v) {
     for (uint32_t i = t; i < words / 4u; i += nthr) reinterpret_cast<uint4*>(gsm + off)[i] = make_uint4(v, v, v, v);
   };
@@ -632,9 +634,8 @@ __device__ __forceinline__ void start_block(const RunArgs& A, const LaunchDev* L
     for (uint32_t i = t; i < words; i += nthr) reinterpret_cast<uint32_t*>(gsm + off)[i] = 0;
   };
   fill4(G.sh, sha + 3u, 0);
-  fill2(G.err);
   if (Ls->uninit) {
-    fill2(G.un);
+    for (uint32_t i = t; i <= ncode; i += nthr) reinterpret_cast<uint2*>(gsm + G.un)[i] = make_uint2(0u, kInf);
     clear(G.wb, (sha + 31u) / 32u);
   }
   const uint32_t tps = tuple_plane_words(sha);
@@ -658,7 +659,7 @@ __device__ __forceinline__ void start_block(const RunArgs& A, const LaunchDev* L
     bv->sreg[3] = 32u;
     SoloConst* sc = reinterpret_cast<SoloConst*>(gsm + kGroupConst);
     sc->irs = smem_u32(ir);
-    sc->rb = smem_u32(ir) + ir_code_bytes(ncode) - smem_u32(ir) / 8u;
+    sc->rb = smem_u32(gsm + G.err) - smem_u32(ir);
     sc->shs = smem_u32(gsm + G.sh);
     sc->sha = sha;
     sc->arena = reinterpret_cast<unsigned long long>(A.arena + Ls->arena_off);
@@ -952,7 +953,7 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
       const uint32_t f = pk_form(in.x);
       // (what touches no memory may run ahead of other agents' earlier rounds)
       if (p < wpc && (solo || !moved || (k < budget && (f > F_ATOMS || f == F_BRZ || f == F_BRNZ)))) {
-      const uint32_t run = f < F_LDS ? lds_u8(irs + ir_code_bytes(ncode) + p) : 0u;
+      const uint32_t run = f < F_LDS ? lds_u8(smem_u32(err) + 8u * p) : 0u;
       if (run) {
         // A run of instructions that touch no memory and do not branch executes in a tight loop,
         // one instruction per round; its last round is published at once (other warps wait on
@@ -1554,7 +1555,7 @@ static BlocksKernel blocks_kernel(uint32_t vec, uint32_t variant, bool fused, bo
 cudaError_t init_interp_attributes(uint32_t smem_optin) {
   cudaError_t e = cudaSuccess;
   for (uint32_t vec = 1; vec <= 4 && e == cudaSuccess; vec *= 2)
-    for (uint32_t variant = 1; variant <= 2 && e == cudaSuccess; ++variant)
+    for (uint32_t variant = 1; variant <= (vec == 4 ? 2u : 1u) && e == cudaSuccess; ++variant)
       for (uint32_t f = 0; f < 3 && e == cudaSuccess; ++f) {
         e = allow_dynamic_smem(plain_kernel(vec, variant, f == 1, f == 2), smem_optin);
         if (e == cudaSuccess) e = allow_dynamic_smem(blocks_kernel(vec, variant, f == 1, f == 2), smem_optin);

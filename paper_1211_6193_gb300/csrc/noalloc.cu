@@ -129,7 +129,7 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
     d.log_cap = (uint32_t)cap;
     d.arena_off = 0;
     d.arena_words = prog->global_words;
-    d.ir_bytes = sr::ir_smem_bytes(ncode);
+    d.ir_bytes = sr::ir_code_bytes(ncode);
     d.nrows = rm.nrows;
     d.sha = pl.shmem_words;                      // (shared_reach takes heap memory)
     d.vec = sr::block_vec(pl.block_dim, d.grid, (uint32_t)sms, false);
@@ -161,7 +161,7 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
   const size_t o_offsets = take(((size_t)nblocks + 1) * 8);
   const size_t o_partials = take(sr::compact_partials_count((uint32_t)nblocks) * 8);
   const uint32_t cctas = std::min<uint32_t>(kCheckCtas, (uint32_t)sms);
-  const size_t o_table = take((size_t)cctas * sr::kScratchWords * 16);
+  const size_t o_table = take((size_t)cctas * sr::check_scratch_words(sr::kCheckBins) * 16);
   if (off >= SR_NOALLOC_SCRATCH_BYTES) return SR_E_RANGE;
   const size_t o_log = off;
   const uint64_t log_records = (SR_NOALLOC_SCRATCH_BYTES - off) / 8;
@@ -227,6 +227,7 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
     ca.log = ra.log;
     ca.blocks = ra.blocks;
     ca.scratch = reinterpret_cast<uint4*>(base + o_table);
+    ca.stage_entries = sr::kCheckBins;
     ca.work_head = heads + wi;
     ca.error_flag = heads + kMaxWaves;
     ca.spin_limit = ra.spin_limit;

@@ -96,7 +96,7 @@ struct sr_batch {
   uint64_t entry_cap = 0;                  // report entries of one wave that fit
   cudaStream_t stream = nullptr;
   bool ran = false;
-  uint32_t check_ctas = 0, check_variant = 0;   // race-check kernel: CTAs, shape
+  uint32_t check_ctas = 0, check_variant = 0, check_stage = 0;   // race-check kernel: CTAs, shape, staged entries per CTA
   // CUDA graph of run_and_check (batched mode with use_graph)
   cudaGraphExec_t graph = nullptr;
   cudaStream_t graph_stream = nullptr;
@@ -241,6 +241,23 @@ sr::GcheckArgs gcheck_args(sr_ctx* c, sr_batch* b, uint32_t wi) {
   return g;
 }
 
+// Side streams a wave's kernels use.
+uint32_t side_streams_of(const sr_batch* b, const Wave& w, bool batched) {
+  const uint32_t n = batched ? w.bk1 - w.bk0 : b->launches[w.li1 - 1].prog - b->launches[w.li0].prog + 1u;
+  return std::min(kSideStreams, n);
+}
+
+// The context's first n side streams and their events (made when a batch first needs them: twelve
+// streams take some 100 us, which a context for small batches need not spend).
+cudaError_t need_side_streams(sr_ctx* c, uint32_t n) {
+  cudaError_t e = cudaSuccess;
+  for (uint32_t i = 0; i < n && e == cudaSuccess; ++i) {
+    if (!c->side[i]) e = cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess && !c->join[i]) e = cudaEventCreateWithFlags(&c->join[i], cudaEventDisableTiming);
+  }
+  return e;
+}
+
 int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
   const sr_opts& o = c->opts;
   b->nevents_used = 0;
@@ -300,8 +317,7 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
     // Independent kernels - the buckets, or in plain mode the programs - run side by side: alone, a
     // kernel of a few blocks leaves the chip idle for the 20 to 90 us that its blocks take.
     const bool batched = o.mode == SR_MODE_BATCHED;
-    const uint32_t nprogs = batched ? 0u : b->launches[w.li1 - 1].prog - b->launches[w.li0].prog + 1u;
-    const uint32_t nside = std::min(kSideStreams, batched ? w.bk1 - w.bk0 : nprogs);
+    const uint32_t nside = side_streams_of(b, w, batched);
     const bool fork = nside > 1;
     if (fork) {
       CUDA_TRY(c, cudaEventRecord(c->fork, s));
@@ -346,6 +362,7 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
       ca.log = ra.log;
       ca.blocks = ra.blocks;
       ca.scratch = (uint4*)b->scratch.p;
+      ca.stage_entries = b->check_stage;
       ca.work_head = (uint32_t*)b->work_head.p + wi;
       ca.error_flag = err_flag(b);
       ca.spin_limit = o.spin_limit;
@@ -405,10 +422,6 @@ int sr_create(sr_ctx** out, const sr_opts* opts) {
   c->smem_per_sm = (size_t)per_sm;
   if (e == cudaSuccess) e = sr::init_kernel_attributes((uint32_t)optin);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
-  for (uint32_t i = 0; i < kSideStreams && e == cudaSuccess; ++i) {
-    e = cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->join[i], cudaEventDisableTiming);
-  }
   if (e == cudaSuccess && !c->custom_alloc) {
     // a pool of its own that keeps freed memory (batch after batch reuses it instead of
     // returning it to the driver at every synchronisation)
@@ -564,7 +577,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       d.ord_off = ord_off;
       d.arena_off = b->arena_off[i];
       d.arena_words = P.global_words;
-      d.ir_bytes = sr::ir_smem_bytes(P.ncode);
+      d.ir_bytes = sr::ir_code_bytes(P.ncode);
       d.nrows = rm.nrows;
       const uint32_t nsw = (L.block_dim + 31) / 32;         // simulated warps
       d.sha = shared_reach(P.code, P.ncode, d.entry, L, ranges);
@@ -599,12 +612,17 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   b->check_variant = o.check_variant ? o.check_variant
                                      : sr::check_variant_for(interval_weight / std::max(1.0, interval_records));
   b->check_ctas = (uint32_t)c->sms * sr::check_ctas_per_sm(b->check_variant);
+  uint32_t max_shw = 0;
   for (LaunchDev& d : b->launches) {             // (at most one item per block)
+    max_shw = std::max(max_shw, d.shw);
     d.check_group = sr::check_group_for(d.log_cap, nblocks / b->check_ctas);
     d.check_item = (uint32_t)check_items;
     check_items += (d.grid + d.check_group - 1) / d.check_group;
   }
   b->check_items = (uint32_t)check_items;
+  b->check_stage = sr::check_stage_entries(max_shw);
+  // (48 to 240 KB of scratch each: none for CTAs that would find no item)
+  b->check_ctas = (uint32_t)std::min<uint64_t>(b->check_ctas, std::max<uint64_t>(1, check_items));
   b->item_launch.resize(check_items);
   for (uint32_t li = 0; li < b->launches.size(); ++li) {
     const LaunchDev& d = b->launches[li];
@@ -733,7 +751,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       {&b->launch_dead, std::max<size_t>(1, b->launches.size()) * 4, "launch stop marks"},
       {&b->counters, sizeof(sr::Counters), "counters"},
       {&b->launch_done, std::max<size_t>(1, nl) * 4, "launch completion"},
-      {&b->scratch, (size_t)b->check_ctas * sr::kScratchWords * 16, "checker scratch"},
+      {&b->scratch, (size_t)b->check_ctas * sr::check_scratch_words(b->check_stage) * 16, "checker scratch"},
       {&b->work_head, (size_t)nwaves * 4, "checker queue"},
       {&b->offsets, ((size_t)b->nblocks + 1) * 8, "report offsets"},
       {&b->partials, sr::compact_partials_count(b->nblocks) * 8, "scan partials"},
@@ -775,7 +793,10 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   auto up = [&](DevBuf& d, const void* src, size_t bytes) -> cudaError_t {
     return bytes ? cudaMemcpyAsync(d.p, src, bytes, cudaMemcpyHostToDevice, s) : cudaSuccess;
   };
-  cudaError_t e = up(b->code, code.data(), code.size() * 8);
+  uint32_t nside = 0;
+  for (const Wave& w : b->waves) nside = std::max(nside, side_streams_of(b, w, batched));
+  cudaError_t e = nside > 1 ? need_side_streams(c, nside) : cudaSuccess;
+  if (e == cudaSuccess) e = up(b->code, code.data(), code.size() * 8);
   if (e == cudaSuccess) e = up(b->launches_d, b->launches.data(), nl * sizeof(LaunchDev));
   if (e == cudaSuccess) e = up(b->item_launch_d, b->item_launch.data(), b->item_launch.size() * 4);
   if (e == cudaSuccess) e = up(b->bq_launch_d, b->bq_launch.data(), b->bq_launch.size() * 4);

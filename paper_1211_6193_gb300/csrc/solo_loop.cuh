@@ -27,8 +27,8 @@ namespace {
 
 // What the loop reads of the block (written at its start, kGroupConst): 16-byte groups.
 struct SoloConst {
-  uint32_t irs, rb, shs, sha;        // shared addresses of the code, its run lengths (less irs / 8), the
-                                     // shared array; its words
+  uint32_t irs, rb, shs, sha;        // shared addresses of the code, the run lengths (8 bytes apart; less irs),
+                                     // the shared array; its words
   unsigned long long arena;
   uint32_t arena_words, spin;
   uint32_t budget4, pad0, nthr, nw;
@@ -267,7 +267,7 @@ enum : uint32_t {
       "setp.lt.u32 pe, k4, bud;\nsetp.lt.and.u32 pe, q, qw, pe;\n@!pe bra.uni LSTOP;\n"                             \
       "LTOP:\n"                                                                                                     \
       "and.b32 u, x, 63;\nsetp.ge.u32 pm, u, 32;\n@pm bra.uni LMEM;\n" /* a run starts */                           \
-      "ld.shared.u32 u, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 4];\nshr.u32 t, q, 3;\nadd.u32 t, t, u;\nld.shared.u8 t, [t];\n"                           \
+      "ld.shared.u32 u, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 4];\nadd.u32 t, q, u;\nld.shared.u8 t, [t];\n"                           \
       "sub.u32 u, bud, k4;\nshr.u32 u, u, 2;\nand.b32 r0, fl, 513;\nsetp.eq.u32 pf, r0, 1;\n@pf mov.u32 u, 255;\n"   \
       "min.u32 t, t, u;\nsub.u32 u, qw, q;\nshr.u32 u, u, 3;\n" /* (up to other agents' round: not cut, see bud) */  \
       "min.u32 t, t, u;\nmad.lo.u32 qend, t, 8, q;\nmad.lo.u32 k4, t, 4, k4;\n"                                     \

@@ -208,10 +208,11 @@ __host__ __device__ inline GroupLayout group_layout(uint32_t nthr, uint32_t shw,
   g.total = o;
   return g;
 }
-// Staged code of a program: its instructions with the EXIT sentinel (an even count), then the run
-// lengths, one byte each.
+// Packed code of a program: its instructions with the EXIT sentinel (an even count), which a block
+// stages, then the run lengths, one byte each, which it puts where the error records of their
+// instructions would be (an instruction of a run reports none).
 __host__ __device__ inline uint32_t ir_code_bytes(uint32_t ncode) { return ((ncode + 2u) & ~1u) * 8u; }
-__host__ __device__ inline uint32_t ir_smem_bytes(uint32_t ncode) { return ir_code_bytes(ncode) + align16(ncode + 1u); }
+__host__ __device__ inline uint32_t packed_bytes(uint32_t ncode) { return ir_code_bytes(ncode) + align16(ncode + 1u); }
 
 // kernel launchers (defined in the .cu files); attributes are set once per process
 cudaError_t init_kernel_attributes(uint32_t smem_optin);
@@ -244,7 +245,8 @@ struct CheckArgs {
   uint32_t item0, item1;        // work items of the wave (launch li owns items from check_item on)
   unsigned long long* log;
   BlockRes* blocks;
-  uint4* scratch;               // per checker CTA: kScratchWords race entries (intervals with many races)
+  uint4* scratch;               // per checker CTA: check_scratch_words(stage_entries) 16-byte words
+  uint32_t stage_entries;       // (check_stage_entries)
   uint32_t* work_head;
   uint32_t* error_flag;
   uint32_t spin_limit;
@@ -259,11 +261,14 @@ uint32_t check_table_cap(uint32_t variant);
 cudaError_t launch_check(const CheckArgs& a, uint32_t variant, uint32_t ctas, cudaStream_t s);
 constexpr uint32_t kCheckBins = 12288;         // the largest shared array (words)
 constexpr uint32_t kCheckTableCap = 4096;      // shared-memory address table entries at most (per variant)
-// per checker CTA in global memory: race entries of an interval staged while its summaries
-// take several rounds (at most kCheckBins), then the spill table (kCheckBins words) for the
-// intervals that touch words past the shared-memory table
-constexpr uint32_t kScratchWords = 1u << 14;
-static_assert(kScratchWords >= kCheckBins + kCheckBins / 4, "spill table must fit behind the staged entries");
+// per checker CTA in global memory, in 16-byte words: race entries of an interval staged while its
+// summaries take several rounds (one per word of the largest shared array), then the spill table
+// (kCheckBins words) for the intervals that touch words past the shared-memory table
+inline uint32_t check_stage_entries(uint32_t max_shw) {
+  const uint32_t m = (max_shw + 15u) & ~15u;
+  return m < kCheckBins ? m : kCheckBins;
+}
+__host__ __device__ inline uint32_t check_scratch_words(uint32_t stage_entries) { return stage_entries + kCheckBins / 4; }
 constexpr uint32_t kCheckItemRecords = 8192;   // log records a check work item aims at
 constexpr uint32_t kCheckMaxGroup = 32;        // blocks per check work item at most
 
