@@ -184,7 +184,7 @@ typedef struct {
                                 Without effect with fused_check or check_global */
   uint32_t loop_log_records; /* log region (records per block) for kernels with loops; 0 = 65536 */
   uint32_t interp_variant;   /* plain-mode interpreter, blocks of eight warps: 1 = registers for three
-                                CTAs per SM, 2 = for four, 0 = the one with more resident */
+                                CTAs per SM, 2 = for four, 0 = chosen by barriers and shared memory */
   uint32_t use_graph;        /* batched mode: capture run_and_check once, replay as a CUDA graph */
   uint32_t profile;          /* record CUDA events between stages (sr_batch_stats) */
   uint32_t spin_limit;       /* device wait iterations before SR_ST_INTERNAL; 0 = 1 << 26 */

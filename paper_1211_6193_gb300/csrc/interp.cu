@@ -1563,15 +1563,18 @@ cudaError_t init_interp_attributes(uint32_t smem_optin) {
   return e;
 }
 
-// variant: 1 = the larger register budget, 2 = more CTAs per SM, 0 = the one with more resident
-// warps for this launch (ties: 1)
+// variant: 1 = the larger register budget, 2 = more CTAs per SM (and more spills), 0 = 2 where its CTAs
+// fit and warps wait much: at four barriers or more.  The reduction of 2^24 values (11 barriers)
+// 1,592 us with 1 and 1,500 with 2, 1501 blocks of 333 threads 81 and 58; 64 generated programs (most
+// with one to three) 1,738 and 1,906, the 2048^2 stencil (one) 5,532 and 6,770.
 cudaError_t launch_interp_plain(const RunArgs& a, uint32_t li, const LaunchDev& L, uint32_t variant,
                                 uint32_t smem_per_sm, cudaStream_t s) {
   const uint32_t threads = L.nw * 32u;
   const uint32_t smem = interp_plain_smem(L);
   const bool global = L.glog_cap != 0;
   const bool fused = L.fused != 0 && !global;
-  if (variant == 0) variant = std::min(32u / L.nw, smem_per_sm / (smem + kBlocksStaticSmem)) > 24u / L.nw ? 2 : 1;
+  if (variant == 0)
+    variant = L.barriers >= 4 && std::min(32u / L.nw, smem_per_sm / (smem + kBlocksStaticSmem)) > 24u / L.nw ? 2 : 1;
   plain_kernel(L.vec, variant, fused, global)<<<L.grid, threads, smem, s>>>(a, li);
   return cudaGetLastError();
 }

@@ -127,6 +127,7 @@ extern "C" int sr_check_program_noalloc(const sr_program* prog, int32_t* d_arena
     const uint64_t cap = launch_log_cap(k, pl.block_dim, 1, 65536);
     if (cap >= (1ull << 31)) return SR_E_RANGE;
     d.log_cap = (uint32_t)cap;
+    d.barriers = k.barriers;
     d.arena_off = 0;
     d.arena_words = prog->global_words;
     d.ir_bytes = sr::ir_code_bytes(ncode);

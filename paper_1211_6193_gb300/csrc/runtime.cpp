@@ -564,6 +564,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
         return fail(c, SR_E_INVAL, "program %u launch %u: access log bound too large", i, l);
       }
       d.log_cap = (uint32_t)cap;
+      d.barriers = k.barriers;
       if (o.check_global) {
         const uint64_t gcap = launch_glog_cap(k, L.block_dim, o.loop_log_records);
         if (gcap >= (1ull << 31)) {

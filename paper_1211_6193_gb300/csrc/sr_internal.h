@@ -109,7 +109,7 @@ struct LaunchDev {
   uint32_t nparams, block_base, log_cap, key_bits;   // log_cap records per block (even)
   uint64_t log_base;                     // record offset of block 0's region
   uint64_t arena_off, arena_words;       // word offset of the program's working arena
-  uint32_t group_bytes, pad0;            // smem of a block beside the staged code
+  uint32_t group_bytes, barriers;        // smem of a block beside the staged code; barriers on the longest path
   uint32_t ir_bytes, nrows;              // smem bytes of the staged code; register rows (zero row last)
   uint32_t check_group, check_item;      // race check: blocks per work item, index of the first item
   uint32_t uninit;                       // 1 = report shared loads of words no thread wrote
