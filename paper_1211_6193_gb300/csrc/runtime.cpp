@@ -490,7 +490,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   double interval_records = 0, interval_weight = 0;   // what the race check will find (bounds)
   uint64_t nblocks = 0, check_items = 0;
   RangeScratch ranges;
-  // shared memory of a CTA of the plain or the persistent batched kernel (one per SM)
+  // shared memory of a CTA (one per SM at least)
   const uint32_t smem_budget =
       (uint32_t)std::min<size_t>(c->smem_optin ? c->smem_optin : 227 * 1024, 227 * 1024) - 1024;
   const bool batched = o.mode == SR_MODE_BATCHED;
