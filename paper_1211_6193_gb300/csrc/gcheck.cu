@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(SC_T) k_count_offsets(const uint32_t* c, uint3
 }
 
 // the same in one CTA, for a few chunks
-constexpr uint32_t SC_ONE = 4;
+constexpr uint32_t SC_ONE = 2;                        // (16384 blocks: 14 us in one CTA, 11 in the three kernels; 4096: 4)
 __global__ void __launch_bounds__(SC_T) k_count_one(const uint32_t* c, uint32_t gb0, uint32_t gb1, unsigned long long* off,
                                                     unsigned long long* total) {
   __shared__ unsigned long long wsum[32];
