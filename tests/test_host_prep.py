@@ -1,4 +1,5 @@
-"""The host's packed instruction forms against the plain code, compiled and run on the CPU."""
+"""The host's preparation of programs, compiled and run on the CPU: the packed instruction forms against
+the plain code, and the reachable words of the shared array against executed accesses."""
 import os
 import subprocess
 
@@ -6,10 +7,23 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 
 
-def test_packed_runs_match_the_plain_code(tmp_path):
-    exe = str(tmp_path / "pack_check")
+def run_check(name, tmp_path):
+    exe = str(tmp_path / name)
     subprocess.run(["g++", "-O1", "-std=c++17", "-I", os.path.join(ROOT, "include"),
                     "-I", os.path.join(ROOT, "paper_1211_6193_gb300", "csrc"), "-I", os.path.join(CUDA, "include"),
-                    os.path.join(ROOT, "tests", "host", "pack_check.cpp"), "-o", exe], check=True)
-    out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()
-    assert out[0] == "ok" and int(out[1]) > 100_000 and int(out[2]) > 10_000, out
+                    os.path.join(ROOT, "tests", "host", name + ".cpp"), "-o", exe], check=True)
+    p = subprocess.run([exe], capture_output=True, text=True)
+    assert p.returncode == 0, p.stdout
+    word, *counts = p.stdout.split()
+    assert word == "ok", p.stdout
+    return [int(c) for c in counts]
+
+
+def test_packed_runs_match_the_plain_code(tmp_path):
+    instrs, chained = run_check("pack_check", tmp_path)
+    assert instrs > 100_000 and chained > 10_000
+
+
+def test_shared_reach_covers_every_access(tmp_path):
+    accesses, below = run_check("reach_check", tmp_path)
+    assert accesses > 20_000 and below > 300
