@@ -443,11 +443,13 @@ enum : uint32_t {
       SR_FLUSH_ANY(E, "A") SR_FLUSH_ANY(E, "B") SR_FLUSH_ANY(E, "C") SR_FLUSH_ANY(E, "D")                           \
       /* A branch forward that parts the threads: those that take it wait at its target, as the lowest-pc rule has   \
          it, while the others go on here, if every agent has some of these - or if a barrier or an exit stands at    \
-         the target, where agents that take it as a whole wait in any case.  Not nested. */                                     \
+         the target, where agents that take it as a whole wait in any case, and the budget has the round in which     \
+         they come to wait there.  Not nested. */                                                                     \
       "LPARTS:\nsetp.eq.u32 pz, u, 34;\nsetp.ne.u32 pc, 0, 0;\n" E(SR_PARTS)                                        \
       "mad.lo.u32 need, y, 8, irs;\nand.b32 t, fl, 512;\nsetp.ne.u32 pa, t, 0;\nsetp.gt.and.u32 pa, need, q, pa;\n"    \
       "setp.eq.and.u32 pa, qw, 0xFFFFFFF8, pa;\nld.shared.u32 t, [need];\nand.b32 t, t, 63;\nsetp.eq.u32 pb, t, 41;\n" \
-      "setp.eq.or.u32 pb, t, 49, pb;\nnot.pred pd, pc;\nor.pred pb, pb, pd;\nand.pred pa, pa, pb;\n"               \
+      "setp.eq.or.u32 pb, t, 49, pb;\nadd.u32 t, k4, 8;\nsetp.le.and.u32 pb, t, bud, pb;\n"                         \
+      "not.pred pd, pc;\nor.pred pb, pb, pd;\nand.pred pa, pa, pb;\n"                                              \
       "selp.u32 t, 14336, 10240, pc;\n@pa or.b32 fl, fl, t;\nbra.uni LEND;\n" /* (kSoloToNest, Nested, Agents) */  \
       "LNEST:\nadd.u32 k4, k4, 4;\nadd.u32 q, q, 8;\nand.b32 t, k4, 0x7FFFFFFF;\nsub.u32 u, t, kst;\nshr.u32 u, u, 2;\n" \
       "mad.lo.u32 ni, u, cnt, ni;\nmov.u32 kst, t;\nmov.u32 qw, need;\nmov.u32 x, nx;\nmov.u32 y, ny;\n"             \
