@@ -548,11 +548,7 @@ __device__ __forceinline__ uint2 alu_run(uint32_t x, uint32_t y, uint32_t q, uin
 // Append one access record per slot of `im` to the block's log (one 32-bit shared atomic per
 // warp and instruction; consecutive 8-byte slots, so coalesced stores).  `low` holds the low
 // record bits of slot 0 without the address.  A warp that found the log full reserves nothing
-// more, so the cursor cannot wrap.  log_all: slots 0 .. ns - 1
-// of every lane, at the place that log_reserve gave lane 0.
-__device__ __forceinline__ uint32_t log_reserve(BlockVars* bv, bool go, uint32_t n, uint32_t lane) {
-  return atom_add_if(go && lane == 0, smem_u32(&bv->cursor), n, 0xFFFFFFFFu);
-}
+// more, here or in solo_loop (entered without kSoloLog then), so the cursor cannot wrap.
 template <int V>
 __device__ __forceinline__ void log_wide(BlockVars* bv, unsigned long long* region, uint32_t front_cap, uint32_t im,
                                          const uint32_t (&ad)[V], uint32_t epoch_hi, uint32_t low, uint32_t lane,
@@ -565,7 +561,7 @@ __device__ __forceinline__ void log_wide(BlockVars* bv, unsigned long long* regi
     total += __popc(m);
   }
   if (total == 0) return;
-  const uint32_t base = same(log_reserve(bv, !full, total, lane));
+  const uint32_t base = same(atom_add_if(!full && lane == 0, smem_u32(&bv->cursor), total, 0xFFFFFFFFu));
   if (base >= front_cap || front_cap - base < total) {
     full = true;
     if (lane == 0) atomicOr(&bv->flags, BF_OVERFLOW);
@@ -574,28 +570,6 @@ __device__ __forceinline__ void log_wide(BlockVars* bv, unsigned long long* regi
   for (int j = 0; j < V; ++j)
     if (((im >> j) & 1u) && base < front_cap && base + pos[j] < front_cap)
       region[base + pos[j]] = rec_of(epoch_hi, low + ((32u * j) << 14), ad[j]);
-}
-
-template <int V>
-__device__ __forceinline__ void log_all(BlockVars* bv, unsigned long long* region, uint32_t front_cap, uint32_t reserved,
-                                        uint32_t ns, const uint32_t (&ad)[V], uint32_t epoch_hi, uint32_t low,
-                                        uint32_t lane, bool& full) {
-  const uint32_t base = same(reserved);
-  if (base < front_cap && front_cap - base >= 32u * ns) {
-    unsigned long long* out = region + base + lane;
-#pragma unroll
-    for (int j = 0; j < V; ++j)
-      if ((uint32_t)j < ns) out[32 * j] = rec_of(epoch_hi, low + ((32u * j) << 14), ad[j]);
-    return;
-  }
-  full = true;                                   // (the part that fits)
-#pragma unroll
-  for (int j = 0; j < V; ++j) {
-    const uint32_t pos = base + 32u * j + lane;
-    if ((uint32_t)j < ns && base < front_cap && pos < front_cap)
-      region[pos] = rec_of(epoch_hi, low + ((32u * j) << 14), ad[j]);
-  }
-  if (lane == 0) atomicOr(&bv->flags, BF_OVERFLOW);
 }
 
 // Sum of a per-lane count over the warp (counts below 2^32, their sum may exceed it).
@@ -901,7 +875,8 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
         const uint32_t k_in = k;
         uint32_t q = same(irs + p * 8u), k4 = same(4u * k + par), eh = same(epoch_hi);
         uint32_t qw = same(wpc == kInf ? 0xFFFFFFF8u : irs + wpc * 8u);
-        uint32_t fl = solo_flags | (whole ? kSoloWhole : 0u) | (ns ? kSoloRegular : 0u) | (lfull ? kSoloFull : 0u);
+        uint32_t fl = solo_flags | (whole ? kSoloWhole : 0u) | (ns ? kSoloRegular : 0u);
+        if (lfull) fl = (fl & ~kSoloLog) | kSoloFull;
         if (solo) fl |= kSoloSolo;
         if (solo || kn) fl |= kSoloPub | solo_mem;
         if (solo && whole && nexit == 0 && !errs && !fused && wpc == kInf) fl |= kSoloBar;

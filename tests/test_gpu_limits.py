@@ -1,12 +1,13 @@
 """Limits of a block at their exact edges: the round budget at every round of a kernel (what each
-thread was doing when the rounds ran out, and how many instructions were executed)."""
+thread was doing when the rounds ran out, and how many instructions were executed), and an access
+log that has been full for billions of accesses."""
 import numpy as np
 import pytest
 
 import oracle
 from test_gpu_blocks import B, random_kernel  # noqa: F401 (the fixture)
 from paper_1211_6193_gb300.workloads import rng
-from paper_1211_6193_gb300.workloads.ir import TID, Asm, Launch, Program, r2, r3, r4
+from paper_1211_6193_gb300.workloads.ir import TID, Asm, Launch, Program, r2, r3, r4, r5, r6, r7
 
 pytestmark = pytest.mark.gpu
 
@@ -64,3 +65,24 @@ def test_round_budget_at_every_round(B, bdim, four):
         progs = [behind_large_block(p) for p in progs]
     for budget in range(1, longest // grid + 2):
         assert_same_at(B, progs, budget, "plain" if budget & 1 and not four else "batched")
+
+
+def test_full_log_stays_full(B):
+    """A block whose log is full after four barrier intervals goes on for 2^32 more accesses, leaving
+    the inner loop (a division by a register) between any two: its races are those of the first
+    intervals, and the other program's results are untouched."""
+    a = Asm().s2r(r2, TID).add(r3, r2, 1).and_(r3, r3, 1023).mov(r5, (1 << 18) + 64).mov(r7, 3)
+    a.label("top").sts(r2, r5)
+    for _ in range(16):
+        a.lds(r4, r3).div(r6, r5, r7)
+    a.bar().sub(r5, r5, 1).brnz(r5, "top").exit()
+    long = Program(a.assemble(), [0], [Launch(0, 1, 1024, 1024, ())], np.zeros(4, np.int32), name="long")
+    a = Asm().s2r(r2, TID).and_(r3, r2, 3).sts(r3, r2).exit()
+    other = Program(a.assemble(), [0], [Launch(0, 5, 96, 8, ())], np.zeros(4, np.int32), name="other")
+    got = B.check([long, other], mode="batched", round_budget=1 << 25, loop_log_records=1 << 16)
+    assert got.status[0] == B.ST_LOG_OVERFLOW and got.status[1] == 0
+    reports = got.report_tuples()
+    mine = [r for r in reports if r[1] == 0]
+    assert mine and {r[4] for r in mine} <= {0, 1, 2, 3}
+    want = [(r[0], 1) + r[2:] for r in oracle.run([other]).report_tuples()]
+    assert [r for r in reports if r[1] == 1] == want and want
