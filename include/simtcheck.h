@@ -25,6 +25,10 @@
  *     memory pool owned by the context) and released by sr_free_batch / sr_destroy.
  *   - `stream` is a cudaStream_t (NULL = legacy default stream).  run_and_check only
  *     enqueues work; fetch_* and sr_batch_status synchronise the batch's stream.
+ *   - Batches may use streams of their own: a run waits for no work enqueued on another stream.
+ *     It spreads independent kernels over streams of the library's behind `stream`, of the
+ *     same priority; behind work that is still pending there it is launched as a CUDA graph
+ *     (captured by the batch's first such run), except with `profile`.
  *   - Races, deadlocks, divergent barriers, out-of-bounds accesses, division by zero and
  *     the round budget are *reports* about the simulated program, never error codes.
  *   - A context and its batches are not thread-safe: use one host thread per context.

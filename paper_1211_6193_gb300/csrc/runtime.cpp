@@ -5,13 +5,14 @@
 //                every launch's per-block access log statically, groups launches into
 //                waves whose logs fit the log budget, and uploads everything.
 // run_and_check  per wave: interpreter (one launch per (program, launch) in plain mode, the
-//                programs on the context's side streams; in batched mode one grid per
+//                programs on side streams of the caller's; in batched mode one grid per
 //                bucket of launches that take the same kernel form, the buckets on the
 //                side streams), race check, report scan and emission.  Everything is
 //                enqueued behind the caller's stream, which waits for the side streams.
 // fetch_*        synchronise the stream and copy results to the host.
 #include <algorithm>
 #include <cstdarg>
+#include <memory>
 #include <new>
 #include <cstdio>
 #include <cstring>
@@ -50,7 +51,22 @@ struct Wave {
 
 }  // namespace
 
-constexpr uint32_t kSideStreams = 12;
+// Streams that a run's independent kernels are spread over: the caller's and up to five more.  Every
+// stream takes one of the hardware's queues (eight by default) and may hold up what shares it; more streams
+// give little (64 generated programs in plain mode 6,209 us in all with one, 4,688 with four, 4,614 with six,
+// 4,583 with twelve; 256 in batched mode 13,787, 13,098, 13,053 and 13,054).
+constexpr uint32_t kLanes = 6, kSideStreams = kLanes - 1;
+
+// Streams on which independent kernels of one run are enqueued side by side: each waits for the
+// caller's stream (fork), which waits for it again (join).  A set serves one caller's stream, at that
+// stream's priority: what is enqueued on another stream does not queue behind it.
+struct SideStreams {
+  unsigned long long owner = 0;   // the caller's stream (cudaStreamGetId: no two streams have the same)
+  uint32_t batches = 0;           // that were last loaded or run there
+  int priority = 0;
+  cudaStream_t side[kSideStreams] = {};
+  cudaEvent_t fork = nullptr, join[kSideStreams] = {};
+};
 
 struct sr_ctx {
   sr_opts opts{};
@@ -62,10 +78,7 @@ struct sr_ctx {
   size_t smem_optin = 0;
   size_t smem_per_sm = 0;
   cudaMemPool_t pool = nullptr;   // without a caller allocator: this context's own memory pool
-  // streams on which independent kernels of one run are enqueued side by side: each waits for
-  // the caller's stream (fork), which waits for it again (join)
-  cudaStream_t side[kSideStreams] = {};
-  cudaEvent_t fork = nullptr, join[kSideStreams] = {};
+  std::vector<std::unique_ptr<SideStreams>> sides;   // one per caller's stream, and idle ones kept for the next
 };
 
 struct sr_batch {
@@ -95,9 +108,11 @@ struct sr_batch {
   uint64_t glog_records = 0;               // largest wave's global-log records
   uint64_t entry_cap = 0;                  // report entries of one wave that fit
   cudaStream_t stream = nullptr;
+  uint32_t lanes = 1;                      // streams a run uses
+  SideStreams* sides = nullptr;            // those of `stream`
   bool ran = false;
   uint32_t check_ctas = 0, check_variant = 0, check_stage = 0;   // race-check kernel: CTAs, shape, staged entries per CTA
-  // CUDA graph of run_and_check (batched mode with use_graph)
+  // CUDA graph of run_and_check (batched mode with use_graph; runs behind pending work)
   cudaGraphExec_t graph = nullptr;
   cudaStream_t graph_stream = nullptr;
   // profiling
@@ -241,20 +256,73 @@ sr::GcheckArgs gcheck_args(sr_ctx* c, sr_batch* b, uint32_t wi) {
   return g;
 }
 
-// Side streams a wave's kernels use.
-uint32_t side_streams_of(const sr_batch* b, const Wave& w, bool batched) {
+// Streams a wave's interpreter kernels use.
+uint32_t lanes_of(const sr_batch* b, const Wave& w, bool batched) {
   const uint32_t n = batched ? w.bk1 - w.bk0 : b->launches[w.li1 - 1].prog - b->launches[w.li0].prog + 1u;
-  return std::min(kSideStreams, n);
+  return std::min(kLanes, n);
 }
 
-// The context's first n side streams and their events (made when a batch first needs them: twelve
-// streams take some 100 us, which a context for small batches need not spend).
-cudaError_t need_side_streams(sr_ctx* c, uint32_t n) {
-  cudaError_t e = cudaSuccess;
-  for (uint32_t i = 0; i < n && e == cudaSuccess; ++i) {
-    if (!c->side[i]) e = cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking);
-    if (e == cudaSuccess && !c->join[i]) e = cudaEventCreateWithFlags(&c->join[i], cudaEventDisableTiming);
+void drop_side_streams(sr_batch* b) {
+  if (b->sides) --b->sides->batches;
+  b->sides = nullptr;
+}
+
+// While this lives, calls of this thread that are closed to stream captures in progress (wherever they
+// are) leave those alone.
+struct OutsideCaptures {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+bool idle(const SideStreams& t) {
+  for (cudaStream_t q : t.side)
+    if (q && cudaStreamQuery(q) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+  return true;
+}
+
+// Gives the batch the side streams of stream s (which is not being captured): its set, or one that no
+// batch uses and whose work is done, or a new one.  Streams are made when a batch first needs them: each
+// takes some 10 us, which a context for small batches need not spend.
+cudaError_t take_side_streams(sr_ctx* c, sr_batch* b, cudaStream_t s) {
+  if (b->lanes < 2) return cudaSuccess;
+  const OutsideCaptures outside;
+  unsigned long long id = 0;
+  cudaError_t e = cudaStreamGetId(s, &id);
+  if (e != cudaSuccess) return e;
+  if (!b->sides || b->sides->owner != id) {
+    int priority = 0;
+    e = cudaStreamGetPriority(s, &priority);
+    if (e != cudaSuccess) return e;
+    drop_side_streams(b);
+    SideStreams* set = nullptr;
+    for (auto& t : c->sides)
+      if (t->owner == id) set = t.get();
+    for (size_t i = 0; !set && i < c->sides.size(); ++i)
+      if (!c->sides[i]->batches && c->sides[i]->priority == priority && idle(*c->sides[i])) set = c->sides[i].get();
+    if (!set) {
+      try {
+        c->sides.push_back(std::make_unique<SideStreams>());
+      } catch (const std::bad_alloc&) {
+        return cudaErrorMemoryAllocation;
+      }
+      set = c->sides.back().get();
+      set->priority = priority;
+    }
+    set->owner = id;
+    ++set->batches;
+    b->sides = set;
   }
+  SideStreams& t = *b->sides;
+  if (!t.fork) e = cudaEventCreateWithFlags(&t.fork, cudaEventDisableTiming);
+  for (uint32_t i = 0; i + 1 < b->lanes && e == cudaSuccess; ++i) {
+    if (!t.side[i]) e = cudaStreamCreateWithPriority(&t.side[i], cudaStreamNonBlocking, t.priority);
+    if (e == cudaSuccess && !t.join[i]) e = cudaEventCreateWithFlags(&t.join[i], cudaEventDisableTiming);
+  }
+  if (e != cudaSuccess) drop_side_streams(b);
   return e;
 }
 
@@ -317,39 +385,37 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
     // Independent kernels - the buckets, or in plain mode the programs - run side by side: alone, a
     // kernel of a few blocks leaves the chip idle for the 20 to 90 us that its blocks take.
     const bool batched = o.mode == SR_MODE_BATCHED;
-    const uint32_t nside = side_streams_of(b, w, batched);
-    const bool fork = nside > 1;
-    if (fork) {
-      CUDA_TRY(c, cudaEventRecord(c->fork, s));
-      for (uint32_t i = 0; i < nside; ++i) CUDA_TRY(c, cudaStreamWaitEvent(c->side[i], c->fork, 0));
+    const uint32_t lanes = lanes_of(b, w, batched);
+    if (lanes > 1) {
+      CUDA_TRY(c, cudaEventRecord(b->sides->fork, s));
+      for (uint32_t i = 0; i + 1 < lanes; ++i) CUDA_TRY(c, cudaStreamWaitEvent(b->sides->side[i], b->sides->fork, 0));
     }
+    auto lane = [&](uint32_t i) { return i % lanes ? b->sides->side[i % lanes - 1] : s; };
     cudaError_t e = cudaSuccess;
     if (batched) {
       for (uint32_t bk = w.bk0; bk < w.bk1 && e == cudaSuccess; ++bk) {
         const Bucket& B = b->buckets[bk];
-        const cudaStream_t bs = fork ? c->side[(bk - w.bk0) % nside] : s;
         ra.bq_launch = (const uint32_t*)b->bq_launch_d.p + B.bq0;
         ra.bq_first = (const uint32_t*)b->bq_first_d.p + B.bq0;
         ra.bq_n = B.bq1 - B.bq0;
         ra.bq_head = B.ordered ? (uint32_t*)b->bq_head.p + bk : nullptr;
         e = sr::launch_interp_blocks(ra, B.vec, B.variant, B.warps, B.blocks, B.smem,
-                                     o.fused_check && o.check_races && !o.check_global, o.check_global != 0, bs);
+                                     o.fused_check && o.check_races && !o.check_global, o.check_global != 0,
+                                     lane(bk - w.bk0));
         b->kernels += 1;
       }
     } else {
       for (uint32_t li = w.li0; li < w.li1 && e == cudaSuccess; ++li) {
         const LaunchDev& L = b->launches[li];
-        e = sr::launch_interp_plain(ra, li, L, o.interp_variant, (uint32_t)c->smem_per_sm,
-                                    fork ? c->side[L.prog % nside] : s);
+        e = sr::launch_interp_plain(ra, li, L, o.interp_variant, (uint32_t)c->smem_per_sm, lane(L.prog));
       }
       b->kernels += w.li1 - w.li0;
     }
-    if (fork)                                    // (also after an error: nothing stays unjoined)
-      for (uint32_t i = 0; i < nside; ++i) {
-        cudaError_t j = cudaEventRecord(c->join[i], c->side[i]);
-        if (j == cudaSuccess) j = cudaStreamWaitEvent(s, c->join[i], 0);
-        if (e == cudaSuccess) e = j;
-      }
+    for (uint32_t i = 0; i + 1 < lanes; ++i) {   // (also after an error: nothing stays unjoined)
+      cudaError_t j = cudaEventRecord(b->sides->join[i], b->sides->side[i]);
+      if (j == cudaSuccess) j = cudaStreamWaitEvent(s, b->sides->join[i], 0);
+      if (e == cudaSuccess) e = j;
+    }
     if (e != cudaSuccess) return fail(c, SR_E_CUDA, "interpreter launch: %s", cudaGetErrorString(e));
     mark();
     if (o.check_races) {
@@ -421,7 +487,6 @@ int sr_create(sr_ctx** out, const sr_opts* opts) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device);
   c->smem_per_sm = (size_t)per_sm;
   if (e == cudaSuccess) e = sr::init_kernel_attributes((uint32_t)optin);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
   if (e == cudaSuccess && !c->custom_alloc) {
     // a pool of its own that keeps freed memory (batch after batch reuses it instead of
     // returning it to the driver at every synchronisation)
@@ -451,11 +516,13 @@ int sr_create(sr_ctx** out, const sr_opts* opts) {
 
 void sr_destroy(sr_ctx* c) {
   if (!c) return;
-  for (uint32_t i = 0; i < kSideStreams; ++i) {
-    if (c->join[i]) cudaEventDestroy(c->join[i]);
-    if (c->side[i]) cudaStreamDestroy(c->side[i]);   // (returns at once; released when its work is done)
+  for (auto& t : c->sides) {
+    for (uint32_t i = 0; i < kSideStreams; ++i) {
+      if (t->join[i]) cudaEventDestroy(t->join[i]);
+      if (t->side[i]) cudaStreamDestroy(t->side[i]);   // (returns at once; released when its work is done)
+    }
+    if (t->fork) cudaEventDestroy(t->fork);
   }
-  if (c->fork) cudaEventDestroy(c->fork);
   if (c->pool) cudaMemPoolDestroy(c->pool);   // released once frees still in flight complete
   delete c;
 }
@@ -794,9 +861,8 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   auto up = [&](DevBuf& d, const void* src, size_t bytes) -> cudaError_t {
     return bytes ? cudaMemcpyAsync(d.p, src, bytes, cudaMemcpyHostToDevice, s) : cudaSuccess;
   };
-  uint32_t nside = 0;
-  for (const Wave& w : b->waves) nside = std::max(nside, side_streams_of(b, w, batched));
-  cudaError_t e = nside > 1 ? need_side_streams(c, nside) : cudaSuccess;
+  for (const Wave& w : b->waves) b->lanes = std::max(b->lanes, lanes_of(b, w, batched));
+  cudaError_t e = take_side_streams(c, b, s);
   if (e == cudaSuccess) e = up(b->code, code.data(), code.size() * 8);
   if (e == cudaSuccess) e = up(b->launches_d, b->launches.data(), nl * sizeof(LaunchDev));
   if (e == cudaSuccess) e = up(b->item_launch_d, b->item_launch.data(), b->item_launch.size() * 4);
@@ -819,6 +885,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     free_batch_buffers(c, b, s);
+    drop_side_streams(b);
     delete b;
     return fail(c, SR_E_CUDA, "upload failed: %s", cudaGetErrorString(e));
   }
@@ -832,7 +899,24 @@ int run_and_check(sr_ctx* c, sr_batch* b, void* stream) {
   b->stream = s;
   b->ran = true;
   const bool profile = c->opts.profile != 0;
-  if (c->opts.use_graph && c->opts.mode == SR_MODE_BATCHED && !profile) {
+  // Side streams that wait for a stream with work pending would hold the hardware's queues (eight in
+  // all by default), and runs on other streams behind these, until that work is done, whatever it waits
+  // for itself.  Behind pending work a run with side streams is therefore launched as a graph, whose
+  // branches come to the queues when it starts (work of 193 ms pending on one stream, 16 programs on it and
+  // 16 on another: the other's run took the 193 ms, and takes 0.2).  Otherwise not:
+  // capturing takes 50 to 100 us, which the first run of a batch on an idle stream need not spend.
+  bool pending = false;
+  if (b->lanes > 1) {
+    const OutsideCaptures outside;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CUDA_TRY(c, cudaStreamIsCapturing(s, &cap));
+    if (cap == cudaStreamCaptureStatusNone) {    // (else the side streams only shape the caller's graph)
+      CUDA_TRY(c, take_side_streams(c, b, s));
+      pending = cudaStreamQuery(s) == cudaErrorNotReady;
+    }
+    if (!b->sides) return fail(c, SR_E_CUDA, "no side streams");   // (an earlier call could not make them)
+  }
+  if (((c->opts.use_graph && c->opts.mode == SR_MODE_BATCHED) || pending) && !profile) {
     if (!b->graph || b->graph_stream != s) {
       if (b->graph) cudaGraphExecDestroy(b->graph);
       b->graph = nullptr;
@@ -997,6 +1081,7 @@ void sr_free_batch(sr_ctx* c, sr_batch* b) {
   for (cudaEvent_t e : b->events) cudaEventDestroy(e);
   free_batch_buffers(c, b, b->stream);
   cudaStreamSynchronize(b->stream);
+  drop_side_streams(b);
   delete b;
 }
 
