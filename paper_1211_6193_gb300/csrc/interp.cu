@@ -640,6 +640,10 @@ __device__ __forceinline__ void start_block(const RunArgs& A, const LaunchDev* L
     sc->arena_words = (uint32_t)Ls->arena_words;
     sc->spin = A.spin_limit;
     sc->budget4 = 4u * A.budget;
+    if (kDebugBounds) {
+      sc->nrows = nrows;
+      sc->ncode = ncode;
+    }
     sc->nthr = nthr;
     sc->nw = nw;
     sc->tup = smem_u32(gsm + G.tup);
@@ -689,6 +693,16 @@ __device__ __forceinline__ void wait_deps(const RunArgs& A, const LaunchDev& L, 
   }
   __syncwarp();
 }
+
+// (debug build) rounds that warps ran in solo_loop, for the test that it is what the build checks
+#if defined(SR_DEBUG_BOUNDS)
+__device__ unsigned long long g_loop_rounds;
+__device__ __forceinline__ void note_loop(uint32_t rounds, uint32_t lane) {
+  if (lane == 0) atomicAdd(&g_loop_rounds, (unsigned long long)rounds);
+}
+#else
+__device__ __forceinline__ void note_loop(uint32_t, uint32_t) {}
+#endif
 
 // Run one simulated block on warps [0, Ls->nw) of the CTA, V simulated warps per warp.  The fused race check is compiled in only where Fused is set, and
 // the logging of global accesses only where Global is set, so that the default kernels keep
@@ -868,7 +882,7 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
         stop = 1;
         break;
       }
-      if (!kDebugBounds) {
+      {
         // Most instructions run in solo_loop; what it does not take is left at (p, k).  While other
         // agents are at later rounds, it runs up to their lowest; with some at the same round, it runs
         // ahead over what touches no memory.
@@ -892,6 +906,16 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
         epoch_hi = same(eh);
         epoch = epoch_hi >> 6;
         moved = k != k_in;
+        if (kDebugBounds) {
+          note_loop(k - k_in, lane);
+          if (fl & kSoloBad) {                   // stop the block the way a wait that gave up does
+            if (lane == 0) atomicOr(&A.prog_status[Ls->prog], (uint32_t)SR_ST_BOUNDS);
+            if (!(fl & kSoloAtBar)) {
+              stop = 2;
+              break;
+            }
+          }
+        }
         if (fl & kSoloNested) {
           // some threads wait at a higher pc (at a barrier or exit: agents without a running thread
           // have executed it)
@@ -1488,6 +1512,13 @@ __global__ void __launch_bounds__(V == 1 ? 64 : 256, MINB) k_interp_blocks(RunAr
 }
 
 }  // namespace
+
+#if defined(SR_DEBUG_BOUNDS)
+// Of the debug build alone: rounds that warps have run in the interpreter's inner loop.
+extern "C" int sr_debug_loop_rounds(unsigned long long* out) {
+  return cudaMemcpyFromSymbol(out, g_loop_rounds, sizeof *out) == cudaSuccess ? SR_OK : SR_E_CUDA;
+}
+#endif
 
 uint32_t interp_plain_smem(const LaunchDev& L) {
   return L.ir_bytes + group_layout(L.nw * 32u * L.vec, L.sha, L.ncode, L.nrows, L.uninit, L.fused).total;

@@ -31,10 +31,10 @@ struct SoloConst {
                                      // the shared array; its words
   unsigned long long arena;
   uint32_t arena_words, spin;
-  uint32_t budget4, pad0, nthr, nw;
+  uint32_t budget4, nrows, nthr, nw;  // (nrows, ncode: set and read in the debug build only)
   uint32_t tup, tps4;                // fused race check: the summaries, bytes per plane
   unsigned long long region;         // the log
-  uint32_t wb, gcap, gblock, pad1;   // uninitialised-read check: the written words; global log: its size, the block
+  uint32_t wb, gcap, gblock, ncode;  // uninitialised-read check: the written words; global log: its size, the block
   unsigned long long gregion, pad2;  // the global log
 };
 static_assert(sizeof(SoloConst) == 96 && sizeof(SoloConst) <= kGroupBv - kGroupConst, "solo constants");
@@ -53,6 +53,7 @@ enum : uint32_t {
   kSoloToNest = 8192, kSoloToMerge = 16384,      // (inside: what follows the writing of kept records)
   kSoloAtBar = 32768, kSoloTimeout = 65536,
   kSoloUninit = 1 << 17, kSoloGlog = 1 << 18,    // (instead of kSoloShared, kSoloGlobal)
+  kSoloBad = 1 << 19,                            // (debug build, out) an index check failed
   kSoloPending = 0x80000000u                     // (inside: records are kept)
 };
 
@@ -75,6 +76,54 @@ enum : uint32_t {
 #define Q_BUD "%15"
 #define SR_STR2(x) #x
 #define SR_STR(x) SR_STR2(x)
+
+// Debug build: every index is checked before its access.  One that is out of range is noted in `bad`, and
+// its access goes to an index in range (an operand's row, a place in the code) or is left out; the loop
+// ends at the next instruction, with kSoloBad.
+#if defined(SR_DEBUG_BOUNDS)
+#define SR_ON(i) "@pg "
+#define SR_D_DECL ".reg .pred px, pg;\n.reg .b32 bad, zrow, ncd, qlast, shr, awr, dx;\n"
+#define SR_D_INIT                                                                                    \
+  "mov.u32 bad, 0;\nld.shared.u32 zrow, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 36];\nsub.u32 zrow, zrow, 1;\n" \
+  "ld.shared.u32 ncd, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 76];\nmad.lo.u32 qlast, ncd, 8, irs;\n" \
+  "mov.u32 shr, sha;\nld.shared.u32 awr, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 24];\n"
+#define SR_D_LIMIT(v, last) "setp.gt.u32 px, " v ", " last ";\n@px mov.u32 bad, 1;\n@px mov.u32 " v ", " last ";\n"
+#define SR_D_ROW SR_D_LIMIT("ro", "zrow")        /* row of an operand */
+#define SR_D_DST                                 /* row of a result that is written (ps) */             \
+  "setp.gt.and.u32 px, ro, zrow, ps;\n@px mov.u32 bad, 1;\nsetp.le.and.u32 ps, ro, zrow, ps;\n"
+#define SR_D_CODE(v) SR_D_LIMIT(v, "qlast")      /* address of an instruction */
+#define SR_D_TARGET SR_D_LIMIT("y", "ncd")       /* pc of a branch's target */
+#define SR_D_CHAIN SR_D_CODE("q") "@px mov.u32 t, 1;\n"
+#define SR_D_SREG SR_D_LIMIT("y", "4")
+#define SR_D_STOP "setp.ne.u32 px, bad, 0;\nvote.sync.any.pred px, px, 0xFFFFFFFF;\n@px bra.uni LDONE;\n"
+#define SR_D_DONE "setp.ne.u32 px, bad, 0;\nvote.sync.any.pred px, px, 0xFFFFFFFF;\n@px or.b32 fl, fl, 0x80000;\n"
+// pg: slot i is active and its index v below the limit
+#define SR_D_BELOW(i, v, limit) "setp.lt.and.u32 pg, " v ", " limit ", s" #i ";\nxor.pred px, pg, s" #i ";\n@px mov.u32 bad, 1;\n"
+#define SR_D_SH(i) SR_D_BELOW(i, "a" #i, "shr")
+#define SR_D_GL(i) SR_D_BELOW(i, "a" #i, "awr")
+#define SR_D_LOG(i) "add.u32 dx, base, lane;\nadd.u32 dx, dx, 32 * " #i ";\n" SR_D_BELOW(i, "dx", Q_FCAP)
+// the written-words bitmap (pf: the lane changes the word at r1)
+#define SR_D_WB                                                                                      \
+  "add.u32 dx, shr, 31;\nshr.u32 dx, dx, 5;\nmad.lo.u32 dx, dx, 4, r0;\nsetp.ge.and.u32 px, r1, dx, pf;\n" \
+  "@px mov.u32 bad, 1;\nsetp.lt.and.u32 px, r1, r0, pf;\n@px mov.u32 bad, 1;\n"                      \
+  "setp.lt.and.u32 pf, r1, dx, pf;\nsetp.ge.and.u32 pf, r1, r0, pf;\n"
+#else
+#define SR_ON(i) "@s" #i " "
+#define SR_D_DECL
+#define SR_D_INIT
+#define SR_D_ROW
+#define SR_D_DST
+#define SR_D_CODE(v)
+#define SR_D_TARGET
+#define SR_D_CHAIN
+#define SR_D_SREG
+#define SR_D_STOP
+#define SR_D_DONE
+#define SR_D_SH(i)
+#define SR_D_GL(i)
+#define SR_D_LOG(i)
+#define SR_D_WB
+#endif
 
 // f for every slot
 #define SR_E1(f) f(0)
@@ -114,11 +163,11 @@ enum : uint32_t {
 #define SR_ADDR(i) "add.u32 a" #i ", a" #i ", y;\n"
 #define SR_MAX(i) "@s" #i " max.u32 m, m, a" #i ";\n"
 #define SR_MAXR(i) "@s" #i " max.u32 r0, r0, a" #i ";\n"
-#define SR_LDSV(i) "mad.lo.u32 t, a" #i ", 4, shs;\n@s" #i " ld.shared.u32 c" #i ", [t];\n"
-#define SR_LDGV(i) "mad.wide.u32 wide, a" #i ", 4, arena;\n@s" #i " ld.global.u32 c" #i ", [wide];\n"
-#define SR_REDV(i) "mad.lo.u32 t, a" #i ", 4, shs;\n@s" #i " red.shared.add.u32 [t], b" #i ";\n"
-#define SR_STSV(i) "mad.lo.u32 t, a" #i ", 4, shs;\n@s" #i " st.shared.u32 [t], b" #i ";\n"
-#define SR_STGV(i) "mad.wide.u32 wide, a" #i ", 4, arena;\n@s" #i " st.global.u32 [wide], b" #i ";\n"
+#define SR_LDSV(i) SR_D_SH(i) "mad.lo.u32 t, a" #i ", 4, shs;\n" SR_ON(i) "ld.shared.u32 c" #i ", [t];\n"
+#define SR_LDGV(i) SR_D_GL(i) "mad.wide.u32 wide, a" #i ", 4, arena;\n" SR_ON(i) "ld.global.u32 c" #i ", [wide];\n"
+#define SR_REDV(i) SR_D_SH(i) "mad.lo.u32 t, a" #i ", 4, shs;\n" SR_ON(i) "red.shared.add.u32 [t], b" #i ";\n"
+#define SR_STSV(i) SR_D_SH(i) "mad.lo.u32 t, a" #i ", 4, shs;\n" SR_ON(i) "st.shared.u32 [t], b" #i ";\n"
+#define SR_STGV(i) SR_D_GL(i) "mad.wide.u32 wide, a" #i ", 4, arena;\n" SR_ON(i) "st.global.u32 [wide], b" #i ";\n"
 #define SR_SREG(i) "add.u32 m, u, 32 * " #i ";\nselp.b32 c" #i ", m, t, pa;\n"
 #define SR_ZERO(i) "mov.u32 c" #i ", 0;\n"
 #define SR_OFF(i) "add.u32 u, m, 32 * " #i ";\nxor.b32 u, u, a" #i ";\n@s" #i " or.b32 n, n, u;\n"
@@ -135,8 +184,9 @@ enum : uint32_t {
 #define SR_BITS(i) "@s" #i " or.b32 m, m, a" #i ";\n@s" #i " min.u32 n, n, a" #i ";\n"
 #define SR_KEEP(i) "mov.u32 l" #i ", a" #i ";\n"
 #define SR_REC(i)                                                                                    \
+  SR_D_LOG(i)                                                                                        \
   "shl.b32 t, l" #i ", 24;\nadd.u32 t, t, lw;\nadd.u32 lw, lw, 0x80000;\nshr.u32 u, l" #i ", 8;\n"   \
-  "or.b32 u, u, eh;\n@s" #i " st.global.v2.u32 [wide + 256 * " #i "], {t, u};\n"
+  "or.b32 u, u, eh;\n" SR_ON(i) "st.global.v2.u32 [wide + 256 * " #i "], {t, u};\n"
 #define SR_REC_ANY(i) /* any set of threads, and a log that may be full */                           \
   "vote.sync.ballot.b32 t, s" #i ", 0xFFFFFFFF;\nand.b32 u, t, r0;\npopc.b32 u, u;\nadd.u32 u, u, m;\n" \
   "popc.b32 t, t;\nadd.u32 m, m, t;\nsetp.lt.and.u32 pf, u, " Q_FCAP ", s" #i ";\n"                  \
@@ -147,17 +197,19 @@ enum : uint32_t {
 // uninitialised-read check (r0: the bitmap of written words): pa, an active thread reads an unwritten
 // word; the words of a store (consecutive within a slot), of an atomic
 #define SR_WBR(i)                                                                                    \
+  SR_D_SH(i)                                                                                         \
   "shr.u32 t, a" #i ", 5;\nmad.lo.u32 t, t, 4, r0;\nand.b32 u, a" #i ", 31;\nmov.u32 n, 0xFFFFFFFF;\n" \
-  "@s" #i " ld.shared.u32 n, [t];\nshr.u32 n, n, u;\nand.b32 n, n, 1;\nsetp.eq.or.u32 pa, n, 0, pa;\n"
+  SR_ON(i) "ld.shared.u32 n, [t];\nshr.u32 n, n, u;\nand.b32 n, n, 1;\nsetp.eq.or.u32 pa, n, 0, pa;\n"
 #define SR_WBS(i)                                                                                    \
   "vote.sync.ballot.b32 t, s" #i ", 0xFFFFFFFF;\nbrev.b32 u, t;\nclz.b32 u, u;\nmin.u32 u, u, 31;\n"  \
   "shfl.sync.idx.b32 r1, a" #i ", u, 31, 0xFFFFFFFF;\nsub.u32 r1, r1, u;\nand.b32 u, r1, 31;\n"       \
   "shl.b32 r2, t, u;\nsub.u32 u, 32, u;\nshr.u32 r3, t, u;\nshr.s32 r1, r1, 5;\nsetp.eq.u32 pa, lane, 1;\n" \
   "@pa mov.u32 r2, r3;\nadd.u32 r1, r1, lane;\nmad.lo.u32 r1, r1, 4, r0;\nsetp.lt.u32 pf, lane, 2;\n" \
-  "setp.ne.and.u32 pf, r2, 0, pf;\n@pf red.shared.or.b32 [r1], r2;\n"
+  "setp.ne.and.u32 pf, r2, 0, pf;\n" SR_D_WB "@pf red.shared.or.b32 [r1], r2;\n"
 #define SR_WBA(i)                                                                                    \
+  SR_D_SH(i)                                                                                         \
   "shr.u32 t, a" #i ", 5;\nmad.lo.u32 t, t, 4, r0;\nand.b32 u, a" #i ", 31;\nmov.u32 r1, 1;\n"        \
-  "shl.b32 r1, r1, u;\n@s" #i " red.shared.or.b32 [t], r1;\n"
+  "shl.b32 r1, r1, u;\n" SR_ON(i) "red.shared.or.b32 [t], r1;\n"
 // the access's records in the global log (as log_global), kind << 12
 #define SR_GREC(i)                                                                                   \
   "vote.sync.ballot.b32 t, s" #i ", 0xFFFFFFFF;\nand.b32 u, t, r0;\npopc.b32 u, u;\nadd.u32 u, u, m;\n" \
@@ -175,9 +227,9 @@ enum : uint32_t {
 // fused race check: the access of slot i into its word's summary (tuple_add), pc in r0, tid r1 (of
 // slot 0); the returned values (in b) are used when every slot's atomics are under way
 #define SR_TUPLE(i, k2)                                                                              \
-  "mad.lo.u32 t, a" #i ", 4, tup;\nmad.lo.u32 u, tps4, 6, t;\n@s" #i " red.shared.min.u32 [u], r0;\n" \
-  "add.u32 u, u, tps4;\n@s" #i " red.shared.max.u32 [u], r0;\nmad.lo.u32 u, tps4, " #k2 ", t;\n"     \
-  "add.u32 b" #i ", r1, 32 * " #i ";\n@s" #i " atom.shared.min.u32 b" #i ", [u], b" #i ";\n"
+  SR_D_SH(i) "mad.lo.u32 t, a" #i ", 4, tup;\nmad.lo.u32 u, tps4, 6, t;\n" SR_ON(i) "red.shared.min.u32 [u], r0;\n" \
+  "add.u32 u, u, tps4;\n" SR_ON(i) "red.shared.max.u32 [u], r0;\nmad.lo.u32 u, tps4, " #k2 ", t;\n"  \
+  "add.u32 b" #i ", r1, 32 * " #i ";\n" SR_ON(i) "atom.shared.min.u32 b" #i ", [u], b" #i ";\n"
 #define SR_TUPLE_OLD(i, k21)                                                                         \
   "add.u32 r2, r1, 32 * " #i ";\nsetp.ne.and.u32 pf, b" #i ", r2, s" #i ";\n"                       \
   "setp.ne.and.u32 pf, b" #i ", 0xFFFFFFFF, pf;\nmax.u32 t, b" #i ", r2;\n"                         \
@@ -197,7 +249,7 @@ enum : uint32_t {
 // instruction or the run's end
 #define SR_TAIL(STC, more)                                                                           \
   "setp.ge.u32 pe, q, qend;\nand.b32 t, x, 128;\nsetp.eq.or.u32 ps, t, 0, pe;\n"                     \
-  "prmt.b32 ro, x, 0, 0x4441;\nsetp.ne.and.u32 ps, ro, 31, ps;\nmad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" \
+  "prmt.b32 ro, x, 0, 0x4441;\nsetp.ne.and.u32 ps, ro, 31, ps;\n" SR_D_DST "mad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" \
   "@!pw bra.uni LPART;\n@ps " STC "mov.u32 x, nx;\nmov.u32 y, ny;\nmov.u32 keep, 64;\n"              \
   "@!pe bra.uni LALU;\n" more
 // end of a memory or control instruction
@@ -207,7 +259,7 @@ enum : uint32_t {
   "@pe bra.uni LTOP;\nbra.uni LSTOP;\n"
 // row d from c (a memory instruction's result)
 #define SR_ROW(STC, part, back)                                                                      \
-  "prmt.b32 ro, x, 0, 0x4441;\nsetp.ne.u32 ps, ro, 31;\nmad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" \
+  "prmt.b32 ro, x, 0, 0x4441;\nsetp.ne.u32 ps, ro, 31;\n" SR_D_DST "mad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" \
   "@!pw bra.uni " part ";\n@ps " STC back ":\n"
 // reserve the log's place for this access and keep its records to be written later
 #define SR_LOG(E, kind)                                                                              \
@@ -248,10 +300,10 @@ enum : uint32_t {
       ".reg .pred pa, pb, pc, pd, pe, pf, ps, pw, pp, pm, pz, s0, s1, s2, s3;\n"                                    \
       ".reg .b32 x, y, nx, ny, m, n, t, u, ro, keep, q, qend, k4, base, lw, eh, n32, clk, need, lane, tid0;\n"      \
       ".reg .b32 gacc, sacc, cnt, r0, r1, r2, r3, r4, r5, irs, shs, sha, awords, bud, tup, tps4, clks, myclk;\n"    \
-      ".reg .b32 ni, kst, qw, wm, fl;\n.reg .b64 wide, arena, region;\n.reg .b32 " REGS ";\n"                      \
+      SR_D_DECL ".reg .b32 ni, kst, qw, wm, fl;\n.reg .b64 wide, arena, region;\n.reg .b32 " REGS ";\n"                      \
       "ld.shared.v4.u32 {irs, t, shs, sha}, [" Q_GB " + " SR_STR(SR_GROUP_CONST) "];\n"                             \
       "ld.shared.u32 t, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 44];\n"                                            \
-      "mov.u32 q, " Q_Q ";\nmov.u32 bud, " Q_BUD ";\nld.shared.v2.u32 {x, y}, [q];\n"                                                        \
+      SR_D_INIT "mov.u32 q, " Q_Q ";\n" SR_D_CODE("q") "mov.u32 bud, " Q_BUD ";\nld.shared.v2.u32 {x, y}, [q];\n"                \
       "mov.u32 k4, " Q_K4 ";\nmov.u32 eh, " Q_EH ";\nmov.u32 fl, " Q_FL ";\nmov.u32 qw, " Q_QW ";\nmov.u32 wm, 0;\n"  \
       "mov.u32 lane, %%laneid;\nmov.u32 gacc, " Q_GACC ";\nmov.u32 sacc, " Q_SACC ";\nmov.u32 ni, " Q_NI ";\n"        \
       "and.b32 kst, k4, 0x7FFFFFFF;\nmad.lo.u32 tid0, " Q_W ", 32 * " #V ", lane;\n"                                \
@@ -265,26 +317,26 @@ enum : uint32_t {
       "LMASK:\n" /* the set has changed: its numbers */                                                             \
       "mov.u32 n32, 0;\nmov.u32 cnt, 0;\n" E(SR_COUNT)                                                             \
       "setp.lt.u32 pe, k4, bud;\nsetp.lt.and.u32 pe, q, qw, pe;\n@!pe bra.uni LSTOP;\n"                             \
-      "LTOP:\n"                                                                                                     \
+      "LTOP:\n" SR_D_CODE("q") SR_D_STOP                                                                                                     \
       "and.b32 u, x, 63;\nsetp.ge.u32 pm, u, 32;\n@pm bra.uni LMEM;\n" /* a run starts */                           \
       "ld.shared.u32 u, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 4];\nadd.u32 t, q, u;\nld.shared.u8 t, [t];\n"                           \
       "sub.u32 u, bud, k4;\nshr.u32 u, u, 2;\nand.b32 r0, fl, 513;\nsetp.eq.u32 pf, r0, 1;\n@pf mov.u32 u, 255;\n"   \
       "min.u32 t, t, u;\nsub.u32 u, qw, q;\nshr.u32 u, u, 3;\n" /* (up to other agents' round: not cut, see bud) */  \
-      "min.u32 t, t, u;\nmad.lo.u32 qend, t, 8, q;\nmad.lo.u32 k4, t, 4, k4;\n"                                     \
+      "min.u32 t, t, u;\nmad.lo.u32 qend, t, 8, q;\n" SR_D_CODE("qend") "mad.lo.u32 k4, t, 4, k4;\n"                                     \
       "min.u32 r0, k4, bud;\n@pp st.release.cta.shared.u32 [myclk], r0;\nmov.u32 keep, 0;\n"                                              \
       "LALU:\n"                                                                                                     \
       "and.b32 t, x, keep;\nsetp.eq.u32 pf, t, 0;\n"                                                                \
-      "prmt.b32 ro, x, 0, 0x4442;\nmad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n@pf " LDC                            \
+      "prmt.b32 ro, x, 0, 0x4442;\n" SR_D_ROW "mad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n@pf " LDC                            \
       "and.b32 u, x, 63;\nsetp.gt.u32 pf, u, 2;\n@pf bra.uni LGEN;\n"                                               \
       /* 0 MOV, 1 ADD, 2 MUL with an immediate: c * m + n, for t instructions in a row */                           \
-      "prmt.b32 t, x, 0, 0x4443;\nmad.lo.u32 q, t, 8, q;\nld.shared.v2.u32 {nx, ny}, [q];\n"                        \
+      "prmt.b32 t, x, 0, 0x4443;\nmad.lo.u32 q, t, 8, q;\n" SR_D_CHAIN "ld.shared.v2.u32 {nx, ny}, [q];\n"                        \
       "setp.eq.u32 pf, u, 2;\nselp.u32 m, y, u, pf;\nselp.u32 n, 0, y, pf;\n" E(SR_MAD)                             \
       "setp.gt.u32 pf, t, 1;\n@pf bra.uni LCHAIN;\nLCHAINED:\n" SR_TAIL(STC, "")                                    \
       "LRUNEND:\nmov.u32 q, qend;\n" /* (cut by its largest length, the rounds left or the lowest waiting pc) */    \
       "setp.lt.u32 pe, k4, bud;\nsetp.lt.and.u32 pe, q, qw, pe;\n@!pe bra.uni LSTOP;\n"                        \
       "and.b32 u, x, 63;\nsetp.lt.u32 pf, u, 32;\n@pf bra.uni LTOP;\n"                                              \
       "LMEM:\n" /* memory and control: u = the form */                                                              \
-      "ld.shared.v2.u32 {nx, ny}, [q + 8];\nprmt.b32 ro, x, 0, 0x4442;\nmad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" LDA \
+      "ld.shared.v2.u32 {nx, ny}, [q + 8];\nprmt.b32 ro, x, 0, 0x4442;\n" SR_D_ROW "mad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" LDA \
       "setp.ge.u32 pf, u, 34;\n@pf bra.uni LMORE;\nld.acquire.cta.shared.u32 clk, [clks];\nmov.u32 qend, u;\n"      \
       "setp.ge.s32 pf, fl, 0;\n@pf bra.uni LMEM1;\n" SR_FLUSH(E, "A")                                                                      \
       "LMEM1:\n" E(SR_ADDR) "setp.eq.u32 pf, qend, 33;\n@pf bra.uni LSTS;\n"                                        \
@@ -302,7 +354,7 @@ enum : uint32_t {
       "bra.uni LLDSW1;\n"                                                        \
       /* 33 STS: consecutive words, one per thread, cannot collide */                                               \
       "LSTS:\n"                                                                                                     \
-      "prmt.b32 ro, x, 0, 0x4443;\nmad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" LDB                                \
+      "prmt.b32 ro, x, 0, 0x4443;\n" SR_D_ROW "mad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" LDB                                \
       "vote.sync.ballot.b32 t, s0, 0xFFFFFFFF;\nsetp.ne.u32 pa, t, 0;\nbrev.b32 t, t;\nclz.b32 t, t;\nmin.u32 t, t, 31;\n" \
       "shfl.sync.idx.b32 need, a0, t, 31, 0xFFFFFFFF;\nsub.u32 need, need, t;\nadd.u32 m, need, lane;\n"      \
       "mov.u32 n, 0;\nmov.u32 r0, 0;\n" E(SR_OFF) E(SR_MAXR)                                                        \
@@ -314,7 +366,7 @@ enum : uint32_t {
       "setp.eq.u32 pa, m, 0;\nsetp.ne.u32 pb, n, 0;\nvote.sync.all.pred pa, pa, 0xFFFFFFFF;\n"                      \
       "vote.sync.all.pred pb, pb, 0xFFFFFFFF;\nor.pred pf, pa, pb;\n@!pf bra.uni LPARTS;\n" /* both ways */           \
       "setp.eq.xor.u32 pf, u, 34, pb;\n@pf bra.uni LTAKE;\n" SR_FIN                                                 \
-      "LTAKE:\nmad.lo.u32 q, y, 8, irs;\nld.shared.v2.u32 {nx, ny}, [q];\nsub.u32 q, q, 8;\n" SR_FIN                \
+      "LTAKE:\n" SR_D_TARGET "mad.lo.u32 q, y, 8, irs;\nld.shared.v2.u32 {nx, ny}, [q];\nsub.u32 q, q, 8;\n" SR_FIN                \
       /* 36 LDG, 37 STG */                                                                                          \
       "LMORE2:\nld.shared.u64 arena, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 16];\n"                                \
       "ld.shared.u32 awords, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 24];\nand.b32 t, fl, 64;\nsetp.eq.u32 pf, t, 0;\n@pf mov.u32 awords, 0;\n"                           \
@@ -329,7 +381,7 @@ enum : uint32_t {
       "LLDGU:\n" SR_REAL("262144", "m", "24") "@!pf bra.uni LEND;\nmov.u32 need, k4;\n" SR_POLL("E")               \
       SR_GLOG(E, 0) "bra.uni LLDGW1;\n"                                                        \
       "LSTG:\n"                                                                                                     \
-      "prmt.b32 ro, x, 0, 0x4443;\nmad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" LDB                                \
+      "prmt.b32 ro, x, 0, 0x4443;\n" SR_D_ROW "mad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" LDB                                \
       "vote.sync.ballot.b32 t, s0, 0xFFFFFFFF;\nsetp.ne.u32 pa, t, 0;\nbrev.b32 t, t;\nclz.b32 t, t;\nmin.u32 t, t, 31;\n" \
       "shfl.sync.idx.b32 need, a0, t, 31, 0xFFFFFFFF;\nsub.u32 need, need, t;\nadd.u32 m, need, lane;\n"      \
       "mov.u32 n, 0;\nmov.u32 r0, 0;\n" E(SR_OFF) E(SR_MAXR)                                                        \
@@ -369,7 +421,7 @@ enum : uint32_t {
       "bra.uni LSTG3;\n"                                                                                           \
       /* 38 ATOMS */                                                                                                \
       "LMORE3:\nsetp.gt.u32 pf, u, 38;\n@pf bra.uni LMORE4;\nsetp.ge.s32 pf, fl, 0;\n@pf bra.uni LATOMS1;\n" SR_FLUSH(E, "C")              \
-      "LATOMS1:\nprmt.b32 ro, x, 0, 0x4443;\nmad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" LDB "mov.u32 m, 0;\n"    \
+      "LATOMS1:\nprmt.b32 ro, x, 0, 0x4443;\n" SR_D_ROW "mad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" LDB "mov.u32 m, 0;\n"    \
       E(SR_ADDR) E(SR_MAX)                                                                                          \
       "setp.lt.u32 pf, m, sha;\nvote.sync.all.pred pf, pf, 0xFFFFFFFF;\n@!pf bra.uni LATOMSU;\n"                    \
       "add.u32 need, k4, 2;\n@pp st.release.cta.shared.u32 [myclk], need;\n" SR_POLL("C")                           \
@@ -379,7 +431,7 @@ enum : uint32_t {
       "ld.shared.u32 r0, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + 64];\n" E(SR_WBA) "bra.uni LATOMS2;\n"                                        \
       /* 39 BRA, 40 S2R, 41 BAR */                                                                                  \
       "LMORE4:\nsetp.eq.u32 pf, u, 39;\n@pf bra.uni LTAKE;\nsetp.eq.u32 pf, u, 40;\n@!pf bra.uni LMORE5;\n"         \
-      "mad.lo.u32 t, y, 4, " Q_GB ";\nld.shared.u32 t, [t + " SR_STR(SR_GROUP_BV) " + 44];\nmov.u32 u, tid0;\nsetp.eq.u32 pa, y, 0;\n"    \
+      SR_D_SREG "mad.lo.u32 t, y, 4, " Q_GB ";\nld.shared.u32 t, [t + " SR_STR(SR_GROUP_BV) " + 44];\nmov.u32 u, tid0;\nsetp.eq.u32 pa, y, 0;\n"    \
       E(SR_SREG) SR_ROW(STC, "LROWC", "LROWC1") SR_FIN                                                              \
       "LMORE5:\nand.b32 t, fl, 2056;\nsetp.eq.u32 pf, t, 8;\nsetp.eq.and.u32 pf, u, 41, pf;\n@!pf bra.uni LDIV;\n"     \
       "setp.ge.s32 pf, fl, 0;\n@pf bra.uni LBAR1;\n" SR_FLUSH(E, "D")       \
@@ -415,8 +467,8 @@ enum : uint32_t {
       "LCHAIN1:\nsetp.eq.u32 pf, t, 0;\n@pf bra.uni LCHAINED;\n"                                                    \
       "ld.shared.v2.u32 {m, n}, [u];\n" E(SR_MAD) "add.u32 u, u, 8;\nsub.u32 t, t, 1;\nbra.uni LCHAIN1;\n"          \
       /* the other ALU groups */                                                                                    \
-      "LGEN:\nadd.u32 q, q, 8;\nld.shared.v2.u32 {nx, ny}, [q];\n"                                                  \
-      "prmt.b32 ro, x, 0, 0x4443;\nmad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\nsetp.ge.u32 pf, u, 8;\n@pf bra.uni LREST;\n" \
+      "LGEN:\nadd.u32 q, q, 8;\n" SR_D_CODE("q") "ld.shared.v2.u32 {nx, ny}, [q];\n"                                                  \
+      "prmt.b32 ro, x, 0, 0x4443;\n" SR_D_ROW "mad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\nsetp.ge.u32 pf, u, 8;\n@pf bra.uni LREST;\n" \
       /* 3 MOV (operand b is zero), 4 ADD, 5 SUB, 6 MUL of registers */                                             \
       LDB "setp.eq.u32 pf, u, 5;\nselp.b32 m, 0xFFFFFFFF, 1, pf;\nsetp.eq.u32 pa, u, 6;\n" E(SR_REGOP)              \
       SR_TAIL(STC, "bra.uni LRUNEND;\n")                                                                            \
@@ -446,7 +498,7 @@ enum : uint32_t {
          the target, where agents that take it as a whole wait in any case, and the budget has the round in which     \
          they come to wait there.  Not nested. */                                                                     \
       "LPARTS:\nsetp.eq.u32 pz, u, 34;\nsetp.ne.u32 pc, 0, 0;\n" E(SR_PARTS)                                        \
-      "mad.lo.u32 need, y, 8, irs;\nand.b32 t, fl, 512;\nsetp.ne.u32 pa, t, 0;\nsetp.gt.and.u32 pa, need, q, pa;\n"    \
+      SR_D_TARGET "mad.lo.u32 need, y, 8, irs;\nand.b32 t, fl, 512;\nsetp.ne.u32 pa, t, 0;\nsetp.gt.and.u32 pa, need, q, pa;\n"    \
       "setp.eq.and.u32 pa, qw, 0xFFFFFFF8, pa;\nld.shared.u32 t, [need];\nand.b32 t, t, 63;\nsetp.eq.u32 pb, t, 41;\n" \
       "setp.eq.or.u32 pb, t, 49, pb;\nadd.u32 t, k4, 8;\nsetp.le.and.u32 pb, t, bud, pb;\n"                         \
       "not.pred pd, pc;\nor.pred pb, pb, pd;\nand.pred pa, pa, pb;\n"                                              \
@@ -465,7 +517,7 @@ enum : uint32_t {
       "LEND:\nsetp.ge.s32 pf, fl, 0;\n@pf bra.uni LENDED;\n" SR_FLUSH(E, "B")                                      \
       "LENDED:\nand.b32 t, fl, 8192;\nsetp.ne.u32 pf, t, 0;\n@pf bra.uni LNEST;\n"                                 \
       "and.b32 t, fl, 16384;\nsetp.ne.u32 pf, t, 0;\n@pf bra.uni LMERGE;\n"                                        \
-      "LDONE:\nand.b32 t, k4, 0x7FFFFFFF;\nsub.u32 u, t, kst;\nshr.u32 u, u, 2;\nmad.lo.u32 ni, u, cnt, ni;\n"       \
+      "LDONE:\n" SR_D_DONE "and.b32 t, k4, 0x7FFFFFFF;\nsub.u32 u, t, kst;\nshr.u32 u, u, 2;\nmad.lo.u32 ni, u, cnt, ni;\n"       \
       "shl.b32 wm, wm, 4;\n" E(SR_OUT) "mov.u32 " Q_MASK ", wm;\nmov.u32 " Q_FL ", fl;\nmov.u32 " Q_QW ", qw;\n"     \
       "mov.u32 " Q_Q ", q;\nmov.u32 " Q_K4 ", k4;\nmov.u32 " Q_GACC ", gacc;\nmov.u32 " Q_SACC ", sacc;\n"           \
       "mov.u32 " Q_EH ", eh;\nmov.u32 " Q_NI ", ni;\n"                                                             \

@@ -59,3 +59,52 @@ def test_debug_build_has_no_failed_index_check_and_matches_the_oracle():
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=1200)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
     assert "debug build ok" in r.stdout
+
+
+LOOP_SCRIPT = r'''
+import ctypes, sys
+sys.path[:0] = [ROOT, HERE]
+import numpy as np
+import oracle
+from paper_1211_6193_gb300 import binding, build
+lib = binding.load_library(build.DEBUG_LIB)
+from paper_1211_6193_gb300.workloads import rng
+from test_gpu_blocks import OPTIONS, random_program
+from test_gpu_limits import behind_large_block
+
+def loop_rounds():
+    n = ctypes.c_ulonglong()
+    assert lib.sr_debug_loop_rounds(ctypes.byref(n)) == 0
+    return n.value
+
+before = loop_rounds()
+for option, (opts, oracle_kw) in OPTIONS.items():
+    for bdim in (33, 64, 97, 128, 255, 640, 1024):
+        progs = [random_program(rng.derive(500 + bdim, i), bdim) for i in range(6)]
+        if opts["mode"] == "batched":
+            progs += [behind_large_block(p) for p in progs]
+        want = oracle.run(progs, **oracle_kw)
+        got = binding.check(progs, **opts)
+        assert not np.any(got.status & (binding.ST_BOUNDS | binding.ST_INTERNAL)), (option, bdim, got.status)
+        assert got.report_tuples() == want.report_tuples(), (option, bdim)
+        for i in range(len(progs)):
+            assert np.array_equal(got.arenas[i], want.arenas[i]), (option, bdim, i)
+    after = loop_rounds()
+    assert after - before > 10_000, (option, after - before)     # the loop, not the general steps
+    before = after
+print("debug loop ok")
+'''
+
+
+def test_debug_build_checks_the_inner_loop():
+    """The debug build runs the inner loop too, with a check before every access: under every option,
+    with one, two and four simulated warps per warp, no check fails and the results are the oracle's."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1211_6193_gb300 import build
+    build.build(debug=True)
+    code = f"ROOT = {ROOT!r}\nHERE = {HERE!r}\n" + LOOP_SCRIPT
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=1200)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+    assert "debug loop ok" in r.stdout
