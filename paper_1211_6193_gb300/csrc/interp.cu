@@ -61,6 +61,10 @@ struct BlockVars {
   uint32_t sreg[4];            // S2R BID, BDIM, GDIM, WARPSIZE
 };
 static_assert(sizeof(BlockVars) <= 64, "block vars");
+static_assert(offsetof(BlockVars, cursor) == 16 && offsetof(BlockVars, flags) == 20 && offsetof(BlockVars, gcursor) == 44 &&
+                  offsetof(BlockVars, sreg) == 48 && BF_OVERFLOW == 1 && SR_SREG_TID == 0 && SR_SREG_BID == 1 &&
+                  SR_SREG_BDIM == 2 && SR_SREG_GDIM == 3 && SR_SREG_WARPSIZE == 4 && K_R == 0 && K_W == 1 && K_A == 2,
+              "block variables, registers and kinds in solo_loop");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));

@@ -20,6 +20,8 @@
 //  - a barrier that every thread of the block waits at, with nothing to report, is passed here,
 //    with one CTA barrier: every warp reads all park entries and draws the same conclusion.
 #pragma once
+#include <cstddef>
+
 #include "sr_internal.h"
 
 namespace sr {
@@ -525,8 +527,30 @@ enum : uint32_t {
       : "+r"(q), "+r"(k4), "+r"(gacc), "+r"(sacc), "+r"(eh), "+r"(ni), "+r"(fl), "+r"(qw), "=r"(mask)               \
       : "r"(gb), "r"(w), "r"(rs), "r"(stride), "r"(am), "r"(fcap), "r"(bud)                                                 \
       : "memory")
-static_assert(F_LDS == 32 && F_STS == 33 && F_BRZ == 34 && F_LDG == 36 && F_ATOMS == 38 && F_S2R == 40 && F_BAR == 41 && F_EXIT == 49 &&
-                  F_DIVR > 41 && kFwdA == 64 && kDeadD == 128 && kNoDest == 31,
+// The numbers in the statement: places of what it reads, flags and masks, forms.
+static_assert(offsetof(SoloConst, irs) == 0 && offsetof(SoloConst, rb) == 4 && offsetof(SoloConst, shs) == 8 &&
+                  offsetof(SoloConst, sha) == 12 && offsetof(SoloConst, arena) == 16 && offsetof(SoloConst, arena_words) == 24 &&
+                  offsetof(SoloConst, spin) == 28 && offsetof(SoloConst, budget4) == 32 && offsetof(SoloConst, nrows) == 36 &&
+                  offsetof(SoloConst, nthr) == 40 && offsetof(SoloConst, nw) == 44 && offsetof(SoloConst, tup) == 48 &&
+                  offsetof(SoloConst, tps4) == 52 && offsetof(SoloConst, region) == 56 && offsetof(SoloConst, wb) == 64 &&
+                  offsetof(SoloConst, gcap) == 68 && offsetof(SoloConst, gblock) == 72 && offsetof(SoloConst, ncode) == 76 &&
+                  offsetof(SoloConst, gregion) == 80,
+              "constants in solo_loop");
+static_assert(kGroupClk == 0 && 32 * kMaxWarps == 1 << (31 - 23) && kMaxWarps == 8, "clocks and park entries in solo_loop");
+static_assert(kSoloPub == 1 && kSoloMany == 2 && kSoloLog == 4 && kSoloBar == 8 && kSoloFull == 16 && kSoloShared == 32 &&
+                  kSoloGlobal == 64 && kSoloWhole == 128 && kSoloSolo == 512 && kSoloFused == 1024 && kSoloNested == 2048 &&
+                  kSoloToNest == 8192 && kSoloToMerge == 16384 && kSoloAtBar == 32768 && kSoloTimeout == 65536 &&
+                  kSoloUninit == 131072 && kSoloGlog == 262144 && kSoloBad == 0x80000 && kSoloPending == 0x80000000u &&
+                  (kSoloLog | kSoloFull) == 20 && (kSoloSolo | kSoloPub) == 513 && (kSoloNested | kSoloBar) == 2056 &&
+                  (kSoloNested | kSoloRegular) == 2304 && kSoloRegular == 256 && (kSoloToNest | kSoloNested) == 10240 &&
+                  (kSoloToNest | kSoloNested | kSoloAgents) == 14336 && ~kSoloLog == 0xFFFFFFFBu && ~kSoloToNest == 0xFFFFDFFFu &&
+                  ~(kSoloNested | kSoloAgents | kSoloToMerge) == 0xFFFFA7FFu && ~kSoloPending == 0x7FFFFFFFu,
+              "flags in solo_loop");
+static_assert(F_MULI == 2 && F_MOVR == 3 && F_SUBR == 5 && F_MULR == 6 && F_AND == 8 && F_OR == 10 && F_XOR == 12 && F_SHL == 14 &&
+                  F_SHR == 16 && F_MIN == 18 && F_MAX == 20 && F_SLT == 22 && F_SLE == 24 && F_SEQ == 26 && F_SNE == 28 &&
+                  F_LDS == 32 && F_STS == 33 && F_BRZ == 34 && F_BRNZ == 35 && F_LDG == 36 && F_STG == 37 && F_ATOMS == 38 &&
+                  F_BRA == 39 && F_S2R == 40 && F_BAR == 41 && F_DIVI == 46 && F_REMI == 48 && F_EXIT == 49 && kFwdA == 64 &&
+                  kDeadD == 128 && kNoDest == 31 && kRunMax == 255,
               "forms in solo_loop");
 
 // Runs the set of the active slots `am` from instruction address q and clock k4 (4 * round with
