@@ -128,14 +128,27 @@ struct RangeScratch {
   struct State {
     int32_t lo[16], hi[16];
     uint32_t visits;             // 0: not reached
+    uint32_t by_params;          // registers whose interval follows from the launch's parameters
   };
   std::vector<int32_t> leader;   // per pc: index of its state, -1 inside a straight line
   std::vector<State> states;
   std::vector<uint8_t> queued;
+  bool by_params = false;        // the last result follows from the parameters (some address's interval does)
+  // the last results for the program at hand (shared_reach_of)
+  struct Seen {
+    uint32_t entry, block_dim, grid, block_begin, block_count, shmem_words, nparams;
+    int32_t params[4];
+    bool by_params;
+    uint32_t reach;
+  };
+  std::vector<Seen> seen;
+  uint64_t analyses = 0;
 };
 inline uint32_t shared_reach(const sr_instr* code, uint32_t ncode, uint32_t entry, const sr_launch& L, RangeScratch& w) {
   const uint32_t shw = L.shmem_words;
+  w.by_params = false;
   if (!shw) return 0;
+  ++w.analyses;
   using State = RangeScratch::State;
   // leaders: the entry, branch targets and what follows a branch
   w.leader.assign(ncode + 1, -1);
@@ -174,14 +187,19 @@ inline uint32_t shared_reach(const sr_instr* code, uint32_t ncode, uint32_t entr
       t.lo[r] = lo;
       t.hi[r] = hi;
     }
-    if (changed) {
-      ++t.visits;
+    const bool more = (s.by_params & ~t.by_params) != 0;
+    t.by_params |= s.by_params;
+    t.visits += changed;
+    if (changed || more) {
       w.queued[pc] = 1;
       next = std::min(next, pc);
     }
   };
   State s{};
-  for (uint32_t q = 0; q < 4 && q < L.nparams; ++q) s.lo[q] = s.hi[q] = L.params[q];
+  for (uint32_t q = 0; q < 4 && q < L.nparams; ++q) {
+    s.lo[q] = s.hi[q] = L.params[q];
+    s.by_params |= 1u << q;
+  }
   flow(s, entry);
   const int64_t first = L.block_begin, blocks = L.block_count ? L.block_count : L.grid;
   while (next < ncode) {
@@ -203,6 +221,7 @@ inline uint32_t shared_reach(const sr_instr* code, uint32_t ncode, uint32_t entr
       int64_t bl = zb ? 0 : s.lo[rb], bh = zb ? 0 : s.hi[rb];
       if (op & SR_BIMM) bl = bh = imm;
       int64_t lo = INT32_MIN, hi = INT32_MAX;    // the result's interval (unknown)
+      const bool pa = !za && ((s.by_params >> ra) & 1u), pb = !(op & SR_BIMM) && !zb && ((s.by_params >> rb) & 1u);
       switch (b) {
         case SR_OP_MOV: lo = bl; hi = bh; break;
         case SR_OP_ADD: lo = al + bl; hi = ah + bh; break;
@@ -258,6 +277,7 @@ inline uint32_t shared_reach(const sr_instr* code, uint32_t ncode, uint32_t entr
           break;
         case SR_OP_LDS: case SR_OP_STS: case SR_OP_ATOMS: {
           const int64_t l = al + imm, h = ah + imm;
+          w.by_params = w.by_params || pa;
           if (l < INT32_MIN || h > INT32_MAX) reach = shw;
           else if (h >= 0 && l < (int64_t)shw) reach = std::max(reach, (uint32_t)std::min<int64_t>(h + 1, shw));
           break;
@@ -268,6 +288,9 @@ inline uint32_t shared_reach(const sr_instr* code, uint32_t ncode, uint32_t entr
         const bool fits = lo >= INT32_MIN && hi <= INT32_MAX;
         s.lo[d] = fits ? (int32_t)lo : INT32_MIN;
         s.hi[d] = fits ? (int32_t)hi : INT32_MAX;
+        // (comparisons and what is loaded, read or counted: the same interval for any parameters)
+        const bool from = b == SR_OP_MOV ? pb : b >= SR_OP_ADD && b <= SR_OP_MAX && (pa || pb);
+        s.by_params = (s.by_params & ~(1u << d)) | (from ? 1u << d : 0u);
       }
       if (reach == shw || b == SR_OP_EXIT) break;
       if (b == SR_OP_BRA || b == SR_OP_BRZ || b == SR_OP_BRNZ) {
@@ -284,6 +307,26 @@ inline uint32_t shared_reach(const sr_instr* code, uint32_t ncode, uint32_t entr
     if (reach == shw) break;
   }
   return reach;
+}
+
+// The same for a program's launches one after the other (w.seen is empty before the first): the analysis
+// (11 us for a kernel of 3,000 instructions) runs once for launches of the same shape
+// whose addresses do not follow from the parameters, or with the same parameters.
+inline uint32_t shared_reach_of(const sr_instr* code, uint32_t ncode, uint32_t entry, const sr_launch& L, RangeScratch& w) {
+  RangeScratch::Seen k{entry, L.block_dim, L.grid, L.block_begin, L.block_count, L.shmem_words, L.nparams, {}, false, 0};
+  for (uint32_t q = 0; q < 4 && q < L.nparams; ++q) k.params[q] = L.params[q];
+  for (size_t i = w.seen.size(); i-- > 0;) {
+    const RangeScratch::Seen& o = w.seen[i];
+    if (o.entry == k.entry && o.block_dim == k.block_dim && o.grid == k.grid && o.block_begin == k.block_begin &&
+        o.block_count == k.block_count && o.shmem_words == k.shmem_words && o.nparams == k.nparams &&
+        (!o.by_params || std::equal(k.params, k.params + 4, o.params)))
+      return o.reach;
+  }
+  k.reach = shared_reach(code, ncode, entry, L, w);
+  k.by_params = w.by_params;
+  if (w.seen.size() >= 16) w.seen.erase(w.seen.begin());
+  w.seen.push_back(k);
+  return k.reach;
 }
 
 inline int validate(const sr_program* p, char* msg, size_t len) {

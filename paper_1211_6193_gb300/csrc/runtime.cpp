@@ -581,6 +581,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       for (uint32_t k = 0; k < P.nkernels; ++k) kb[k] = bound_kernel(P.code, P.ncode, P.kernel_entry[k], ws);
     }
     const uint32_t first_launch = (uint32_t)b->launches.size();   // the program's launches are contiguous
+    ranges.seen.clear();
     bool one_all = wide && P.nlaunches > 0;    // every launch's blocks are large
     // batched mode: a program's launches run in one grid, so they share the kernel form
     uint32_t pvec = 0;
@@ -648,7 +649,7 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
       d.ir_bytes = sr::ir_code_bytes(P.ncode);
       d.nrows = rm.nrows;
       const uint32_t nsw = (L.block_dim + 31) / 32;         // simulated warps
-      d.sha = shared_reach(P.code, P.ncode, d.entry, L, ranges);
+      d.sha = shared_reach_of(P.code, P.ncode, d.entry, L, ranges);
       d.vec = pvec ? pvec : sr::block_vec(L.block_dim, d.grid, (uint32_t)c->sms, fused);
       d.nw = sr::block_warps(L.block_dim, d.vec);
       const uint32_t lanes = d.nw * 32 * d.vec;

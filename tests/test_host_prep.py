@@ -27,3 +27,8 @@ def test_packed_runs_match_the_plain_code(tmp_path):
 def test_shared_reach_covers_every_access(tmp_path):
     accesses, below = run_check("reach_check", tmp_path)
     assert accesses > 20_000 and below > 300
+
+
+def test_shared_reach_is_analysed_once_for_alike_launches(tmp_path):
+    launches, analyses = run_check("reach_memo_check", tmp_path)
+    assert launches == 48_000 and analyses == 1
