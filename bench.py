@@ -464,7 +464,7 @@ def run_native(args):
         gbs = 32 * gst.global_records / (ms_g / 1e3) / 1e9 if ms_g > 0 else 0.0
         global_leg = {"workload": WORKLOADS["reduction"], "records_per_step": gst.global_records,
                       "stage_ms": gstage, "ms_per_step": statistics.mean(gper), "reports_per_step": gn,
-                      "roofline": {"bound": "hbm", "kernels": "k_ggather, k_rs_upsweep, k_rs_pass, k_grun",
+                      "roofline": {"bound": "hbm", "kernels": "k_ggather, k_rs_upsweep, k_rs_pass, k_grun, k_grun_long",
                                    "achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
                                    "algorithmic_bytes": "32 B per logged global access (16 B record written, "
                                                         "read once); radix passes beyond that are "

@@ -613,6 +613,8 @@ struct GrunArgs {
   unsigned long long gcap;          // entries that fit
   unsigned long long* gn;           // entries produced (may exceed gcap: the run is repeated)
   uint32_t* gcount;                 // per global block: its entries
+  unsigned long long* longs;        // first records of long runs (room for one in eight records)
+  uint32_t* nlongs;                 // their number (zero before the launch)
 };
 
 __device__ __forceinline__ uint32_t find_launch(const GrunArgs& A, uint32_t gb) {
@@ -683,6 +685,111 @@ __device__ __forceinline__ bool ordered(const GrunArgs& A, const LaunchDev& P0, 
   return (A.ord_bits[P0.ord_off + (bit >> 5)] >> (bit & 31u)) & 1u;
 }
 
+// The run of equal (program, word) that starts at record i of n, by one thread; rec(j) is record j.
+template <class RecAt>
+__device__ __forceinline__ void scan_run(const GrunArgs& A, unsigned long long n, unsigned long long i, const RecAt& rec) {
+  const uint4 r0 = rec(i);
+  uint32_t li = find_launch(A, r0.w);
+  const uint32_t prog = A.launches[li].prog;
+  uint32_t base = A.launches[li].block_base, grid = A.launches[li].grid;   // of launch li
+  const uint32_t word = r0.x;
+  const LaunchDev& P0 = A.launches[A.launches[li].first_launch];    // the program's launch 0
+  const bool pairs = P0.ord_off != kNoDep;                          // unordered launches exist
+  // interval summary: the two smallest distinct reader and writer tids, pc range
+  uint32_t igb = kInf, iep = 0, iR = NONE16 << 16 | NONE16, iW = NONE16 << 16 | NONE16, ipl = kInf, iph = 0;
+  // launch summary: the two smallest distinct reader and writer blocks, pc range
+  uint32_t lcur = kInf, lR[2] = {kInf, kInf}, lW[2] = {kInf, kInf}, lpl = kInf, lph = 0;
+  // launch pairs: kinds of the current launch, start of its sub-run, best pair and classes
+  uint32_t lk = 0, b1 = kInf, b2 = kInf, pcls = 0;
+  unsigned long long lstart = i;
+  for (unsigned long long j = i;; ++j) {
+    bool end = j >= n;
+    uint4 q = make_uint4(0, 0, 0, 0);
+    uint32_t qli = li;
+    if (!end) {
+      q = rec(j);
+      end = q.x != word;
+      if (!end && (q.w < base || q.w - base >= grid)) {
+        qli = find_launch(A, q.w);
+        end = A.launches[qli].prog != prog;
+      }
+    }
+    // interval boundary: (block, epoch) changes
+    if (igb != kInf && (end || q.w != igb || q.y != iep)) {
+      const uint32_t W[2] = {iW & 0xFFFFu, iW >> 16}, R[2] = {iR & 0xFFFFu, iR >> 16};
+      uint32_t t1, t2;
+      const uint32_t cls = pair_classes(W, R, NONE16, t1, t2);
+      if (cls) emit_entry(A, igb, iep << 2, word, t1 << 16 | t2, cls << 24 | (ipl & 0xFFFu) << 12 | (iph & 0xFFFu));
+      igb = kInf;
+    }
+    // launch boundary
+    if (lcur != kInf && (end || qli != lcur)) {
+      const LaunchDev& L = A.launches[lcur];
+      uint32_t p1, p2;
+      const uint32_t cls = pair_classes(lW, lR, kInf, p1, p2);
+      if (cls)
+        emit_entry(A, L.block_base + p1, 1u, word, p2 + L.block_off,
+                   cls << 24 | (lpl & 0xFFFu) << 12 | (lph & 0xFFFu));
+      if (pairs) {
+        // this launch against every earlier launch of the run that nothing orders before it
+        const uint32_t l = L.launch;
+        unsigned long long k = i;
+        while (k < lstart) {
+          const uint32_t mli = find_launch(A, rec(k).w);
+          const LaunchDev& M = A.launches[mli];
+          uint32_t mk = 1u << grec_write(rec(k));      // (the first record is M's: progress)
+          for (++k; k < lstart && rec(k).w >= M.block_base && rec(k).w - M.block_base < M.grid; ++k)
+            mk |= 1u << grec_write(rec(k));
+          const uint32_t m = M.launch;
+          if (ordered(A, P0, m, l)) continue;
+          uint32_t c = 0;
+          if ((mk & 2u) && (lk & 2u)) c |= SR_CLS_WW;
+          if (((mk & 2u) && (lk & 1u)) || ((mk & 1u) && (lk & 2u))) c |= SR_CLS_WR;
+          if (!c) continue;
+          pcls |= c;
+          if (m < b1 || (m == b1 && l < b2)) {
+            b1 = m;
+            b2 = l;
+          }
+        }
+      }
+      lcur = kInf;
+    }
+    if (end) break;
+    // accumulate record q
+    const uint32_t t = grec_tid(q), wr = grec_write(q), pc = grec_pc(q);
+    if (igb == kInf) {
+      igb = q.w;
+      iep = q.y;
+      iR = iW = NONE16 << 16 | NONE16;
+      ipl = kInf;
+      iph = 0;
+    }
+    if (wr) iW = min2_16(iW, t); else iR = min2_16(iR, t);
+    ipl = min(ipl, pc);
+    iph = max(iph, pc);
+    if (lcur == kInf) {
+      lcur = qli;
+      lR[0] = lR[1] = lW[0] = lW[1] = kInf;
+      lpl = kInf;
+      lph = 0;
+      lk = 0;
+      lstart = j;
+    }
+    if (qli != li) {
+      li = qli;
+      base = A.launches[li].block_base;
+      grid = A.launches[li].grid;
+    }
+    const uint32_t blk = q.w - base;
+    if (wr) min2_32(lW[0], lW[1], blk); else min2_32(lR[0], lR[1], blk);
+    lpl = min(lpl, pc);
+    lph = max(lph, pc);
+    lk |= 1u << wr;
+  }
+  if (pcls) emit_entry(A, A.launches[P0.first_launch + b1].block_base, 2u, word, b2, pcls << 24);
+}
+
 // One thread per run of equal (program, word) of two records or more (one record holds no pair);
 // records of a run are in (launch, block, epoch) order.  What bounds it is latency: a run is a chain
 // of dependent reads, and runs start at a few lanes of a warp only.  So a CTA takes GR_T records
@@ -690,7 +797,13 @@ __device__ __forceinline__ bool ordered(const GrunArgs& A, const LaunchDev& P0, 
 // collects the places where runs start, and then every thread has a run.  With a thread per record
 // and no tile this kernel took 348 us for 6.3 M records of a stencil; the whole check of the
 // 1024^2 stencil's eight launches went from 2,230 to 1,310 us.
-constexpr uint32_t GR_T = 1024, GR_HALO = 256, GR_N = 256, GR_PROGS = 512;
+// A run of more than GR_LONG records (a word that many threads use, as of a table) would hold up its
+// CTA: it is left to k_grun_long.  10.8 M loads of a table of 64, 1,024, 16,384 and 131,072 words, the
+// check with all runs here 62,046, 11,738, 3,570 and 1,006 us, now 55,641, 4,281, 1,014 and 733 (with
+// a limit of 128 or 256: 1,006 the last; with a thread per record and no tile 65,454, 5,787,
+// 2,729 and 1,967); checks without long runs take 4 us more for the second kernel.
+constexpr uint32_t GR_T = 1024, GR_HALO = 256, GR_N = 256, GR_PROGS = 512, GR_LONG = 64;
+static_assert(GR_LONG <= GR_HALO && GR_LONG >= 8, "a long run shows in the tile, and the list has room");
 __global__ void __launch_bounds__(GR_N) k_grun(GrunArgs A) {
   __shared__ uint4 tile[GR_T + GR_HALO + 1];       // records t0 - 1 .. t0 + GR_T + GR_HALO - 1
   __shared__ uint16_t start[GR_T];
@@ -745,110 +858,23 @@ __global__ void __launch_bounds__(GR_N) k_grun(GrunArgs A) {
   __syncthreads();
   const uint32_t nst = nstart;
   for (uint32_t x = tid; x < nst; x += GR_N) {
-    const unsigned long long i = t0 + start[x];
-    auto rec = [&](unsigned long long j) { return j - t0 < nt ? tile[j - t0 + 1] : A.rec[j]; };
-    const uint4 r0 = rec(i);
-    uint32_t li = find_launch(A, r0.w);
-    const uint32_t prog = A.launches[li].prog;
-    uint32_t base = A.launches[li].block_base, grid = A.launches[li].grid;   // of launch li
-    const uint32_t word = r0.x;
-    const LaunchDev& P0 = A.launches[A.launches[li].first_launch];    // the program's launch 0
-    const bool pairs = P0.ord_off != kNoDep;                          // unordered launches exist
-    // interval summary: the two smallest distinct reader and writer tids, pc range
-    uint32_t igb = kInf, iep = 0, iR = NONE16 << 16 | NONE16, iW = NONE16 << 16 | NONE16, ipl = kInf, iph = 0;
-    // launch summary: the two smallest distinct reader and writer blocks, pc range
-    uint32_t lcur = kInf, lR[2] = {kInf, kInf}, lW[2] = {kInf, kInf}, lpl = kInf, lph = 0;
-    // launch pairs: kinds of the current launch, start of its sub-run, best pair and classes
-    uint32_t lk = 0, b1 = kInf, b2 = kInf, pcls = 0;
-    unsigned long long lstart = i;
-    for (unsigned long long j = i;; ++j) {
-      bool end = j >= n;
-      uint4 q = make_uint4(0, 0, 0, 0);
-      uint32_t qli = li;
-      if (!end) {
-        q = rec(j);
-        end = q.x != word;
-        if (!end && (q.w < base || q.w - base >= grid)) {
-          qli = find_launch(A, q.w);
-          end = A.launches[qli].prog != prog;
-        }
-      }
-      // interval boundary: (block, epoch) changes
-      if (igb != kInf && (end || q.w != igb || q.y != iep)) {
-        const uint32_t W[2] = {iW & 0xFFFFu, iW >> 16}, R[2] = {iR & 0xFFFFu, iR >> 16};
-        uint32_t t1, t2;
-        const uint32_t cls = pair_classes(W, R, NONE16, t1, t2);
-        if (cls) emit_entry(A, igb, iep << 2, word, t1 << 16 | t2, cls << 24 | (ipl & 0xFFFu) << 12 | (iph & 0xFFFu));
-        igb = kInf;
-      }
-      // launch boundary
-      if (lcur != kInf && (end || qli != lcur)) {
-        const LaunchDev& L = A.launches[lcur];
-        uint32_t p1, p2;
-        const uint32_t cls = pair_classes(lW, lR, kInf, p1, p2);
-        if (cls)
-          emit_entry(A, L.block_base + p1, 1u, word, p2 + L.block_off,
-                     cls << 24 | (lpl & 0xFFFu) << 12 | (lph & 0xFFFu));
-        if (pairs) {
-          // this launch against every earlier launch of the run that nothing orders before it
-          const uint32_t l = L.launch;
-          unsigned long long k = i;
-          while (k < lstart) {
-            const uint32_t mli = find_launch(A, rec(k).w);
-            const LaunchDev& M = A.launches[mli];
-            uint32_t mk = 1u << grec_write(rec(k));      // (the first record is M's: progress)
-            for (++k; k < lstart && rec(k).w >= M.block_base && rec(k).w - M.block_base < M.grid; ++k)
-              mk |= 1u << grec_write(rec(k));
-            const uint32_t m = M.launch;
-            if (ordered(A, P0, m, l)) continue;
-            uint32_t c = 0;
-            if ((mk & 2u) && (lk & 2u)) c |= SR_CLS_WW;
-            if (((mk & 2u) && (lk & 1u)) || ((mk & 1u) && (lk & 2u))) c |= SR_CLS_WR;
-            if (!c) continue;
-            pcls |= c;
-            if (m < b1 || (m == b1 && l < b2)) {
-              b1 = m;
-              b2 = l;
-            }
-          }
-        }
-        lcur = kInf;
-      }
-      if (end) break;
-      // accumulate record q
-      const uint32_t t = grec_tid(q), wr = grec_write(q), pc = grec_pc(q);
-      if (igb == kInf) {
-        igb = q.w;
-        iep = q.y;
-        iR = iW = NONE16 << 16 | NONE16;
-        ipl = kInf;
-        iph = 0;
-      }
-      if (wr) iW = min2_16(iW, t); else iR = min2_16(iR, t);
-      ipl = min(ipl, pc);
-      iph = max(iph, pc);
-      if (lcur == kInf) {
-        lcur = qli;
-        lR[0] = lR[1] = lW[0] = lW[1] = kInf;
-        lpl = kInf;
-        lph = 0;
-        lk = 0;
-        lstart = j;
-      }
-      if (qli != li) {
-        li = qli;
-        base = A.launches[li].block_base;
-        grid = A.launches[li].grid;
-      }
-      const uint32_t blk = q.w - base;
-      if (wr) min2_32(lW[0], lW[1], blk); else min2_32(lR[0], lR[1], blk);
-      lpl = min(lpl, pc);
-      lph = max(lph, pc);
-      lk |= 1u << wr;
+    const uint32_t s0 = start[x] + 1u;             // its first record in the tile
+    if (start[x] + GR_LONG < nt && tile[s0 + GR_LONG].x == tile[s0].x && (one_prog || pr[s0 + GR_LONG] == pr[s0])) {
+      A.longs[atomicAdd(A.nlongs, 1u)] = t0 + start[x];
+      continue;
     }
-    if (pcls) emit_entry(A, A.launches[P0.first_launch + b1].block_base, 2u, word, b2, pcls << 24);
+    scan_run(A, n, t0 + start[x], [&](unsigned long long j) { return j - t0 < nt ? tile[j - t0 + 1] : A.rec[j]; });
   }
   }
+}
+
+// The long runs, one thread each, a warp's lanes last: one thread per warp while there are few.
+__global__ void __launch_bounds__(GR_N) k_grun_long(GrunArgs A) {
+  const unsigned long long n = *A.n_ptr;
+  const uint32_t m = *A.nlongs, warps = gridDim.x * (GR_N / 32u);
+  const uint32_t w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  for (unsigned long long x = w + (unsigned long long)(threadIdx.x & 31u) * warps; x < m; x += 32ull * warps)
+    scan_run(A, n, A.longs[x], [&](unsigned long long j) { return A.rec[j]; });
 }
 
 uint32_t g_pass_ctas16 = 0, g_pass_ctas32 = 0;
@@ -954,10 +980,13 @@ cudaError_t launch_gcheck(const GcheckArgs& G, uint32_t& kernels, cudaStream_t s
   R.gcap = G.entry_cap;
   R.gn = G.gn;
   R.gcount = G.gcount;
+  R.longs = G.status;                              // (the sort's tile states: free between the two sorts)
+  R.nlongs = G.tile_ctr + MAX_PASSES - 1;          // (an address has at most four digits: the sort's last counter)
   {
     const uint32_t ctas = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((G.rec_cap + GR_T - 1) / GR_T, 8ull * G.sms));
     k_grun<<<ctas, GR_N, 0, s>>>(R);
-    ++kernels;
+    k_grun_long<<<std::min(ctas, 4u * G.sms), GR_N, 0, s>>>(R);
+    kernels += 2;
   }
   // 4. the entries in (block, epoch, kind, word) order, and each block's first entry
   e = radix_sort<Rec32, EntryDigit, true>(reinterpret_cast<Rec32*>(G.entries_a), reinterpret_cast<Rec32*>(G.entries_b),

@@ -159,6 +159,28 @@ def test_global_check_groups_by_program(B):
     assert len(assert_same(B, [deep], {"check_global": True}, {"check_global": True}).reports) == 1
 
 
+@pytest.mark.parametrize("mode", ["plain", "batched"])
+def test_global_check_run_lengths(B, mode):
+    """Words used by one block to all of 1,400, the lengths around the run scan's limits (64 records, its
+    tile of 1,024 and 256 behind it), odd words stored to, in launches that nothing orders too."""
+    lengths = [1, 2, 3, 31, 62, 63, 64, 65, 66, 67, 127, 128, 129, 255, 256, 257, 258, 500, 640, 767, 768, 1000, 1022, 1023,
+               1024, 1025, 1278, 1279, 1280, 1281, 1399, 1400]
+    def prog(shift, unordered):
+        a = Asm().s2r(r2, TID).s2r(r3, BID).ldg(r4, r2, 64).slt(r5, r3, r4).brz(r5, "end")
+        a.and_(r9, r2, 1).brz(r9, "load").stg(r2, r3, 32).label("load").ldg(r10, r2, 32).label("end").exit()
+        arena = np.zeros(96, np.int32)
+        arena[64:] = np.roll(lengths, shift)
+        launches = [Launch(0, 1400, 32, 1, (), stream=0)]
+        if unordered:
+            launches += [Launch(0, 1400, 32, 1, (), stream=1), Launch(0, 7, 32, 1, (), stream=2)]
+        return Program(a.assemble(), [0], launches, arena, name=f"lengths_{shift}_{unordered}")
+    progs = [prog(0, False), prog(5, True), prog(11, False)]
+    want = oracle.run(progs, check_global=True)
+    got = B.check(progs, mode=mode, check_global=True)
+    assert not np.any(got.status)
+    assert got.report_tuples() == want.report_tuples() and len(want.reports) > 60
+
+
 def test_global_check_in_a_graph(B):
     """The sort's cooperative kernel under capture, and the graph run again."""
     progs = [random_program(rng.derive(7, i), 96) for i in range(6)]
