@@ -720,7 +720,7 @@ __device__ __forceinline__ void note_loop(uint32_t, uint32_t) {}
 // lowest such pc).  Otherwise the agents' states sit in lanes 0..V-1 (ap next pc, ak round,
 // aw lowest waiting pc) and the set with the lowest round runs, at one round first loads and
 // everything that touches no memory, then stores, then atomics.
-template <int V, bool Fused, bool Global>
+template <int V, bool Fused, bool Global, bool Div>
 __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls, uint32_t block,
                                           const uint2* __restrict__ ir, unsigned char* gsm) {
   const uint32_t w = same(threadIdx.x >> 5), nw = same(Ls->nw);
@@ -899,7 +899,7 @@ __device__ __forceinline__ void run_block(const RunArgs& A, const LaunchDev* Ls,
         if (solo || kn) fl |= kSoloPub | solo_mem;
         if (solo && whole && nexit == 0 && !errs && !fused && wpc == kInf) fl |= kSoloBar;
         fl = same(fl);
-        const uint32_t mask = solo_loop<V, Fused>(q, k4, n_gacc, n_sacc, eh, n_instr, fl, qw, gb, w, rs, rstride, am,
+        const uint32_t mask = solo_loop<V, Fused, Div>(q, k4, n_gacc, n_sacc, eh, n_instr, fl, qw, gb, w, rs, rstride, am,
                                                   same(front_cap), same(4u * (solo || !kn ? budget : kn) + par));
         fl = same(fl);
         lfull = (fl & kSoloFull) != 0;
@@ -1412,7 +1412,7 @@ __device__ __forceinline__ void copy_launch(LaunchDev* dst, const LaunchDev* src
 
 // The CTA's block once its launch is known and its code is under way: clear, wait for the code,
 // run (unless warp 0 has found, before it comes here, that the launch is skipped).
-template <int V, bool Fused, bool Global>
+template <int V, bool Fused, bool Global, bool Div>
 __device__ __forceinline__ void run_staged(const RunArgs& A, const LaunchDev* Ls, uint32_t block, unsigned char* smem,
                                            unsigned long long* mbar, const uint32_t* skip) {
   // every thread must take the same branch before the block's named barriers
@@ -1422,7 +1422,7 @@ __device__ __forceinline__ void run_staged(const RunArgs& A, const LaunchDev* Ls
   if (!__any_sync(FULL, stage_wait(mbar, 0, drained))) {           // (its barrier also ends the clearing)
     if (threadIdx.x == 0) atomicOr(&A.prog_status[Ls->prog], (uint32_t)SR_ST_INTERNAL);
   } else if (mine && !same(*skip)) {
-    run_block<V, Fused, Global>(A, Ls, block, reinterpret_cast<const uint2*>(smem), smem + Ls->ir_bytes);
+    run_block<V, Fused, Global, Div>(A, Ls, block, reinterpret_cast<const uint2*>(smem), smem + Ls->ir_bytes);
   }
 }
 
@@ -1449,7 +1449,7 @@ __global__ void __launch_bounds__(V == 1 ? 64 : 256, MINB) k_interp_plain(RunArg
   }
   __syncthreads();
   if (same(s_skip)) return;
-  run_staged<V, Fused, Global>(A, &Ls, blockIdx.x, smem, &mbar, &s_skip);
+  run_staged<V, Fused, Global, MINB != 4>(A, &Ls, blockIdx.x, smem, &mbar, &s_skip);
 }
 
 // Batched mode: the blocks of many launches in one grid, one simulated block per CTA.  The host
@@ -1506,7 +1506,7 @@ __global__ void __launch_bounds__(V == 1 ? 64 : 256, MINB) k_interp_blocks(RunAr
   } else {
     asm volatile("bar.sync 2, %0;" ::"r"(blockDim.x) : "memory");
   }
-  if (!same(s_bad)) run_staged<V, Fused, Global>(A, &Ls, s_block, smem, &mbar, &s_skip);
+  if (!same(s_bad)) run_staged<V, Fused, Global, MINB != 4>(A, &Ls, s_block, smem, &mbar, &s_skip);
   if (!A.bq_head) return;
   __syncthreads();
   if (threadIdx.x == 0) {

@@ -183,6 +183,16 @@ enum : uint32_t {
 #define SR_STGO(i) SR_STGV(i) "bar.warp.sync 0xFFFFFFFF;\n"
 #define SR_DIVV(i) "div.s32 c" #i ", a" #i ", y;\n"
 #define SR_REMV(i) "rem.s32 c" #i ", a" #i ", y;\n"
+#define SR_DIVOK(i) "add.u32 t, b" #i ", 1;\nsetp.le.and.u32 pf, t, 1, s" #i ";\nor.pred pc, pc, pf;\n"
+#define SR_DIVRV(i) "div.s32 c" #i ", a" #i ", b" #i ";\n"
+#define SR_REMRV(i) "rem.s32 c" #i ", a" #i ", b" #i ";\n"
+// 45 DIV, 47 REM by registers that are neither 0 nor -1 in any active thread
+#define SR_NO_DIVR(E, LDB) "bra.uni LEND;\n"
+#define SR_DIVR(E, LDB)                                                                              \
+  "setp.eq.u32 pa, u, 45;\nsetp.eq.or.u32 pf, u, 47, pa;\n@!pf bra.uni LEND;\nprmt.b32 ro, x, 0, 0x4443;\n"   \
+  SR_D_ROW "mad.lo.u32 ro, ro, " Q_STRIDE ", " Q_RS ";\n" LDB "setp.ne.u32 pc, 0, 0;\n" E(SR_DIVOK)    \
+  "vote.sync.any.pred pc, pc, 0xFFFFFFFF;\n@pc bra.uni LEND;\n@!pa bra.uni LREMR;\n" E(SR_DIVRV)      \
+  "bra.uni LDIV1;\nLREMR:\n" E(SR_REMRV) "bra.uni LDIV1;\n"
 #define SR_BITS(i) "@s" #i " or.b32 m, m, a" #i ";\n@s" #i " min.u32 n, n, a" #i ";\n"
 #define SR_KEEP(i) "mov.u32 l" #i ", a" #i ";\n"
 #define SR_REC(i)                                                                                    \
@@ -296,7 +306,7 @@ enum : uint32_t {
 #define SR_REAL(flag, v, at)                                                                         \
   "and.b32 t, fl, " flag ";\nsetp.ne.u32 pf, t, 0;\nld.shared.u32 t, [" Q_GB " + " SR_STR(SR_GROUP_CONST) " + " at "];\n" \
   "setp.lt.and.u32 pf, " v ", t, pf;\nvote.sync.all.pred pf, pf, 0xFFFFFFFF;\n"
-#define SR_SOLO_ASM(V, REGS, LDC, LDB, STC, LDA, E, TUP)                                                            \
+#define SR_SOLO_ASM(V, REGS, LDC, LDB, STC, LDA, E, TUP, DIVR)                                                            \
   asm volatile(                                                                                                     \
       "{\n"                                                                                                         \
       ".reg .pred pa, pb, pc, pd, pe, pf, ps, pw, pp, pm, pz, s0, s1, s2, s3;\n"                                    \
@@ -457,9 +467,11 @@ enum : uint32_t {
       "LBAR2:\nadd.u32 eh, eh, 64;\nsub.u32 k4, k4, 4;\n" SR_FIN                                                    \
       "LBARFULL:\nor.b32 fl, fl, 32768;\nbra.uni LDONE;\n"                                                                \
       /* 46 DIV, 48 REM by an immediate other than 0 and -1 */                                                      \
-      "LDIV:\nsetp.eq.u32 pa, u, 46;\nsetp.eq.or.u32 pf, u, 48, pa;\nadd.u32 t, y, 1;\nsetp.gt.and.u32 pf, t, 1, pf;\n" \
-      "@!pf bra.uni LEND;\n@!pa bra.uni LREM;\n" E(SR_DIVV) "LDIV1:\n" SR_ROW(STC, "LROWD", "LROWD1") SR_FIN         \
+      "LDIV:\nsetp.eq.u32 pa, u, 46;\nsetp.eq.or.u32 pf, u, 48, pa;\n@!pf bra.uni LDIVR;\nadd.u32 t, y, 1;\n"        \
+      "setp.gt.u32 pf, t, 1;\n@!pf bra.uni LEND;\n@!pa bra.uni LREM;\n" E(SR_DIVV) "LDIV1:\n"                      \
+      SR_ROW(STC, "LROWD", "LROWD1") SR_FIN                                                                         \
       "LREM:\n" E(SR_REMV) "bra.uni LDIV1;\n"                                                                       \
+      "LDIVR:\n" DIVR(E, LDB)                                                                                       \
       /* a chain's other factors and addends stand in the slots of its instructions, up to q */                     \
       "LCHAIN:\nsub.u32 t, t, 1;\nshl.b32 u, t, 3;\nsub.u32 u, q, u;\n"                                             \
       "setp.lt.u32 pf, t, 4;\n@pf bra.uni LCHAIN1;\n"                                                               \
@@ -560,25 +572,29 @@ static_assert(F_MULI == 2 && F_MOVR == 3 && F_SUBR == 5 && F_MULR == 6 && F_AND 
 // q, k4, eh (the epoch field of log records), fl (flags), qw and the per-lane counts of global and
 // (fused) shared accesses and of executed instructions are updated.  gb: the block's shared memory;
 // rs, stride: this lane's row 0 and the row stride; fcap: log records that fit.  Returns the slots
-// active at the end, << 4 those that wait at qw.
-template <int V, bool Fused>
+// active at the end, << 4 those that wait at qw.  Div: divisions by registers run here (with V = 4; in 64
+// registers they would cost what does not divide 1%: the reduction of 2^24 values 2,490 us, with them
+// 2,522).
+template <int V, bool Fused, bool Div>
 __device__ __forceinline__ uint32_t solo_loop(uint32_t& q, uint32_t& k4, uint32_t& gacc, uint32_t& sacc, uint32_t& eh,
                                               uint32_t& ni, uint32_t& fl, uint32_t& qw, uint32_t gb, uint32_t w,
                                               uint32_t rs, uint32_t stride, uint32_t am, uint32_t fcap, uint32_t bud) {
   uint32_t mask;
-#define SR_SOLO_4(TUP)                                                                                              \
+#define SR_SOLO_4(TUP, DIVR)                                                                                              \
   SR_SOLO_ASM(4, "c0, c1, c2, c3, b0, b1, b2, b3, a0, a1, a2, a3, l0, l1, l2, l3",                                  \
               "ld.shared.v4.u32 {c0, c1, c2, c3}, [ro];\n", "ld.shared.v4.u32 {b0, b1, b2, b3}, [ro];\n",           \
-              "st.shared.v4.u32 [ro], {c0, c1, c2, c3};\n", "ld.shared.v4.u32 {a0, a1, a2, a3}, [ro];\n", SR_E4, TUP)
+              "st.shared.v4.u32 [ro], {c0, c1, c2, c3};\n", "ld.shared.v4.u32 {a0, a1, a2, a3}, [ro];\n", SR_E4, TUP, DIVR)
 #define SR_SOLO_2(TUP)                                                                                              \
   SR_SOLO_ASM(2, "c0, c1, b0, b1, a0, a1, l0, l1", "ld.shared.v2.u32 {c0, c1}, [ro];\n",                            \
               "ld.shared.v2.u32 {b0, b1}, [ro];\n", "st.shared.v2.u32 [ro], {c0, c1};\n",                           \
-              "ld.shared.v2.u32 {a0, a1}, [ro];\n", SR_E2, TUP)
+              "ld.shared.v2.u32 {a0, a1}, [ro];\n", SR_E2, TUP, SR_DIVR)
 #define SR_SOLO_1(TUP)                                                                                              \
   SR_SOLO_ASM(1, "c0, b0, a0, l0", "ld.shared.u32 c0, [ro];\n", "ld.shared.u32 b0, [ro];\n",                        \
-              "st.shared.u32 [ro], c0;\n", "ld.shared.u32 a0, [ro];\n", SR_E1, TUP)
-  if constexpr (V == 4 && Fused) SR_SOLO_4(SR_TUP);
-  else if constexpr (V == 4) SR_SOLO_4(SR_NO_TUP);
+              "st.shared.u32 [ro], c0;\n", "ld.shared.u32 a0, [ro];\n", SR_E1, TUP, SR_DIVR)
+  if constexpr (V == 4 && Fused && Div) SR_SOLO_4(SR_TUP, SR_DIVR);
+  else if constexpr (V == 4 && Fused) SR_SOLO_4(SR_TUP, SR_NO_DIVR);
+  else if constexpr (V == 4 && Div) SR_SOLO_4(SR_NO_TUP, SR_DIVR);
+  else if constexpr (V == 4) SR_SOLO_4(SR_NO_TUP, SR_NO_DIVR);
   else if constexpr (V == 2 && Fused) SR_SOLO_2(SR_TUP);
   else if constexpr (V == 2) SR_SOLO_2(SR_NO_TUP);
   else if constexpr (Fused) SR_SOLO_1(SR_TUP);

@@ -69,9 +69,9 @@ def test_round_budget_at_every_round(B, bdim, four):
 
 def test_full_log_stays_full(B):
     """A block whose log is full after four barrier intervals goes on for 2^32 more accesses, leaving
-    the inner loop (a division by a register) between any two: its races are those of the first
+    the inner loop (a division by -1) between any two: its races are those of the first
     intervals, and the other program's results are untouched."""
-    a = Asm().s2r(r2, TID).add(r3, r2, 1).and_(r3, r3, 1023).mov(r5, (1 << 18) + 64).mov(r7, 3)
+    a = Asm().s2r(r2, TID).add(r3, r2, 1).and_(r3, r3, 1023).mov(r5, (1 << 18) + 64).mov(r7, -1)
     a.label("top").sts(r2, r5)
     for _ in range(16):
         a.lds(r4, r3).div(r6, r5, r7)
