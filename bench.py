@@ -222,6 +222,11 @@ def run_reference(args):
 
 
 # ----------------------------------------------------------------- GPU
+# What a capture's kernels are compiled from, and the code they run is packed by: a change voids the entry.
+INTERP_SOURCES = ("interp.cu", "solo_loop.cuh", "host_prep.h", "sr_internal.h")
+CHECK_SOURCES = ("check.cu", "sr_internal.h")
+
+
 def src_sha(*names):
     h = hashlib.sha1()
     for n in names:
@@ -233,11 +238,13 @@ def src_sha(*names):
 def traffic_per_launch(workload: str, kernel: str, src: str, units: dict):
     """DRAM bytes per launch of `kernel` on `workload` from the committed ncu capture (taken
     on a smaller case of the same workload and scaled by its unit, blocks or logged records),
-    if one was taken on this source; else None."""
+    if one was taken on this source; else None.  `steps` holds kernels of which a step launches
+    several grids (batched mode: one per bucket), with the sums over a step."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(path):
         return None
-    for t in json.load(open(path)).get("captures", []):
+    data = json.load(open(path))
+    for t in data.get("captures", []) + data.get("steps", []):
         if t["workload"] == workload and t["kernel"] == kernel and t["src_sha1"] == src:
             return (t["dram_read"] + t["dram_write"]) / t["units"] * units[t["unit"]]
     return None
@@ -421,7 +428,7 @@ def run_native(args):
     # (batched mode: one launch of it per bucket of alike blocks, side by side)
     interp_kernel = "k_interp_plain" if mode == "plain" else "k_interp_blocks"
     achieved = step_bytes / (stage["interp"] / 1e3) / 1e9
-    isha, csha = src_sha("interp.cu", "sr_internal.h"), src_sha("check.cu", "sr_internal.h")
+    isha, csha = src_sha(*INTERP_SOURCES), src_sha(*CHECK_SOURCES)
     fused = bool(opts.get("fused_check"))
     units = {"block": nblocks, "record": st.shared_accesses}
     int_peak = 152 * 128 * sm_max * 1e6            # int32 lane-ops/s: 152 SMs x 128 lanes x max clock
