@@ -21,7 +21,7 @@ variant behind the fastest interpreter, then the fused check behind that interpr
 shape, kept only if its whole run beats interpreter plus checker.  Every candidate must
 produce the same reports
 (any difference is a bug, not a tuning outcome).  Choices are cached per workload
-signature (device, mode, program shapes) in a JSON file.
+signature (device, mode, program shapes, the library's sources) in a JSON file.
 """
 from __future__ import annotations
 
@@ -59,9 +59,20 @@ class Tuned:
     cached: bool = False
 
 
+def library_version() -> str:
+    """Digest of the library's sources: what an option's value stands for may change with them."""
+    from . import build
+    h = hashlib.sha256()
+    for path in sorted(build._inputs()):
+        h.update(os.path.basename(path).encode())
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def signature(programs: Sequence[Program], mode: str, device: str, fused: bool = True) -> str:
-    """Digest of what the choice depends on: device, mode and every launch's shape."""
-    h = hashlib.sha256(f"{device}|{mode}|{fused}".encode())
+    """Digest of what the choice depends on: device, mode, the library and every launch's shape."""
+    h = hashlib.sha256(f"{device}|{mode}|{fused}|{library_version()}".encode())
     for p in programs:
         h.update(np.int64(p.ncode).tobytes())
         for l in p.launches:

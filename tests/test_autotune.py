@@ -95,6 +95,21 @@ def test_cache_round_trip_and_signature(tmp_path):
     assert s != autotune.signature(progs[:-1], "batched", "fake")
 
 
+def test_choices_of_another_library_are_not_used(tmp_path, monkeypatch):
+    from paper_1211_6193_gb300 import build
+    progs = [fig1.program()]
+    source = tmp_path / "kernel.cu"
+    source.write_text("first")
+    monkeypatch.setattr(build, "_inputs", lambda: [str(source)])
+    path = str(tmp_path / "tune.json")
+    m, _ = _fake({}, {4: 0.5})
+    assert autotune.tune(progs, "batched", measure=m, cache_path=path, device="fake").options["check_variant"] == 4
+    source.write_text("second")
+    m, _ = _fake({}, {2: 0.5})
+    t = autotune.tune(progs, "batched", measure=m, cache_path=path, device="fake")
+    assert not t.cached and t.options["check_variant"] == 2
+
+
 @pytest.mark.gpu
 def test_tuned_options_on_the_gpu_match_the_oracle():
     import torch
