@@ -1,11 +1,12 @@
 """Limits of a block at their exact edges: the round budget at every round of a kernel (what each
 thread was doing when the rounds ran out, and how many instructions were executed), and an access
-log that has been full for billions of accesses."""
+log that has been full for billions of accesses.  And the kernel form that carries most generated
+batches, blocks of 129 to 512 threads with four simulated warps per warp, on random kernels."""
 import numpy as np
 import pytest
 
 import oracle
-from test_gpu_blocks import B, random_kernel  # noqa: F401 (the fixture)
+from test_gpu_blocks import OPTIONS, B, assert_same, random_kernel, random_program  # noqa: F401 (the fixture)
 from paper_1211_6193_gb300.workloads import rng
 from paper_1211_6193_gb300.workloads.ir import TID, Asm, Launch, Program, r2, r3, r4, r5, r6, r7
 
@@ -86,3 +87,29 @@ def test_full_log_stays_full(B):
     assert mine and {r[4] for r in mine} <= {0, 1, 2, 3}
     want = [(r[0], 1) + r[2:] for r in oracle.run([other]).report_tuples()]
     assert [r for r in reports if r[1] == 1] == want and want
+
+
+@pytest.mark.parametrize("option", [o for o in OPTIONS if OPTIONS[o][0]["mode"] == "batched"])
+@pytest.mark.parametrize("bdim", [129, 160, 255, 257, 384, 511, 512])
+def test_four_simulated_warps_per_warp(B, bdim, option):
+    opts, oracle_kw = OPTIONS[option]
+    assert_same(B, [behind_large_block(random_program(rng.derive(700 + bdim, i), bdim)) for i in range(10)], opts, oracle_kw)
+
+
+@pytest.mark.parametrize("option", ["plain", "global"])
+@pytest.mark.parametrize("bdim", [129, 288, 512])
+def test_four_simulated_warps_per_warp_in_large_grids(B, bdim, option):
+    """Grids too large for the form of two simulated warps per warp (16 warps of it per SM)."""
+    import torch
+    opts, oracle_kw = OPTIONS[option]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    grid, words = 16 * sms // ((bdim + 63) // 64) + 1, bdim + 40
+    n = grid * bdim
+    progs = []
+    for i in range(2):
+        seed = rng.derive(800 + bdim, i)
+        arena = np.zeros(3 * n, dtype=np.int32)
+        arena[:n] = rng.uniform_mod(seed, n, 50)
+        progs.append(Program(random_kernel(seed, bdim, n, words).assemble(), [0], [Launch(0, grid, bdim, words, (0, 0))],
+                             arena, name=f"random_{i}"))
+    assert_same(B, progs, opts, oracle_kw)
