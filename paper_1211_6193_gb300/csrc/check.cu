@@ -1080,7 +1080,9 @@ constexpr uint32_t kDefaultVariant = 4, kSmallVariant = 6;
 // it needs no barrier at an interval's end.  6.3 M records in full intervals of 1536: 32 us (shape
 // 4) against 30 (shape 6), of 768 40 against 26, of 192 110 against 46, of 3072 30 against 36; the
 // reduction of 1501 blocks of 333 threads 47 against 26; generated batches, whose records are mostly
-// in long intervals, 590 against 716.
+// in long intervals, 590 against 716.  What the runtime gives is a bound, every thread taking every access:
+// for the reduction of 2^24 values 2,979, where its intervals hold some 340, so it takes shape 4 (427 us;
+// shape 6: 317).
 constexpr double kSmallInterval = 1536;
 
 const VariantEntry& variant_entry(uint32_t v) {

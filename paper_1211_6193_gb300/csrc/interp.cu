@@ -117,8 +117,7 @@ __device__ __forceinline__ bool stage_wait(unsigned long long* bar, uint32_t pha
   return ok;
 }
 
-// A value that is the same in every lane, through a broadcast: the compiler then knows it to be
-// warp-uniform, and what depends on it needs no handling of divergence.
+// A value that is the same in every lane, through a broadcast, which says so to the compiler.
 __device__ __forceinline__ uint32_t same(uint32_t v) { return __shfl_sync(FULL, v, 0); }
 
 // Shared-memory accesses by 32-bit shared-window address (cheaper address arithmetic than
@@ -136,8 +135,7 @@ __device__ __forceinline__ uint32_t lds_acquire(uint32_t a) {
   asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
   return v;
 }
-// The same under a predicate inside the statement: around a statement that the compiler cannot
-// look into, an `if` becomes a branch with its reconvergence instead of a predicated access.
+// The same under a predicate inside the statement.
 __device__ __forceinline__ uint32_t lds_if(bool p, uint32_t a) {
   uint32_t v;
   asm volatile("{ .reg .pred q; setp.ne.u32 q, %2, 0; mov.u32 %0, 0; @q ld.shared.u32 %0, [%1]; }"
@@ -227,7 +225,7 @@ __device__ __forceinline__ unsigned long long rec_of(uint32_t epoch_hi, uint32_t
 }
 
 // Append one 16-byte global-log record per lane with `me` to the block's global log (the
-// same warp-aggregated reservation as log_access).
+// same warp-aggregated reservation as log_wide).
 __device__ __forceinline__ void log_global(BlockVars* bv, uint4* region, uint32_t cap, bool me, uint4 rec,
                                            uint32_t lane) {
   const uint32_t m = __ballot_sync(FULL, me);
@@ -1576,7 +1574,11 @@ cudaError_t init_interp_attributes(uint32_t smem_optin) {
 // variant: 1 = the larger register budget, 2 = more CTAs per SM (and more spills), 0 = 2 where its CTAs
 // fit and warps wait much: at four barriers or more.  The reduction of 2^24 values (11 barriers)
 // 1,592 us with 1 and 1,500 with 2, 1501 blocks of 333 threads 81 and 58; 64 generated programs (most
-// with one to three) 1,738 and 1,906, the 2048^2 stencil (one) 5,532 and 6,770.
+// with one to three) 1,738 and 1,906, the 2048^2 stencil (one) 5,532 and 6,770.  Intervals of one store
+// and 2 to 12 ALU instructions in full grids, time with 1 over time with 2: blocks of 256 threads 0.92 to
+// 0.94 at one barrier, 0.97 to 1.07 at three, 1.02 to 1.10 at four, 1.09 to 1.12 at eight; of 1024 threads
+// 0.90 to 0.92, 0.94 to 1.00, 0.96 to 1.02, 1.02 to 1.05.  A kernel with a loop counts as without
+// barriers: with 24 turns of two barriers each it would be 1.06 to 1.10 times as fast with 2.
 cudaError_t launch_interp_plain(const RunArgs& a, uint32_t li, const LaunchDev& L, uint32_t variant,
                                 uint32_t smem_per_sm, cudaStream_t s) {
   const uint32_t threads = L.nw * 32u;

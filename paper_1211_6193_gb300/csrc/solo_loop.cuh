@@ -3,9 +3,8 @@
 //
 // In PTX, because what bounds it is latency.  Shared memory and registers hold 20 to 30 warps per
 // SM; a taken branch costs a warp some 24 cycles, an indexed jump 90 and an instruction in
-// straight line 1 (measured), and the compiled form of these steps took two to four times the
-// instructions: a dispatch switch predicated every operation's code into one stream, and each
-// condition that the compiler could not see to be warp-uniform brought its reconvergence.  Here:
+// straight line 1 (timed in loops of them), and the same steps written in C++ executed two to four
+// times the instructions (smsp__inst_executed).  Here:
 //  - MOV, ADD and MUL with an immediate (SUB and SHL become them) are one multiply-add, and a
 //    chain of them, each on the previous one's result, is a loop over its factors and addends
 //    (set_runs lays them out); each group of the other operations is computed in straight line

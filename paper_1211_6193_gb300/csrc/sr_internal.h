@@ -49,7 +49,8 @@ __host__ __device__ constexpr bool pk_imm(uint32_t form) { return form < F_LDS &
 // line the other way round: 1449 of 192 59 -> 74, 1501 of 333 58 -> 102 (blocks above 512 threads
 // would need more than 8 warps).  A block keeps two warps from 64 threads on.
 // With the fused check a block's summaries leave room for few blocks per SM, whose warps are then too
-// few with four: 1178 blocks of 192 in 497 -> 212 us, 3% over 48 drawn cases.
+// few with four: 1178 blocks of 192 in 497 -> 212 us, 3% over 48 random workloads.  The line is drawn for
+// one launch by itself, also where launches of other programs run beside it.
 __host__ __device__ constexpr uint32_t block_warps(uint32_t bdim, uint32_t vec) { return (bdim + 32u * vec - 1u) / (32u * vec); }
 __host__ __device__ constexpr uint32_t block_vec(uint32_t bdim, uint64_t blocks, uint32_t sms, bool fused) {
   return bdim <= 64 ? 1u
