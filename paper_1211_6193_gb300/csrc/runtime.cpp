@@ -276,57 +276,70 @@ struct OutsideCaptures {
 };
 
 bool idle(const SideStreams& t) {
-  for (cudaStream_t q : t.side)
-    if (q && cudaStreamQuery(q) != cudaSuccess) {
+  for (cudaStream_t q : t.side) {
+    if (!q) continue;
+    cudaStreamCaptureStatus status;              // (a query would end the capture that a stream is part of)
+    if (cudaStreamIsCapturing(q, &status) != cudaSuccess || status != cudaStreamCaptureStatusNone ||
+        cudaStreamQuery(q) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
+  }
   return true;
 }
 
-// Gives the batch the side streams of stream s (which is not being captured): its set, or one that no
-// batch uses and whose work is done, or a new one.  Streams are made when a batch first needs them: each
+// The context's set for `owner` at a priority: its own, or one that no batch uses and whose work is done,
+// or a new one, with streams for so many lanes.  Streams are made when a batch first needs them: each
 // takes some 10 us, which a context for small batches need not spend.
-cudaError_t take_side_streams(sr_ctx* c, sr_batch* b, cudaStream_t s) {
-  if (b->lanes < 2) return cudaSuccess;
-  const OutsideCaptures outside;
-  unsigned long long id = 0;
-  cudaError_t e = cudaStreamGetId(s, &id);
-  if (e != cudaSuccess) return e;
-  if (!b->sides || b->sides->owner != id) {
-    int priority = 0;
-    e = cudaStreamGetPriority(s, &priority);
-    if (e != cudaSuccess) return e;
-    drop_side_streams(b);
-    SideStreams* set = nullptr;
-    for (auto& t : c->sides)
-      if (t->owner == id) set = t.get();
-    for (size_t i = 0; !set && i < c->sides.size(); ++i)
-      if (!c->sides[i]->batches && c->sides[i]->priority == priority && idle(*c->sides[i])) set = c->sides[i].get();
-    if (!set) {
-      try {
-        c->sides.push_back(std::make_unique<SideStreams>());
-      } catch (const std::bad_alloc&) {
-        return cudaErrorMemoryAllocation;
-      }
-      set = c->sides.back().get();
-      set->priority = priority;
+cudaError_t find_side_streams(sr_ctx* c, unsigned long long owner, int priority, uint32_t lanes, SideStreams** out) {
+  SideStreams* set = nullptr;
+  for (auto& t : c->sides)
+    if (t->owner == owner && t->priority == priority) set = t.get();
+  for (size_t i = 0; !set && i < c->sides.size(); ++i)
+    if (!c->sides[i]->batches && c->sides[i]->priority == priority && idle(*c->sides[i])) set = c->sides[i].get();
+  if (!set) {
+    try {
+      c->sides.push_back(std::make_unique<SideStreams>());
+    } catch (const std::bad_alloc&) {
+      return cudaErrorMemoryAllocation;
     }
-    set->owner = id;
-    ++set->batches;
-    b->sides = set;
+    set = c->sides.back().get();
+    set->priority = priority;
   }
-  SideStreams& t = *b->sides;
-  if (!t.fork) e = cudaEventCreateWithFlags(&t.fork, cudaEventDisableTiming);
-  for (uint32_t i = 0; i + 1 < b->lanes && e == cudaSuccess; ++i) {
-    if (!t.side[i]) e = cudaStreamCreateWithPriority(&t.side[i], cudaStreamNonBlocking, t.priority);
-    if (e == cudaSuccess && !t.join[i]) e = cudaEventCreateWithFlags(&t.join[i], cudaEventDisableTiming);
+  set->owner = owner;
+  cudaError_t e = set->fork ? cudaSuccess : cudaEventCreateWithFlags(&set->fork, cudaEventDisableTiming);
+  for (uint32_t i = 0; i + 1 < lanes && e == cudaSuccess; ++i) {
+    if (!set->side[i]) e = cudaStreamCreateWithPriority(&set->side[i], cudaStreamNonBlocking, priority);
+    if (e == cudaSuccess && !set->join[i]) e = cudaEventCreateWithFlags(&set->join[i], cudaEventDisableTiming);
   }
-  if (e != cudaSuccess) drop_side_streams(b);
+  *out = set;
   return e;
 }
 
-int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
+// The side streams of a run on stream s.  Being captured, these stay part of the capture until it ends,
+// so a capture has a set of its own (capture ids are no stream's; a set that has left its capture is idle).
+cudaError_t side_streams(sr_ctx* c, sr_batch* b, cudaStream_t s, bool* captured, SideStreams** out) {
+  const OutsideCaptures outside;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  int priority = 0;
+  cudaError_t e = cudaStreamGetPriority(s, &priority);
+  if (e == cudaSuccess) e = cudaStreamGetCaptureInfo(s, &status, &id);
+  if (e != cudaSuccess) return e;
+  *captured = status != cudaStreamCaptureStatusNone;
+  if (*captured) return find_side_streams(c, id | 1ull << 63, priority, b->lanes, out);
+  e = cudaStreamGetId(s, &id);
+  if (e != cudaSuccess) return e;
+  if (!b->sides || b->sides->owner != id) drop_side_streams(b);
+  e = find_side_streams(c, id, priority, b->lanes, out);
+  if (e == cudaSuccess && !b->sides) {
+    b->sides = *out;
+    ++b->sides->batches;
+  }
+  return e;
+}
+
+int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, SideStreams* sides, bool profile) {
   const sr_opts& o = c->opts;
   b->nevents_used = 0;
   b->kernels = 0;
@@ -387,10 +400,10 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
     const bool batched = o.mode == SR_MODE_BATCHED;
     const uint32_t lanes = lanes_of(b, w, batched);
     if (lanes > 1) {
-      CUDA_TRY(c, cudaEventRecord(b->sides->fork, s));
-      for (uint32_t i = 0; i + 1 < lanes; ++i) CUDA_TRY(c, cudaStreamWaitEvent(b->sides->side[i], b->sides->fork, 0));
+      CUDA_TRY(c, cudaEventRecord(sides->fork, s));
+      for (uint32_t i = 0; i + 1 < lanes; ++i) CUDA_TRY(c, cudaStreamWaitEvent(sides->side[i], sides->fork, 0));
     }
-    auto lane = [&](uint32_t i) { return i % lanes ? b->sides->side[i % lanes - 1] : s; };
+    auto lane = [&](uint32_t i) { return i % lanes ? sides->side[i % lanes - 1] : s; };
     cudaError_t e = cudaSuccess;
     if (batched) {
       for (uint32_t bk = w.bk0; bk < w.bk1 && e == cudaSuccess; ++bk) {
@@ -412,8 +425,8 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, bool profile) {
       b->kernels += w.li1 - w.li0;
     }
     for (uint32_t i = 0; i + 1 < lanes; ++i) {   // (also after an error: nothing stays unjoined)
-      cudaError_t j = cudaEventRecord(b->sides->join[i], b->sides->side[i]);
-      if (j == cudaSuccess) j = cudaStreamWaitEvent(s, b->sides->join[i], 0);
+      cudaError_t j = cudaEventRecord(sides->join[i], sides->side[i]);
+      if (j == cudaSuccess) j = cudaStreamWaitEvent(s, sides->join[i], 0);
       if (e == cudaSuccess) e = j;
     }
     if (e != cudaSuccess) return fail(c, SR_E_CUDA, "interpreter launch: %s", cudaGetErrorString(e));
@@ -863,7 +876,9 @@ int load_programs(sr_ctx* c, const sr_program* progs, uint32_t n, void* stream, 
     return bytes ? cudaMemcpyAsync(d.p, src, bytes, cudaMemcpyHostToDevice, s) : cudaSuccess;
   };
   for (const Wave& w : b->waves) b->lanes = std::max(b->lanes, lanes_of(b, w, batched));
-  cudaError_t e = take_side_streams(c, b, s);
+  bool captured = false;
+  SideStreams* sides = nullptr;                // (made here: the first run need not)
+  cudaError_t e = b->lanes > 1 ? side_streams(c, b, s, &captured, &sides) : cudaSuccess;
   if (e == cudaSuccess) e = up(b->code, code.data(), code.size() * 8);
   if (e == cudaSuccess) e = up(b->launches_d, b->launches.data(), nl * sizeof(LaunchDev));
   if (e == cudaSuccess) e = up(b->item_launch_d, b->item_launch.data(), b->item_launch.size() * 4);
@@ -906,25 +921,22 @@ int run_and_check(sr_ctx* c, sr_batch* b, void* stream) {
   // branches come to the queues when it starts (work of 193 ms pending on one stream, 16 programs on it and
   // 16 on another: the other's run took the 193 ms, and takes 0.2).  Otherwise not:
   // capturing takes 50 to 100 us, which the first run of a batch on an idle stream need not spend.
-  bool pending = false;
+  bool pending = false, captured = false;
+  SideStreams* sides = nullptr;
   if (b->lanes > 1) {
+    CUDA_TRY(c, side_streams(c, b, s, &captured, &sides));
     const OutsideCaptures outside;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CUDA_TRY(c, cudaStreamIsCapturing(s, &cap));
-    if (cap == cudaStreamCaptureStatusNone) {    // (else the side streams only shape the caller's graph)
-      CUDA_TRY(c, take_side_streams(c, b, s));
-      pending = cudaStreamQuery(s) == cudaErrorNotReady;
-    }
-    if (!b->sides) return fail(c, SR_E_CUDA, "no side streams");   // (an earlier call could not make them)
+    pending = !captured && cudaStreamQuery(s) == cudaErrorNotReady;
   }
   if (((c->opts.use_graph && c->opts.mode == SR_MODE_BATCHED) || pending) && !profile) {
     if (!b->graph || b->graph_stream != s) {
+      const OutsideCaptures outside;
       if (b->graph) cudaGraphExecDestroy(b->graph);
       b->graph = nullptr;
       cudaStream_t cap;
       CUDA_TRY(c, cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
       CUDA_TRY(c, cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
-      int rc = enqueue_run(c, b, cap, false);
+      int rc = enqueue_run(c, b, cap, sides, false);
       cudaGraph_t g = nullptr;
       cudaError_t e = cudaStreamEndCapture(cap, &g);
       cudaStreamDestroy(cap);
@@ -938,7 +950,7 @@ int run_and_check(sr_ctx* c, sr_batch* b, void* stream) {
     CUDA_TRY(c, cudaGraphLaunch(b->graph, s));
     return SR_OK;
   }
-  return enqueue_run(c, b, s, profile);
+  return enqueue_run(c, b, s, sides, profile);
 }
 
 int fetch_reports(sr_ctx* c, sr_batch* b, sr_report* dst, uint64_t cap, uint64_t* n_total) {

@@ -70,3 +70,39 @@ def test_a_batch_runs_on_other_streams_than_it_was_loaded_on(B, mode, options):
                     g.replay()
                     torch.cuda.synchronize()
                     same(a)
+
+
+@pytest.mark.parametrize("mode", ["plain", "batched"])
+def test_runs_beside_a_callers_capture(B, mode):
+    """While a caller's stream is captured, with one batch's run or two on it, other batches run on the
+    streams that all were loaded on, behind pending work and not; the graph is replayed afterwards."""
+    import torch
+    progs = [random_program(rng.derive(47, i), bdim) for i, bdim in enumerate([33, 96, 257, 640])]
+    want = oracle.run(progs)
+
+    def same(batch):
+        assert [tuple(int(x) for x in r) for r in batch.fetch_reports()] == want.report_tuples()
+        for i, arena in enumerate(batch.fetch_all_memory()):
+            assert np.array_equal(arena, want.arenas[i]), i
+
+    s0, s1, s = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.Stream()
+    with B.Context(mode=mode) as ctx, ctx.load_programs(progs, s0) as a, ctx.load_programs(progs, s0) as b, \
+            ctx.load_programs(progs, s1) as c:
+        for batch, q in ((a, s0), (b, s0), (c, s1)):
+            batch.run_and_check(q)
+            same(batch)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            a.run_and_check(s)
+            c.run_and_check(s1)
+            c.run_and_check(s1)                      # (behind the first)
+            b.run_and_check(s)
+            c.run_and_check(s0)
+        same(c)
+        for _ in range(2):
+            g.replay()
+            torch.cuda.synchronize()
+            same(a)
+            same(b)
+        a.run_and_check(s0)
+        same(a)
