@@ -13,29 +13,36 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("reverse", [False, True])
 def test_a_run_does_not_wait_for_another_stream(B, mode, reverse):
     """While a kernel of a second or so holds the first stream, a run enqueued behind it must not hold
-    up a run on the second: that one is done while the first stream is still held."""
+    up a run on the second: that one is done while the first stream is still held.  (Any two streams may
+    share one of the few hardware queues by chance: the best of three pairs of streams counts.)"""
     import torch
     progs = [random_program(rng.derive(41, i), bdim) for i, bdim in enumerate([33, 64, 96, 128, 257, 512, 640, 1024] * 2)]
     want = oracle.run(progs)
-    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
-    if reverse:
-        s1, s2 = s2, s1
-    with B.Context(mode=mode) as ctx, ctx.load_programs(progs, s1) as a, ctx.load_programs(progs, s2) as b:
-        for batch, s in ((a, s1), (b, s2)):          # (kernels are loaded at their first launch)
-            batch.run_and_check(s)
-            batch.fetch_reports()
-        held = torch.cuda.Event()
-        with torch.cuda.stream(s1):
-            torch.cuda._sleep(2_000_000_000)
-        held.record(s1)
-        a.run_and_check(s1)
-        b.run_and_check(s2)
-        s2.synchronize()
-        assert not held.query()
-        for batch in (b, a):
-            assert [tuple(int(x) for x in r) for r in batch.fetch_reports()] == want.report_tuples()
-            for i, arena in enumerate(batch.fetch_all_memory()):
-                assert np.array_equal(arena, want.arenas[i]), i
+
+    def done_meanwhile(s1, s2):
+        with B.Context(mode=mode) as ctx, ctx.load_programs(progs, s1) as a, ctx.load_programs(progs, s2) as b:
+            for batch, s in ((a, s1), (b, s2)):          # (kernels are loaded at their first launch)
+                batch.run_and_check(s)
+                batch.fetch_reports()
+            held = torch.cuda.Event()
+            with torch.cuda.stream(s1):
+                torch.cuda._sleep(2_000_000_000)
+            held.record(s1)
+            a.run_and_check(s1)
+            b.run_and_check(s2)
+            s2.synchronize()
+            meanwhile = not held.query()
+            for batch in (b, a):
+                assert [tuple(int(x) for x in r) for r in batch.fetch_reports()] == want.report_tuples()
+                for i, arena in enumerate(batch.fetch_all_memory()):
+                    assert np.array_equal(arena, want.arenas[i]), i
+        return meanwhile
+
+    for _ in range(3):
+        pair = torch.cuda.Stream(), torch.cuda.Stream()
+        if done_meanwhile(*(reversed(pair) if reverse else pair)):
+            return
+    assert False, "every run on the second stream waited for the first"
 
 
 @pytest.mark.parametrize("mode, options", [("plain", {}), ("plain", {"check_global": True}), ("batched", {}),
@@ -87,8 +94,8 @@ def test_runs_beside_a_callers_capture(B, mode):
 
     s0, s1, s = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.Stream()
     with B.Context(mode=mode) as ctx, ctx.load_programs(progs, s0) as a, ctx.load_programs(progs, s0) as b, \
-            ctx.load_programs(progs, s1) as c:
-        for batch, q in ((a, s0), (b, s0), (c, s1)):
+            ctx.load_programs(progs, s1) as c, ctx.load_programs(progs, s0) as d:
+        for batch, q in ((a, s0), (b, s0), (c, s1), (d, s0)):
             batch.run_and_check(q)
             same(batch)
         g = torch.cuda.CUDAGraph()
@@ -97,8 +104,9 @@ def test_runs_beside_a_callers_capture(B, mode):
             c.run_and_check(s1)
             c.run_and_check(s1)                      # (behind the first)
             b.run_and_check(s)
-            c.run_and_check(s0)
+            d.run_and_check(s0)
         same(c)
+        same(d)
         for _ in range(2):
             g.replay()
             torch.cuda.synchronize()
