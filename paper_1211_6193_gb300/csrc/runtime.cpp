@@ -256,6 +256,12 @@ sr::GcheckArgs gcheck_args(sr_ctx* c, sr_batch* b, uint32_t wi) {
   return g;
 }
 
+// Lane of the i-th bucket (they come by falling work): the largest shares its lane with the smallest.
+uint32_t to_and_fro(uint32_t i, uint32_t lanes) {
+  i %= 2u * lanes;
+  return i < lanes ? i : 2u * lanes - 1u - i;
+}
+
 // Streams a wave's interpreter kernels use.
 uint32_t lanes_of(const sr_batch* b, const Wave& w, bool batched) {
   const uint32_t n = batched ? w.bk1 - w.bk0 : b->launches[w.li1 - 1].prog - b->launches[w.li0].prog + 1u;
@@ -414,7 +420,7 @@ int enqueue_run(sr_ctx* c, sr_batch* b, cudaStream_t s, SideStreams* sides, bool
         ra.bq_head = B.ordered ? (uint32_t*)b->bq_head.p + bk : nullptr;
         e = sr::launch_interp_blocks(ra, B.vec, B.variant, B.warps, B.blocks, B.smem,
                                      o.fused_check && o.check_races && !o.check_global, o.check_global != 0,
-                                     lane(bk - w.bk0));
+                                     lane(to_and_fro(bk - w.bk0, lanes)));
         b->kernels += 1;
       }
     } else {
